@@ -207,7 +207,9 @@ void gsm_query_destroy(gsm_query *q);
  * Errors: GSM_ERR_INVALID_ARG (u out of range, lo > hi, negative bound). */
 gsm_status gsm_query_restrict(gsm_query *q, int32_t u, int32_t lo, int32_t hi);
 
-/* Counts the embeddings of q in the loaded graph.
+/* Counts the embeddings of q in the loaded graph.  Query vertices of degree 1
+ * are counted in closed form where that is possible, so a count may exceed
+ * 64 bits (GSM_ERR_OVERFLOW).
  * Errors: GSM_ERR_NO_GRAPH, GSM_ERR_BUDGET, GSM_ERR_OOM, GSM_ERR_OVERFLOW,
  * GSM_ERR_CUDA. */
 gsm_status gsm_count(gsm_ctx *ctx, const gsm_query *q, uint64_t *count);
@@ -484,8 +486,9 @@ typedef struct gsm_run_stats {
   int32_t k;
   int32_t order[16];
   uint64_t cand_size[16];    /* |C(u)| per query vertex id */
-  uint64_t frontier[16];     /* rows at level i (i = 1..k; [0] unused) */
-  uint64_t candidates[16];   /* candidates checked while extending level i -> i+1 */
+  uint64_t frontier[16];     /* partial embeddings of i vertices (i = 1..k; [0] unused) */
+  uint64_t candidates[16];   /* candidates checked while extending level i -> i+1 (0 for
+                                levels counted in closed form) */
   uint64_t chunks;           /* extend sub-chunks launched */
   uint64_t peak_bytes;       /* high-water mark of budgeted device memory */
   uint64_t kernel_launches;  /* kernels launched by the call */

@@ -64,6 +64,8 @@ struct Block {
 
 }  // namespace
 
+constexpr size_t kSmallBytes = 512;  // gsm_ctx::d_small
+
 struct gsm_query {
   int32_t k = 0, m = 0;
   std::vector<int32_t> edges;
@@ -106,7 +108,7 @@ struct gsm_ctx {
   size_t bitmaps2_cap = 0;
   void *mfilter = nullptr;  // gsm_enumerate_many: descriptors, sizes and bitmaps of all queries
   size_t mfilter_cap = 0;
-  unsigned long long *d_small = nullptr;  // [0..15] sizes, [16] total, [17] err
+  unsigned long long *d_small = nullptr;  // [0..15] sizes, [16..34] a count (kCountWords), [17] err
   void *acc[2] = {nullptr, nullptr};
   size_t acc_cap[2] = {0, 0};
   // gsm_enumerate_many: the result buffers (acc, sort_keys) come in several
@@ -700,8 +702,10 @@ struct Run {
   size_t acc_row_bytes() const {
     return acc_mode == kSinkKeys ? (size_t)key_nw * sizeof(uint64_t) : (size_t)k * sizeof(int32_t);
   }
-  unsigned __int128 count = 0;
   unsigned long long *d_total;
+  // counts: the query's leaves that are not extended but counted in closed
+  // form per embedding of the others; k is then the number of the others
+  LeafDesc leaf{};
   // the last level's keys carry the dense rank of the prefix (query vertices
   // 0..rank_p-1, placed first in that order) when rank_p > 0: ranks of the
   // rows of the last level's input piece in `rank`, running state in prefix
@@ -790,7 +794,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   if (count_only) {
     timed(ctx, K_COUNT, read_bytes, (uint64_t)W, 1, [&] {
       launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nullptr,
-                          nullptr, R.d_total, ctx->stream);
+                          nullptr, R.d_total, ctx->stream, R.leaf.nleaves ? &R.leaf : nullptr);
     });
     return;
   }
@@ -1186,6 +1190,76 @@ bool dense_labels(gsm_ctx *ctx, const gsm_query *q, int32_t *dense) {
   return true;
 }
 
+// Splits off the leaves that a count need not extend (LeafDesc): moves them to
+// the end of the order (positions and parents of the others keep their
+// sequence) and returns the number of the others.  A leaf is a query vertex
+// with one query edge that is not placed first.  An unrestricted one never
+// removes a partial embedding other than by injectivity, so it can wait until
+// the end; a restricted one prunes and stays where the plan put it, unless
+// that is the end.  Leaves of one parent, label and restriction form a group;
+// of several groups with one label (their images could coincide) the largest
+// is split off.
+int32_t split_leaves(const gsm_ctx *ctx, const gsm_query *q, const int32_t *dense,
+                     int32_t *order, LeafDesc *leaf) {
+  struct Group {
+    int32_t parent, lab, lo, hi;
+    uint32_t mask;  // query vertices
+    int32_t last;   // position of the last of them
+  };
+  const int32_t k = q->k;
+  std::vector<Group> groups;
+  for (int32_t i = 1; i < k; ++i) {
+    const int32_t u = order[i];
+    if (popc(q->adj[u]) != 1) continue;
+    const int32_t lo = std::max<int32_t>(0, q->lo[u]), hi = std::min<int32_t>(ctx->n, q->hi[u]);
+    if ((lo > 0 || hi < ctx->n) && i != k - 1) continue;
+    const int32_t p = __builtin_ctz(q->adj[u]);
+    size_t t = 0;
+    while (t < groups.size() && !(groups[t].parent == p && groups[t].lab == dense[u] &&
+                                  groups[t].lo == lo && groups[t].hi == hi))
+      ++t;
+    if (t == groups.size()) groups.push_back(Group{p, dense[u], lo, hi, 0u, 0});
+    groups[t].mask |= 1u << u;
+    groups[t].last = i;
+  }
+  // one group per label: the largest, then the one placed later
+  std::vector<Group> take;
+  for (const Group &x : groups) {
+    bool best = true;
+    for (const Group &y : groups)
+      if (y.lab == x.lab && (popc(y.mask) > popc(x.mask) ||
+                             (popc(y.mask) == popc(x.mask) && y.last > x.last)))
+        best = false;
+    if (best) take.push_back(x);
+  }
+  uint32_t gone = 0;
+  for (const Group &x : take) gone |= x.mask;
+  int32_t kc = 0, next[kMaxK], nl = 0;
+  for (size_t t = 0; t < take.size(); ++t)
+    for (int32_t i = 0; i < k; ++i)
+      if (take[t].mask >> order[i] & 1u) {
+        leaf->of[nl] = (int32_t)t;
+        next[nl++] = order[i];
+      }
+  for (int32_t i = 0; i < k; ++i)
+    if (!(gone >> order[i] & 1u)) order[kc++] = order[i];
+  for (int32_t j = 0; j < nl; ++j) order[kc + j] = next[j];
+  leaf->nleaves = nl;
+  for (size_t t = 0; t < take.size(); ++t) {
+    const Group &x = take[t];
+    LeafGroup &gr = leaf->grp[t];
+    gr = LeafGroup{0, x.lab, x.lo, x.hi, 0u, 0u};
+    for (int32_t j = 0; j < kc; ++j) {
+      const int32_t u = order[j];
+      if (u == x.parent)
+        gr.pos = j;
+      else if (dense[u] == x.lab)
+        (q->adj[x.parent] >> u & 1u ? gr.in_mask : gr.chk_mask) |= 1u << j;
+    }
+  }
+  return kc;
+}
+
 // Filtering step: fills the k candidate bitmaps and returns |C(u)|; then
 // opt.filter_rounds refinement rounds (double-buffered, so every round reads
 // the previous round's sets only).
@@ -1285,6 +1359,19 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   for (int32_t u = 0; u < q->k; ++u)
     if (sizes[u] == 0) return;
   plan(q->k, q->adj, sizes, R.order, R.parent);
+  // counts multiply leaves out instead of checking every image (LeafDesc).
+  // Compressed frontiers keep their own last level, and `less` its
+  // constraints on leaves.
+  // With look-ahead the leaves come last too, but are extended; fault
+  // injection keeps every level, so that its wait is reached.
+  if (!enumerate && !less &&
+      !(ctx->opt.flags & (GSM_OPT_COMPRESSED_FRONTIERS | GSM_OPT_INJECT_SCAN_STALL))) {
+    R.k = split_leaves(ctx, q, dense, R.order, &R.leaf);
+    if (ctx->opt.lookahead > 0) {
+      R.k = q->k;
+      R.leaf.nleaves = 0;
+    }
+  }
   for (int32_t i = 0; i < q->k; ++i) ctx->run.order[i] = R.order[i];
   // The levels emit rows in lexicographic order of the matching order.  If
   // query vertices sort_cols .. k-1 are placed in increasing id order, rows
@@ -1322,7 +1409,7 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
 
   const int32_t nw = (ctx->n + 31) / 32;
   const uint32_t *bm = pre ? pre->bitmaps : (const uint32_t *)ctx->bitmaps;
-  for (int32_t i = 1; i < q->k; ++i) {
+  for (int32_t i = 1; i < R.k; ++i) {
     LevelDesc &d = R.lv[i];
     std::memset(&d, 0, sizeof(d));
     const int32_t u = R.order[i];
@@ -1377,7 +1464,7 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     }
   }
 
-  CU(cudaMemsetAsync(R.d_total, 0, sizeof(unsigned long long), ctx->stream));
+  CU(cudaMemsetAsync(R.d_total, 0, sizeof(unsigned long long) * kCountWords, ctx->stream));
   const Mark mk = stack_mark(ctx);
   const int64_t R1 = (int64_t)sizes[R.order[0]];
   int32_t *F1 = (int32_t *)stack_push(ctx, sizeof(int32_t) * R1);
@@ -1391,9 +1478,12 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
                             (int64_t *)(sc + o_off), (int64_t *)(sc + o_tmp), F1, ctx->stream);
     });
   }
-  ctx->run.frontier[1] = (uint64_t)R1;
+  if (R.k == 1) ctx->run.frontier[1] = (uint64_t)R1;  // (recurse counts the rows of every level)
   R.acc_ld = (int64_t)(ctx->acc_cap[0] / R.acc_row_bytes());
-  if (q->k == 1) {
+  if (R.k == 1 && R.leaf.nleaves) {
+    timed(ctx, K_COUNT, 12.0 * R1, (uint64_t)R1, 1,
+          [&] { launch_leaf_rows(R.g, R.leaf, F1, R1, R1, R.d_total, ctx->stream); });
+  } else if (q->k == 1) {
     if (enumerate) {
       ensure_acc(R, (uint64_t)R1);
       CU(cudaMemcpyAsync(ctx->acc[0], F1, sizeof(int32_t) * R1, cudaMemcpyDeviceToDevice,
@@ -1413,8 +1503,14 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   if (enumerate || q->k == 1) {
     total = R.acc_rows;
   } else {
-    fetch(ctx, R.d_total, sizeof(uint64_t));
-    total = (uint64_t)ctx->h_stage[0];
+    fetch(ctx, R.d_total, sizeof(uint64_t) * kCountWords);
+    uint64_t w[kCountWords];
+    std::memcpy(w, ctx->h_stage, sizeof(w));
+    // (without leaves word 0 is the count itself)
+    const unsigned __int128 sum = (unsigned __int128)w[0] + ((unsigned __int128)w[1] << 32);
+    if (w[2] || sum >> 64) FAIL(GSM_ERR_OVERFLOW, "more than 2^64 - 1 embeddings");
+    total = (uint64_t)sum;
+    for (int32_t l = 0; l < R.leaf.nleaves; ++l) ctx->run.frontier[R.k + l] = w[3 + l];
   }
   ctx->run.frontier[q->k] = total;
   *count_out = total;
@@ -2591,7 +2687,7 @@ gsm_status gsm_create(gsm_ctx **out, int32_t device, const gsm_options *opt) {
     ctx->d_flags = (uint32_t *)((char *)ctx->d_stage + 4096);
     std::memset(ctx->h_flags, 0, 64);
     CU(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device));
-    ctx->d_small = (unsigned long long *)dev_alloc(ctx, 256);
+    ctx->d_small = (unsigned long long *)dev_alloc(ctx, kSmallBytes);
   });
   if (st != GSM_OK) {
     gsm_destroy(ctx);
@@ -2626,7 +2722,7 @@ void gsm_destroy(gsm_ctx *ctx) {
       dev_free(ctx, p.acc[1], p.acc_cap[1]);
       dev_free(ctx, p.sort_keys, p.sort_keys_cap);
     }
-    dev_free(ctx, ctx->d_small, 256);
+    dev_free(ctx, ctx->d_small, kSmallBytes);
   } catch (...) {
   }
   for (auto e : ctx->event_pool) cudaEventDestroy(e);

@@ -500,16 +500,18 @@ __global__ void k_tile_rows(const int64_t *__restrict__ woff, int64_t ra, int64_
 // consecutive, so its candidate loads cover contiguous bytes.  The survivor
 // bits stay in candidate order: each lane's 4-bit group is shifted into place
 // and OR-ed across the 8 lanes that share a 32-bit mask word.
-template <bool kMasks>
+// kLeaves > 0: a survivor adds its leaf number (LeafSums) instead of one.
+template <bool kMasks, int kLeaves>
 __global__ void __launch_bounds__(1024) k_extend_count(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
     int32_t W, uint32_t *__restrict__ masks, int32_t *__restrict__ tile_cnt,
-    unsigned long long *__restrict__ total) {
+    unsigned long long *__restrict__ total, const __grid_constant__ LeafDesc leaf) {
   static_assert(kItemsPerThread == 4, "one 4-bit group per lane");
   extern __shared__ int32_t s_woff[];
   __shared__ int32_t s_count;
+  LeafSums<kLeaves ? kLeaves : 1> sums;
   const int32_t B = blockDim.x;
   const int32_t tile_items = B * kItemsPerThread;
   const int32_t x0 = blockIdx.x * tile_items;
@@ -539,9 +541,19 @@ __global__ void __launch_bounds__(1024) k_extend_count(
       }
       const int32_t w = __ldg(g.lcol + pst + (x - rs));
       if (check_candidate(g, d, ColumnRow{F, ld, r}, w, slot) &&
-          (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w)))
-        bits |= 1u << j;
+          (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w))) {
+        if constexpr (kLeaves > 0) {
+          const ColumnRow row{F, ld, r};
+          sums.add(g, leaf, ExtendedRow<ColumnRow>{row, d.i, w});
+        } else {
+          bits |= 1u << j;
+        }
+      }
     }
+  }
+  if constexpr (kLeaves > 0) {
+    sums.flush(leaf, total);
+    return;
   }
   uint32_t word = bits << (4 * (lane & 7));
   word |= __shfl_xor_sync(kFull, word, 1);
@@ -559,6 +571,21 @@ __global__ void __launch_bounds__(1024) k_extend_count(
     if (tile_cnt) tile_cnt[blockIdx.x] = s_count;
     if (total && s_count) atomicAdd(total, (unsigned long long)s_count);
   }
+}
+
+// Leaf numbers of the rows of a core frontier (a core of one vertex: its
+// candidate list).
+template <int kLeaves>
+__global__ void __launch_bounds__(256) k_leaf_rows(GraphDev g,
+                                                   const __grid_constant__ LeafDesc leaf,
+                                                   const int32_t *__restrict__ F, int32_t ld,
+                                                   int32_t rows,
+                                                   unsigned long long *__restrict__ total) {
+  LeafSums<kLeaves> sums;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += stride)
+    sums.add(g, leaf, ColumnRow{F, ld, (int32_t)r});
+  sums.flush(leaf, total);
 }
 
 // Position (0..31) of the n-th (0-based) set bit of m; m has more than n.
@@ -1138,18 +1165,38 @@ void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
                          uint32_t *masks, int32_t *tile_cnt, unsigned long long *total,
-                         cudaStream_t s) {
+                         cudaStream_t s, const LeafDesc *leaf) {
   const int64_t tiles = extend_tiles(wa, wb, block);
   if (tiles <= 0) return;
   const size_t smem = (size_t)((int64_t)block * kItemsPerThread + 1) * sizeof(int32_t);
-  if (masks)
-    k_extend_count<true><<<(unsigned)tiles, block, smem, s>>>(
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)tiles, block, smem, s>>>(
         g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, (int32_t)(wb - wa), masks,
-        tile_cnt, total);
+        tile_cnt, total, leaf ? *leaf : LeafDesc{});
+  };
+  if (!leaf)
+    masks ? go(k_extend_count<true, 0>) : go(k_extend_count<false, 0>);
+  else if (leaf->nleaves == 1)
+    go(k_extend_count<false, 1>);
+  else if (leaf->nleaves <= 3)
+    go(k_extend_count<false, 3>);
   else
-    k_extend_count<false><<<(unsigned)tiles, block, smem, s>>>(
-        g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, (int32_t)(wb - wa), masks,
-        tile_cnt, total);
+    go(k_extend_count<false, kMaxK>);
+}
+
+void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,
+                      int64_t rows, unsigned long long *total, cudaStream_t s) {
+  if (rows <= 0) return;
+  auto go = [&](auto kernel) {
+    kernel<<<grid_for(rows, 256, 152 * 8), 256, 0, s>>>(g, leaf, F, (int32_t)ld, (int32_t)rows,
+                                                        total);
+  };
+  if (leaf.nleaves == 1)
+    go(k_leaf_rows<1>);
+  else if (leaf.nleaves <= 3)
+    go(k_leaf_rows<3>);
+  else
+    go(k_leaf_rows<kMaxK>);
 }
 
 void launch_extend_write(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,

@@ -43,6 +43,32 @@ __device__ __forceinline__ int2 label_segment(const GraphDev &g, int32_t x, int3
   return make_int2(lo, hi);
 }
 
+// The part of an id-sorted segment of lcol with ids in [lo, hi).
+__device__ __forceinline__ int2 cut_segment(const GraphDev &g, int2 seg, int32_t lo, int32_t hi) {
+  int32_t a = seg.x, len = seg.y - seg.x;
+  while (len > 0) {
+    const int32_t half = len >> 1;
+    if (__ldg(g.lcol + a + half) < lo) {
+      a += half + 1;
+      len -= half + 1;
+    } else {
+      len = half;
+    }
+  }
+  int32_t b = a;
+  len = seg.y - a;
+  while (len > 0) {
+    const int32_t half = len >> 1;
+    if (__ldg(g.lcol + b + half) < hi) {
+      b += half + 1;
+      len -= half + 1;
+    } else {
+      len = half;
+    }
+  }
+  return make_int2(a, b);
+}
+
 // Is w (label l) a neighbour of x?  One bit of x's adjacency bitmap when x
 // is a hub, else one binary search on the (label, id) order of x's row.
 __device__ __forceinline__ bool row_contains_l(const GraphDev &g, int32_t x, int32_t l,

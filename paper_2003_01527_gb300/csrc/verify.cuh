@@ -62,6 +62,14 @@ __device__ __forceinline__ int32_t item_row(const TileRows &t, const int32_t *s_
   return t.r0 + lo;
 }
 
+// A row extended by one vertex at position i.
+template <typename Row>
+struct ExtendedRow {
+  const Row &row;
+  int32_t i, w;
+  __device__ __forceinline__ int32_t operator()(int c) const { return c == i ? w : row(c); }
+};
+
 // Position c of row r of a column-major frontier (leading dimension ld).
 struct ColumnRow {
   const int32_t *__restrict__ F;
@@ -80,12 +88,13 @@ __device__ __forceinline__ int32_t parent_index(const Row &) {
 // The checks of Sec. 3.2 verification that need no adjacency search, for
 // candidate w of a partial embedding (row(c) = the image of pi_c): label +
 // signature (bitmap of C(pi_i)), injectivity against same-label, non-adjacent
-// positions, and the ordering constraints of distinct counting.  Desc is a
+// positions, and the ordering constraints of distinct counting.  A null
+// bitmap: the label segment's entries are all candidates.  Desc is a
 // level description with the fields of LevelDesc used here (the single-query
 // LevelDesc or the batched form's BatchLevel).
 template <typename Desc, typename Row>
 __device__ __forceinline__ bool check_local(const Desc &d, const Row &row, int32_t w) {
-  if (!bitmap_has(d.bitmap, w)) return false;
+  if (d.bitmap && !bitmap_has(d.bitmap, w)) return false;
   for (int t = 0; t < d.ninj; ++t)
     if (row(d.inj[t]) == w) return false;
   for (int t = 0; t < d.nlt; ++t)
@@ -126,6 +135,69 @@ __device__ __forceinline__ bool check_candidate_probes(const GraphDev &g, const 
   }
   return true;
 }
+
+// One thread's sums of the leaf numbers of core embeddings; kLeaves = an
+// upper bound of the query's leaves.
+template <int kLeaves>
+struct LeafSums {
+  unsigned long long lo = 0, hi = 0;  // of the numbers' 32-bit halves
+  unsigned long long part[kLeaves] = {};  // partial embeddings with l leaves placed
+  bool over = false;
+
+  // Adds the images of the leaves for one core embedding (row(c) = the image
+  // of core position c): the product over the groups (LeafDesc).
+  template <typename Row>
+  __device__ __forceinline__ void add(const GraphDev &g, const LeafDesc &leaf, const Row &row) {
+    unsigned long long v = 1;
+    bool big = false;
+    int32_t a = 0;
+#pragma unroll
+    for (int l = 0; l < kLeaves; ++l) {
+      if (l >= leaf.nleaves) break;
+      if (l == 0 || leaf.of[l] != leaf.of[l - 1]) {
+        const LeafGroup &gr = leaf.grp[leaf.of[l]];
+        const int32_t x = row(gr.pos);
+        int2 seg = label_segment(g, x, gr.lab);
+        if (gr.lo > 0 || gr.hi < g.n) seg = cut_segment(g, seg, gr.lo, gr.hi);
+        a = seg.y - seg.x;
+        for (uint32_t m = gr.in_mask; m; m &= m - 1) {
+          const int32_t y = row(__ffs(m) - 1);
+          a -= y >= gr.lo && y < gr.hi;
+        }
+        for (uint32_t m = gr.chk_mask; m && a > 0; m &= m - 1) {
+          const int32_t y = row(__ffs(m) - 1);
+          if (y >= gr.lo && y < gr.hi && row_contains_l(g, x, gr.lab, y)) --a;
+        }
+      } else {
+        --a;
+      }
+      part[l] += v;
+      if (a <= 0) return;  // this leaf has no image
+      big = big || __umul64hi(v, (unsigned long long)a);
+      v *= (unsigned long long)a;
+    }
+    over = over || big;
+    lo += (uint32_t)v;
+    hi += v >> 32;
+  }
+
+  // Adds the warp's sums into the count's words (all lanes call it).
+  __device__ __forceinline__ void flush(const LeafDesc &leaf, unsigned long long *total) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const bool first = (threadIdx.x & 31) == 0;
+    auto sum = [&](unsigned long long v, unsigned long long *to) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kAll, v, o);
+      if (first && v) atomicAdd(to, v);
+    };
+    sum(lo, total);
+    sum(hi, total + 1);
+    if (__any_sync(kAll, over) && first) atomicOr(total + 2, 1ull);
+#pragma unroll
+    for (int l = 0; l < kLeaves; ++l)
+      if (l < leaf.nleaves) sum(part[l], total + 3 + l);
+  }
+};
 
 // Entries of w's (label, id)-ordered row scanned at most per group by the
 // 2-look-ahead before it gives up (and keeps the candidate).

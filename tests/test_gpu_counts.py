@@ -1,0 +1,88 @@
+"""gsm_count's closed forms against the oracle: queries whose leaves are
+multiplied out instead of extended (one and several parents, equal and
+different labels, restricted leaves), and counts past 64 bits."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2003_01527_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {
+    "edge": (2, [(0, 1)]),
+    "path3": (3, [(0, 1), (1, 2)]),
+    "path5": (5, [(0, 1), (1, 2), (2, 3), (3, 4)]),
+    "star5": (6, [(0, 1), (0, 2), (0, 3), (0, 4), (0, 5)]),
+    "tailed_triangle": (5, [(0, 1), (1, 2), (0, 2), (2, 3), (3, 4)]),
+    "bull": (5, [(0, 1), (1, 2), (0, 2), (0, 3), (1, 4)]),
+    "triangle_two_tails": (5, [(0, 1), (1, 2), (0, 2), (2, 3), (2, 4)]),
+    "caterpillar": (7, [(0, 1), (1, 2), (0, 3), (1, 4), (1, 5), (2, 6)]),
+    "square_with_tails": (6, [(0, 1), (1, 2), (2, 3), (0, 3), (0, 4), (2, 5)]),
+}
+
+
+def er(n, m, labels, seed):
+    _, rp, col = I.erdos_renyi(n, m, seed=seed)
+    lab = I.uniform_labels(n, labels, seed + 1) if labels > 1 else np.zeros(n, np.int32)
+    return I.make_graph(n, rp, col, lab)
+
+
+@pytest.mark.parametrize("labels", [1, 2, 3])
+@pytest.mark.parametrize("shape", sorted(SHAPES))
+def test_counts_with_leaves(gsm_lib, cuda, shape, labels):
+    g = er(90, 330, labels, seed=50 + labels)
+    k, edges = SHAPES[shape]
+    rng = np.random.default_rng(labels)
+    m = gsm_lib.Matcher(device=0)
+    m.load_graph(g.row_ptr, g.col, g.labels, validate=True)
+    small = gsm_lib.Matcher(device=0, mem_budget_bytes=1 << 18, chunk_rows=37)
+    small.load_graph(g.row_ptr, g.col, g.labels)
+    for trial in range(4 if labels > 1 else 1):
+        q = I.query_from_edges(k, edges, rng.integers(0, labels, k))
+        want = oracle.count(g, q)
+        for x in (m, small):
+            assert x.count(x.query(q.k, q.edges, q.labels)) == want
+        # a range of every vertex in turn: results of the two parts add up
+        for u in range(k):
+            parts = [m.count(m.query(q.k, q.edges, q.labels).restrict(u, *r))
+                     for r in ((0, 31), (31, g.n))]
+            assert sum(parts) == want
+        # every vertex restricted: the listing agrees
+        Q = m.query(q.k, q.edges, q.labels)
+        for u in range(k):
+            Q.restrict(u, 5, 60 + 3 * u)
+        assert m.count(Q) == m.enumerate(Q, cap_rows=0)[1]
+    m.close()
+    small.close()
+
+
+def test_counts_past_64_bits(gsm_lib, cuda):
+    """A star with d leaves has perm(d, m) maps of an m-leaf star onto its
+    centre (m >= 2): exact below 2^64, an error above."""
+    d = 2000
+    g = I.graph_from_edges(d + 1, [(0, v) for v in range(1, d + 1)])
+    m = gsm_lib.Matcher(device=0)
+    m.load_graph(g.row_ptr, g.col, g.labels)
+
+    def star(leaves):
+        return m.query(leaves + 1, [(0, j + 1) for j in range(leaves)])
+
+    assert math.perm(d, 5) < 2 ** 64 < math.perm(d, 6)
+    assert m.count(star(5)) == math.perm(d, 5)
+    for leaves in (6, 9, 15):
+        with pytest.raises(gsm_lib.GsmError) as e:
+            m.count(star(leaves))
+        assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+    assert m.count(star(3)) == math.perm(d, 3)  # the context is still usable
+    # 40 hubs of 2,000 leaves: every hub's number fits in 64 bits, and their sum
+    hubs = I.graph_from_edges(40 * 2001, [(2001 * h, 2001 * h + v) for h in range(40)
+                                          for v in range(1, 2001)])
+    m.load_graph(hubs.row_ptr, hubs.col, hubs.labels)
+    assert m.count(star(4)) == 40 * math.perm(2000, 4)
+    with pytest.raises(gsm_lib.GsmError) as e:
+        m.count(star(6))
+    assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+    m.close()
