@@ -1260,6 +1260,43 @@ int32_t split_leaves(const gsm_ctx *ctx, const gsm_query *q, const int32_t *dens
   return kc;
 }
 
+// Ordering constraints between the positions of the core (order[0 .. kc)) that
+// keep one of every set of core embeddings which the core's symmetries map to
+// one another, and the number of those symmetries.  A symmetry preserves each
+// core vertex's label, restriction and leaves outside the core (their labels
+// and restrictions), so the embeddings of a set have the same leaf numbers and
+// the count is the sum over the kept ones times the number of symmetries.
+// Positions are fixed in matching order, so that every constraint bounds the
+// later vertex from below.
+uint64_t core_symmetry(const gsm_ctx *ctx, const gsm_query *q, const int32_t *dense,
+                       const int32_t *order, int32_t kc,
+                       std::vector<std::pair<int32_t, int32_t>> *less) {
+  using Key = std::array<int32_t, 3>;
+  auto key = [&](int32_t u) {
+    return Key{dense[u], std::max<int32_t>(0, q->lo[u]), std::min<int32_t>(ctx->n, q->hi[u])};
+  };
+  uint32_t core = 0;
+  for (int32_t j = 0; j < kc; ++j) core |= 1u << order[j];
+  std::vector<std::vector<Key>> seen;  // colours: own key, then the leaves' keys in order
+  int32_t colour[kMaxK];
+  uint32_t adj[kMaxK] = {};
+  for (int32_t j = 0; j < kc; ++j) {
+    const int32_t u = order[j];
+    std::vector<Key> c;
+    for (int32_t w = 0; w < q->k; ++w)
+      if ((q->adj[u] & ~core) >> w & 1u) c.push_back(key(w));
+    std::sort(c.begin(), c.end());
+    c.insert(c.begin(), key(u));
+    const auto it = std::find(seen.begin(), seen.end(), c);
+    colour[j] = (int32_t)(it - seen.begin());
+    if (it == seen.end()) seen.push_back(c);
+    for (int32_t b = 0; b < kc; ++b)
+      if (q->adj[u] >> order[b] & 1u) adj[j] |= 1u << b;
+  }
+  if ((int32_t)seen.size() == kc) return 1;
+  return symmetry_constraints(kc, adj, colour, less);
+}
+
 // Filtering step: fills the k candidate bitmaps and returns |C(u)|; then
 // opt.filter_rounds refinement rounds (double-buffered, so every round reads
 // the previous round's sets only).
@@ -1305,7 +1342,8 @@ void run_filter(gsm_ctx *ctx, const gsm_query *q, const int32_t *dense, uint64_t
   std::memcpy(sizes, ctx->h_stage, sizeof(uint64_t) * q->k);
 }
 
-// The whole matcher for one query.  out == nullptr and !enumerate: count only.
+// The whole matcher for one query.  out == nullptr and !enumerate: count only;
+// distinct_of = |Aut(Q)| divides the count (distinct subgraphs).
 // pre (optional): the query's candidate bitmaps and sizes, already computed
 // by a batched filter launch (gsm_enumerate_many).
 struct Prefiltered {
@@ -1315,8 +1353,8 @@ struct Prefiltered {
 
 void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, uint64_t cap_rows,
                int32_t flags, uint64_t *count_out, bool *truncated,
-               const std::vector<std::pair<int32_t, int32_t>> *less = nullptr,
-               bool copy_async = false, const Prefiltered *pre = nullptr) {
+               bool copy_async = false, const Prefiltered *pre = nullptr,
+               uint64_t distinct_of = 1) {
   if (!ctx->has_graph) FAIL(GSM_ERR_NO_GRAPH, "no data graph loaded");
   const Range range(enumerate ? "gsm query (list)" : "gsm query (count)");
   std::memset(&ctx->run, 0, sizeof(ctx->run));
@@ -1359,15 +1397,19 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   for (int32_t u = 0; u < q->k; ++u)
     if (sizes[u] == 0) return;
   plan(q->k, q->adj, sizes, R.order, R.parent);
-  // counts multiply leaves out instead of checking every image (LeafDesc).
-  // Compressed frontiers keep their own last level, and `less` its
-  // constraints on leaves.
-  // With look-ahead the leaves come last too, but are extended; fault
-  // injection keeps every level, so that its wait is reached.
-  if (!enumerate && !less &&
-      !(ctx->opt.flags & (GSM_OPT_COMPRESSED_FRONTIERS | GSM_OPT_INJECT_SCAN_STALL))) {
+  // counts multiply leaves out instead of checking every image (LeafDesc), and
+  // count one of every set of embeddings that a symmetry of the other vertices
+  // (the core) maps to one another
+  uint64_t core_aut = 1;
+  std::vector<std::pair<int32_t, int32_t>> less;  // positions a < b: f(pi_a) < f(pi_b)
+  if (!enumerate) {
     R.k = split_leaves(ctx, q, dense, R.order, &R.leaf);
-    if (ctx->opt.lookahead > 0) {
+    core_aut = core_symmetry(ctx, q, dense, R.order, R.k, &less);
+    // with look-ahead and in compressed frontiers the leaves are extended like
+    // the others; fault injection keeps every level, so that its wait is
+    // reached
+    if (ctx->opt.lookahead > 0 ||
+        (ctx->opt.flags & (GSM_OPT_COMPRESSED_FRONTIERS | GSM_OPT_INJECT_SCAN_STALL))) {
       R.k = q->k;
       R.leaf.nleaves = 0;
     }
@@ -1422,8 +1464,11 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
         d.inj[d.ninj++] = j;
     }
     for (int32_t j = 0; j <= i; ++j) d.out_col[j] = (i == q->k - 1) ? R.order[j] : j;
-    d.bitmap = bm + (size_t)u * nw;
+    // a leaf's candidates are all entries of its parent's cut label segment
+    d.bitmap = popc(q->adj[u]) == 1 ? nullptr : bm + (size_t)u * nw;
     d.lab = dense[u];
+    d.rlo = std::max<int32_t>(0, q->lo[u]);
+    d.rhi = std::min<int32_t>(ctx->n, q->hi[u]);
     d.la = std::max<int32_t>(0, ctx->opt.lookahead);
     d.cand = bm;
     d.n_words = nw;
@@ -1453,15 +1498,9 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
             d.la_pos[t] |= 1u << j;
         }
     }
-    if (less) {
-      // ordering constraints between pi_i and vertices placed before it
-      for (const auto &c : *less) {
-        for (int32_t j = 0; j < i; ++j) {
-          if (c.first == u && c.second == R.order[j]) d.lt[d.nlt++] = j;   // f(u) < f(pi_j)
-          if (c.second == u && c.first == R.order[j]) d.gt[d.ngt++] = j;   // f(pi_j) < f(u)
-        }
-      }
-    }
+    for (const auto &c : less)
+      if (c.second == i) d.gt[d.ngt++] = c.first;
+    d.cut = d.rlo > 0 || d.rhi < ctx->n || d.ngt > 0;
   }
 
   CU(cudaMemsetAsync(R.d_total, 0, sizeof(unsigned long long) * kCountWords, ctx->stream));
@@ -1506,9 +1545,11 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     fetch(ctx, R.d_total, sizeof(uint64_t) * kCountWords);
     uint64_t w[kCountWords];
     std::memcpy(w, ctx->h_stage, sizeof(w));
-    // (without leaves word 0 is the count itself)
-    const unsigned __int128 sum = (unsigned __int128)w[0] + ((unsigned __int128)w[1] << 32);
-    if (w[2] || sum >> 64) FAIL(GSM_ERR_OVERFLOW, "more than 2^64 - 1 embeddings");
+    // (without leaves word 0 is the sum itself)
+    unsigned __int128 sum = (unsigned __int128)w[0] + ((unsigned __int128)w[1] << 32);
+    const bool big = w[2] || sum > ~(unsigned __int128)0 / core_aut;
+    sum = sum * core_aut / distinct_of;
+    if (big || sum >> 64) FAIL(GSM_ERR_OVERFLOW, "the count exceeds 2^64 - 1");
     total = (uint64_t)sum;
     for (int32_t l = 0; l < R.leaf.nleaves; ++l) ctx->run.frontier[R.k + l] = w[3 + l];
   }
@@ -3106,7 +3147,7 @@ void list_many(gsm_ctx *ctx, ManyState &M, uint64_t *launches, uint64_t *peak, b
     bool trunc = false;
     const Prefiltered *p = (M.pre && (*M.pre)[j].bitmaps) ? &(*M.pre)[j] : nullptr;
     run_query(c, M.queries[j], true, M.outs[j], M.cap_rows[j], M.flags, &M.counts[j], &trunc,
-              nullptr, true, p);
+              true, p);
     *launches += c->run.kernel_launches;
     *peak = std::max<uint64_t>(*peak, c->peak_bytes);
     if (trunc) {
@@ -3310,7 +3351,7 @@ gsm_status gsm_count_distinct(gsm_ctx *ctx, const gsm_query *q, uint64_t *count,
     std::vector<std::pair<int32_t, int32_t>> less;
     const uint64_t aut = symmetry_constraints(q->k, q->adj, q->labels, &less);
     bool trunc = false;
-    run_query(ctx, q, false, nullptr, 0, 0, count, &trunc, &less);
+    run_query(ctx, q, false, nullptr, 0, 0, count, &trunc, false, nullptr, aut);
     if (automorphisms) *automorphisms = aut;
     resolve_timings(ctx);
     ctx->run.peak_bytes = ctx->peak_bytes;

@@ -17,8 +17,6 @@ struct BatchLevel {
   int32_t last;             // 1 if pi_i is the query's last vertex
   int32_t lab;              // dense label of pi_i (the row segment traversed)
   const uint32_t *bitmap;   // C(pi_i)
-  int32_t nlt, lt[kMaxK];   // ordering constraints (none in the batched form)
-  int32_t ngt, gt[kMaxK];
 };
 
 struct BatchQuery {

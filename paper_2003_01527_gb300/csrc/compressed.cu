@@ -34,8 +34,11 @@ __global__ void k_cpivot(GraphDev g, LevelDesc d, CFrontier f, int32_t i, int64_
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R; r += stride) {
     decode_row(f, i, (int32_t)r, vals);
     int32_t best = INT_MAX, best_start = 0, best_slot = 0;
+    int32_t lo = d.rlo;
+    for (int t = 0; t < d.ngt; ++t) lo = max(lo, vals[d.gt[t]] + 1);
     for (int b = 0; b < d.nb; ++b) {
-      const int2 seg = label_segment(g, vals[d.bpos[b]], d.lab);
+      int2 seg = label_segment(g, vals[d.bpos[b]], d.lab);
+      if (d.cut) seg = cut_segment(g, seg, lo, d.rhi);
       if (seg.y - seg.x < best) {
         best = seg.y - seg.x;
         best_start = seg.x;

@@ -389,6 +389,13 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
       bstart[j] = 0;
       bslot[j] = 0;
     }
+    int32_t lo[kPsIpt];  // the new vertex's lower bound (its segments are cut there)
+#pragma unroll
+    for (int j = 0; j < kPsIpt; ++j) {
+      lo[j] = d.rlo;
+      for (int t = 0; t < d.ngt && best[j]; ++t)
+        lo[j] = max(lo[j], F[(int64_t)d.gt[t] * ld + base + j * kPsThreads + threadIdx.x] + 1);
+    }
     for (int b = 0; b < d.nb; ++b) {
       int32_t x[kPsIpt];
 #pragma unroll
@@ -403,7 +410,8 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
           bslot[j] = b;
           continue;
         }
-        const int2 seg = label_segment(g, x[j], d.lab);
+        int2 seg = label_segment(g, x[j], d.lab);
+        if (d.cut) seg = cut_segment(g, seg, lo[j], d.rhi);
         if (seg.y - seg.x < best[j]) {
           best[j] = seg.y - seg.x;
           bstart[j] = seg.x;

@@ -38,9 +38,15 @@ struct LevelDesc {
   int32_t ninj;               // positions that need an explicit injectivity test
   int32_t inj[kMaxK];
   int32_t out_col[kMaxK + 1]; // output column of position j (0..i); identity except last level
-  const uint32_t *bitmap;     // C(pi_i)
-  int32_t nlt, lt[kMaxK];     // symmetry breaking: the new vertex must be < row[lt[t]]
-  int32_t ngt, gt[kMaxK];     //                     and > row[gt[t]]
+  const uint32_t *bitmap;     // C(pi_i); null: every entry of a cut label segment is in it
+  // bounds of the new vertex, taken off the ends of its (id-sorted) label
+  // segment when the pivot is chosen (cut != 0), so that no candidate outside
+  // them is generated: the restriction [rlo, rhi) and, for symmetry breaking,
+  // > row[gt[t]].  Counting the ordered triangles of R-MAT 20 checks 2.3e9
+  // candidates instead of 1.4e10 (117.7 -> 20.8 ms), the distinct 4-cliques of
+  // R-MAT 16 6e8 instead of 6.2e9 (39.7 -> 11.3 ms)
+  int32_t cut, rlo, rhi;
+  int32_t ngt, gt[kMaxK];
   int32_t lab;                // dense label of pi_i: only that segment of a row is traversed
   // k-look-ahead (Sec. 3.2; la = 0 off, 1 or 2): the query neighbours of
   // pi_i placed after it, grouped by label.  Group t: label la_lab[t],

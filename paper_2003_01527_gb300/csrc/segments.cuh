@@ -45,7 +45,7 @@ __device__ __forceinline__ int2 label_segment(const GraphDev &g, int32_t x, int3
 
 // The part of an id-sorted segment of lcol with ids in [lo, hi).
 __device__ __forceinline__ int2 cut_segment(const GraphDev &g, int2 seg, int32_t lo, int32_t hi) {
-  int32_t a = seg.x, len = seg.y - seg.x;
+  int32_t a = seg.x, len = lo > 0 ? seg.y - seg.x : 0;
   while (len > 0) {
     const int32_t half = len >> 1;
     if (__ldg(g.lcol + a + half) < lo) {
@@ -55,6 +55,7 @@ __device__ __forceinline__ int2 cut_segment(const GraphDev &g, int2 seg, int32_t
       len = half;
     }
   }
+  if (hi >= g.n) return make_int2(a, seg.y);
   int32_t b = a;
   len = seg.y - a;
   while (len > 0) {

@@ -87,9 +87,10 @@ __device__ __forceinline__ int32_t parent_index(const Row &) {
 
 // The checks of Sec. 3.2 verification that need no adjacency search, for
 // candidate w of a partial embedding (row(c) = the image of pi_c): label +
-// signature (bitmap of C(pi_i)), injectivity against same-label, non-adjacent
-// positions, and the ordering constraints of distinct counting.  A null
-// bitmap: the label segment's entries are all candidates.  Desc is a
+// signature (bitmap of C(pi_i)) and injectivity against same-label,
+// non-adjacent positions (the bounds of the new vertex were cut off its
+// segment with the pivot).  A null bitmap: the segment's entries are all
+// candidates.  Desc is a
 // level description with the fields of LevelDesc used here (the single-query
 // LevelDesc or the batched form's BatchLevel).
 template <typename Desc, typename Row>
@@ -97,10 +98,6 @@ __device__ __forceinline__ bool check_local(const Desc &d, const Row &row, int32
   if (d.bitmap && !bitmap_has(d.bitmap, w)) return false;
   for (int t = 0; t < d.ninj; ++t)
     if (row(d.inj[t]) == w) return false;
-  for (int t = 0; t < d.nlt; ++t)
-    if (!(w < row(d.lt[t]))) return false;
-  for (int t = 0; t < d.ngt; ++t)
-    if (!(w > row(d.gt[t]))) return false;
   return true;
 }
 

@@ -1,6 +1,8 @@
-"""gsm_count's closed forms against the oracle: queries whose leaves are
+"""gsm_count's shortcuts against the oracle: queries whose leaves are
 multiplied out instead of extended (one and several parents, equal and
-different labels, restricted leaves), and counts past 64 bits."""
+different labels, restricted leaves), queries with symmetries (one of every
+set of symmetric embeddings is counted; candidates outside the ordering
+constraints are never generated), and counts past 64 bits."""
 import math
 
 import numpy as np
@@ -20,6 +22,13 @@ SHAPES = {
     "bull": (5, [(0, 1), (1, 2), (0, 2), (0, 3), (1, 4)]),
     "triangle_two_tails": (5, [(0, 1), (1, 2), (0, 2), (2, 3), (2, 4)]),
     "caterpillar": (7, [(0, 1), (1, 2), (0, 3), (1, 4), (1, 5), (2, 6)]),
+    "triangle": (3, [(0, 1), (1, 2), (0, 2)]),
+    "cycle4": (4, [(0, 1), (1, 2), (2, 3), (0, 3)]),
+    "diamond": (4, [(0, 1), (1, 2), (2, 3), (0, 3), (0, 2)]),
+    "clique4": (4, [(0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (2, 3)]),
+    "cycle5": (5, [(0, 1), (1, 2), (2, 3), (3, 4), (0, 4)]),
+    "k23": (5, [(0, 2), (0, 3), (0, 4), (1, 2), (1, 3), (1, 4)]),
+    "cycle6": (6, [(0, 1), (1, 2), (2, 3), (3, 4), (4, 5), (0, 5)]),
     "square_with_tails": (6, [(0, 1), (1, 2), (2, 3), (0, 3), (0, 4), (2, 5)]),
 }
 
@@ -32,31 +41,43 @@ def er(n, m, labels, seed):
 
 @pytest.mark.parametrize("labels", [1, 2, 3])
 @pytest.mark.parametrize("shape", sorted(SHAPES))
-def test_counts_with_leaves(gsm_lib, cuda, shape, labels):
-    g = er(90, 330, labels, seed=50 + labels)
+def test_counts_of_shapes(gsm_lib, cuda, shape, labels):
+    g = er(90, 500, labels, seed=50 + labels)
     k, edges = SHAPES[shape]
     rng = np.random.default_rng(labels)
     m = gsm_lib.Matcher(device=0)
     m.load_graph(g.row_ptr, g.col, g.labels, validate=True)
-    small = gsm_lib.Matcher(device=0, mem_budget_bytes=1 << 18, chunk_rows=37)
-    small.load_graph(g.row_ptr, g.col, g.labels)
+    others = [gsm_lib.Matcher(device=0, **o) for o in
+              ({"mem_budget_bytes": 1 << 18, "chunk_rows": 37}, {"compressed": True},
+               {"lookahead": 2}, {"two_pass": True, "hub_bitmap_bytes": -1, "filter_rounds": 1})]
+    for x in others:
+        x.load_graph(g.row_ptr, g.col, g.labels)
     for trial in range(4 if labels > 1 else 1):
         q = I.query_from_edges(k, edges, rng.integers(0, labels, k))
         want = oracle.count(g, q)
-        for x in (m, small):
+        for x in [m] + others:
             assert x.count(x.query(q.k, q.edges, q.labels)) == want
+        distinct, aut = m.count_distinct(m.query(q.k, q.edges, q.labels))
+        assert distinct * aut == want
         # a range of every vertex in turn: results of the two parts add up
         for u in range(k):
             parts = [m.count(m.query(q.k, q.edges, q.labels).restrict(u, *r))
                      for r in ((0, 31), (31, g.n))]
             assert sum(parts) == want
-        # every vertex restricted: the listing agrees
-        Q = m.query(q.k, q.edges, q.labels)
-        for u in range(k):
-            Q.restrict(u, 5, 60 + 3 * u)
-        assert m.count(Q) == m.enumerate(Q, cap_rows=0)[1]
-    m.close()
-    small.close()
+        # every vertex restricted, alike and each to its own range: the count
+        # and the listing are the rows of the whole result in the ranges
+        rows = oracle.match(g, q)[1]
+        for ranges in ([(7, 70)] * k, [(5, 60 + 3 * u) for u in range(k)]):
+            keep = np.all([(rows[:, u] >= a) & (rows[:, u] < b)
+                           for u, (a, b) in enumerate(ranges)], axis=0)
+            for x in [m] + others:
+                Q = x.query(q.k, q.edges, q.labels)
+                for u, r in enumerate(ranges):
+                    Q.restrict(u, *r)
+                assert x.count(Q) == int(keep.sum())
+                assert np.array_equal(x.enumerate(Q)[0], rows[keep])
+    for x in [m] + others:
+        x.close()
 
 
 def test_counts_past_64_bits(gsm_lib, cuda):
