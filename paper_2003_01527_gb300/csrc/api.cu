@@ -97,6 +97,8 @@ struct gsm_ctx {
   size_t hub_seg_bytes = 0;
   uint8_t *d_nlc = nullptr;        // neighbour label counts, nlc_stride per vertex
   int32_t nlc_stride = 0;
+  uint32_t *d_thr = nullptr;       // threshold bitmaps, then the label bitmaps
+  size_t thr_bytes = 0;
   int32_t hub_count = 0, hub_min_deg = 0;
   size_t hub_bits_bytes = 0;
   std::vector<int32_t> label_values;  // sorted distinct labels; dense id = index
@@ -240,6 +242,10 @@ GraphDev graph_dev(const gsm_ctx *ctx) {
                   ctx->hub_count ? ctx->d_hub_seg : nullptr,
                   ctx->d_nlc,
                   ctx->nlc_stride,
+                  ctx->d_thr,
+                  ctx->d_thr ? ctx->d_thr + (size_t)kThrLevels * ctx->label_values.size() *
+                                               ((ctx->n + 31) / 32)
+                             : nullptr,
                   ctx->d_flags ? ctx->d_flags + 1 : nullptr};
 }
 
@@ -1698,6 +1704,7 @@ void free_graph(gsm_ctx *ctx) {
     ctx->d_hub_seg = nullptr;
     ctx->d_nlc = nullptr;
     ctx->nlc_stride = 0;
+    ctx->d_thr = nullptr;
     ctx->hub_count = 0;
     ctx->has_graph = false;
     ctx->borrowed_graph = false;
@@ -1713,8 +1720,10 @@ void free_graph(gsm_ctx *ctx) {
   if (ctx->d_hub_bits) dev_free(ctx, ctx->d_hub_bits, ctx->hub_bits_bytes);
   if (ctx->d_hub_seg) dev_free(ctx, ctx->d_hub_seg, ctx->hub_seg_bytes);
   if (ctx->d_nlc) dev_free(ctx, ctx->d_nlc, (size_t)ctx->n * ctx->nlc_stride);
+  if (ctx->d_thr) dev_free(ctx, ctx->d_thr, ctx->thr_bytes);
   ctx->d_nlc = nullptr;
   ctx->nlc_stride = 0;
+  ctx->d_thr = nullptr;
   ctx->d_hub = nullptr;
   ctx->d_hub_bits = nullptr;
   ctx->d_hub_seg = nullptr;
@@ -2933,8 +2942,17 @@ gsm_status gsm_load_graph(gsm_ctx *ctx, int32_t n, int64_t nnz, const int32_t *r
       ctx->d_nlc = (uint8_t *)dev_alloc(ctx, std::max<size_t>((size_t)n * L, 1));
       launch_label_counts(graph_dev(ctx), ctx->d_nlc, L, ctx->stream);
       CU(cudaGetLastError());
-      CU(cudaStreamSynchronize(ctx->stream));
     }
+    if (n > 0 && (L == 1 || ctx->d_nlc)) {
+      // (kThrLevels + 1) bitmaps per label, less than the count table's bytes
+      const size_t words = (size_t)(n + 31) / 32;
+      ctx->thr_bytes = sizeof(uint32_t) * words * L * (kThrLevels + 1);
+      ctx->d_thr = (uint32_t *)dev_alloc(ctx, ctx->thr_bytes);
+      launch_threshold_bits(graph_dev(ctx), ctx->d_thr, ctx->d_thr + words * L * kThrLevels,
+                            ctx->stream);
+      CU(cudaGetLastError());
+    }
+    CU(cudaStreamSynchronize(ctx->stream));
     ctx->has_graph = true;
   });
 }
@@ -3094,6 +3112,7 @@ void share_graph(const gsm_ctx *ctx, gsm_ctx *w) {
   w->d_hub_seg = ctx->d_hub_seg;
   w->d_nlc = ctx->d_nlc;
   w->nlc_stride = ctx->nlc_stride;
+  w->d_thr = ctx->d_thr;
   w->hub_count = ctx->hub_count;
   w->label_values = ctx->label_values;
   w->has_graph = ctx->has_graph;

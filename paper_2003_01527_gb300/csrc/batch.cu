@@ -147,6 +147,19 @@ __global__ void __launch_bounds__(256) k_b_filter(GraphDev g, const FilterDesc *
                ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
 
+// The same from the graph's bitmaps (a thread per word, a CTA row per query).
+__global__ void __launch_bounds__(256) k_b_filter_bits(GraphDev g,
+                                                       const FilterDesc *__restrict__ fds,
+                                                       uint32_t *const *__restrict__ bm_out,
+                                                       unsigned long long *__restrict__ sizes) {
+  __shared__ FilterDesc s_d;
+  const int32_t q = blockIdx.y;
+  for (int j = threadIdx.x; j < (int)(sizeof(FilterDesc) / 4); j += blockDim.x)
+    reinterpret_cast<int32_t *>(&s_d)[j] = reinterpret_cast<const int32_t *>(fds + q)[j];
+  __syncthreads();
+  filter_words(g, s_d, bm_out[q], sizes ? sizes + (int64_t)q * kMaxK : nullptr, 0, 1);
+}
+
 // Word counts of every query's root bitmap; one-vertex queries are counted
 // here and contribute no rows.
 __global__ void k_b_list_popc(const BatchQuery *__restrict__ qs, int32_t nq, int32_t n_words,
@@ -597,7 +610,11 @@ void launch_filter_many(const GraphDev &g, const FilterDesc *fds, uint32_t *cons
                         unsigned long long *sizes, int32_t nq, int32_t n_words,
                         cudaStream_t s) {
   if (nq <= 0) return;
-  cudaMemsetAsync(sizes, 0, sizeof(unsigned long long) * nq * kMaxK, s);
+  if (sizes) cudaMemsetAsync(sizes, 0, sizeof(unsigned long long) * nq * kMaxK, s);
+  if (g.thr && n_words > 0) {
+    k_b_filter_bits<<<dim3((n_words + 255) / 256, nq), 256, 0, s>>>(g, fds, bm_out, sizes);
+    return;
+  }
   const int gx = (int)std::min<int64_t>((n_words + 7) / 8, 128);
   k_b_filter<<<dim3(std::max(gx, 1), nq), 256, 0, s>>>(g, fds, bm_out, sizes);
 }
@@ -608,12 +625,10 @@ int batch_enqueue(const GraphDev &g, const BatchArgs &a, cudaStream_t s) {
   const size_t smem = (size_t)(tile_items + 1) * sizeof(int32_t);
   int launches = 0;
   cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.nq, s);
-  cudaMemsetAsync(a.sizes, 0, sizeof(unsigned long long) * a.nq * kMaxK, s);
   cudaMemsetAsync(a.overflow, 0, sizeof(int32_t), s);
   k_b_init<<<1, 32, 0, s>>>(a.state, (int64_t)a.nq * a.n_words);
-  // filter: one CTA row per query
-  const int gx = (int)std::min<int64_t>((a.n_words + 7) / 8, 128);
-  k_b_filter<<<dim3(std::max(gx, 1), a.nq), 256, 0, s>>>(g, a.fds, a.bm_out, a.sizes);
+  // filter: one CTA row per query (nothing reads the sizes here)
+  launch_filter_many(g, a.fds, a.bm_out, g.thr ? nullptr : a.sizes, a.nq, a.n_words, s);
   ++launches;
   // level 1: every query's candidate list for its first matched vertex
   k_b_list_popc<<<G, 256, 0, s>>>(a.qs, a.nq, a.n_words, a.wcnt, a.counts);

@@ -106,6 +106,39 @@ __global__ void __launch_bounds__(256) k_filter(GraphDev g, FilterDesc d,
                ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
 
+// The same from the graph's bitmaps: a thread per word, a CTA row per query
+// vertex.
+__global__ void __launch_bounds__(256) k_filter_bits(GraphDev g,
+                                                     const __grid_constant__ FilterDesc d,
+                                                     uint32_t *__restrict__ bitmaps,
+                                                     unsigned long long *__restrict__ sizes) {
+  filter_words(g, d, bitmaps, sizes, blockIdx.y, gridDim.y);
+}
+
+// One warp per 32 vertices: ballots of the threshold and label tests.
+__global__ void __launch_bounds__(256) k_threshold_bits(GraphDev g, uint32_t *__restrict__ thr,
+                                                        uint32_t *__restrict__ lab_bits) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < g.hub_words;
+       w += warps) {
+    const int64_t v = w * 32 + lane;
+    const bool valid = v < g.n;
+    const int32_t lv = valid ? g.lab[v] : -1;
+    for (int32_t l = 0; l < g.num_labels; ++l) {
+      int32_t c = 0;
+      if (valid) c = g.num_labels == 1 ? g.rp[v + 1] - g.rp[v] : g.nlc[v * g.nlc_stride + l];
+#pragma unroll
+      for (int t = 0; t < kThrLevels; ++t) {
+        const uint32_t word = __ballot_sync(kFull, c > t);
+        if (lane == t) thr[((int64_t)l * kThrLevels + t) * g.hub_words + w] = word;
+      }
+      const uint32_t word = __ballot_sync(kFull, lv == l);
+      if (lane == 0) lab_bits[(int64_t)l * g.hub_words + w] = word;
+    }
+  }
+}
+
 // ------------------------------------------------------------ refinement
 
 // One warp per (query vertex u, word of 32 data vertices).  Each candidate v
@@ -1086,9 +1119,20 @@ void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int3
   k_hub_segments<<<grid_for((int64_t)H * 32, 256, 152 * 8), 256, 0, s>>>(g, hubs, H, seg);
 }
 
+void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits, cudaStream_t s) {
+  if (g.n <= 0) return;
+  k_threshold_bits<<<grid_for((int64_t)g.hub_words * 32, 256, 152 * 16), 256, 0, s>>>(g, thr,
+                                                                                      lab_bits);
+}
+
 void launch_filter(const GraphDev &g, const FilterDesc &d, uint32_t *bitmaps,
                    unsigned long long *sizes, cudaStream_t s) {
   const int threads = 256;
+  if (g.thr && d.n_words > 0) {
+    k_filter_bits<<<dim3((d.n_words + threads - 1) / threads, d.k), threads, 0, s>>>(g, d, bitmaps,
+                                                                                     sizes);
+    return;
+  }
   int64_t warps_needed = d.n_words;
   int blocks = grid_for(warps_needed * 32, threads, 152 * 16);
   k_filter<<<blocks, threads, 0, s>>>(g, d, bitmaps, sizes);

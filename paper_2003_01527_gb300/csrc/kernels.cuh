@@ -80,7 +80,7 @@ struct GraphDev {
   // neighbour of v.  hub = null: no bitmaps, every test searches the row.
   const int32_t *hub;
   const uint32_t *hub_bits;
-  int32_t hub_words;
+  int32_t hub_words;  // ceil(n/32), also without hubs
   // label segments of the hubs' rows (null: none): the neighbours of hub h
   // with label l are lcol[hub_seg[h * (num_labels + 1) + l] .. the next entry)
   const int32_t *hub_seg;
@@ -89,6 +89,11 @@ struct GraphDev {
   // 15, so the saturated count decides every requirement exactly)
   const uint8_t *nlc;
   int32_t nlc_stride;
+  // the same as bitmaps over the vertices (null: none): bit v of
+  // thr[(l * kThrLevels + c - 1) * hub_words ..] is set iff v has at least c
+  // neighbours with label l, bit v of lab_bits[l * hub_words ..] iff v's label
+  // is l.  One label: its neighbours are all, so thr holds degrees.
+  const uint32_t *thr, *lab_bits;
   // GSM_DEBUG builds: the mapped word a failed bounds check writes its site
   // to (null: not reported)
   uint32_t *dbg;
@@ -144,6 +149,12 @@ void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int3
 // stride), from the label-segmented rows.
 constexpr int32_t kNlcMaxLabels = 64;
 void launch_label_counts(const GraphDev &g, uint8_t *nlc, int32_t stride, cudaStream_t s);
+
+// The threshold and label bitmaps of GraphDev (thr: num_labels * kThrLevels,
+// lab_bits: num_labels bitmaps of hub_words words), from the neighbour label
+// counts, or with one label from the degrees.
+constexpr int32_t kThrLevels = 4;
+void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits, cudaStream_t s);
 
 // Writes k bitmaps of n_words words and adds |C(u)| into sizes[u].
 void launch_filter(const GraphDev &g, const FilterDesc &d, uint32_t *bitmaps,
