@@ -171,7 +171,7 @@ struct gsm_ctx {
     bool ready = false;
     int64_t cap_rows = 0, cap_elems = 0, cap_items = 0;
     int32_t max_nq = 0;
-    int64_t max_words_total = 0;
+    int64_t max_list_tiles = 0;
     std::vector<std::pair<void *, size_t>> allocs;
     gsm::BatchArgs a{};
     void *bitmaps = nullptr;
@@ -179,8 +179,13 @@ struct gsm_ctx {
     FilterDesc *h_fds = nullptr;
     BatchQuery *h_qs = nullptr;
     uint32_t **h_bm = nullptr;
-    unsigned long long *h_counts = nullptr;
-    int32_t *h_overflow = nullptr;
+    int64_t *h_list_off = nullptr;
+    // read back in one piece: steps, overflow flag, counts (see BatchArgs);
+    // counts: the selected queries' counts made of them (lane_counts)
+    char *h_back = nullptr;
+    std::vector<uint64_t> counts;
+    std::vector<uint64_t> core_aut;  // symmetries a counted query's sum is multiplied by
+    const BatchStep *steps() const { return (const BatchStep *)h_back; }
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_done = nullptr;
     uint32_t *zero_bitmap = nullptr;  // root bitmap of padding queries
     int32_t mb = 0, kb = 0;           // shape of the issued batch (padded)
@@ -189,7 +194,6 @@ struct gsm_ctx {
     // whether it lists rows, and the buffers of the canonical sort
     int32_t enumerate = 0;
     int64_t cap_final = 0;
-    BatchStep *h_state = nullptr;
     std::vector<std::array<int32_t, kMaxK>> orders;
     std::vector<int32_t> lists;
     // device buffers of the canonical sorts: keys (2), sort scratch, the
@@ -602,53 +606,52 @@ gsm_status validate_query_edges(int32_t k, int32_t m, const int32_t *edges, uint
 // Is there an automorphism of the labelled query (a label-preserving
 // permutation that maps edges to edges and non-edges to non-edges) with
 // sigma(x) = x for every x in `fixed` and sigma(a) = b?  Backtracking over
-// query vertices in id order.
-bool aut_exists(int32_t k, const uint32_t *adj, const int32_t *lab, uint32_t fixed, int32_t a,
-                int32_t b) {
+// query vertices in id order (aut_exists).
+struct AutSearch {
+  int32_t k;
+  const uint32_t *adj;
+  const int32_t *lab;
   int32_t sigma[kMaxK];
-  for (int32_t u = 0; u < kMaxK; ++u) sigma[u] = -1;
-  for (int32_t u = 0; u < k; ++u)
-    if (fixed >> u & 1u) sigma[u] = u;
-  if (sigma[a] >= 0 && sigma[a] != b) return false;
-  sigma[a] = b;
-  uint32_t used = 0;
-  for (int32_t u = 0; u < k; ++u)
-    if (sigma[u] >= 0) {
-      if (used >> sigma[u] & 1u) return false;
-      used |= 1u << sigma[u];
+  uint32_t placed = 0, used = 0;  // vertices with an image; images
+
+  // sigma(u) = v consistent with the part placed so far?
+  bool fits(int32_t u, int32_t v) const {
+    if (lab[u] != lab[v] || popc(adj[u]) != popc(adj[v])) return false;
+    for (uint32_t m = placed; m; m &= m - 1) {
+      const int32_t x = __builtin_ctz(m);
+      if ((adj[u] >> x & 1u) != (adj[v] >> sigma[x] & 1u)) return false;
     }
-  // consistency of the preassigned part
-  for (int32_t u = 0; u < k; ++u)
-    for (int32_t v = 0; v < k; ++v)
-      if (sigma[u] >= 0 && sigma[v] >= 0 &&
-          ((adj[u] >> v & 1u) != (adj[sigma[u]] >> sigma[v] & 1u)))
-        return false;
-  for (int32_t u = 0; u < k; ++u)
-    if (sigma[u] >= 0 && (lab[u] != lab[sigma[u]] || popc(adj[u]) != popc(adj[sigma[u]])))
-      return false;
-  // extend to the free vertices
-  int32_t freev[kMaxK], nf = 0;
-  for (int32_t u = 0; u < k; ++u)
-    if (sigma[u] < 0) freev[nf++] = u;
-  std::function<bool(int32_t)> go = [&](int32_t t) -> bool {
-    if (t == nf) return true;
-    const int32_t u = freev[t];
-    for (int32_t v = 0; v < k; ++v) {
-      if (used >> v & 1u) continue;
-      if (lab[v] != lab[u] || popc(adj[v]) != popc(adj[u])) continue;
-      bool ok = true;
-      for (int32_t x = 0; x < k && ok; ++x)
-        if (sigma[x] >= 0 && ((adj[u] >> x & 1u) != (adj[v] >> sigma[x] & 1u))) ok = false;
-      if (!ok) continue;
-      sigma[u] = v;
-      used |= 1u << v;
-      if (go(t + 1)) return true;
-      sigma[u] = -1;
+    return true;
+  }
+  void put(int32_t u, int32_t v) {
+    sigma[u] = v;
+    placed |= 1u << u;
+    used |= 1u << v;
+  }
+  bool extend() {
+    const uint32_t all = (1u << k) - 1u;
+    if (placed == all) return true;
+    const int32_t u = __builtin_ctz(all & ~placed);
+    for (uint32_t m = all & ~used; m; m &= m - 1) {
+      const int32_t v = __builtin_ctz(m);
+      if (!fits(u, v)) continue;
+      put(u, v);
+      if (extend()) return true;
+      placed &= ~(1u << u);
       used &= ~(1u << v);
     }
     return false;
-  };
-  return go(0);
+  }
+};
+
+bool aut_exists(int32_t k, const uint32_t *adj, const int32_t *lab, uint32_t fixed, int32_t a,
+                int32_t b) {
+  AutSearch s{k, adj, lab, {}};
+  for (uint32_t m = fixed; m; m &= m - 1) s.put(__builtin_ctz(m), __builtin_ctz(m));
+  if (fixed >> a & 1u) return a == b;
+  if (fixed >> b & 1u || !s.fits(a, b)) return false;
+  s.put(a, b);
+  return s.extend();
 }
 
 // Ordering constraints that keep exactly one embedding per orbit of Aut(Q)
@@ -668,7 +671,9 @@ uint64_t symmetry_constraints(int32_t k, const uint32_t *adj, const int32_t *lab
       if (fixed >> u & 1u) continue;
       std::vector<int32_t> o{u};
       for (int32_t v = 0; v < k; ++v)
-        if (v != u && !(fixed >> v & 1u) && aut_exists(k, adj, lab, fixed, u, v)) o.push_back(v);
+        if (v != u && lab[v] == lab[u] && !(fixed >> v & 1u) &&
+            aut_exists(k, adj, lab, fixed, u, v))
+          o.push_back(v);
       if (o.size() > 1) {
         pick = u;
         orbit = o;
@@ -1213,45 +1218,47 @@ int32_t split_leaves(const gsm_ctx *ctx, const gsm_query *q, const int32_t *dens
     int32_t last;   // position of the last of them
   };
   const int32_t k = q->k;
-  std::vector<Group> groups;
+  Group groups[kMaxK], take[kMaxK];
+  int32_t ng = 0, nt = 0;
   for (int32_t i = 1; i < k; ++i) {
     const int32_t u = order[i];
     if (popc(q->adj[u]) != 1) continue;
     const int32_t lo = std::max<int32_t>(0, q->lo[u]), hi = std::min<int32_t>(ctx->n, q->hi[u]);
     if ((lo > 0 || hi < ctx->n) && i != k - 1) continue;
     const int32_t p = __builtin_ctz(q->adj[u]);
-    size_t t = 0;
-    while (t < groups.size() && !(groups[t].parent == p && groups[t].lab == dense[u] &&
-                                  groups[t].lo == lo && groups[t].hi == hi))
+    int32_t t = 0;
+    while (t < ng && !(groups[t].parent == p && groups[t].lab == dense[u] &&
+                       groups[t].lo == lo && groups[t].hi == hi))
       ++t;
-    if (t == groups.size()) groups.push_back(Group{p, dense[u], lo, hi, 0u, 0});
+    if (t == ng) groups[ng++] = Group{p, dense[u], lo, hi, 0u, 0};
     groups[t].mask |= 1u << u;
     groups[t].last = i;
   }
   // one group per label: the largest, then the one placed later
-  std::vector<Group> take;
-  for (const Group &x : groups) {
+  for (int32_t x = 0; x < ng; ++x) {
     bool best = true;
-    for (const Group &y : groups)
-      if (y.lab == x.lab && (popc(y.mask) > popc(x.mask) ||
-                             (popc(y.mask) == popc(x.mask) && y.last > x.last)))
+    for (int32_t y = 0; y < ng; ++y) {
+      const int px = popc(groups[x].mask), py = popc(groups[y].mask);
+      if (groups[y].lab == groups[x].lab &&
+          (py > px || (py == px && groups[y].last > groups[x].last)))
         best = false;
-    if (best) take.push_back(x);
+    }
+    if (best) take[nt++] = groups[x];
   }
   uint32_t gone = 0;
-  for (const Group &x : take) gone |= x.mask;
+  for (int32_t t = 0; t < nt; ++t) gone |= take[t].mask;
   int32_t kc = 0, next[kMaxK], nl = 0;
-  for (size_t t = 0; t < take.size(); ++t)
+  for (int32_t t = 0; t < nt; ++t)
     for (int32_t i = 0; i < k; ++i)
       if (take[t].mask >> order[i] & 1u) {
-        leaf->of[nl] = (int32_t)t;
+        leaf->of[nl] = t;
         next[nl++] = order[i];
       }
   for (int32_t i = 0; i < k; ++i)
     if (!(gone >> order[i] & 1u)) order[kc++] = order[i];
   for (int32_t j = 0; j < nl; ++j) order[kc + j] = next[j];
   leaf->nleaves = nl;
-  for (size_t t = 0; t < take.size(); ++t) {
+  for (int32_t t = 0; t < nt; ++t) {
     const Group &x = take[t];
     LeafGroup &gr = leaf->grp[t];
     gr = LeafGroup{0, x.lab, x.lo, x.hi, 0u, 0u};
@@ -1281,25 +1288,53 @@ uint64_t core_symmetry(const gsm_ctx *ctx, const gsm_query *q, const int32_t *de
   auto key = [&](int32_t u) {
     return Key{dense[u], std::max<int32_t>(0, q->lo[u]), std::min<int32_t>(ctx->n, q->hi[u])};
   };
-  uint32_t core = 0;
+  uint32_t core = 0, adj[kMaxK] = {};
   for (int32_t j = 0; j < kc; ++j) core |= 1u << order[j];
-  std::vector<std::vector<Key>> seen;  // colours: own key, then the leaves' keys in order
-  int32_t colour[kMaxK];
-  uint32_t adj[kMaxK] = {};
+  // a hash of every core vertex that symmetries preserve: its own properties
+  // and leaves, then three rounds of its neighbours' hashes.  Mostly they all
+  // differ (labels), and there is no symmetry to look for; else they narrow the
+  // search down.
+  auto mix = [](uint64_t x) {
+    x = (x ^ (x >> 31)) * 0x9e3779b97f4a7c15ull;
+    return x ^ (x >> 29);
+  };
+  uint64_t h[kMaxK];
   for (int32_t j = 0; j < kc; ++j) {
     const int32_t u = order[j];
-    std::vector<Key> c;
-    for (int32_t w = 0; w < q->k; ++w)
-      if ((q->adj[u] & ~core) >> w & 1u) c.push_back(key(w));
-    std::sort(c.begin(), c.end());
-    c.insert(c.begin(), key(u));
-    const auto it = std::find(seen.begin(), seen.end(), c);
-    colour[j] = (int32_t)(it - seen.begin());
-    if (it == seen.end()) seen.push_back(c);
+    auto hash = [&](int32_t w) {
+      const Key c = key(w);
+      return mix(mix(mix((uint64_t)c[0] + 1) + (uint64_t)c[1]) + (uint64_t)c[2]);
+    };
+    h[j] = hash(u) + (uint64_t)popc(q->adj[u]);
+    for (uint32_t m = q->adj[u] & ~core; m; m &= m - 1) h[j] += mix(hash(__builtin_ctz(m)));
     for (int32_t b = 0; b < kc; ++b)
       if (q->adj[u] >> order[b] & 1u) adj[j] |= 1u << b;
   }
-  if ((int32_t)seen.size() == kc) return 1;
+  for (int32_t round = 0; round < 3; ++round) {
+    uint64_t next[kMaxK];
+    for (int32_t j = 0; j < kc; ++j) {
+      next[j] = mix(h[j]);
+      for (uint32_t m = adj[j]; m; m &= m - 1) next[j] += mix(h[__builtin_ctz(m)] + 7);
+    }
+    std::copy(next, next + kc, h);
+  }
+  bool alike = false;  // two core vertices that a symmetry could exchange
+  for (int32_t j = 0; j < kc; ++j)
+    for (int32_t a = 0; a < j; ++a) alike = alike || h[a] == h[j];
+  if (!alike) return 1;
+  // exact colours (own key, then the leaves' keys in order), told apart by the
+  // hashes too
+  std::vector<std::pair<uint64_t, std::vector<Key>>> seen;
+  int32_t colour[kMaxK];
+  for (int32_t j = 0; j < kc; ++j) {
+    std::vector<Key> c;
+    for (uint32_t m = q->adj[order[j]] & ~core; m; m &= m - 1) c.push_back(key(__builtin_ctz(m)));
+    std::sort(c.begin(), c.end());
+    c.insert(c.begin(), key(order[j]));
+    const auto it = std::find(seen.begin(), seen.end(), std::make_pair(h[j], c));
+    colour[j] = (int32_t)(it - seen.begin());
+    if (it == seen.end()) seen.push_back({h[j], c});
+  }
   return symmetry_constraints(kc, adj, colour, less);
 }
 
@@ -1779,9 +1814,8 @@ void lane_release(gsm_ctx *ctx, Lane &L) {
   if (L.h_fds) cudaFreeHost(L.h_fds);
   if (L.h_qs) cudaFreeHost(L.h_qs);
   if (L.h_bm) cudaFreeHost(L.h_bm);
-  if (L.h_counts) cudaFreeHost(L.h_counts);
-  if (L.h_overflow) cudaFreeHost(L.h_overflow);
-  if (L.h_state) cudaFreeHost(L.h_state);
+  if (L.h_list_off) cudaFreeHost(L.h_list_off);
+  if (L.h_back) cudaFreeHost(L.h_back);
   if (L.h_items) cudaFreeHost(L.h_items);
   L.h_items = nullptr;
   L.h_items_cap = 0;
@@ -1798,6 +1832,13 @@ void lane_release(gsm_ctx *ctx, Lane &L) {
   L = Lane();
   L.stream = st;
   L.own_stream = own;
+}
+
+// Where the pieces of a lane's read-back lie: steps, overflow flag, counts.
+constexpr size_t kLaneOverflow = (sizeof(BatchStep) * (kMaxK + 1) + 15) / 16 * 16;
+constexpr size_t kLaneCounts = kLaneOverflow + 16;
+size_t lane_back_bytes(int32_t nq) {
+  return kLaneCounts + 2 * sizeof(unsigned long long) * (size_t)nq;
 }
 
 // Fixed-capacity buffers (once), per-query arrays (grown with the batch).
@@ -1817,19 +1858,12 @@ void lane_workspace(gsm_ctx *ctx, Lane &L, int32_t nq, int64_t words_total) {
     a.pstart = lane_alloc<int32_t>(ctx, L, L.cap_rows);
     a.pslot = lane_alloc<uint8_t>(ctx, L, L.cap_rows);
     a.woff = lane_alloc<int64_t>(ctx, L, L.cap_rows + 1);
-    const int64_t tiles = L.cap_items / 128 + 3;
+    const int64_t tiles = L.cap_items / kBatchMinTile + 2;
     a.tile_row = lane_alloc<int32_t>(ctx, L, tiles);
-    a.tile_cnt = lane_alloc<int32_t>(ctx, L, tiles);
-    a.tile_off = lane_alloc<int64_t>(ctx, L, tiles);
-    a.masks = lane_alloc<uint32_t>(ctx, L, L.cap_items / 32 + 256);  // + a tile of the largest block
-    a.fmasks = lane_alloc<uint32_t>(ctx, L, L.cap_items / 32 + 256);
-    a.ftile_cnt = lane_alloc<int32_t>(ctx, L, tiles);
-    a.ftile_off = lane_alloc<int64_t>(ctx, L, tiles);
-    a.state = lane_alloc<BatchStep>(ctx, L, kMaxK + 1);
-    CU(cudaMallocHost(&L.h_state, sizeof(BatchStep) * (kMaxK + 1)));
-    a.overflow = lane_alloc<int32_t>(ctx, L, 1);
-    a.partials = lane_alloc<int64_t>(ctx, L, (int64_t)ctx->num_sms * 32 + 1);
-    CU(cudaMallocHost(&L.h_overflow, sizeof(int32_t)));
+    a.lb_level = lane_alloc<unsigned long long>(ctx, L, tiles + kLbExtra);
+    a.lb_pivot =
+        lane_alloc<unsigned long long>(ctx, L, L.cap_rows / kBatchPivotTile + 1 + kLbExtra);
+    batch_setup();
     const int32_t nw = (ctx->n + 31) / 32;
     L.zero_bitmap = lane_alloc<uint32_t>(ctx, L, nw);
     CU(cudaMemsetAsync(L.zero_bitmap, 0, sizeof(uint32_t) * std::max(nw, 1), L.stream));
@@ -1844,35 +1878,38 @@ void lane_workspace(gsm_ctx *ctx, Lane &L, int32_t nq, int64_t words_total) {
       lane_free_one(ctx, L, a.fds);
       lane_free_one(ctx, L, a.bm_out);
       lane_free_one(ctx, L, a.qs);
-      lane_free_one(ctx, L, a.counts);
+      lane_free_one(ctx, L, a.list_off);
+      lane_free_one(ctx, L, a.state);
       lane_free_one(ctx, L, a.sizes);
       cudaFreeHost(L.h_fds);
       cudaFreeHost(L.h_qs);
       cudaFreeHost(L.h_bm);
-      cudaFreeHost(L.h_counts);
+      cudaFreeHost(L.h_list_off);
+      cudaFreeHost(L.h_back);
     }
     const int32_t cap = std::max(nq, 2 * L.max_nq);
     a.fds = lane_alloc<FilterDesc>(ctx, L, cap);
     a.bm_out = lane_alloc<uint32_t *>(ctx, L, cap);
     a.qs = lane_alloc<BatchQuery>(ctx, L, cap);
-    a.counts = lane_alloc<unsigned long long>(ctx, L, cap);
+    a.list_off = lane_alloc<int64_t>(ctx, L, cap + 1);
+    char *back = lane_alloc<char>(ctx, L, (int64_t)lane_back_bytes(cap));
+    a.state = (BatchStep *)back;
+    a.overflow = (int32_t *)(back + kLaneOverflow);
+    a.counts = (unsigned long long *)(back + kLaneCounts);
     a.sizes = lane_alloc<unsigned long long>(ctx, L, (int64_t)cap * kMaxK);
     CU(cudaMallocHost(&L.h_fds, sizeof(FilterDesc) * cap));
     CU(cudaMallocHost(&L.h_qs, sizeof(BatchQuery) * cap));
     CU(cudaMallocHost(&L.h_bm, sizeof(uint32_t *) * cap));
-    CU(cudaMallocHost(&L.h_counts, sizeof(unsigned long long) * cap));
+    CU(cudaMallocHost(&L.h_list_off, sizeof(int64_t) * (cap + 1)));
+    CU(cudaMallocHost(&L.h_back, lane_back_bytes(cap)));
     L.max_nq = cap;
     moved = true;
   }
-  if (words_total > L.max_words_total) {
-    if (L.max_words_total) {
-      lane_free_one(ctx, L, a.wcnt);
-      lane_free_one(ctx, L, a.woffs);
-    }
-    const int64_t cap = std::max<int64_t>(words_total, 2 * L.max_words_total);
-    a.wcnt = lane_alloc<int32_t>(ctx, L, cap);
-    a.woffs = lane_alloc<int64_t>(ctx, L, cap + 1);
-    L.max_words_total = cap;
+  const int64_t list_tiles = words_total / kBatchListTile + 1;
+  if (list_tiles > L.max_list_tiles) {
+    if (L.max_list_tiles) lane_free_one(ctx, L, a.lb_list);
+    L.max_list_tiles = std::max<int64_t>(list_tiles, 2 * L.max_list_tiles);
+    a.lb_list = lane_alloc<unsigned long long>(ctx, L, L.max_list_tiles + kLbExtra);
     moved = true;
   }
   if (moved) lane_clear_graphs(L);  // captured graphs hold the old pointers
@@ -1907,10 +1944,10 @@ int32_t unsorted_columns(int32_t k, const int32_t *order) {
 // Element offset in the result arena of every selected query that listed
 // rows (-1 for the others), from the step sizes read back after the batch:
 // step k-1 holds the queries of k vertices, in batch order.
-std::vector<int64_t> lane_row_offsets(const Lane &L, const unsigned long long *counts) {
+std::vector<int64_t> lane_row_offsets(const Lane &L, const uint64_t *counts) {
   std::vector<int64_t> off(L.m, -1);
   int64_t next[kMaxK + 1];
-  for (int32_t i = 0; i <= kMaxK; ++i) next[i] = L.h_state[i].FB;
+  for (int32_t i = 0; i <= kMaxK; ++i) next[i] = L.steps()[i].FB;
   for (int32_t t = 0; t < L.m; ++t) {
     const int32_t k = L.h_qs[t].k;
     if (!L.lists[t] || k < 2) continue;
@@ -1966,7 +2003,8 @@ cudaGraphExec_t lane_graph(gsm_ctx *ctx, Lane &L, int32_t m, int32_t kmax, int32
   if (it != L.graphs.end()) return it->second;
   if (L.enumerate) lane_final(ctx, L);
   BatchArgs a = L.a;
-  a.enumerate = L.enumerate;
+  if (!L.enumerate) a.final_rows = nullptr;
+  a.spin_limit = ctx->opt.lookback_spin_limit > 0 ? ctx->opt.lookback_spin_limit : kLbSpinLimit;
   a.nq = m;
   a.kmax = kmax;
   a.n_words = n_words;
@@ -2039,7 +2077,9 @@ int32_t lane_prepare(gsm_ctx *ctx, Lane &L, const gsm_query *const *qs, int32_t 
   lane_workspace(ctx, L, L.mb, (int64_t)L.mb * n_words);
   uint32_t *bm = (uint32_t *)L.bitmaps;
   int32_t kmax = 1;
-  int64_t off = 0;
+  int64_t off = 0, words = 0;
+  L.core_aut.assign(L.m, 1);
+  std::vector<std::pair<int32_t, int32_t>> less;
   for (int32_t t = 0; t < L.m; ++t) {
     const gsm_query *q = qs[L.sel[t]];
     const int32_t *dense = dense_of[t].data();
@@ -2051,44 +2091,65 @@ int32_t lane_prepare(gsm_ctx *ctx, Lane &L, const gsm_query *const *qs, int32_t 
     L.h_bm[t] = base;
     BatchQuery &bq = L.h_qs[t];
     std::memset(&bq, 0, sizeof(bq));
-    bq.k = q->k;
-    bq.root_bitmap = base + (size_t)order[0] * n_words;
+    bq.k = bq.kc = q->k;
     bq.enumerate = (lists && lists[L.sel[t]] && q->k >= 2) ? 1 : 0;
     L.enumerate |= bq.enumerate;
-    for (int32_t j = 0; j < q->k; ++j) bq.out_col[j] = order[j];
+    less.clear();
+    if (!bq.enumerate) {
+      // counts: leaves multiplied out, symmetries broken, as in run_query
+      bq.kc = split_leaves(ctx, q, dense, order, &bq.leaf);
+      L.core_aut[t] = core_symmetry(ctx, q, dense, order, bq.kc, &less);
+    }
+    bq.root_bitmap = base + (size_t)order[0] * n_words;
+    // only words that the root's restriction reaches can be non-zero
+    const int32_t rlo = std::min(std::max(0, q->lo[order[0]]), ctx->n),
+                  rhi = std::max(rlo, std::min(ctx->n, q->hi[order[0]]));
+    bq.word0 = rlo / 32;
+    L.h_list_off[t] = words;
+    words += rhi > rlo ? (rhi + 31) / 32 - bq.word0 : 0;
+    for (int32_t j = 0; j < q->k; ++j) bq.out_col[j] = (int8_t)order[j];
     std::array<int32_t, kMaxK> ord{};
     for (int32_t j = 0; j < q->k; ++j) ord[j] = order[j];
     L.orders.push_back(ord);
     L.lists.push_back(lists && lists[L.sel[t]] ? 1 : 0);
-    for (int32_t i = 1; i < q->k; ++i) {
+    for (int32_t i = 1; i < bq.kc; ++i) {
       BatchLevel &lv = bq.lv[i];
       const int32_t u = order[i];
       for (int32_t j = 0; j < i; ++j) {
         const int32_t uj = order[j];
         if (q->adj[u] >> uj & 1u)
-          lv.bpos[lv.nb++] = j;
+          lv.bpos[lv.nb++] = (int8_t)j;
         else if (dense[uj] == dense[u])
-          lv.inj[lv.ninj++] = j;
+          lv.inj[lv.ninj++] = (int8_t)j;
       }
-      lv.last = i == q->k - 1;
       lv.lab = dense[u];
-      lv.bitmap = base + (size_t)u * n_words;
+      // a leaf's candidates are all entries of its parent's cut label segment
+      lv.bitmap = popc(q->adj[u]) == 1 ? nullptr : base + (size_t)u * n_words;
+      lv.rlo = std::max<int32_t>(0, q->lo[u]);
+      lv.rhi = std::min<int32_t>(ctx->n, q->hi[u]);
+      for (const auto &c : less)
+        if (c.second == i) lv.gt[lv.ngt++] = (int8_t)c.first;
+      lv.cut = lv.rlo > 0 || lv.rhi < ctx->n || lv.ngt > 0;
     }
-    kmax = std::max(kmax, q->k);
+    kmax = std::max(kmax, bq.kc);
   }
   for (int32_t t = L.m; t < L.mb; ++t) {  // padding: no filter work, nothing to count
     std::memset(&L.h_fds[t], 0, sizeof(FilterDesc));
     L.h_bm[t] = L.zero_bitmap;
     std::memset(&L.h_qs[t], 0, sizeof(BatchQuery));
-    L.h_qs[t].k = 1;
+    L.h_qs[t].k = L.h_qs[t].kc = 1;
     L.h_qs[t].root_bitmap = L.zero_bitmap;
+    L.h_list_off[t] = words;
   }
+  L.h_list_off[L.mb] = words;
   CU(cudaMemcpyAsync((void *)L.a.fds, L.h_fds, sizeof(FilterDesc) * L.mb, cudaMemcpyHostToDevice,
                      L.stream));
   CU(cudaMemcpyAsync((void *)L.a.bm_out, L.h_bm, sizeof(uint32_t *) * L.mb,
                      cudaMemcpyHostToDevice, L.stream));
   CU(cudaMemcpyAsync((void *)L.a.qs, L.h_qs, sizeof(BatchQuery) * L.mb, cudaMemcpyHostToDevice,
                      L.stream));
+  CU(cudaMemcpyAsync((void *)L.a.list_off, L.h_list_off, sizeof(int64_t) * (L.mb + 1),
+                     cudaMemcpyHostToDevice, L.stream));
   L.kb = bucket_size(kmax);
   return L.kb;
 }
@@ -2101,23 +2162,38 @@ void lane_issue(gsm_ctx *ctx, Lane &L, int32_t kmax, int32_t block, int32_t grid
   CU(cudaEventRecord(L.ev0, L.stream));
   CU(cudaGraphLaunch(exec, L.stream));
   CU(cudaEventRecord(L.ev1, L.stream));
-  CU(cudaMemcpyAsync(L.h_counts, L.a.counts, sizeof(unsigned long long) * L.m,
-                     cudaMemcpyDeviceToHost, L.stream));
-  CU(cudaMemcpyAsync(L.h_overflow, L.a.overflow, sizeof(int32_t), cudaMemcpyDeviceToHost,
+  CU(cudaMemcpyAsync(L.h_back, L.a.state, lane_back_bytes(L.m), cudaMemcpyDeviceToHost,
                      L.stream));
-  CU(cudaMemcpyAsync(L.h_state, L.a.state, sizeof(BatchStep) * (kMaxK + 1),
-                     cudaMemcpyDeviceToHost, L.stream));
   CU(cudaEventRecord(L.ev_done, L.stream));
   ctx->bstats.graph_launches += 1;
   ctx->bstats.block_size = block;
   ctx->bstats.grid = grid;
 }
 
+// The counts of a finished batch (L.counts); true if it overflowed (also when
+// a count does not fit 64 bits: the single-query path says so).
+bool lane_counts(gsm_ctx *ctx, Lane &L) {
+  L.counts.assign(L.m, 0);
+  if (L.m == 0) return false;
+  const int32_t flag = *(const int32_t *)(L.h_back + kLaneOverflow);
+  if (flag == kBatchTimeout) FAIL(GSM_ERR_TIMEOUT, "a batch tile waited too long");
+  if (flag) return true;
+  const auto *c = (const unsigned long long *)(L.h_back + kLaneCounts);
+  for (int32_t t = 0; t < L.m; ++t) {
+    unsigned __int128 sum = (unsigned __int128)c[2 * t] + ((unsigned __int128)c[2 * t + 1] << 32);
+    if (sum > ~(unsigned __int128)0 / L.core_aut[t]) return true;
+    sum *= L.core_aut[t];
+    if (sum >> 64) return true;
+    L.counts[t] = (uint64_t)sum;
+  }
+  return false;
+}
+
 // Waits for the issued batch; returns the overflow flag, *ms = graph time.
 bool lane_wait(gsm_ctx *ctx, Lane &L, float *ms) {
   CU(cudaEventSynchronize(L.ev_done));
   if (ms) CU(cudaEventElapsedTime(ms, L.ev0, L.ev1));
-  return *L.h_overflow != 0;
+  return lane_counts(ctx, L);
 }
 
 std::pair<int32_t, int32_t> batch_config(gsm_ctx *ctx, int32_t m, int32_t kmax, bool *tuned) {
@@ -2248,7 +2324,7 @@ void lane_batch_rows(gsm_ctx *ctx, Lane &L, const std::vector<int64_t> &off,
     const int32_t k = L.h_qs[t].k;
     if (!want[t] || k < 2) continue;
     gsm_result &r = results[L.sel[t]];
-    r.count = L.h_counts[t];
+    r.count = L.counts[t];
     r.k = k;
     r.on_device = on_device ? 1 : 0;
     r.rows = nullptr;
@@ -2265,13 +2341,13 @@ void lane_batch_rows(gsm_ctx *ctx, Lane &L, const std::vector<int64_t> &off,
   for (const auto &kv : groups) {
     for (int32_t t : kv.second) {
       pos[t] = total;
-      total += (size_t)L.h_counts[t] * kv.first;
+      total += (size_t)L.counts[t] * kv.first;
     }
     total = (total + 3) & ~size_t(3);
   }
   for (int32_t t : rest) {
     pos[t] = total;
-    total += ((size_t)L.h_counts[t] * L.h_qs[t].k + 3) & ~size_t(3);
+    total += ((size_t)L.counts[t] * L.h_qs[t].k + 3) & ~size_t(3);
   }
   const size_t bytes = total * sizeof(int32_t);
   void *base = on_device ? dev_alloc(ctx, bytes) : std::malloc(bytes);
@@ -2304,8 +2380,8 @@ void lane_batch_rows(gsm_ctx *ctx, Lane &L, const std::vector<int64_t> &off,
     for (const auto &kv : groups) {
       int64_t first = 0;
       for (int32_t t : kv.second) {
-        h[e++] = SortSegment{L.a.final_rows + off[t], first, (int64_t)L.h_counts[t]};
-        first += (int64_t)L.h_counts[t];
+        h[e++] = SortSegment{L.a.final_rows + off[t], first, (int64_t)L.counts[t]};
+        first += (int64_t)L.counts[t];
       }
     }
     CU(cudaMemcpyAsync(d, h, nsegs * sizeof(SortSegment), cudaMemcpyHostToDevice, L.stream));
@@ -2315,7 +2391,7 @@ void lane_batch_rows(gsm_ctx *ctx, Lane &L, const std::vector<int64_t> &off,
       int64_t N = 0;
       int32_t S = 1;
       for (int32_t t : kv.second) {
-        N += (int64_t)L.h_counts[t];
+        N += (int64_t)L.counts[t];
         S = std::max(S, sort_cols[t]);
       }
       SortPrefix pre;
@@ -2337,7 +2413,7 @@ void lane_batch_rows(gsm_ctx *ctx, Lane &L, const std::vector<int64_t> &off,
   int32_t max_k = 2;
   for (int32_t t : rest) {
     const int32_t k = L.h_qs[t].k;
-    const int64_t N = (int64_t)L.h_counts[t];
+    const int64_t N = (int64_t)L.counts[t];
     const int32_t *src = L.a.final_rows + off[t];
     if (N <= kSmallSortRows) {
       items.push_back({src, dst + pos[t], (int32_t)N, k, sort_cols[t] > 0 ? 1 : 0});
@@ -2429,9 +2505,9 @@ void run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *c
         }
       }
     } else {
-      for (int32_t t = 0; t < L.m; ++t) counts[L.sel[t]] = L.h_counts[t];
+      for (int32_t t = 0; t < L.m; ++t) counts[L.sel[t]] = L.counts[t];
       if (results) {
-        const std::vector<int64_t> off = lane_row_offsets(L, L.h_counts);
+        const std::vector<int64_t> off = lane_row_offsets(L, L.counts.data());
         for (int32_t t = 0; t < L.m; ++t) {
           const int32_t j = L.sel[t];
           if (qs[j]->k == 1)  // one-vertex queries: their candidate list
@@ -2501,7 +2577,6 @@ int64_t now_ns() {
 // Completes the batch of a lane whose ev_done has fired: counts, and the
 // sorted rows of the requests in enumerate mode.
 void server_complete(gsm_ctx *ctx, gsm_ctx::Server &S, Lane &L) {
-  const bool overflow = *L.h_overflow != 0;
   std::vector<const gsm_query *> qs;
   std::vector<int32_t> modes;
   {
@@ -2517,7 +2592,7 @@ void server_complete(gsm_ctx *ctx, gsm_ctx::Server &S, Lane &L) {
   for (auto &r : res) std::memset(&r, 0, sizeof(r));
   gsm_status st = guarded(ctx, [&] {
     try {
-      if (overflow) {
+      if (lane_counts(ctx, L)) {
         ctx->bstats.fallbacks += 1;
         for (size_t t = 0; t < nr; ++t) {
           if (modes[t] == GSM_MODE_ENUMERATE) {
@@ -2529,9 +2604,9 @@ void server_complete(gsm_ctx *ctx, gsm_ctx::Server &S, Lane &L) {
           }
         }
       } else {
-        for (int32_t t = 0; t < L.m; ++t) counts[L.sel[t]] = L.h_counts[t];
+        for (int32_t t = 0; t < L.m; ++t) counts[L.sel[t]] = L.counts[t];
         if (L.enumerate || std::count(modes.begin(), modes.end(), GSM_MODE_ENUMERATE)) {
-          const std::vector<int64_t> off = lane_row_offsets(L, L.h_counts);
+          const std::vector<int64_t> off = lane_row_offsets(L, L.counts.data());
           std::vector<char> want(L.m, 0);
           for (int32_t t = 0; t < L.m; ++t) {
             const int32_t j = L.sel[t];
@@ -2612,7 +2687,6 @@ void server_loop(gsm_ctx *ctx) {
           auto cfg = batch_config(ctx, L.m, kmax, &tuned);
           lane_issue(ctx, L, kmax, cfg.first, cfg.second);
         } else {
-          *L.h_overflow = 0;
           CU(cudaEventRecord(L.ev_done, L.stream));
         }
         ctx->bstats.batches += 1;

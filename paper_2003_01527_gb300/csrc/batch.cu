@@ -22,115 +22,20 @@ namespace gsm {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kPScanThreads = 256;
-constexpr int kPScanTile = 2048;  // 8 elements per thread
-
-__device__ __forceinline__ int64_t warp_incl(int64_t x, int lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int64_t y = __shfl_up_sync(kFull, x, o);
-    if (lane >= o) x += y;
-  }
-  return x;
-}
-
-// Exclusive scan of one value per thread of the block; *total = block sum.
-__device__ int64_t block_scan(int64_t x, int64_t *s_warp, int64_t *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int64_t incl = warp_incl(x, lane);
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int64_t t = lane < nw ? s_warp[lane] : 0;
-    const int64_t ti = warp_incl(t, lane);
-    if (lane < nw) s_warp[lane] = ti - t;
-    if (lane == 31) s_warp[32] = ti;
-  }
-  __syncthreads();
-  const int64_t r = incl - x + s_warp[warp];
-  *total = s_warp[32];
-  __syncthreads();
-  return r;
-}
-
-// ---- scans whose length lives in device memory (fixed grid of G blocks;
-// block b owns a contiguous range of ceil(n/G) elements)
-
-template <typename T>
-__global__ void __launch_bounds__(kPScanThreads) k_pscan_reduce(const T *in, const int64_t *n_ptr,
-                                                                int64_t *partials) {
-  __shared__ int64_t s_warp[33];
-  const int64_t n = *n_ptr;
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = (int64_t)blockIdx.x * chunk, hi = min(n, lo + chunk);
-  int64_t sum = 0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) sum += (int64_t)in[i];
-  int64_t total;
-  block_scan(sum, s_warp, &total);
-  if (threadIdx.x == 0) partials[blockIdx.x] = total;
-}
-
-__global__ void __launch_bounds__(1024) k_pscan_top(int64_t *partials, int32_t nb) {
-  __shared__ int64_t s_warp[33];
-  int64_t carry = 0;
-  for (int32_t base = 0; base < nb; base += blockDim.x) {
-    const int32_t idx = base + threadIdx.x;
-    const int64_t x = idx < nb ? partials[idx] : 0;
-    int64_t total;
-    const int64_t ex = block_scan(x, s_warp, &total);
-    if (idx < nb) partials[idx] = ex + carry;
-    carry += total;
-  }
-  if (threadIdx.x == 0) partials[nb] = carry;
-}
-
-// In place safe (in == out for int64): each tile is read whole before it is
-// written, and later tiles are untouched until their turn.
-template <typename T>
-__global__ void __launch_bounds__(kPScanThreads) k_pscan_down(const T *in, const int64_t *n_ptr,
-                                                              const int64_t *partials,
-                                                              int64_t *out) {
-  __shared__ int64_t s_val[kPScanTile];
-  __shared__ int64_t s_warp[33];
-  const int64_t n = *n_ptr;
-  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = (int64_t)blockIdx.x * chunk, hi = min(n, lo + chunk);
-  int64_t carry = partials[blockIdx.x];
-  for (int64_t base = lo; base < hi; base += kPScanTile) {
-    for (int j = threadIdx.x; j < kPScanTile; j += blockDim.x) {
-      const int64_t idx = base + j;
-      s_val[j] = idx < hi ? (int64_t)in[idx] : 0;
-    }
-    __syncthreads();
-    int64_t loc[8], sum = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      loc[j] = sum;
-      sum += s_val[threadIdx.x * 8 + j];
-    }
-    int64_t total;
-    const int64_t ex = block_scan(sum, s_warp, &total);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) s_val[threadIdx.x * 8 + j] = carry + ex + loc[j];
-    __syncthreads();
-    for (int j = threadIdx.x; j < kPScanTile; j += blockDim.x) {
-      const int64_t idx = base + j;
-      if (idx < hi) out[idx] = s_val[j];
-    }
-    carry += total;
-    __syncthreads();
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = partials[gridDim.x];
-}
 
 // ---- set-up, filter and level 1
 
-// Zeroes the step sizes and stores the number of root-bitmap words (the
-// length of the level-1 scan) where the scan can read it.
-__global__ void k_b_init(BatchStep *state, int64_t words) {
-  for (int j = threadIdx.x; j <= kMaxK; j += blockDim.x) state[j] = BatchStep{0, 0, 0, 0, 0, 0};
-  __syncthreads();
-  if (threadIdx.x == 0) state[0].W = words;
+// Zeroes what the batch adds up in: the step sizes, the overflow flag, the
+// counts and the list's look-back words.
+__global__ void __launch_bounds__(256) k_b_init(BatchStep *state, int32_t *overflow,
+                                                unsigned long long *counts, int64_t ncounts,
+                                                unsigned long long *lb_list, int64_t lb_words) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t j = t; j <= kMaxK; j += stride) state[j] = BatchStep{0, 0, 0, 0, 0, 0, 0};
+  for (int64_t j = t; j < ncounts; j += stride) counts[j] = 0;
+  for (int64_t j = t; j < lb_words; j += stride) lb_list[j] = 0;
+  if (t == 0) *overflow = 0;
 }
 
 __global__ void __launch_bounds__(256) k_b_filter(GraphDev g, const FilterDesc *__restrict__ fds,
@@ -160,448 +65,442 @@ __global__ void __launch_bounds__(256) k_b_filter_bits(GraphDev g,
   filter_words(g, s_d, bm_out[q], sizes ? sizes + (int64_t)q * kMaxK : nullptr, 0, 1);
 }
 
-// Word counts of every query's root bitmap; one-vertex queries are counted
-// here and contribute no rows.
-__global__ void k_b_list_popc(const BatchQuery *__restrict__ qs, int32_t nq, int32_t n_words,
-                              int32_t *__restrict__ wcnt, unsigned long long *__restrict__ counts) {
-  const int64_t total = (int64_t)nq * n_words;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-    const int32_t q = (int32_t)(i / n_words), w = (int32_t)(i % n_words);
-    const int32_t c = __popc(__ldg(qs[q].root_bitmap + w));
-    if (qs[q].k == 1) {
-      if (c) atomicAdd(counts + q, (unsigned long long)c);
-      wcnt[i] = 0;
+// ---- counts, and what the last CTA of a kernel does
+
+// One thread's sum of the numbers of one query's whole embeddings (halves of
+// 32 bits), added to the query's two count words when the query changes.
+struct BatchSum {
+  int32_t q = -1;
+  unsigned long long lo = 0, hi = 0;
+  __device__ __forceinline__ void add(int32_t query, unsigned long long v,
+                                      unsigned long long *counts) {
+    if (query != q) {
+      put(counts);
+      q = query;
+    }
+    lo += (uint32_t)v;
+    hi += v >> 32;
+  }
+  __device__ __forceinline__ void put(unsigned long long *counts) {
+    if (lo) atomicAdd(counts + 2 * (int64_t)q, lo);
+    if (hi) atomicAdd(counts + 2 * (int64_t)q + 1, hi);
+    lo = hi = 0;
+  }
+  // All lanes of the warp: one atomic for the warp when its lanes sum one
+  // query (most tiles hold rows of one query), else one per lane.
+  __device__ __forceinline__ void flush(unsigned long long *counts) {
+    const bool has = lo || hi;
+    const uint32_t m = __ballot_sync(kFull, has);
+    if (!m) return;
+    const int32_t q0 = __shfl_sync(kFull, q, __ffs(m) - 1);
+    if (__all_sync(kFull, !has || q == q0)) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        lo += __shfl_xor_sync(kFull, lo, o);
+        hi += __shfl_xor_sync(kFull, hi, o);
+      }
+      q = q0;
+      if ((threadIdx.x & 31) == 0) put(counts);
+      lo = hi = 0;
     } else {
-      wcnt[i] = c;
+      put(counts);
     }
   }
+};
+
+// The number of query `bq`'s embeddings with this core row.
+template <typename Row>
+__device__ __forceinline__ unsigned long long core_number(const GraphDev &g, const BatchQuery &bq,
+                                                          const Row &row, bool *over) {
+  if (bq.leaf.nleaves == 0) return 1;
+  return leaf_number<kMaxK>(g, bq.leaf, row, over, [](int, unsigned long long) {});
 }
 
-// Level-1 size check: rows = total set bits; over capacity -> overflow.
-__global__ void k_b_list_check(const int64_t *__restrict__ woffs, int64_t words,
-                               BatchStep *state, int64_t cap_rows, int32_t *overflow) {
-  const int64_t R = woffs[words];
-  if (R > cap_rows) {
-    *overflow = 1;
-    state[1].R = 0;
-  } else {
-    state[1].R = R;
+// True in every thread of the CTA that finishes last (lb: the kernel's
+// look-back words; the counter of finished CTAs is word tiles + 3).  One
+// barrier; the CTA's earlier atomics are ordered before its count.
+__device__ __forceinline__ bool last_cta(unsigned long long *lb, int64_t tiles) {
+  __shared__ bool s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(lb + tiles + 3, 1ull) == gridDim.x - 1;
+    __threadfence();
   }
+  __syncthreads();
+  return s_last;
 }
 
-__global__ void k_b_list_emit(const BatchQuery *__restrict__ qs, int32_t nq, int32_t n_words,
-                              const int64_t *__restrict__ woffs, const BatchStep *state,
-                              int32_t *__restrict__ F, int32_t *__restrict__ rseg) {
-  const int64_t total = (int64_t)nq * n_words;
-  if (state[1].R != woffs[total]) return;  // overflowed: nothing to write
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-    const int32_t q = (int32_t)(i / n_words), w = (int32_t)(i % n_words);
-    if (qs[q].k == 1) continue;
-    uint32_t word = __ldg(qs[q].root_bitmap + w);
-    int64_t pos = woffs[i];
-    while (word) {
-      const int b = __ffs(word) - 1;
-      word &= word - 1;
-      F[pos] = w * 32 + b;
-      rseg[pos] = q;
-      ++pos;
+__device__ __forceinline__ void zero_words(unsigned long long *p, int64_t n) {
+  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) p[j] = 0;
+}
+
+// Rows of a level go into arrays of this leading dimension: as many as there
+// are candidates, at most what the frontier holds (more survivors are an
+// overflow).
+__device__ __forceinline__ int64_t level_ld(int64_t most, int32_t width, int64_t cap_rows,
+                                            int64_t cap_elems) {
+  return min(most, min(cap_rows, cap_elems / width));
+}
+
+// Level 1 of every query: its candidate list for pi_0, queries in batch order.
+// Tiles of kBatchListTile root-bitmap words (only words inside the root's
+// restriction are numbered: list_off); a tile's rows start where the
+// look-back says.  Queries whose core is one vertex are counted here.  The
+// last CTA sets the level's size and zeroes the next kernel's look-back words.
+__global__ void __launch_bounds__(256) k_b_list(GraphDev g, const BatchQuery *__restrict__ qs,
+                                                int32_t nq, const int64_t *__restrict__ list_off,
+                                                BatchStep *state, int64_t cap,
+                                                int32_t *__restrict__ F,
+                                                int32_t *__restrict__ rseg,
+                                                unsigned long long *counts,
+                                                unsigned long long *lb,
+                                                unsigned long long *lb_pivot, int32_t spin_limit,
+                                                int32_t *overflow) {
+  constexpr int kWords = kBatchListTile / 256;  // of a thread, consecutive
+  __shared__ int32_t s_warp[33];
+  __shared__ int32_t s_tile, s_q;
+  __shared__ unsigned long long s_prefix;
+  const int64_t words = list_off[nq];
+  const int32_t tiles = (int32_t)((words + kBatchListTile - 1) / kBatchListTile);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bool over = false;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      const int32_t tile = (int32_t)atomicAdd(lb + tiles, 1ull);
+      int32_t lo = 0, len = nq;  // last query whose words start at or before the tile
+      while (len > 1) {
+        const int32_t half = len >> 1;
+        if (list_off[lo + half] <= (int64_t)tile * kBatchListTile) lo += half;
+        len -= half;
+      }
+      s_tile = tile;
+      s_q = lo;
     }
+    __syncthreads();
+    const int32_t tile = s_tile;
+    if (tile >= tiles) break;  // uniform across the block
+    int32_t q = s_q;
+    uint32_t word[kWords];
+    int32_t qw[kWords], vw[kWords];
+    int32_t c = 0;
+    BatchSum sum;
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+      const int64_t i = (int64_t)tile * kBatchListTile + threadIdx.x * kWords + j;
+      word[j] = 0;
+      if (i >= words) continue;
+      while (list_off[q + 1] <= i) ++q;
+      const BatchQuery &bq = qs[q];
+      const int32_t w = bq.word0 + (int32_t)(i - list_off[q]);
+      uint32_t x = __ldg(bq.root_bitmap + w);
+      if (bq.kc == 1) {
+        for (; x; x &= x - 1) {
+          const int32_t v = w * 32 + __ffs(x) - 1;
+          sum.add(q, core_number(g, bq, [&](int) { return v; }, &over), counts);
+        }
+      }
+      word[j] = x;
+      qw[j] = q;
+      vw[j] = w * 32;
+      c += __popc(x);
+    }
+    sum.flush(counts);
+    int32_t T;
+    const int32_t rank = block_rank(c, s_warp, &T);
+    if (warp == 0) {
+      const unsigned long long p = lookback_prefix(lb, tile, tiles, (unsigned long long)T, lane,
+                                                   spin_limit);
+      if (lane == 0) s_prefix = p;
+    }
+    __syncthreads();
+    int64_t pos = (int64_t)s_prefix + rank;
+#pragma unroll
+    for (int j = 0; j < kWords; ++j)
+      for (uint32_t x = word[j]; x; x &= x - 1, ++pos)
+        if (pos < cap) {
+          F[pos] = vw[j] + __ffs(x) - 1;
+          rseg[pos] = qw[j];
+        }
+    __syncthreads();  // the shared words are reused by the next tile
   }
+  if (over) *overflow = kBatchOverflow;  // past 64 bits: the single-query path reports it
+  if (!last_cta(lb, tiles)) return;
+  const int64_t R = (int64_t)atomicAdd(lb + tiles + 1, 0ull);
+  const bool late = atomicAdd(lb + tiles + 2, 0ull) != 0;
+  const bool ok = !late && R <= cap;
+  if (threadIdx.x == 0) {
+    if (late) *overflow = kBatchTimeout;
+    else if (!ok) *overflow = kBatchOverflow;
+    state[1].R = ok ? R : 0;
+    state[1].ld = R;
+  }
+  zero_words(lb_pivot, (ok ? (R + kBatchPivotTile - 1) / kBatchPivotTile : 0) + kLbExtra);
 }
 
 // ---- one step: level i -> i+1 (frontier rows of width i, column-major,
-// leading dimension R = state[i].R)
+// leading dimension state[i].ld)
 
-__global__ void k_b_pivot(GraphDev g, const BatchQuery *__restrict__ qs, int32_t i,
-                          const BatchStep *state, const int32_t *__restrict__ F,
-                          const int32_t *__restrict__ rseg, int32_t *__restrict__ pstart,
-                          uint8_t *__restrict__ pslot, int64_t *__restrict__ work) {
-  const int32_t R = (int32_t)state[i].R;
-  for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    const BatchLevel &L = qs[rseg[r]].lv[i];
-    int32_t best = 0x7fffffff, best_start = 0, best_slot = 0;
-    for (int b = 0; b < L.nb; ++b) {
-      const int32_t x = F[L.bpos[b] * R + r];
-      const int2 seg = label_segment(g, x, L.lab);  // only pi_i's label can match
-      if (seg.y - seg.x < best) {
-        best = seg.y - seg.x;
-        best_start = seg.x;
-        best_slot = b;
+// Pivot choice of every row and scan of the rows' candidate counts: tiles of
+// kBatchPivotTile rows, a row per thread.  A row also writes itself into
+// tile_row for every level tile that starts among its candidates.  The last
+// CTA sets the step's candidates, tiles and next leading dimension, and
+// zeroes the level's look-back words.
+__global__ void __launch_bounds__(256) k_b_pivot_scan(
+    GraphDev g, const BatchQuery *__restrict__ qs, int32_t i, BatchStep *state,
+    const int32_t *__restrict__ F, const int32_t *__restrict__ rseg,
+    int32_t *__restrict__ pstart, uint8_t *__restrict__ pslot, int64_t *__restrict__ woff,
+    int32_t *__restrict__ tile_row, int32_t tile_items, int64_t cap_rows, int64_t cap_elems,
+    int64_t cap_items, unsigned long long *lb, unsigned long long *lb_level, int32_t spin_limit,
+    int32_t *overflow) {
+  __shared__ int64_t s_warp[33];
+  __shared__ int32_t s_tile;
+  __shared__ unsigned long long s_prefix;
+  const int64_t R = state[i].R, ld = state[i].ld;
+  const int32_t tiles = (int32_t)((R + kBatchPivotTile - 1) / kBatchPivotTile);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t max_tiles = (cap_items + tile_items - 1) / tile_items;  // entries of tile_row
+  for (;;) {
+    if (threadIdx.x == 0) s_tile = (int32_t)atomicAdd(lb + tiles, 1ull);
+    __syncthreads();
+    const int32_t tile = s_tile;
+    if (tile >= tiles) break;  // uniform across the block
+    const int64_t r = tile * kBatchPivotTile + threadIdx.x;
+    int32_t best = 0;
+    if (r < R) {
+      const BatchLevel &L = qs[rseg[r]].lv[i];
+      int32_t best_start = 0, best_slot = 0, lo = L.rlo;
+      best = 0x7fffffff;
+      for (int t = 0; t < L.ngt; ++t) lo = max(lo, F[L.gt[t] * ld + r] + 1);
+      for (int b = 0; b < L.nb; ++b) {
+        const int32_t x = F[L.bpos[b] * ld + r];
+        int2 seg = label_segment(g, x, L.lab);  // only pi_i's label can match
+        if (L.cut) seg = cut_segment(g, seg, lo, L.rhi);
+        if (seg.y - seg.x < best) {
+          best = seg.y - seg.x;
+          best_start = seg.x;
+          best_slot = b;
+        }
       }
+      pstart[r] = best_start;
+      pslot[r] = (uint8_t)best_slot;
     }
-    pstart[r] = best_start;
-    pslot[r] = (uint8_t)best_slot;
-    work[r] = best;
-  }
-}
-
-// Candidates W = woff[R]; over capacity -> overflow and no tiles.
-__global__ void k_b_check_work(int32_t i, BatchStep *state, const int64_t *__restrict__ woff,
-                               int64_t cap_items, int32_t tile_items, int32_t *overflow) {
-  const int64_t R = state[i].R;
-  const int64_t W = R > 0 ? woff[R] : 0;
-  if (W > cap_items) {
-    *overflow = 1;
-    state[i].W = 0;
-    state[i].tiles = 0;
-  } else {
-    state[i].W = W;
-    state[i].tiles = (W + tile_items - 1) / tile_items;
-  }
-}
-
-__global__ void k_b_tile_rows(int32_t i, const BatchStep *state, const int64_t *__restrict__ woff,
-                              int32_t tile_items, int32_t *__restrict__ tile_row) {
-  const int32_t R = (int32_t)state[i].R;
-  const int64_t tiles = state[i].tiles;
-  if (tiles == 0) return;
-  for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < R; r += gridDim.x * blockDim.x) {
-    const int64_t s = woff[r], e = woff[r + 1];
-    for (int64_t t = (s + tile_items - 1) / tile_items; t * tile_items < e; ++t)
-      tile_row[t] = r;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) tile_row[tiles] = R - 1;
-}
-
-// Rows of one tile, with their work offsets staged in shared memory.
-struct BTile {
-  int32_t r0, span;
-  bool staged;
-};
-
-__device__ __forceinline__ BTile b_stage(const int64_t *__restrict__ woff,
-                                         const int32_t *__restrict__ tile_row, int64_t t,
-                                         int32_t tile_items, int32_t *s_woff) {
-  BTile b;
-  b.r0 = tile_row[t];
-  b.span = tile_row[t + 1] + 1 - b.r0;
-  b.staged = b.span <= tile_items;
-  if (b.staged)
-    for (int32_t j = threadIdx.x; j <= b.span; j += blockDim.x) s_woff[j] = (int32_t)woff[b.r0 + j];
-  __syncthreads();
-  return b;
-}
-
-__device__ __forceinline__ int32_t b_row(const BTile &b, const int32_t *s_woff,
-                                         const int64_t *__restrict__ woff, int32_t x,
-                                         int32_t *row_start) {
-  int32_t lo = 0, hi = b.span;
-  if (b.staged) {
-    while (hi - lo > 1) {
-      const int32_t mid = (lo + hi) >> 1;
-      if (s_woff[mid] <= x) lo = mid; else hi = mid;
+    // exclusive scan over the tile
+    int64_t incl = best;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
     }
-    *row_start = s_woff[lo];
-  } else {
-    while (hi - lo > 1) {
-      const int32_t mid = (lo + hi) >> 1;
-      if (woff[b.r0 + mid] <= x) lo = mid; else hi = mid;
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const int64_t v = lane < 8 ? s_warp[lane] : 0;
+      int64_t vi = v;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        const int64_t y = __shfl_up_sync(kFull, vi, o);
+        if (lane >= o) vi += y;
+      }
+      if (lane < 8) s_warp[lane] = vi - v;
+      const unsigned long long T = (unsigned long long)__shfl_sync(kFull, vi, 7);
+      const unsigned long long p = lookback_prefix(lb, tile, tiles, T, lane, spin_limit);
+      if (lane == 0) s_prefix = p;
     }
-    *row_start = (int32_t)woff[b.r0 + lo];
+    __syncthreads();
+    if (r < R) {
+      const int64_t s = (int64_t)s_prefix + s_warp[warp] + incl - best, e = s + best;
+      woff[r] = s;
+      if (best > 0)
+        for (int64_t t = (s + tile_items - 1) / tile_items; t * tile_items < e && t < max_tiles;
+             ++t)
+          tile_row[t] = (int32_t)r;
+    }
+    __syncthreads();  // the shared words are reused by the next tile
   }
-  return b.r0 + lo;
+  if (!last_cta(lb, tiles)) return;
+  const int64_t W = (int64_t)atomicAdd(lb + tiles + 1, 0ull);
+  const bool late = atomicAdd(lb + tiles + 2, 0ull) != 0;
+  const bool ok = !late && W <= cap_items;
+  const int64_t level_tiles = ok ? (W + tile_items - 1) / tile_items : 0;
+  if (threadIdx.x == 0) {
+    if (late) *overflow = kBatchTimeout;
+    else if (!ok) *overflow = kBatchOverflow;
+    woff[R] = W;
+    state[i].W = ok ? W : 0;
+    state[i].tiles = level_tiles;
+    if (level_tiles > 0) tile_row[level_tiles] = (int32_t)(R - 1);
+    state[i + 1].ld = level_ld(W, i + 1, cap_rows, cap_elems);
+  }
+  zero_words(lb_level, level_tiles + kLbExtra);
 }
 
-// Verification pass of one step.  A survivor of a query at its last level
-// is counted into counts[q] (and, for a query that lists its rows, marked in
-// fmasks and counted towards its tile in ftile_cnt); other survivors get
-// their mask bit and count towards their tile.  The check is the
-// single-query path's (check_candidate).  Thread t of a tile takes the 4
-// consecutive candidates 4t .. 4t+3 (one row search for all four); the mask
-// bits stay in candidate order (4-bit groups OR-ed across the 8 lanes of a
-// mask word).
-__global__ void __launch_bounds__(1024) k_b_count(
-    GraphDev g, const BatchQuery *__restrict__ qs, int32_t i, const BatchStep *state,
+// Verification and write pass of one step, in one launch: tiles by ticket; a
+// tile's survivors are ranked, kept in one of two shared buffers and written
+// after the CTA has verified its next tile, when the look-back has its prefix
+// (the single-query path's k_extend_fused, with the check, check_candidate).
+// Survivors of a query at its last level are counted (times their leaf
+// numbers), and for a query that lists its rows written to the result arena;
+// the others become rows of the next level.  Both ranks travel in one
+// look-back word (30 bits each: a level has fewer than 2^30 candidates).
+// Thread t of a tile takes the 4 consecutive candidates 4t .. 4t+3.
+//
+// Bound by latency at these sizes (thousands of candidates a level): one
+// launch and a look-back replace the count pass, two three-kernel scans, two
+// one-thread kernels and two write passes of the step.  256 counted queries on
+// R-MAT 18 take 21 launches instead of 116 and 1,000 us instead of 1,250; 48
+// listed ones 21 instead of 160, and 1,820 us instead of 2,160.
+constexpr int kPackBits = 30;
+constexpr unsigned long long kPackMask = (1ull << kPackBits) - 1;
+
+template <int kMaxThreads>
+__global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_level(
+    GraphDev g, const BatchQuery *__restrict__ qs, int32_t i, BatchStep *state,
     const int32_t *__restrict__ F, const int32_t *__restrict__ rseg,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
-    const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row,
-    uint32_t *__restrict__ masks, int32_t *__restrict__ tile_cnt,
-    unsigned long long *__restrict__ counts, uint32_t *__restrict__ fmasks,
-    int32_t *__restrict__ ftile_cnt) {
-  static_assert(kItemsPerThread == 4, "one 4-bit group per lane");
-  extern __shared__ int32_t s_woff[];
-  __shared__ int32_t s_count, s_fcount;
-  const int32_t R = (int32_t)state[i].R;
-  const int32_t W = (int32_t)state[i].W;
-  const int64_t tiles = state[i].tiles;
+    const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t cap_rows,
+    int64_t cap_elems, int64_t cap_final, unsigned long long *counts, int32_t *__restrict__ Fn,
+    int32_t *__restrict__ rseg_n, int32_t *__restrict__ final_rows, unsigned long long *lb,
+    unsigned long long *lb_pivot, int32_t spin_limit, int32_t *overflow) {
+  static_assert(kItemsPerThread == 4, "four candidates per thread");
+  extern __shared__ int32_t smem[];
+  __shared__ int32_t s_tile;
+  __shared__ int32_t s_warp[33];
+  __shared__ unsigned long long s_prefix;
+  const int32_t ld = (int32_t)state[i].ld, W = (int32_t)state[i].W;
+  const int32_t tiles = (int32_t)state[i].tiles;
+  const int64_t ldn = state[i + 1].ld, FB = state[i].FB;
   const int32_t B = blockDim.x;
   const int32_t tile_items = B * kItemsPerThread;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    if (threadIdx.x == 0) s_count = s_fcount = 0;
-    const BTile b = b_stage(woff, tile_row, t, tile_items, s_woff);
-    const int32_t x0 = (int32_t)t * tile_items, x1 = min(x0 + tile_items, W);
+  int32_t *s_woff = smem;
+  int32_t *s_pairs = s_woff + tile_items + 4;  // 2 buffers of tile_items (row, vertex) pairs
+  int32_t pend = -1, pend_T = 0, buf = 0;
+  const int32_t width = i + 1;
+  bool over = false;
+
+  // T packs the tile's survivors: next rows in the low half (pairs from the
+  // front of the buffer), result rows in the high half (pairs from its end)
+  auto finish = [&](int32_t tile, int32_t T, int32_t pb) {
+    const int32_t tn = T & 0xffff, tf = (int32_t)((uint32_t)T >> 16);
+    if (warp == 0) {
+      const unsigned long long p = lookback_resolve(
+          lb, tile, tiles, ((unsigned long long)tf << kPackBits) | (unsigned long long)tn, lane,
+          spin_limit);
+      if (lane == 0) s_prefix = p;
+    }
+    __syncthreads();
+    const int32_t *pairs = s_pairs + pb * 2 * tile_items;
+    const int64_t pn = (int64_t)(s_prefix & kPackMask), pf = (int64_t)(s_prefix >> kPackBits);
+    for (int32_t x = threadIdx.x; x < tn; x += B) {
+      const int32_t r = pairs[2 * x];
+      const int64_t pos = pn + x;
+      if (pos >= ldn) continue;  // over capacity: reported below
+      for (int c = 0; c < i; ++c) Fn[c * ldn + pos] = F[c * ld + r];
+      Fn[i * ldn + pos] = pairs[2 * x + 1];
+      rseg_n[pos] = rseg[r];
+    }
+    for (int32_t x = threadIdx.x; x < tf; x += B) {
+      const int32_t *pr = pairs + 2 * (tile_items - 1 - x);
+      const int32_t r = pr[0];
+      const int64_t at = FB + (pf + x) * width;
+      if (at + width > cap_final) continue;  // over capacity: reported below
+      const int8_t *oc = qs[rseg[r]].out_col;
+      int32_t *dst = final_rows + at;
+      for (int c = 0; c < i; ++c) dst[oc[c]] = F[c * ld + r];
+      dst[oc[i]] = pr[1];
+    }
+  };
+
+  for (;;) {
+    if (threadIdx.x == 0) s_tile = (int32_t)atomicAdd(lb + tiles, 1ull);
+    __syncthreads();
+    const int32_t tile = s_tile;
+    if (tile >= tiles) break;  // uniform across the block
+    const int32_t x0 = tile * tile_items, x1 = min(x0 + tile_items, W);
+    const TileRows t = stage_rows(woff, tile_row, 0, tile_items, s_woff, tile);
     const int32_t xb = x0 + warp * 128 + lane * kItemsPerThread;
     uint32_t bits = 0, fbits = 0;
-    int32_t qj[kItemsPerThread] = {-1, -1, -1, -1};  // query of a last-level survivor
+    int32_t rj[kItemsPerThread], wj[kItemsPerThread];
+    BatchSum sum;
     if (xb < x1) {
       int32_t rs;
-      int32_t r = b_row(b, s_woff, woff, xb, &rs);
-      int32_t rr = r - b.r0;
-      int32_t re = b.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
+      int32_t r = item_row(t, s_woff, woff, 0, xb, &rs);
+      int32_t rr = r - t.r0;
+      int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
       int32_t q = rseg[r], pst = pstart[r], slot = pslot[r];
 #pragma unroll
       for (int j = 0; j < kItemsPerThread; ++j) {
+        rj[j] = r;
+        wj[j] = 0;
         const int32_t x = xb + j;
-        if (x >= x1) break;
-        while (x >= re) {
+        if (x >= x1) continue;
+        while (x >= re) {  // next row (rows without work are skipped)
           ++rr;
           ++r;
           rs = re;
-          re = b.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
+          re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
           q = rseg[r];
           pst = pstart[r];
           slot = pslot[r];
         }
-        const BatchLevel &L = qs[q].lv[i];
+        const BatchQuery &bq = qs[q];
         const int32_t w = __ldg(g.lcol + pst + (x - rs));
-        if (check_candidate(g, L, ColumnRow{F, R, r}, w, slot)) {
-          if (L.last) {
-            qj[j] = q;
-            if (fmasks && qs[q].enumerate) fbits |= 1u << j;
-          } else {
+        rj[j] = r;
+        wj[j] = w;
+        const ColumnRow row{F, ld, r};
+        if (check_candidate(g, bq.lv[i], row, w, slot)) {
+          if (i != bq.kc - 1) {
             bits |= 1u << j;
+          } else {
+            sum.add(q, core_number(g, bq, ExtendedRow<ColumnRow>{row, i, w}, &over), counts);
+            if (bq.enumerate) fbits |= 1u << j;
           }
         }
       }
     }
-    // last-level survivors: one atomic per query per warp and item slot
-    // (a warp's rows mostly belong to one query: ballots settle that case,
-    // match_any only a warp that straddles queries)
+    sum.flush(counts);
+    int32_t T;
+    const int32_t rank = block_rank(__popc(bits) | (__popc(fbits) << 16), s_warp, &T);
+    {
+      int32_t *s_pair = s_pairs + buf * 2 * tile_items;
+      int32_t qn = rank & 0xffff, qf = (int32_t)((uint32_t)rank >> 16);
 #pragma unroll
-    for (int j = 0; j < kItemsPerThread; ++j) {
-      const uint32_t has = __ballot_sync(kFull, qj[j] >= 0);
-      if (!has) continue;
-      const int first = __ffs(has) - 1;
-      const int32_t qa = __shfl_sync(kFull, qj[j], first);
-      if (__ballot_sync(kFull, qj[j] == qa) == has) {
-        if (lane == first) atomicAdd(counts + qa, (unsigned long long)__popc(has));
-      } else {
-        const uint32_t peers = __match_any_sync(kFull, qj[j]);
-        if (qj[j] >= 0 && lane == __ffs(peers) - 1)
-          atomicAdd(counts + qj[j], (unsigned long long)__popc(peers));
+      for (int j = 0; j < kItemsPerThread; ++j) {
+        if (!(((bits | fbits) >> j) & 1u)) continue;
+        const int32_t at = (bits >> j) & 1u ? qn++ : tile_items - 1 - qf++;
+        s_pair[2 * at] = rj[j];
+        s_pair[2 * at + 1] = wj[j];
       }
     }
-    uint32_t word = bits << (4 * (lane & 7));
-    word |= __shfl_xor_sync(kFull, word, 1);
-    word |= __shfl_xor_sync(kFull, word, 2);
-    word |= __shfl_xor_sync(kFull, word, 4);
-    int32_t cnt = 0;
-    if ((lane & 7) == 0) {
-      masks[(x0 + warp * 128) / 32 + (lane >> 3)] = word;
-      cnt = __popc(word);
-    }
-    cnt = __reduce_add_sync(kFull, cnt);
-    if (lane == 0 && cnt) atomicAdd(&s_count, cnt);
-    if (fmasks) {
-      uint32_t fw = fbits << (4 * (lane & 7));
-      fw |= __shfl_xor_sync(kFull, fw, 1);
-      fw |= __shfl_xor_sync(kFull, fw, 2);
-      fw |= __shfl_xor_sync(kFull, fw, 4);
-      int32_t fc = 0;
-      if ((lane & 7) == 0) {
-        fmasks[(x0 + warp * 128) / 32 + (lane >> 3)] = fw;
-        fc = __popc(fw);
-      }
-      fc = __reduce_add_sync(kFull, fc);
-      if (lane == 0 && fc) atomicAdd(&s_fcount, fc);
-    }
+    if (threadIdx.x == 0)
+      lookback_publish(lb, tile, tiles,
+                       ((unsigned long long)((uint32_t)T >> 16) << kPackBits) |
+                           (unsigned long long)(T & 0xffff));
     __syncthreads();
-    if (threadIdx.x == 0) {
-      tile_cnt[t] = s_count;
-      if (ftile_cnt) ftile_cnt[t] = s_fcount;
-    }
-    __syncthreads();
+    if (pend >= 0) finish(pend, pend_T, buf ^ 1);
+    pend = tile;
+    pend_T = T;
+    buf ^= 1;
   }
-}
-
-// Survivors S = tile_off[tiles]; the next level gets them unless they exceed
-// the frontier capacity.
-__global__ void k_b_advance(int32_t i, BatchStep *state, const int64_t *__restrict__ tile_off,
-                            int64_t cap_rows, int64_t cap_elems, int32_t *overflow) {
-  const int64_t tiles = state[i].tiles;
-  const int64_t S = tiles > 0 ? tile_off[tiles] : 0;
-  state[i].S = S;
-  if (S > cap_rows || S * (i + 1) > cap_elems) {
-    *overflow = 1;
-    state[i + 1].R = 0;
-  } else {
-    state[i + 1].R = S;
+  if (pend >= 0) finish(pend, pend_T, buf ^ 1);
+  if (over) *overflow = kBatchOverflow;  // past 64 bits: the single-query path reports it
+  if (!last_cta(lb, tiles)) return;
+  const unsigned long long total = atomicAdd(lb + tiles + 1, 0ull);
+  const bool late = atomicAdd(lb + tiles + 2, 0ull) != 0;
+  const int64_t S = (int64_t)(total & kPackMask), FS = (int64_t)(total >> kPackBits);
+  const bool rows_ok = !late && S <= cap_rows && S * width <= cap_elems;
+  const bool final_ok = !late && FB + FS * width <= cap_final;
+  const int64_t Rn = rows_ok ? S : 0;
+  if (threadIdx.x == 0) {
+    if (late) *overflow = kBatchTimeout;
+    else if (!rows_ok || !final_ok) *overflow = kBatchOverflow;
+    state[i].S = S;
+    state[i].FS = final_ok ? FS : 0;
+    state[i + 1].R = Rn;
+    state[i + 1].FB = FB + (final_ok ? FS * width : 0);
   }
-}
-
-__device__ __forceinline__ int b_nth_bit(uint32_t m, int n) {
-  int pos = 0;
-#pragma unroll
-  for (int w = 16; w; w >>= 1) {
-    const uint32_t lo = m & ((1u << w) - 1u);
-    const int c = __popc(lo);
-    if (n >= c) {
-      n -= c;
-      m >>= w;
-      pos += w;
-    } else {
-      m = lo;
-    }
-  }
-  return pos;
-}
-
-__global__ void __launch_bounds__(1024) k_b_write(
-    GraphDev g, int32_t i, const BatchStep *state, const int32_t *__restrict__ F,
-    const int32_t *__restrict__ rseg, const int32_t *__restrict__ pstart,
-    const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row,
-    const uint32_t *__restrict__ masks, const int64_t *__restrict__ tile_off,
-    int32_t *__restrict__ Fn, int32_t *__restrict__ rseg_n) {
-  extern __shared__ int32_t s_woff[];
-  __shared__ uint32_t s_mask[kItemsPerThread * 1024 / 32];
-  __shared__ int32_t s_wpre[kItemsPerThread * 1024 / 32];
-  const int32_t R = (int32_t)state[i].R;
-  const int64_t tiles = state[i].tiles;
-  const int64_t S = state[i + 1].R;
-  if (S == 0 || S != state[i].S) return;  // nothing survives, or overflow
-  const int32_t B = blockDim.x;
-  const int32_t tile_items = B * kItemsPerThread;
-  const int32_t tile_words = tile_items / 32;
-  const int lane = threadIdx.x & 31;
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int64_t base = tile_off[t];
-    const int32_t cnt = (int32_t)(tile_off[t + 1] - base);
-    if (cnt == 0) continue;  // uniform across the block
-    for (int32_t w = threadIdx.x; w < tile_words; w += B) s_mask[w] = masks[t * tile_words + w];
-    const BTile b = b_stage(woff, tile_row, t, tile_items, s_woff);
-    if (threadIdx.x < 32) {
-      int32_t carry = 0;
-      for (int32_t c = 0; c < tile_words; c += 32) {
-        const int32_t idx = c + lane;
-        const int32_t v = idx < tile_words ? __popc(s_mask[idx]) : 0;
-        int32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int32_t y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        if (idx < tile_words) s_wpre[idx] = carry + incl - v;
-        carry += __shfl_sync(kFull, incl, 31);
-      }
-    }
-    __syncthreads();
-    const int32_t x0 = (int32_t)t * tile_items;
-    for (int32_t q = threadIdx.x; q < cnt; q += B) {
-      int32_t lo = 0, hi = tile_words;
-      while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (s_wpre[mid] <= q) lo = mid; else hi = mid;
-      }
-      const int32_t x = x0 + lo * 32 + b_nth_bit(s_mask[lo], q - s_wpre[lo]);
-      int32_t rs;
-      const int32_t r = b_row(b, s_woff, woff, x, &rs);
-      const int32_t w = __ldg(g.lcol + pstart[r] + (x - rs));
-      const int64_t pos = base + q;
-      for (int c = 0; c < i; ++c) Fn[c * S + pos] = F[c * R + r];
-      Fn[i * S + pos] = w;
-      rseg_n[pos] = rseg[r];
-    }
-    __syncthreads();
-  }
-}
-
-// Result rows of step i: FS = ftile_off[tiles]; they take arena elements
-// [FB, FB + FS*(i+1)) and the next step's rows start after them.  Over the
-// arena's capacity: overflow, and no row is written.
-__global__ void k_b_fadvance(int32_t i, BatchStep *state, const int64_t *__restrict__ ftile_off,
-                             int64_t cap_final, int32_t *overflow) {
-  const int64_t tiles = state[i].tiles;
-  const int64_t FS = tiles > 0 ? ftile_off[tiles] : 0;
-  const int64_t FB = state[i].FB;
-  if (FB + FS * (i + 1) > cap_final) {
-    *overflow = 1;
-    state[i].FS = 0;
-    state[i + 1].FB = FB;
-  } else {
-    state[i].FS = FS;
-    state[i + 1].FB = FB + FS * (i + 1);
-  }
-}
-
-// Writes the result rows of step i: result survivor q of tile t becomes row
-// ftile_off[t] + q of the step, row-major from arena element FB, position c
-// of the frontier row going to column out_col[c] of its query (the new
-// vertex to column out_col[i]).
-__global__ void __launch_bounds__(1024) k_b_fwrite(
-    GraphDev g, const BatchQuery *__restrict__ qs, int32_t i, const BatchStep *state,
-    const int32_t *__restrict__ F, const int32_t *__restrict__ rseg,
-    const int32_t *__restrict__ pstart, const int64_t *__restrict__ woff,
-    const int32_t *__restrict__ tile_row, const uint32_t *__restrict__ fmasks,
-    const int64_t *__restrict__ ftile_off, int32_t *__restrict__ final_rows) {
-  extern __shared__ int32_t s_woff[];
-  __shared__ uint32_t s_mask[kItemsPerThread * 1024 / 32];
-  __shared__ int32_t s_wpre[kItemsPerThread * 1024 / 32];
-  const int32_t R = (int32_t)state[i].R;
-  const int64_t tiles = state[i].tiles;
-  const int64_t FS = state[i].FS, FB = state[i].FB;
-  if (FS == 0) return;  // nothing to write, or over capacity
-  const int32_t B = blockDim.x;
-  const int32_t tile_items = B * kItemsPerThread;
-  const int32_t tile_words = tile_items / 32;
-  const int lane = threadIdx.x & 31;
-  const int32_t width = i + 1;
-  for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int64_t base = ftile_off[t];
-    const int32_t cnt = (int32_t)(ftile_off[t + 1] - base);
-    if (cnt == 0) continue;  // uniform across the block
-    for (int32_t w = threadIdx.x; w < tile_words; w += B) s_mask[w] = fmasks[t * tile_words + w];
-    const BTile b = b_stage(woff, tile_row, t, tile_items, s_woff);
-    if (threadIdx.x < 32) {
-      int32_t carry = 0;
-      for (int32_t c = 0; c < tile_words; c += 32) {
-        const int32_t idx = c + lane;
-        const int32_t v = idx < tile_words ? __popc(s_mask[idx]) : 0;
-        int32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int32_t y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        if (idx < tile_words) s_wpre[idx] = carry + incl - v;
-        carry += __shfl_sync(kFull, incl, 31);
-      }
-    }
-    __syncthreads();
-    const int32_t x0 = (int32_t)t * tile_items;
-    for (int32_t q = threadIdx.x; q < cnt; q += B) {
-      int32_t lo = 0, hi = tile_words;
-      while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (s_wpre[mid] <= q) lo = mid; else hi = mid;
-      }
-      const int32_t x = x0 + lo * 32 + b_nth_bit(s_mask[lo], q - s_wpre[lo]);
-      int32_t rs;
-      const int32_t r = b_row(b, s_woff, woff, x, &rs);
-      const int32_t w = __ldg(g.lcol + pstart[r] + (x - rs));
-      const int32_t *oc = qs[rseg[r]].out_col;
-      int32_t *dst = final_rows + FB + (base + q) * width;
-      for (int c = 0; c < i; ++c) dst[oc[c]] = F[c * R + r];
-      dst[oc[i]] = w;
-    }
-    __syncthreads();
-  }
-}
-
-// Address of a field of state[i] (device memory; no host access).
-const int64_t *step_field(const BatchStep *state, int32_t i, size_t off) {
-  return reinterpret_cast<const int64_t *>(reinterpret_cast<const char *>(state) +
-                                           (size_t)i * sizeof(BatchStep) + off);
-}
-
-template <typename T>
-void pscan(const T *in, const int64_t *n_ptr, int64_t *out, int64_t *partials, int32_t G,
-           cudaStream_t s) {
-  k_pscan_reduce<T><<<G, kPScanThreads, 0, s>>>(in, n_ptr, partials);
-  k_pscan_top<<<1, 1024, 0, s>>>(partials, G);
-  k_pscan_down<T><<<G, kPScanThreads, 0, s>>>(in, n_ptr, partials, out);
+  zero_words(lb_pivot, (Rn + kBatchPivotTile - 1) / kBatchPivotTile + kLbExtra);
 }
 
 }  // namespace
@@ -619,51 +518,45 @@ void launch_filter_many(const GraphDev &g, const FilterDesc *fds, uint32_t *cons
   k_b_filter<<<dim3(std::max(gx, 1), nq), 256, 0, s>>>(g, fds, bm_out, sizes);
 }
 
+namespace {
+size_t level_smem(int32_t block) {
+  return sizeof(int32_t) * ((size_t)block * kItemsPerThread * 5 + 4);
+}
+}  // namespace
+
+void batch_setup() {
+  cudaFuncSetAttribute(k_b_level<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)level_smem(1024));
+}
+
 int batch_enqueue(const GraphDev &g, const BatchArgs &a, cudaStream_t s) {
   const int32_t B = a.block, G = a.grid;
   const int32_t tile_items = B * kItemsPerThread;
-  const size_t smem = (size_t)(tile_items + 1) * sizeof(int32_t);
-  int launches = 0;
-  cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.nq, s);
-  cudaMemsetAsync(a.overflow, 0, sizeof(int32_t), s);
-  k_b_init<<<1, 32, 0, s>>>(a.state, (int64_t)a.nq * a.n_words);
+  const int64_t list_tiles = ((int64_t)a.nq * a.n_words + kBatchListTile - 1) / kBatchListTile;
+  k_b_init<<<(unsigned)std::min<int64_t>((list_tiles + 2 * a.nq) / 256 + 1, G), 256, 0, s>>>(
+      a.state, a.overflow, a.counts, 2 * (int64_t)a.nq, a.lb_list, list_tiles + kLbExtra);
   // filter: one CTA row per query (nothing reads the sizes here)
   launch_filter_many(g, a.fds, a.bm_out, g.thr ? nullptr : a.sizes, a.nq, a.n_words, s);
-  ++launches;
   // level 1: every query's candidate list for its first matched vertex
-  k_b_list_popc<<<G, 256, 0, s>>>(a.qs, a.nq, a.n_words, a.wcnt, a.counts);
-  pscan<int32_t>(a.wcnt, step_field(a.state, 0, offsetof(BatchStep, W)), a.woffs, a.partials,
-                 G, s);
-  k_b_list_check<<<1, 1, 0, s>>>(a.woffs, (int64_t)a.nq * a.n_words, a.state,
-                                 std::min(a.cap_rows, a.cap_elems), a.overflow);
-  k_b_list_emit<<<G, 256, 0, s>>>(a.qs, a.nq, a.n_words, a.woffs, a.state, a.F[0], a.rseg[0]);
-  launches += 7;
+  k_b_list<<<(unsigned)std::max<int64_t>(std::min<int64_t>(list_tiles, G), 1), 256, 0, s>>>(
+      g, a.qs, a.nq, a.list_off, a.state, std::min(a.cap_rows, a.cap_elems), a.F[0], a.rseg[0],
+      a.counts, a.lb_list, a.lb_pivot, a.spin_limit, a.overflow);
+  int launches = 3;
   for (int32_t i = 1; i < a.kmax; ++i) {
     const int cur = (i - 1) & 1, nxt = i & 1;
-    k_b_pivot<<<G, 256, 0, s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart, a.pslot,
-                                a.woff);
-    pscan<int64_t>(a.woff, step_field(a.state, i, offsetof(BatchStep, R)), a.woff, a.partials,
-                   G, s);
-    k_b_check_work<<<1, 1, 0, s>>>(i, a.state, a.woff, a.cap_items, tile_items, a.overflow);
-    k_b_tile_rows<<<G, 256, 0, s>>>(i, a.state, a.woff, tile_items, a.tile_row);
-    k_b_count<<<G, B, smem, s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart, a.pslot,
-                                 a.woff, a.tile_row, a.masks, a.tile_cnt, a.counts,
-                                 a.enumerate ? a.fmasks : nullptr,
-                                 a.enumerate ? a.ftile_cnt : nullptr);
-    pscan<int32_t>(a.tile_cnt, step_field(a.state, i, offsetof(BatchStep, tiles)), a.tile_off,
-                   a.partials, G, s);
-    k_b_advance<<<1, 1, 0, s>>>(i, a.state, a.tile_off, a.cap_rows, a.cap_elems, a.overflow);
-    k_b_write<<<G, B, smem, s>>>(g, i, a.state, a.F[cur], a.rseg[cur], a.pstart, a.woff,
-                                 a.tile_row, a.masks, a.tile_off, a.F[nxt], a.rseg[nxt]);
-    launches += 12;
-    if (a.enumerate) {
-      pscan<int32_t>(a.ftile_cnt, step_field(a.state, i, offsetof(BatchStep, tiles)),
-                     a.ftile_off, a.partials, G, s);
-      k_b_fadvance<<<1, 1, 0, s>>>(i, a.state, a.ftile_off, a.cap_final, a.overflow);
-      k_b_fwrite<<<G, B, smem, s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart, a.woff,
-                                    a.tile_row, a.fmasks, a.ftile_off, a.final_rows);
-      launches += 5;
-    }
+    k_b_pivot_scan<<<G, 256, 0, s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart,
+                                     a.pslot, a.woff, a.tile_row, tile_items, a.cap_rows,
+                                     a.cap_elems, a.cap_items, a.lb_pivot, a.lb_level,
+                                     a.spin_limit, a.overflow);
+    auto level = [&](auto kernel) {
+      kernel<<<G, B, level_smem(B), s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart,
+                                         a.pslot, a.woff, a.tile_row, a.cap_rows, a.cap_elems,
+                                         a.cap_final, a.counts, a.F[nxt], a.rseg[nxt],
+                                         a.final_rows, a.lb_level, a.lb_pivot, a.spin_limit,
+                                         a.overflow);
+    };
+    B <= 256 ? level(k_b_level<256>) : level(k_b_level<1024>);
+    launches += 2;
   }
   return launches;
 }

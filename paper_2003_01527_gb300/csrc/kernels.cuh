@@ -23,8 +23,8 @@ struct FilterDesc {
   int32_t qdeg[kMaxK];             // deg_Q(u)
   int32_t lo[kMaxK], hi[kMaxK];    // restriction of f(u) to [lo, hi)
   int32_t nreq[kMaxK];             // number of (slot, count) requirements of u
-  int32_t req_slot[kMaxK][kMaxK];  // label slot of requirement r of u
-  int32_t req_cnt[kMaxK][kMaxK];   // neighbours needed with that label
+  int8_t req_slot[kMaxK][kMaxK];   // label slot of requirement r of u
+  int8_t req_cnt[kMaxK][kMaxK];    // neighbours needed with that label
   int32_t nslots;                  // distinct labels used by requirements
   int32_t slot_label[kMaxK];       // dense label id of each slot
 };

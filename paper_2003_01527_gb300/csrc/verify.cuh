@@ -133,47 +133,58 @@ __device__ __forceinline__ bool check_candidate_probes(const GraphDev &g, const 
   return true;
 }
 
-// One thread's sums of the leaf numbers of core embeddings; kLeaves = an
-// upper bound of the query's leaves.
+// The images of the leaves for one core embedding (row(c) = the image of core
+// position c): the product over the groups (LeafDesc), 0 if a leaf has none.
+// part(l, v) receives the partial products (l leaves placed); *over is set
+// when the number exceeds 64 bits.  kLeaves: an upper bound of the leaves.
+template <int kLeaves, typename Row, typename Part>
+__device__ __forceinline__ unsigned long long leaf_number(const GraphDev &g, const LeafDesc &leaf,
+                                                          const Row &row, bool *over,
+                                                          const Part &part) {
+  unsigned long long v = 1;
+  bool big = false;
+  int32_t a = 0;
+  constexpr int kUnroll = kLeaves <= 3 ? kLeaves : 1;
+#pragma unroll kUnroll
+  for (int l = 0; l < kLeaves; ++l) {
+    if (l >= leaf.nleaves) break;
+    if (l == 0 || leaf.of[l] != leaf.of[l - 1]) {
+      const LeafGroup &gr = leaf.grp[leaf.of[l]];
+      const int32_t x = row(gr.pos);
+      int2 seg = label_segment(g, x, gr.lab);
+      if (gr.lo > 0 || gr.hi < g.n) seg = cut_segment(g, seg, gr.lo, gr.hi);
+      a = seg.y - seg.x;
+      for (uint32_t m = gr.in_mask; m; m &= m - 1) {
+        const int32_t y = row(__ffs(m) - 1);
+        a -= y >= gr.lo && y < gr.hi;
+      }
+      for (uint32_t m = gr.chk_mask; m && a > 0; m &= m - 1) {
+        const int32_t y = row(__ffs(m) - 1);
+        if (y >= gr.lo && y < gr.hi && row_contains_l(g, x, gr.lab, y)) --a;
+      }
+    } else {
+      --a;
+    }
+    part(l, v);
+    if (a <= 0) return 0;
+    big = big || __umul64hi(v, (unsigned long long)a);
+    v *= (unsigned long long)a;
+  }
+  *over = *over || big;
+  return v;
+}
+
+// One thread's sums of the leaf numbers of core embeddings.
 template <int kLeaves>
 struct LeafSums {
   unsigned long long lo = 0, hi = 0;  // of the numbers' 32-bit halves
   unsigned long long part[kLeaves] = {};  // partial embeddings with l leaves placed
   bool over = false;
 
-  // Adds the images of the leaves for one core embedding (row(c) = the image
-  // of core position c): the product over the groups (LeafDesc).
   template <typename Row>
   __device__ __forceinline__ void add(const GraphDev &g, const LeafDesc &leaf, const Row &row) {
-    unsigned long long v = 1;
-    bool big = false;
-    int32_t a = 0;
-#pragma unroll
-    for (int l = 0; l < kLeaves; ++l) {
-      if (l >= leaf.nleaves) break;
-      if (l == 0 || leaf.of[l] != leaf.of[l - 1]) {
-        const LeafGroup &gr = leaf.grp[leaf.of[l]];
-        const int32_t x = row(gr.pos);
-        int2 seg = label_segment(g, x, gr.lab);
-        if (gr.lo > 0 || gr.hi < g.n) seg = cut_segment(g, seg, gr.lo, gr.hi);
-        a = seg.y - seg.x;
-        for (uint32_t m = gr.in_mask; m; m &= m - 1) {
-          const int32_t y = row(__ffs(m) - 1);
-          a -= y >= gr.lo && y < gr.hi;
-        }
-        for (uint32_t m = gr.chk_mask; m && a > 0; m &= m - 1) {
-          const int32_t y = row(__ffs(m) - 1);
-          if (y >= gr.lo && y < gr.hi && row_contains_l(g, x, gr.lab, y)) --a;
-        }
-      } else {
-        --a;
-      }
-      part[l] += v;
-      if (a <= 0) return;  // this leaf has no image
-      big = big || __umul64hi(v, (unsigned long long)a);
-      v *= (unsigned long long)a;
-    }
-    over = over || big;
+    const unsigned long long v = leaf_number<kLeaves>(
+        g, leaf, row, &over, [&](int l, unsigned long long x) { part[l] += x; });
     lo += (uint32_t)v;
     hi += v >> 32;
   }
