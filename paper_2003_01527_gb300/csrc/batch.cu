@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(256) k_b_pivot_scan(
 // Verification and write pass of one step, in one launch: tiles by ticket; a
 // tile's survivors are ranked, kept in one of two shared buffers and written
 // after the CTA has verified its next tile, when the look-back has its prefix
-// (the single-query path's k_extend_fused, with the check, check_candidate).
+// (the single-query path's k_extend_fused, with its check, check_candidate).
 // Survivors of a query at its last level are counted (times their leaf
 // numbers), and for a query that lists its rows written to the result arena;
 // the others become rows of the next level.  Both ranks travel in one
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
         rj[j] = r;
         wj[j] = w;
         const ColumnRow row{F, ld, r};
-        if (check_candidate(g, bq.lv[i], row, w, slot)) {
+        if (check_candidate(g, bq.lv[i], row, w, slot, re - rs <= kFewCandidates)) {
           if (i != bq.kc - 1) {
             bits |= 1u << j;
           } else {

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(1024) k_cextend(
       const int32_t w = __ldg(g.lcol + pst + (x - rs));
       rj[j] = r;
       wj[j] = w;
-      if (check_candidate(g, d, ArrayRow{vals}, w, slot) &&
+      if (check_candidate(g, d, ArrayRow{vals}, w, slot, re - rs <= kFewCandidates) &&
           (!d.la || lookahead_ok(g, d, ArrayRow{vals}, w)))
         bits |= 1u << j;
     }

@@ -542,8 +542,8 @@ __global__ void k_tile_rows(const int64_t *__restrict__ woff, int64_t ra, int64_
 // bits stay in candidate order: each lane's 4-bit group is shifted into place
 // and OR-ed across the 8 lanes that share a 32-bit mask word.
 // kLeaves > 0: a survivor adds its leaf number (LeafSums) instead of one.
-template <bool kMasks, int kLeaves>
-__global__ void __launch_bounds__(1024) k_extend_count(
+template <bool kMasks, int kLeaves, int kNb>
+__global__ void __launch_bounds__(kNb ? 256 : 1024, kNb ? 6 : 1) k_extend_count(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
@@ -568,23 +568,27 @@ __global__ void __launch_bounds__(1024) k_extend_count(
     int32_t rr = r - t.r0;
     int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
     int32_t pst = pstart[r], slot = pslot[r];
+    RowCheck<kNb> check;
+    check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
 #pragma unroll
     for (int j = 0; j < kItemsPerThread; ++j) {
       const int32_t x = xb + j;
       if (x >= x1) break;
-      while (x >= re) {  // next row (rows without work are skipped)
-        ++rr;
-        ++r;
-        rs = re;
-        re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+      if (x >= re) {
+        do {  // next row (rows without work are skipped)
+          ++rr;
+          ++r;
+          rs = re;
+          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+        } while (x >= re);
         pst = pstart[r];
         slot = pslot[r];
+        check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
       }
       const int32_t w = __ldg(g.lcol + pst + (x - rs));
-      if (check_candidate(g, d, ColumnRow{F, ld, r}, w, slot) &&
-          (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w))) {
+      const ColumnRow row{F, ld, r};
+      if (check.ok(g, d, row, w, slot)) {
         if constexpr (kLeaves > 0) {
-          const ColumnRow row{F, ld, r};
           sums.add(g, leaf, ExtendedRow<ColumnRow>{row, d.i, w});
         } else {
           bits |= 1u << j;
@@ -734,7 +738,8 @@ constexpr size_t kFusedStageMax = 96 * 1024;   // ... with the tile's result row
 
 // kMaxThreads = 256: up to 256 threads per CTA, registers capped so that six
 // CTAs fit on an SM; 1024: any block size.
-template <int kMode, int kMaxThreads, bool kProbes>
+// kNb: the RowCheck (0 with kProbes).
+template <int kMode, int kMaxThreads, bool kProbes, int kNb>
 __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_extend_fused(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
@@ -825,19 +830,24 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_ext
       int32_t rr = r - t.r0;
       int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
       int32_t pst = pstart[r], slot = pslot[r];
+      RowCheck<kNb> check;
+      check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
 #pragma unroll
       for (int j = 0; j < kItemsPerThread; ++j) {
         rj[j] = r;
         wj[j] = 0;
         const int32_t x = xb + j;
         if (x >= x1) continue;
-        while (x >= re) {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+        if (x >= re) {
+          do {  // next row (rows without work are skipped)
+            ++rr;
+            ++r;
+            rs = re;
+            re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+          } while (x >= re);
           pst = pstart[r];
           slot = pslot[r];
+          check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
         }
         if (!GSM_IN_BOUNDS(g.dbg, pst + (x - rs) >= 0 && pst + (x - rs) < g.nnz, kDbgCandidate) ||
             !GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
@@ -847,10 +857,12 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_ext
         wj[j] = w;
         bool ok;
         if constexpr (kProbes)
-          ok = check_candidate_probes(g, d, ColumnRow{F, ld, r}, w, slot, &probes);
+          ok = check_candidate_probes(g, d, ColumnRow{F, ld, r}, w, slot, re - rs <= kFewCandidates,
+                                      &probes) &&
+               (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w));
         else
-          ok = check_candidate(g, d, ColumnRow{F, ld, r}, w, slot);
-        if (ok && (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w))) bits |= 1u << j;
+          ok = check.ok(g, d, ColumnRow{F, ld, r}, w, slot);
+        if (ok) bits |= 1u << j;
       }
     }
     if constexpr (kProbes) {
@@ -1213,6 +1225,12 @@ void launch_tile_rows(const int64_t *woff, int64_t ra, int64_t rb, int64_t wa, i
       woff, ra, rb, wa, (int64_t)block * kItemsPerThread, tiles, tile_row, lookback, lb_words);
 }
 
+// The RowCheck a level's launches take: by the level's shape, for CTAs of up to
+// 256 threads (the default; the instances are bounded to it).
+static int row_check_nb(const LevelDesc &d, int32_t block) {
+  return block <= 256 && d.nb <= kMaxRowCheck && d.ninj <= 2 && !d.la && !d.count_probes ? d.nb : 0;
+}
+
 void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
@@ -1226,14 +1244,28 @@ void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F
         g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, (int32_t)(wb - wa), masks,
         tile_cnt, total, leaf ? *leaf : LeafDesc{});
   };
-  if (!leaf)
-    masks ? go(k_extend_count<true, 0>) : go(k_extend_count<false, 0>);
+  const int nb = row_check_nb(d, block);
+  auto by_nb = [&](auto masked, auto leaves) {
+    constexpr bool kM = decltype(masked)::value;
+    constexpr int kL = decltype(leaves)::value;
+    switch (nb) {
+      case 1: return go(k_extend_count<kM, kL, 1>);
+      case 2: return go(k_extend_count<kM, kL, 2>);
+      case 3: return go(k_extend_count<kM, kL, 3>);
+      default: return go(k_extend_count<kM, kL, 0>);
+    }
+  };
+  using std::integral_constant;
+  if (masks)
+    by_nb(std::true_type{}, integral_constant<int, 0>{});
+  else if (!leaf)
+    by_nb(std::false_type{}, integral_constant<int, 0>{});
   else if (leaf->nleaves == 1)
-    go(k_extend_count<false, 1>);
+    by_nb(std::false_type{}, integral_constant<int, 1>{});
   else if (leaf->nleaves <= 3)
-    go(k_extend_count<false, 3>);
+    go(k_extend_count<false, 3, 0>);
   else
-    go(k_extend_count<false, kMaxK>);
+    go(k_extend_count<false, kMaxK, 0>);
 }
 
 void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,
@@ -1271,10 +1303,10 @@ void launch_extend_write(const GraphDev &g, const LevelDesc &d, const int32_t *F
 }
 
 namespace {
-// One persistent launch of k_extend_fused<kMode, ..., kProbes>: as many CTAs as fit on the
+// One persistent launch of k_extend_fused<kMode, ...>: as many CTAs as fit on the
 // device at once (at most one per tile).  The dynamic shared-memory limit is
 // raised once per device for this instance.
-template <int kMode, int kMaxThreads, bool kProbes>
+template <int kMode, int kMaxThreads, bool kProbes, int kNb>
 void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                        const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                        const int32_t *tile_row, int64_t wa, int32_t W, int32_t tiles,
@@ -1291,7 +1323,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int di = dev & 63;
   if (!((attr_set.load() >> di) & 1ull)) {
-    cudaFuncSetAttribute(k_extend_fused<kMode, kMaxThreads, kProbes>,
+    cudaFuncSetAttribute(k_extend_fused<kMode, kMaxThreads, kProbes, kNb>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemAttr);
     attr_set.fetch_or(1ull << di);
   }
@@ -1299,7 +1331,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
   if (blocks_cache[di] == block && smem_cache[di] == smem && per_sm_cache[di][0]) {
     per_sm = per_sm_cache[di][1];
   } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_extend_fused<kMode, kMaxThreads, kProbes>,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_extend_fused<kMode, kMaxThreads, kProbes, kNb>,
                                                   block, smem);
     blocks_cache[di] = block;
     smem_cache[di] = smem;
@@ -1307,7 +1339,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
     per_sm_cache[di][1] = per_sm;
   }
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)std::max(per_sm, 1) * sms);
-  k_extend_fused<kMode, kMaxThreads, kProbes><<<(unsigned)grid, block, smem, s>>>(
+  k_extend_fused<kMode, kMaxThreads, kProbes, kNb><<<(unsigned)grid, block, smem, s>>>(
       g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, W, tiles, lookback, sink, stage,
       spin_limit, stall_tile);
 }
@@ -1331,32 +1363,41 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
   const size_t smem_rows = (base_ints + (size_t)items * sink.k) * sizeof(int32_t);
   const bool stage = sink.mode == kSinkRows && (sink.k & 1) && smem_rows <= kFusedStageMax;
   if (stage) smem = smem_rows;
-  auto go = [&](auto small, auto probes) {
+  auto go = [&](auto small, auto probes, auto nb) {
     constexpr int kMax = decltype(small)::value ? 256 : 1024;
     constexpr bool kP = decltype(probes)::value;
+    constexpr int kNb = decltype(nb)::value;
     if (sink.mode == kSinkRows)
-      launch_fused_mode<kSinkRows, kMax, kP>(g, d, F, ld, pstart, pslot, woff, tile_row, wa, W,
-                                             T, block, smem, lookback, sink, stage, spin_limit,
-                                             stall_tile, s);
+      launch_fused_mode<kSinkRows, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
+                                                  W, T, block, smem, lookback, sink, stage,
+                                                  spin_limit, stall_tile, s);
     else if (sink.mode == kSinkKeys)
-      launch_fused_mode<kSinkKeys, kMax, kP>(g, d, F, ld, pstart, pslot, woff, tile_row, wa, W,
-                                             T, block, smem, lookback, sink, false, spin_limit,
-                                             stall_tile, s);
+      launch_fused_mode<kSinkKeys, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
+                                                  W, T, block, smem, lookback, sink, false,
+                                                  spin_limit, stall_tile, s);
     else
-      launch_fused_mode<kSinkColumns, kMax, kP>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
-                                                W, T, block, smem, lookback, sink, false,
-                                                spin_limit, stall_tile, s);
+      launch_fused_mode<kSinkColumns, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row,
+                                                     wa, W, T, block, smem, lookback, sink, false,
+                                                     spin_limit, stall_tile, s);
   };
   // the probe-byte accounting is a separate instance, so the default one
   // carries no trace of it
-  if (block <= 256 && !d.count_probes)
-    go(std::true_type{}, std::false_type{});
+  const int nb = row_check_nb(d, block);
+  using std::integral_constant;
+  if (nb == 1)
+    go(std::true_type{}, std::false_type{}, integral_constant<int, 1>{});
+  else if (nb == 2)
+    go(std::true_type{}, std::false_type{}, integral_constant<int, 2>{});
+  else if (nb == 3)
+    go(std::true_type{}, std::false_type{}, integral_constant<int, 3>{});
+  else if (block <= 256 && !d.count_probes)
+    go(std::true_type{}, std::false_type{}, integral_constant<int, 0>{});
   else if (block <= 256)
-    go(std::true_type{}, std::true_type{});
+    go(std::true_type{}, std::true_type{}, integral_constant<int, 0>{});
   else if (!d.count_probes)
-    go(std::false_type{}, std::false_type{});
+    go(std::false_type{}, std::false_type{}, integral_constant<int, 0>{});
   else
-    go(std::false_type{}, std::true_type{});
+    go(std::false_type{}, std::true_type{}, integral_constant<int, 0>{});
 }
 
 void launch_split_points(const int64_t *woff, int64_t R, int64_t step, int64_t J,
