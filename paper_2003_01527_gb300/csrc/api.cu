@@ -804,8 +804,8 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   });
   if (count_only) {
     timed(ctx, K_COUNT, read_bytes, (uint64_t)W, 1, [&] {
-      launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nullptr,
-                          nullptr, R.d_total, ctx->stream, R.leaf.nleaves ? &R.leaf : nullptr);
+      launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nrows,
+                          nullptr, nullptr, R.d_total, ctx->stream, R.leaf.nleaves ? &R.leaf : nullptr);
     });
     return;
   }
@@ -814,7 +814,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   int64_t *tile_off = (int64_t *)(sc + o_off);
   int64_t *tmp = (int64_t *)(sc + o_tmp);
   timed(ctx, K_COUNT, read_bytes + W / 8.0, (uint64_t)W, 1, [&] {
-    launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, masks,
+    launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nrows, masks,
                         tile_cnt, nullptr, ctx->stream);
   });
   timed(ctx, K_PIVOT, 12.0 * tiles, (uint64_t)tiles, scan_kernels(tiles),
@@ -901,8 +901,8 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
     sink = RowSink{kSinkColumns, w_out, 0, 0, W, 0, Fn};
   }
   timed(ctx, K_FUSED, read_bytes, (uint64_t)W, 1, [&] {
-    launch_extend_fused(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, lb, sink,
-                        R.spin_limit, R.stall_tile, ctx->stream);
+    launch_extend_fused(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nrows, lb,
+                        sink, R.spin_limit, R.stall_tile, ctx->stream);
   });
   const int64_t *S_dev = (const int64_t *)(lb + tiles + 1);
   if (last) {

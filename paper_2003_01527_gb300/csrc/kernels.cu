@@ -542,8 +542,14 @@ __global__ void k_tile_rows(const int64_t *__restrict__ woff, int64_t ra, int64_
 // bits stay in candidate order: each lane's 4-bit group is shifted into place
 // and OR-ed across the 8 lanes that share a 32-bit mask word.
 // kLeaves > 0: a survivor adds its leaf number (LeafSums) instead of one.
-template <bool kMasks, int kLeaves, int kNb>
-__global__ void __launch_bounds__(kNb ? 256 : 1024, kNb ? 6 : 1) k_extend_count(
+// The forms that check a row's candidates one after the other hide the probes'
+// latency with warps: eight CTAs of 256 threads an SM (32 registers).  At 34
+// registers, six CTAs, the distinct 4-cliques of R-MAT 16 took 11.8 instead
+// of 9.8 ms.
+template <bool kMasks, int kLeaves, int kCheck>
+__global__ void __launch_bounds__(kCheck ? 256 : 1024,
+                                  kCheck > kCheckGroup ? 4 : !kCheck ? 1 : kLeaves ? 6 : 8)
+    k_extend_count(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
@@ -563,37 +569,15 @@ __global__ void __launch_bounds__(kNb ? 256 : 1024, kNb ? 6 : 1) k_extend_count(
   const int32_t xb = x0 + warp * 128 + lane * kItemsPerThread;
   uint32_t bits = 0;
   if (xb < x1) {
-    int32_t rs;
-    int32_t r = item_row(t, s_woff, woff, wa, xb, &rs);
-    int32_t rr = r - t.r0;
-    int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-    int32_t pst = pstart[r], slot = pslot[r];
-    RowCheck<kNb> check;
-    check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
+    int32_t rj[kItemsPerThread], wj[kItemsPerThread];
+    bits = check_group<kCheck>(g, d, F, ld, t, s_woff, woff, wa, pstart, pslot, xb, x1, rj, wj);
+    if constexpr (kLeaves > 0) {
 #pragma unroll
-    for (int j = 0; j < kItemsPerThread; ++j) {
-      const int32_t x = xb + j;
-      if (x >= x1) break;
-      if (x >= re) {
-        do {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-        } while (x >= re);
-        pst = pstart[r];
-        slot = pslot[r];
-        check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
-      }
-      const int32_t w = __ldg(g.lcol + pst + (x - rs));
-      const ColumnRow row{F, ld, r};
-      if (check.ok(g, d, row, w, slot)) {
-        if constexpr (kLeaves > 0) {
-          sums.add(g, leaf, ExtendedRow<ColumnRow>{row, d.i, w});
-        } else {
-          bits |= 1u << j;
+      for (int j = 0; j < kItemsPerThread; ++j)
+        if ((bits >> j) & 1u) {
+          const ColumnRow row{F, ld, rj[j]};
+          sums.add(g, leaf, ExtendedRow<ColumnRow>{row, d.i, wj[j]});
         }
-      }
     }
   }
   if constexpr (kLeaves > 0) {
@@ -738,9 +722,11 @@ constexpr size_t kFusedStageMax = 96 * 1024;   // ... with the tile's result row
 
 // kMaxThreads = 256: up to 256 threads per CTA, registers capped so that six
 // CTAs fit on an SM; 1024: any block size.
-// kNb: the RowCheck (0 with kProbes).
-template <int kMode, int kMaxThreads, bool kProbes, int kNb>
-__global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_extend_fused(
+// kCheck: the form of check_group (kCheckAny with kProbes).
+template <int kMode, int kMaxThreads, bool kProbes, int kCheck>
+__global__ void __launch_bounds__(kMaxThreads,
+                                  kMaxThreads == 256 ? (kCheck > kCheckGroup ? 4 : 6) : 1)
+    k_extend_fused(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
@@ -825,45 +811,8 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_ext
     uint32_t bits = 0, probes = 0;
     int32_t rj[kItemsPerThread], wj[kItemsPerThread];
     if (xb < x1) {
-      int32_t rs;
-      int32_t r = item_row(t, s_woff, woff, wa, xb, &rs);
-      int32_t rr = r - t.r0;
-      int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-      int32_t pst = pstart[r], slot = pslot[r];
-      RowCheck<kNb> check;
-      check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
-#pragma unroll
-      for (int j = 0; j < kItemsPerThread; ++j) {
-        rj[j] = r;
-        wj[j] = 0;
-        const int32_t x = xb + j;
-        if (x >= x1) continue;
-        if (x >= re) {
-          do {  // next row (rows without work are skipped)
-            ++rr;
-            ++r;
-            rs = re;
-            re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-          } while (x >= re);
-          pst = pstart[r];
-          slot = pslot[r];
-          check.load(g, d, ColumnRow{F, ld, r}, slot, re - rs);
-        }
-        if (!GSM_IN_BOUNDS(g.dbg, pst + (x - rs) >= 0 && pst + (x - rs) < g.nnz, kDbgCandidate) ||
-            !GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
-          continue;
-        const int32_t w = __ldg(g.lcol + pst + (x - rs));
-        rj[j] = r;
-        wj[j] = w;
-        bool ok;
-        if constexpr (kProbes)
-          ok = check_candidate_probes(g, d, ColumnRow{F, ld, r}, w, slot, re - rs <= kFewCandidates,
-                                      &probes) &&
-               (!d.la || lookahead_ok(g, d, ColumnRow{F, ld, r}, w));
-        else
-          ok = check.ok(g, d, ColumnRow{F, ld, r}, w, slot);
-        if (ok) bits |= 1u << j;
-      }
+      bits = check_group<kCheck, kProbes>(g, d, F, ld, t, s_woff, woff, wa, pstart, pslot, xb, x1,
+                                       rj, wj, &probes);
     }
     if constexpr (kProbes) {
 #pragma unroll
@@ -1225,17 +1174,19 @@ void launch_tile_rows(const int64_t *woff, int64_t ra, int64_t rb, int64_t wa, i
       woff, ra, rb, wa, (int64_t)block * kItemsPerThread, tiles, tile_row, lookback, lb_words);
 }
 
-// The RowCheck a level's launches take: by the level's shape, for CTAs of up to
-// 256 threads (the default; the instances are bounded to it).
-static int row_check_nb(const LevelDesc &d, int32_t block) {
-  return block <= 256 && d.nb <= kMaxRowCheck && d.ninj <= 2 && !d.la && !d.count_probes ? d.nb : 0;
+// The form of check_group for a level's launch over W candidates of `rows`
+// rows, for CTAs of up to 256 threads (the default; the other instances are
+// bounded to it).
+static int check_form(const LevelDesc &d, int32_t block, int64_t W, int64_t rows) {
+  if (block > 256 || d.nb > kMaxRowCheck || d.ninj > 2 || d.la || d.count_probes) return kCheckAny;
+  return d.nb >= 2 && W <= kFewCandidates * rows ? kCheckGroup + d.nb : kCheckRow + d.nb;
 }
 
 void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                         uint32_t *masks, int32_t *tile_cnt, unsigned long long *total,
-                         cudaStream_t s, const LeafDesc *leaf) {
+                         int64_t rows, uint32_t *masks, int32_t *tile_cnt,
+                         unsigned long long *total, cudaStream_t s, const LeafDesc *leaf) {
   const int64_t tiles = extend_tiles(wa, wb, block);
   if (tiles <= 0) return;
   const size_t smem = (size_t)((int64_t)block * kItemsPerThread + 1) * sizeof(int32_t);
@@ -1244,28 +1195,30 @@ void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F
         g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, (int32_t)(wb - wa), masks,
         tile_cnt, total, leaf ? *leaf : LeafDesc{});
   };
-  const int nb = row_check_nb(d, block);
-  auto by_nb = [&](auto masked, auto leaves) {
+  const int form = check_form(d, block, wb - wa, rows);
+  auto by_form = [&](auto masked, auto leaves) {
     constexpr bool kM = decltype(masked)::value;
     constexpr int kL = decltype(leaves)::value;
-    switch (nb) {
-      case 1: return go(k_extend_count<kM, kL, 1>);
-      case 2: return go(k_extend_count<kM, kL, 2>);
-      case 3: return go(k_extend_count<kM, kL, 3>);
-      default: return go(k_extend_count<kM, kL, 0>);
+    switch (form) {
+      case kCheckRow + 1: return go(k_extend_count<kM, kL, kCheckRow + 1>);
+      case kCheckRow + 2: return go(k_extend_count<kM, kL, kCheckRow + 2>);
+      case kCheckRow + 3: return go(k_extend_count<kM, kL, kCheckRow + 3>);
+      case kCheckGroup + 2: return go(k_extend_count<kM, kL, kCheckGroup + 2>);
+      case kCheckGroup + 3: return go(k_extend_count<kM, kL, kCheckGroup + 3>);
+      default: return go(k_extend_count<kM, kL, kCheckAny>);
     }
   };
   using std::integral_constant;
   if (masks)
-    by_nb(std::true_type{}, integral_constant<int, 0>{});
+    by_form(std::true_type{}, integral_constant<int, 0>{});
   else if (!leaf)
-    by_nb(std::false_type{}, integral_constant<int, 0>{});
+    by_form(std::false_type{}, integral_constant<int, 0>{});
   else if (leaf->nleaves == 1)
-    by_nb(std::false_type{}, integral_constant<int, 1>{});
+    by_form(std::false_type{}, integral_constant<int, 1>{});
   else if (leaf->nleaves <= 3)
-    go(k_extend_count<false, 3, 0>);
+    go(k_extend_count<false, 3, kCheckAny>);
   else
-    go(k_extend_count<false, kMaxK, 0>);
+    go(k_extend_count<false, kMaxK, kCheckAny>);
 }
 
 void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,
@@ -1306,7 +1259,7 @@ namespace {
 // One persistent launch of k_extend_fused<kMode, ...>: as many CTAs as fit on the
 // device at once (at most one per tile).  The dynamic shared-memory limit is
 // raised once per device for this instance.
-template <int kMode, int kMaxThreads, bool kProbes, int kNb>
+template <int kMode, int kMaxThreads, bool kProbes, int kCheck>
 void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                        const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                        const int32_t *tile_row, int64_t wa, int32_t W, int32_t tiles,
@@ -1323,7 +1276,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int di = dev & 63;
   if (!((attr_set.load() >> di) & 1ull)) {
-    cudaFuncSetAttribute(k_extend_fused<kMode, kMaxThreads, kProbes, kNb>,
+    cudaFuncSetAttribute(k_extend_fused<kMode, kMaxThreads, kProbes, kCheck>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmemAttr);
     attr_set.fetch_or(1ull << di);
   }
@@ -1331,7 +1284,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
   if (blocks_cache[di] == block && smem_cache[di] == smem && per_sm_cache[di][0]) {
     per_sm = per_sm_cache[di][1];
   } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_extend_fused<kMode, kMaxThreads, kProbes, kNb>,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_extend_fused<kMode, kMaxThreads, kProbes, kCheck>,
                                                   block, smem);
     blocks_cache[di] = block;
     smem_cache[di] = smem;
@@ -1339,7 +1292,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
     per_sm_cache[di][1] = per_sm;
   }
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)std::max(per_sm, 1) * sms);
-  k_extend_fused<kMode, kMaxThreads, kProbes, kNb><<<(unsigned)grid, block, smem, s>>>(
+  k_extend_fused<kMode, kMaxThreads, kProbes, kCheck><<<(unsigned)grid, block, smem, s>>>(
       g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, W, tiles, lookback, sink, stage,
       spin_limit, stall_tile);
 }
@@ -1348,8 +1301,8 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
 void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                         unsigned long long *lookback, const RowSink &sink, int32_t spin_limit,
-                         int32_t stall_tile, cudaStream_t s) {
+                         int64_t rows, unsigned long long *lookback, const RowSink &sink,
+                         int32_t spin_limit, int32_t stall_tile, cudaStream_t s) {
   const int64_t tiles = extend_tiles(wa, wb, block);
   if (tiles <= 0) return;
   const int32_t W = (int32_t)(wb - wa), T = (int32_t)tiles;
@@ -1363,41 +1316,47 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
   const size_t smem_rows = (base_ints + (size_t)items * sink.k) * sizeof(int32_t);
   const bool stage = sink.mode == kSinkRows && (sink.k & 1) && smem_rows <= kFusedStageMax;
   if (stage) smem = smem_rows;
-  auto go = [&](auto small, auto probes, auto nb) {
+  auto go = [&](auto small, auto probes, auto check) {
     constexpr int kMax = decltype(small)::value ? 256 : 1024;
     constexpr bool kP = decltype(probes)::value;
-    constexpr int kNb = decltype(nb)::value;
+    constexpr int kC = decltype(check)::value;
     if (sink.mode == kSinkRows)
-      launch_fused_mode<kSinkRows, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
-                                                  W, T, block, smem, lookback, sink, stage,
-                                                  spin_limit, stall_tile, s);
+      launch_fused_mode<kSinkRows, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
+                                                 W, T, block, smem, lookback, sink, stage,
+                                                 spin_limit, stall_tile, s);
     else if (sink.mode == kSinkKeys)
-      launch_fused_mode<kSinkKeys, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
-                                                  W, T, block, smem, lookback, sink, false,
-                                                  spin_limit, stall_tile, s);
+      launch_fused_mode<kSinkKeys, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
+                                                 W, T, block, smem, lookback, sink, false,
+                                                 spin_limit, stall_tile, s);
     else
-      launch_fused_mode<kSinkColumns, kMax, kP, kNb>(g, d, F, ld, pstart, pslot, woff, tile_row,
-                                                     wa, W, T, block, smem, lookback, sink, false,
-                                                     spin_limit, stall_tile, s);
+      launch_fused_mode<kSinkColumns, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row,
+                                                    wa, W, T, block, smem, lookback, sink, false,
+                                                    spin_limit, stall_tile, s);
   };
   // the probe-byte accounting is a separate instance, so the default one
   // carries no trace of it
-  const int nb = row_check_nb(d, block);
+  using std::false_type;
   using std::integral_constant;
-  if (nb == 1)
-    go(std::true_type{}, std::false_type{}, integral_constant<int, 1>{});
-  else if (nb == 2)
-    go(std::true_type{}, std::false_type{}, integral_constant<int, 2>{});
-  else if (nb == 3)
-    go(std::true_type{}, std::false_type{}, integral_constant<int, 3>{});
-  else if (block <= 256 && !d.count_probes)
-    go(std::true_type{}, std::false_type{}, integral_constant<int, 0>{});
+  using std::true_type;
+  switch (check_form(d, block, W, rows)) {
+    case kCheckRow + 1: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 1>{});
+    case kCheckRow + 2: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 2>{});
+    case kCheckRow + 3: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 3>{});
+    case kCheckGroup + 2:
+      return go(true_type{}, false_type{}, integral_constant<int, kCheckGroup + 2>{});
+    case kCheckGroup + 3:
+      return go(true_type{}, false_type{}, integral_constant<int, kCheckGroup + 3>{});
+    default: break;
+  }
+  const integral_constant<int, kCheckAny> any;
+  if (block <= 256 && !d.count_probes)
+    go(true_type{}, false_type{}, any);
   else if (block <= 256)
-    go(std::true_type{}, std::true_type{}, integral_constant<int, 0>{});
+    go(true_type{}, true_type{}, any);
   else if (!d.count_probes)
-    go(std::false_type{}, std::false_type{}, integral_constant<int, 0>{});
+    go(false_type{}, false_type{}, any);
   else
-    go(std::false_type{}, std::true_type{}, integral_constant<int, 0>{});
+    go(false_type{}, true_type{}, any);
 }
 
 void launch_split_points(const int64_t *woff, int64_t R, int64_t step, int64_t J,

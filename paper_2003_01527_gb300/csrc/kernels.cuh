@@ -260,7 +260,7 @@ constexpr int32_t kCountWords = 3 + kMaxK;
 void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,
                       int64_t rows, unsigned long long *total, cudaStream_t s);
 
-// Verification pass over candidates [wa, wb): writes one survivor bit per
+// Verification pass over candidates [wa, wb) of `rows` rows: writes one survivor bit per
 // candidate into masks (if non-null), one survivor count per tile into
 // tile_cnt (if non-null), and adds the total into *total (if non-null).  With
 // leaf (null masks and tile_cnt), each survivor adds its leaf number into the
@@ -268,8 +268,9 @@ void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F,
 void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                         uint32_t *masks, int32_t *tile_cnt, unsigned long long *total,
-                         cudaStream_t s, const LeafDesc *leaf = nullptr);
+                         int64_t rows, uint32_t *masks, int32_t *tile_cnt,
+                         unsigned long long *total, cudaStream_t s,
+                         const LeafDesc *leaf = nullptr);
 
 // Where the write pass puts a row.  kSinkColumns: column-major int32 (the
 // frontier layout), column c of row r at out[c*ld + r].  kSinkRows: row-major
@@ -335,8 +336,8 @@ constexpr int32_t kLbSpinLimit = 1 << 20;  // default bound of a look-back wait 
 void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                         unsigned long long *lookback, const RowSink &sink, int32_t spin_limit,
-                         int32_t stall_tile, cudaStream_t s);
+                         int64_t rows, unsigned long long *lookback, const RowSink &sink,
+                         int32_t spin_limit, int32_t stall_tile, cudaStream_t s);
 
 // Row boundaries for work-bounded sub-chunks: bounds[j] = the row r with
 // woff[r] <= j*step < woff[r+1] (clamped to [0, R]); bounds[J] = R.

@@ -116,73 +116,6 @@ __device__ __forceinline__ bool check_candidate(const GraphDev &g, const Desc &d
   return true;
 }
 
-template <typename Row>
-__device__ __forceinline__ bool lookahead_ok(const GraphDev &g, const LevelDesc &d,
-                                             const Row &row, int32_t w);
-
-// The check of one row's candidates.  kNb = 0: check_candidate and the
-// look-ahead, everything of the row read again for every candidate.  kNb = 1
-// to 3 (that many mapped neighbours, at most two injectivity tests, no
-// look-ahead): what the check needs of the row is loaded once per row and kept
-// in registers, with where the other neighbours' adjacency is.  The last level of
-// a 5-cycle listing on R-MAT 20 (67 M candidates, four a row) went from 2.00 to
-// 1.67 ms with it, the distinct 4-cliques of R-MAT 16 from 11.3 to 9.8 ms.
-constexpr int kMaxRowCheck = 3;
-template <int kNb>
-struct RowCheck {
-  static constexpr int kOthers = kNb > 1 ? kNb - 1 : 1;
-  int32_t inj0 = -1, inj1 = -1;  // same-label images
-  // neighbours besides the pivot: x, and its row [b, e) or, when x is a hub,
-  // e = -1 and b = its bitmap's index
-  int32_t x[kOthers], b[kOthers], e[kOthers];
-  bool few = false;
-
-  __device__ __forceinline__ void load(const GraphDev &g, const LevelDesc &d,
-                                       const ColumnRow &row, int slot, int32_t candidates) {
-    few = candidates <= kFewCandidates;
-    if constexpr (kNb > 0) {
-      if (d.ninj > 0) inj0 = row(d.inj[0]);
-      if (d.ninj > 1) inj1 = row(d.inj[1]);
-    }
-    if constexpr (kNb > 1) {
-#pragma unroll
-      for (int o = 0; o < kOthers; ++o) {
-        x[o] = row(d.bpos[o + (o >= slot)]);
-        b[o] = e[o] = 0;
-        if (!GSM_IN_BOUNDS(g.dbg, x[o] >= 0 && x[o] < g.n, kDbgNeighbour)) continue;
-        const int32_t h = g.hub ? __ldg(g.hub + x[o]) : -1;
-        if (h >= 0) {
-          b[o] = h;
-          e[o] = -1;
-        } else {
-          b[o] = __ldg(g.rp + x[o]);
-          e[o] = __ldg(g.rp + x[o] + 1);
-        }
-      }
-    }
-  }
-
-  __device__ __forceinline__ bool ok(const GraphDev &g, const LevelDesc &d, const ColumnRow &row,
-                                     int32_t w, int slot) const {
-    if constexpr (kNb == 0) {
-      return check_candidate(g, d, row, w, slot, few) && (!d.la || lookahead_ok(g, d, row, w));
-    } else {
-      if (w == inj0 || w == inj1) return false;
-      if (d.bitmap && !bitmap_has(d.bitmap, w)) return false;
-      if constexpr (kNb > 1) {
-#pragma unroll
-        for (int o = 0; o < kOthers; ++o) {
-          const bool in = e[o] < 0 ? hub_bit(g, b[o], w)
-                          : few    ? row_contains_few(g, x[o], b[o], e[o], d.lab, w)
-                                   : row_search(g, b[o], e[o], d.lab, w);
-          if (!in) return false;
-        }
-      }
-      return true;
-    }
-  }
-};
-
 // check_candidate that also adds to *probe_bytes 4 * ceil(log2 deg(x)) for
 // every non-tree edge check it makes against a mapped vertex x (the bytes a
 // binary search of x's row reads; the check itself may be one bitmap probe).
@@ -332,6 +265,272 @@ __device__ __forceinline__ bool lookahead_ok(const GraphDev &g, const LevelDesc 
     }
   }
   return true;
+}
+
+// The check of one row's candidates for 1 to 3 mapped neighbours, at most two
+// injectivity tests and no look-ahead: what it needs of the row is loaded once
+// per row and kept in registers, with where the other neighbours' adjacency is.  The last level of
+// a 5-cycle listing on R-MAT 20 (67 M candidates, four a row) went from 2.00 to
+// 1.67 ms with it, the distinct 4-cliques of R-MAT 16 from 11.3 to 9.8 ms.
+template <int kNb>
+struct RowCheck {
+  static constexpr int kOthers = kNb > 1 ? kNb - 1 : 1;
+  int32_t inj0 = -1, inj1 = -1;  // same-label images
+  // the neighbours besides the pivot: row [b, e), or, of a hub, e = -1 and b =
+  // its bitmap's index
+  int32_t b[kOthers], e[kOthers];
+
+  __device__ __forceinline__ void load(const GraphDev &g, const LevelDesc &d,
+                                       const ColumnRow &row, int slot) {
+    if (d.ninj > 0) inj0 = row(d.inj[0]);
+    if (d.ninj > 1) inj1 = row(d.inj[1]);
+    if constexpr (kNb > 1) {
+#pragma unroll
+      for (int o = 0; o < kOthers; ++o) {
+        const int32_t x = row(d.bpos[o + (o >= slot)]);
+        b[o] = e[o] = 0;
+        if (!GSM_IN_BOUNDS(g.dbg, x >= 0 && x < g.n, kDbgNeighbour)) continue;
+        const int32_t h = g.hub ? __ldg(g.hub + x) : -1;
+        if (h >= 0) {
+          b[o] = h;
+          e[o] = -1;
+        } else {
+          b[o] = __ldg(g.rp + x);
+          e[o] = __ldg(g.rp + x + 1);
+        }
+      }
+    }
+  }
+
+  __device__ __forceinline__ bool ok(const GraphDev &g, const LevelDesc &d, int32_t w) const {
+    if (w == inj0 || w == inj1) return false;
+    if (d.bitmap && !bitmap_has(d.bitmap, w)) return false;
+    if constexpr (kNb > 1) {
+#pragma unroll
+      for (int o = 0; o < kOthers; ++o)
+        if (!(e[o] < 0 ? hub_bit(g, b[o], w) : row_search(g, b[o], e[o], d.lab, w))) return false;
+    }
+    return true;
+  }
+};
+
+// How a level's launch checks its candidates.
+//   kCheckAny      every shape: check_candidate and the look-ahead, one
+//                  candidate after the other, the row read again for each
+//   kCheckRow + n  n = 1..3 mapped neighbours, at most two injectivity tests,
+//                  no look-ahead: RowCheck
+//   kCheckGroup+n  the same shapes, n = 2, 3: the loads of a thread's four
+//                  candidates are issued together, stage by stage -- candidate
+//                  bitmap, images of the row, hub indexes, adjacency words, and
+//                  the steps of the binary searches
+// A check is a chain of dependent loads.  With few candidates a row they miss
+// L1 and the chains' latency bounds the level: grouped, the last level of a
+// 5-cycle listing on R-MAT 20 (four candidates a row) takes 1.46 instead of
+// 1.67 ms.  With many, the row's adjacency stays in L1 and the grouped form's
+// registers cost more warps than it gains: ordered triangles of R-MAT 20 (146
+// a row) 24.1 against 19.9 ms, 4-cliques of R-MAT 16 12.5 against 9.8 ms.
+// Hence grouped up to kFewCandidates candidates a row on average.
+constexpr int kCheckAny = 0, kCheckRow = 0, kCheckGroup = 3;
+constexpr int kMaxRowCheck = 3;
+
+// The candidates x = xb .. xb + 3 of one thread, below x1: returns a bit for
+// each that passes the level's checks; rj, wj: their rows and vertices.
+// kProbes (kCheckAny only): adds the checks' probe bytes to *probe_bytes.
+template <int kCheck, bool kProbes = false>
+__device__ __forceinline__ uint32_t check_group(
+    const GraphDev &g, const LevelDesc &d, const int32_t *__restrict__ F, int32_t ld,
+    const TileRows &t, const int32_t *s_woff, const int64_t *__restrict__ woff, int64_t wa,
+    const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot, int32_t xb, int32_t x1,
+    int32_t (&rj)[kItemsPerThread], int32_t (&wj)[kItemsPerThread],
+    uint32_t *probe_bytes = nullptr) {
+  constexpr int kN = kItemsPerThread;
+  constexpr int kNb = kCheck > kCheckGroup ? kCheck - kCheckGroup : 0;
+  int32_t rs;
+  int32_t r = item_row(t, s_woff, woff, wa, xb, &rs);
+  int32_t rr = r - t.r0;
+  int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+  int32_t pst = pstart[r], slot = pslot[r];
+  if constexpr (kCheck > kCheckRow && kCheck <= kCheckRow + kMaxRowCheck) {
+    RowCheck<kCheck - kCheckRow> check;
+    check.load(g, d, ColumnRow{F, ld, r}, slot);
+    uint32_t bits = 0;
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {  // (rj, wj: only of candidates that pass)
+      const int32_t x = xb + j;
+      if (x >= x1) break;
+      if (x >= re) {
+        do {  // next row (rows without work are skipped)
+          ++rr;
+          ++r;
+          rs = re;
+          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+        } while (x >= re);
+        pst = pstart[r];
+        slot = pslot[r];
+        check.load(g, d, ColumnRow{F, ld, r}, slot);
+      }
+      if (!GSM_IN_BOUNDS(g.dbg, pst + (x - rs) >= 0 && pst + (x - rs) < g.nnz, kDbgCandidate) ||
+          !GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
+        continue;
+      const int32_t w = __ldg(g.lcol + pst + (x - rs));
+      rj[j] = r;
+      wj[j] = w;
+      if (check.ok(g, d, w)) bits |= 1u << j;
+    }
+    return bits;
+  }
+  int32_t at[kN], sj[kN];
+  uint32_t alive = 0, few = 0;
+#pragma unroll
+  for (int j = 0; j < kN; ++j) {
+    const int32_t x = xb + j;
+    if (x < x1) {
+      if (x >= re) {
+        do {  // next row (rows without work are skipped)
+          ++rr;
+          ++r;
+          rs = re;
+          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
+        } while (x >= re);
+        pst = pstart[r];
+        slot = pslot[r];
+      }
+      if (GSM_IN_BOUNDS(g.dbg, pst + (x - rs) >= 0 && pst + (x - rs) < g.nnz, kDbgCandidate) &&
+          GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
+        alive |= 1u << j;
+      if (re - rs <= kFewCandidates) few |= 1u << j;
+    }
+    rj[j] = r;
+    sj[j] = slot;
+    at[j] = pst + (x - rs);
+  }
+#pragma unroll
+  for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
+  if constexpr (kCheck == kCheckAny) {
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      if (!((alive >> j) & 1u)) continue;
+      const ColumnRow row{F, ld, rj[j]};
+      bool ok;
+      if constexpr (kProbes)
+        ok = check_candidate_probes(g, d, row, wj[j], sj[j], (few >> j) & 1u, probe_bytes);
+      else
+        ok = check_candidate(g, d, row, wj[j], sj[j], (few >> j) & 1u);
+      if (!ok || (d.la && !lookahead_ok(g, d, row, wj[j]))) alive &= ~(1u << j);
+    }
+    return alive;
+  }
+  if (d.bitmap) {
+    uint32_t word[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      word[j] = (alive >> j) & 1u ? __ldg(d.bitmap + (wj[j] >> 5)) : 0u;
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (!((word[j] >> (wj[j] & 31)) & 1u)) alive &= ~(1u << j);
+  }
+  for (int i = 0; i < d.ninj; ++i) {
+    const int32_t *col = F + d.inj[i] * ld;
+    int32_t y[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) y[j] = (alive >> j) & 1u ? col[rj[j]] : -1;
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (y[j] == wj[j]) alive &= ~(1u << j);
+  }
+#pragma unroll
+  for (int o = 0; o + 1 < kNb; ++o) {  // neighbours besides the pivot
+    int32_t x[kN], h[kN];
+    uint32_t word[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      x[j] = (alive >> j) & 1u ? F[d.bpos[o + (o >= sj[j])] * ld + rj[j]] : 0;
+      if (!GSM_IN_BOUNDS(g.dbg, x[j] >= 0 && x[j] < g.n, kDbgNeighbour)) {
+        alive &= ~(1u << j);
+        x[j] = 0;
+      }
+    }
+    uint32_t open = alive;  // candidates no bitmap has decided
+    if (g.hub) {
+#pragma unroll
+      for (int j = 0; j < kN; ++j) h[j] = (alive >> j) & 1u ? __ldg(g.hub + x[j]) : -1;
+      uint32_t rev = 0;  // taken from the candidate's bitmap
+#pragma unroll
+      for (int j = 0; j < kN; ++j)
+        if (h[j] < 0 && (alive & few) >> j & 1u) {
+          h[j] = __ldg(g.hub + wj[j]);
+          rev |= 1u << j;
+        }
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        const int32_t v = (rev >> j) & 1u ? x[j] : wj[j];
+        word[j] = h[j] >= 0 ? __ldg(g.hub_bits + (size_t)h[j] * g.hub_words + (v >> 5)) >> (v & 31)
+                            : 0u;
+      }
+#pragma unroll
+      for (int j = 0; j < kN; ++j)
+        if (h[j] >= 0) {
+          open &= ~(1u << j);
+          if (!(word[j] & 1u)) alive &= ~(1u << j);
+        }
+    }
+    if (open) {  // binary searches, step by step together
+      int32_t lo[kN], len[kN], end[kN], key[kN], lab[kN];
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        const bool on = (open >> j) & 1u;
+        lo[j] = on ? __ldg(g.rp + x[j]) : 0;
+        end[j] = on ? __ldg(g.rp + x[j] + 1) : 0;
+        key[j] = wj[j];
+        lab[j] = d.lab;
+      }
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        if ((few & open) >> j & 1u && end[j] - lo[j] > kLongRow) {
+          const int32_t wb = __ldg(g.rp + wj[j]), we = __ldg(g.rp + wj[j] + 1);
+          if (we - wb < end[j] - lo[j]) {  // the candidate's row is shorter: x in it
+            lo[j] = wb;
+            end[j] = we;
+            key[j] = x[j];
+            lab[j] = __ldg(g.lab + x[j]);
+          }
+        }
+        len[j] = end[j] - lo[j];
+      }
+      const bool one = g.num_labels == 1;
+      bool more = true;
+      while (more) {
+        more = false;
+        int32_t v[kN], m[kN];
+#pragma unroll
+        for (int j = 0; j < kN; ++j) {
+          const int32_t mid = lo[j] + (len[j] >> 1);
+          v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
+          m[j] = len[j] > 0 && !one ? __ldg(g.llab + mid) : lab[j];
+        }
+#pragma unroll
+        for (int j = 0; j < kN; ++j) {
+          if (len[j] <= 0) continue;
+          const int32_t half = len[j] >> 1;
+          if (m[j] < lab[j] || (m[j] == lab[j] && v[j] < key[j])) {
+            lo[j] += half + 1;
+            len[j] -= half + 1;
+          } else {
+            len[j] = half;
+          }
+          more = more || len[j] > 0;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        if (!((open >> j) & 1u)) continue;
+        const bool in = lo[j] < end[j] && __ldg(g.lcol + lo[j]) == key[j] &&
+                        (one || __ldg(g.llab + lo[j]) == lab[j]);
+        if (!in) alive &= ~(1u << j);
+      }
+    }
+  }
+  return alive;
 }
 
 // Writes the partial embedding `src` (src(c) = image of pi_c, c < d.i)
