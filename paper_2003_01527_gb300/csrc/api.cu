@@ -65,6 +65,7 @@ struct Block {
 }  // namespace
 
 constexpr size_t kSmallBytes = 512;  // gsm_ctx::d_small
+constexpr int32_t kSmallCount = 18;  // where a count's words (kCountWords) start in it
 
 struct gsm_query {
   int32_t k = 0, m = 0;
@@ -110,7 +111,7 @@ struct gsm_ctx {
   size_t bitmaps2_cap = 0;
   void *mfilter = nullptr;  // gsm_enumerate_many: descriptors, sizes and bitmaps of all queries
   size_t mfilter_cap = 0;
-  unsigned long long *d_small = nullptr;  // [0..15] sizes, [16..34] a count (kCountWords), [17] err
+  unsigned long long *d_small = nullptr;  // [0..15] sizes, [16] finished CTAs, [17] err, then a count
   void *acc[2] = {nullptr, nullptr};
   size_t acc_cap[2] = {0, 0};
   // gsm_enumerate_many: the result buffers (acc, sort_keys) come in several
@@ -156,6 +157,7 @@ struct gsm_ctx {
   // (the copy engines stay free for result copies in flight)
   int64_t *h_stage = nullptr;
   void *d_stage = nullptr;  // device view of h_stage
+  int64_t stage_seq = 0;    // number of the last read-back a kernel makes by itself (Stage)
   // mapped flag words after the 4 KB of h_stage: [0] = a sort's look-back
   // wait ran out (set by the sort kernels, read and cleared by the host)
   uint32_t *h_flags = nullptr, *d_flags = nullptr;
@@ -431,6 +433,34 @@ void fetch(gsm_ctx *ctx, const void *dptr, size_t bytes) {
   ctx->run.kernel_launches += 1;
   CU(cudaGetLastError());
   CU(cudaStreamSynchronize(ctx->stream));
+}
+
+// The next read-back a kernel makes by itself, and the wait for it: polls the
+// sequence number in the mapped page (every other access of the kernel's CTAs
+// is done by then; what the stream does next is ordered after the kernel).
+// The stream is asked now and then, so that a failed launch ends the wait.
+Stage next_stage(gsm_ctx *ctx) { return Stage{(long long *)ctx->d_stage, ++ctx->stage_seq}; }
+
+void wait_stage(gsm_ctx *ctx) {
+  CU(cudaGetLastError());
+  const volatile int64_t *seq = ctx->h_stage + kStageSeq;
+  for (int32_t asked = 0;; ++asked) {
+    for (int32_t n = 0; n < 20000; ++n)
+      if (*seq == ctx->stage_seq) {
+        std::atomic_thread_fence(std::memory_order_acquire);
+        return;
+      }
+    if (asked >= 64) {
+      CU(cudaStreamSynchronize(ctx->stream));  // a long kernel: no more polling
+    } else {
+      const cudaError_t e = cudaStreamQuery(ctx->stream);
+      if (e == cudaErrorNotReady) continue;
+      CU(e);
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    if (*seq == ctx->stage_seq) return;
+    FAIL(GSM_ERR_CUDA, "a kernel finished without its read-back");
+  }
 }
 
 // GSM_OPT_INJECT_SORT_STALL: the tile of every sort pass that withholds its
@@ -727,10 +757,29 @@ struct Run {
 
 void recurse(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows);
 void recurse_rest(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows,
-                  const int32_t *pstart, const uint8_t *pslot, const int64_t *woff, int64_t W);
+                  const int32_t *pstart, const uint8_t *pslot, const int64_t *woff, int64_t W,
+                  const LevelSetup &setup);
 void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t *pstart,
                    const uint8_t *pslot, const int64_t *woff, int64_t ra, int64_t rb, int64_t wa,
-                   int64_t wb);
+                   int64_t wb, const LevelSetup &setup);
+
+// Room on the stack for what a level's pivot scan prepares (LevelSetup), for
+// rows of the level (at most); none if it does not fit the budget.  Enough for
+// 128 candidates a row on average, at most 8,192 tiles (8 M candidates, 0.4 ms
+// of checks, beside which one more launch does not count).
+LevelSetup push_setup(Run &R, int64_t rows) {
+  gsm_ctx *ctx = R.ctx;
+  LevelSetup st;
+  st.tile_items = R.block * kItemsPerThread;
+  st.cap = (int32_t)std::min<int64_t>(8192, 64 + rows / 8);
+  const size_t words = sizeof(unsigned long long) * level_setup_words(st.cap, st.tile_items);
+  const size_t bytes = align_up(words) + align_up(sizeof(int32_t) * (size_t)(st.cap + 1));
+  if (!stack_fits(ctx, bytes)) return LevelSetup();
+  char *p = (char *)stack_push(ctx, bytes);
+  st.lb = (unsigned long long *)p;
+  st.tile_row = (int32_t *)(p + align_up(words));
+  return st;
+}
 
 // Largest result staging (bytes) the single-pass last level may reserve for
 // its upper bound of one row per candidate.
@@ -760,7 +809,7 @@ void ensure_acc(Run &R, uint64_t rows) {
 
 void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t *pstart,
                  const uint8_t *pslot, const int64_t *woff, int64_t ra, int64_t rb, int64_t wa,
-                 int64_t wb) {
+                 int64_t wb, const LevelSetup &setup = LevelSetup()) {
   gsm_ctx *ctx = R.ctx;
   const Range range(level_range(i));
   const LevelDesc &d = R.lv[i];
@@ -787,21 +836,23 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
       fits = (int64_t)W * w_out < (int64_t(1) << 31) - 1 && stack_fits(ctx, need);
     }
     if (fits) {
-      process_fused(R, i, F, ld, pstart, pslot, woff, ra, rb, wa, wb);
+      process_fused(R, i, F, ld, pstart, pslot, woff, ra, rb, wa, wb, setup);
       return;
     }
   }
   Carve cv;
-  const size_t o_row = cv.add<int32_t>(tiles + 1);
+  const bool ready = tiles <= setup.cap;  // the pivot scan has written tile_row
+  const size_t o_row = cv.add<int32_t>(ready ? 0 : tiles + 1);
   const size_t o_mask = count_only ? 0 : cv.add<uint32_t>(tiles * (tile_items / 32));
   const size_t o_cnt = count_only ? 0 : cv.add<int32_t>(tiles);
   const size_t o_off = count_only ? 0 : cv.add<int64_t>(tiles + 1);
   const size_t o_tmp = count_only ? 0 : cv.add<int64_t>(scan_tmp_elems(tiles));
   char *sc = (char *)scratch_get(ctx, cv.off);
-  int32_t *tile_row = (int32_t *)(sc + o_row);
-  timed(ctx, K_PIVOT, 8.0 * (nrows + tiles), (uint64_t)tiles, 1, [&] {
-    launch_tile_rows(woff, ra, rb, wa, wb, R.block, tile_row, nullptr, ctx->stream);
-  });
+  int32_t *tile_row = ready ? setup.tile_row : (int32_t *)(sc + o_row);
+  if (!ready)
+    timed(ctx, K_PIVOT, 8.0 * (nrows + tiles), (uint64_t)tiles, 1, [&] {
+      launch_tile_rows(woff, ra, rb, wa, wb, R.block, tile_row, nullptr, ctx->stream);
+    });
   if (count_only) {
     timed(ctx, K_COUNT, read_bytes, (uint64_t)W, 1, [&] {
       launch_extend_count(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nrows,
@@ -865,7 +916,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
 // (k_extend_fused); the caller checked that the output has room for W rows.
 void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t *pstart,
                    const uint8_t *pslot, const int64_t *woff, int64_t ra, int64_t rb, int64_t wa,
-                   int64_t wb) {
+                   int64_t wb, const LevelSetup &setup) {
   gsm_ctx *ctx = R.ctx;
   const Range range(level_range(i));
   const LevelDesc &d = R.lv[i];
@@ -873,19 +924,23 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   const int64_t W = wb - wa, nrows = rb - ra;
   const int64_t tiles = extend_tiles(wa, wb, R.block);
   const int32_t w_out = i + 1;
-  Carve cv;
-  const size_t o_row = cv.add<int32_t>(tiles + 1);
   // the level's look-back words, then (not last) those of the next level's
-  // pivot choice and work scan (sized for up to W rows); k_tile_rows zeroes
-  // both
-  const int64_t pwords = last ? 0 : pivot_scan_words(W);
-  const size_t o_lb = cv.add<unsigned long long>(tiles + kLbExtra + pwords);
-  char *sc = (char *)scratch_get(ctx, cv.off);
-  int32_t *tile_row = (int32_t *)(sc + o_row);
-  unsigned long long *lb = (unsigned long long *)(sc + o_lb);
-  timed(ctx, K_PIVOT, 8.0 * (nrows + tiles) + 8.0 * (tiles + pwords), (uint64_t)tiles, 1, [&] {
-    launch_tile_rows(woff, ra, rb, wa, wb, R.block, tile_row, lb, ctx->stream, pwords);
-  });
+  // pivot choice and work scan (sized for up to W rows): zeroed by the pivot
+  // scan (setup), else by k_tile_rows
+  int32_t *tile_row = setup.tile_row;
+  unsigned long long *lb = setup.lb;
+  if (tiles > setup.cap) {
+    Carve cv;
+    const size_t o_row = cv.add<int32_t>(tiles + 1);
+    const int64_t pwords = last ? 0 : pivot_scan_words(W);
+    const size_t o_lb = cv.add<unsigned long long>(tiles + kLbExtra + pwords);
+    char *sc = (char *)scratch_get(ctx, cv.off);
+    tile_row = (int32_t *)(sc + o_row);
+    lb = (unsigned long long *)(sc + o_lb);
+    timed(ctx, K_PIVOT, 8.0 * (nrows + tiles) + 8.0 * (tiles + pwords), (uint64_t)tiles, 1, [&] {
+      launch_tile_rows(woff, ra, rb, wa, wb, R.block, tile_row, lb, ctx->stream, pwords);
+    });
+  }
   const double read_bytes = (double)nrows * (4.0 * i + 13.0) + 4.0 * (double)W;
   const Mark mk = stack_mark(ctx);
   RowSink sink;
@@ -902,11 +957,12 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   }
   timed(ctx, K_FUSED, read_bytes, (uint64_t)W, 1, [&] {
     launch_extend_fused(R.g, d, F, ld, pstart, pslot, woff, tile_row, wa, wb, R.block, nrows, lb,
-                        sink, R.spin_limit, R.stall_tile, ctx->stream);
+                        sink, R.spin_limit, R.stall_tile, last ? next_stage(ctx) : Stage(),
+                        ctx->stream);
   });
   const int64_t *S_dev = (const int64_t *)(lb + tiles + 1);
   if (last) {
-    fetch(ctx, S_dev, 3 * sizeof(unsigned long long));
+    wait_stage(ctx);
     const int64_t S = ((volatile int64_t *)ctx->h_stage)[0];
     if (((volatile int64_t *)ctx->h_stage)[1])
       FAIL(GSM_ERR_TIMEOUT, "a verification tile waited too long for its predecessors");
@@ -924,12 +980,12 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   int32_t *pstart2 = (int32_t *)stack_push(ctx, sizeof(int32_t) * W);
   uint8_t *pslot2 = (uint8_t *)stack_push(ctx, W);
   int64_t *woff2 = (int64_t *)stack_push(ctx, sizeof(int64_t) * (W + 1));
+  const LevelSetup next = push_setup(R, W);
   timed(ctx, K_PIVOT, 0.0, 0, 1, [&] {
     launch_pivot_scan(R.g, dn, Fn, W, W, pstart2, pslot2, woff2, lb + tiles + kLbExtra,
-                      R.spin_limit, ctx->d_stage, R.scan_stall_tile, ctx->stream, S_dev);
+                      R.spin_limit, next_stage(ctx), next, R.scan_stall_tile, ctx->stream, S_dev);
   });
-  CU(cudaGetLastError());
-  CU(cudaStreamSynchronize(ctx->stream));
+  wait_stage(ctx);
   const int64_t S = ((volatile int64_t *)ctx->h_stage)[0];
   if (((volatile int64_t *)ctx->h_stage)[1])
     FAIL(GSM_ERR_TIMEOUT,
@@ -940,7 +996,7 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   ctx->kstats[K_FUSED].probe_bytes += probes;
   ctx->kstats[K_PIVOT].algo_bytes += (double)S * (4.0 * dn.nb + 8.0 * dn.nb + 13.0);
   ctx->kstats[K_PIVOT].items += (uint64_t)S;
-  if (S > 0) recurse_rest(R, i + 1, Fn, W, S, pstart2, pslot2, woff2, W2);
+  if (S > 0) recurse_rest(R, i + 1, Fn, W, S, pstart2, pslot2, woff2, W2, next);
   stack_release(ctx, mk);
 }
 
@@ -1004,23 +1060,24 @@ void recurse(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows) {
   const int64_t pwords = pivot_scan_words(rows);
   auto *plb = (unsigned long long *)scratch_get(ctx, sizeof(unsigned long long) * pwords);
   CU(cudaMemsetAsync(plb, 0, sizeof(unsigned long long) * pwords, ctx->stream));
+  const LevelSetup setup = push_setup(R, rows);
   timed(ctx, K_PIVOT, (double)rows * (4.0 * d.nb + 8.0 * d.nb + 13.0), (uint64_t)rows, 1,
         [&] {
     launch_pivot_scan(R.g, d, F, ld, rows, pstart, pslot, woff, plb, R.spin_limit,
-                      ctx->d_stage, R.scan_stall_tile, ctx->stream);
+                      next_stage(ctx), setup, R.scan_stall_tile, ctx->stream);
   });
-  CU(cudaGetLastError());
-  CU(cudaStreamSynchronize(ctx->stream));
+  wait_stage(ctx);
   if (((volatile int64_t *)ctx->h_stage)[1])
     FAIL(GSM_ERR_TIMEOUT, "a work-scan tile waited too long for its predecessors");
   const int64_t W = ((volatile int64_t *)ctx->h_stage)[2];
-  recurse_rest(R, i, F, ld, rows, pstart, pslot, woff, W);
+  recurse_rest(R, i, F, ld, rows, pstart, pslot, woff, W, setup);
   stack_release(ctx, mk);
 }
 
 // The part of recurse after the pivot and work scan (W = total candidates).
 void recurse_rest(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows,
-                  const int32_t *pstart, const uint8_t *pslot, const int64_t *woff, int64_t W) {
+                  const int32_t *pstart, const uint8_t *pslot, const int64_t *woff, int64_t W,
+                  const LevelSetup &setup) {
   R.ctx->run.frontier[i] += (uint64_t)rows;
   R.ctx->run.candidates[i] += (uint64_t)W;
   if (i == R.k - 1 && R.rank_p > 0 && rows > 0) {
@@ -1038,8 +1095,9 @@ void recurse_rest(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows,
   }
   std::vector<int64_t> bnd, bw;
   level_chunks(R, woff, rows, W, bnd, bw);
-  for (size_t j = 0; j + 1 < bnd.size(); ++j)
-    process_sub(R, i, F, ld, pstart, pslot, woff, bnd[j], bnd[j + 1], bw[j], bw[j + 1]);
+  for (size_t j = 0; j + 1 < bnd.size(); ++j)  // (the setup is of the level in one piece)
+    process_sub(R, i, F, ld, pstart, pslot, woff, bnd[j], bnd[j + 1], bw[j], bw[j + 1],
+                bnd.size() == 2 ? setup : LevelSetup());
   if (i == R.k - 1) R.rank = nullptr;
 }
 
@@ -1347,12 +1405,14 @@ void run_filter(gsm_ctx *ctx, const gsm_query *q, const int32_t *dense, uint64_t
   fill_filter(ctx, q, dense, fd);
   const size_t bytes = (size_t)q->k * fd.n_words * sizeof(uint32_t);
   ensure_buf(ctx, &ctx->bitmaps, &ctx->bitmaps_cap, bytes, false, 0);
-  CU(cudaMemsetAsync(ctx->d_small, 0, sizeof(unsigned long long) * kMaxK, ctx->stream));
+  CU(cudaMemsetAsync(ctx->d_small, 0, kSmallBytes, ctx->stream));
   GraphDev g = graph_dev(ctx);
-  timed(ctx, K_FILTER, 12.0 * ctx->n + bytes, (uint64_t)ctx->n, 1, [&] {
-    launch_filter(g, fd, (uint32_t *)ctx->bitmaps, ctx->d_small, ctx->stream);
-  });
   const int32_t rounds = std::max<int32_t>(0, ctx->opt.filter_rounds);
+  const bool staged = filter_stages(g) && !(rounds > 0 && q->k > 1);
+  timed(ctx, K_FILTER, 12.0 * ctx->n + bytes, (uint64_t)ctx->n, 1, [&] {
+    launch_filter(g, fd, (uint32_t *)ctx->bitmaps, ctx->d_small, ctx->stream,
+                  staged ? next_stage(ctx) : Stage());
+  });
   if (rounds > 0 && q->k > 1) {
     RefineDesc rd;
     std::memset(&rd, 0, sizeof(rd));
@@ -1379,7 +1439,10 @@ void run_filter(gsm_ctx *ctx, const gsm_query *q, const int32_t *dense, uint64_t
       std::swap(ctx->bitmaps_cap, ctx->bitmaps2_cap);
     }
   }
-  fetch(ctx, ctx->d_small, sizeof(uint64_t) * q->k);
+  if (staged)
+    wait_stage(ctx);
+  else
+    fetch(ctx, ctx->d_small, sizeof(uint64_t) * q->k);
   std::memcpy(sizes, ctx->h_stage, sizeof(uint64_t) * q->k);
 }
 
@@ -1422,7 +1485,7 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   R.wcap = std::max<int64_t>((int64_t)ctx->max_deg + 1,
                              std::min<int64_t>((int64_t(1) << 30) - 4096,
                                                (int64_t)(ctx->scratch_limit / 2) * 7));
-  R.d_total = ctx->d_small + kMaxK;
+  R.d_total = ctx->d_small + kSmallCount;
   ctx->run.k = q->k;
   *truncated = false;
   *count_out = 0;
@@ -1544,11 +1607,18 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     d.cut = d.rlo > 0 || d.rhi < ctx->n || d.ngt > 0;
   }
 
-  CU(cudaMemsetAsync(R.d_total, 0, sizeof(unsigned long long) * kCountWords, ctx->stream));
+  // (run_filter has zeroed the count's words; a listing adds up none)
   const Mark mk = stack_mark(ctx);
   const int64_t R1 = (int64_t)sizes[R.order[0]];
   int32_t *F1 = (int32_t *)stack_push(ctx, sizeof(int32_t) * R1);
-  {
+  // only words that the root's restriction reaches can be non-zero
+  const int32_t w0 = std::min(std::max(0, q->lo[R.order[0]]), ctx->n) / 32,
+                w1 = (int32_t)(((int64_t)std::min(ctx->n, q->hi[R.order[0]]) + 31) / 32);
+  if (w1 - w0 <= kListDirectWords) {
+    timed(ctx, K_LIST, (w1 - w0) * 4.0 + 4.0 * R1, (uint64_t)R1, 1, [&] {
+      launch_list_direct(bm + (size_t)R.order[0] * nw, w0, w1, F1, ctx->stream);
+    });
+  } else {
     Carve cv;
     const size_t o_cnt = cv.add<int32_t>(nw), o_off = cv.add<int64_t>(nw + 1),
                  o_tmp = cv.add<int64_t>(scan_tmp_elems(nw));
@@ -2809,7 +2879,7 @@ gsm_status gsm_create(gsm_ctx **out, int32_t device, const gsm_options *opt) {
     CU(cudaHostGetDevicePointer(&ctx->d_stage, ctx->h_stage, 0));
     ctx->h_flags = (uint32_t *)((char *)ctx->h_stage + 4096);
     ctx->d_flags = (uint32_t *)((char *)ctx->d_stage + 4096);
-    std::memset(ctx->h_flags, 0, 64);
+    std::memset((void *)ctx->h_stage, 0, 4096 + 64);
     CU(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device));
     ctx->d_small = (unsigned long long *)dev_alloc(ctx, kSmallBytes);
   });

@@ -111,8 +111,19 @@ __global__ void __launch_bounds__(256) k_filter(GraphDev g, FilterDesc d,
 __global__ void __launch_bounds__(256) k_filter_bits(GraphDev g,
                                                      const __grid_constant__ FilterDesc d,
                                                      uint32_t *__restrict__ bitmaps,
-                                                     unsigned long long *__restrict__ sizes) {
+                                                     unsigned long long *sizes, Stage stage) {
   filter_words(g, d, bitmaps, sizes, blockIdx.y, gridDim.y);
+  if (!stage.words) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();  // the CTA's sizes before its count
+    if (atomicAdd(sizes + kMaxK, 1ull) == (unsigned long long)gridDim.x * gridDim.y - 1) {
+      __threadfence();
+      for (int u = 0; u < d.k; ++u) stage.words[u] = (long long)atomicAdd(sizes + u, 0ull);
+      __threadfence_system();
+      *(volatile long long *)(stage.words + kStageSeq) = stage.seq;
+    }
+  }
 }
 
 // One warp per 32 vertices: ballots of the threshold and label tests.
@@ -363,6 +374,42 @@ __global__ void k_bitmap_emit(const uint32_t *__restrict__ bm, int32_t n_words,
   }
 }
 
+// The list in one launch: CTA b adds up the words before its 1,024 itself, so
+// there is no scan to wait for.  Latency-bound; for the 2,048 words of an
+// R-MAT 16 graph it replaces three launches, and up to kListDirectWords words
+// (a CTA reads at most 128 KB of L2) it stays near 3 us.
+__global__ void __launch_bounds__(256) k_list_direct(const uint32_t *__restrict__ bm, int32_t w0,
+                                                     int32_t w1, int32_t *__restrict__ out) {
+  __shared__ int64_t s_scan[33];
+  __shared__ int32_t s_warp[33];
+  const int32_t base = w0 + blockIdx.x * 1024;
+  int64_t sum = 0, before;
+#pragma unroll 8
+  for (int32_t w = w0 + threadIdx.x; w < base; w += 256) sum += __popc(__ldg(bm + w));
+  block_excl_scan(sum, s_scan, &before);
+  uint32_t word[4];
+  int32_t c = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int32_t w = base + threadIdx.x * 4 + j;
+    word[j] = w < w1 ? __ldg(bm + w) : 0u;
+    c += __popc(word[j]);
+  }
+  int32_t total;
+  int64_t pos = before + block_rank(c, s_warp, &total);
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    for (uint32_t x = word[j]; x; x &= x - 1)
+      out[pos++] = (base + threadIdx.x * 4 + j) * 32 + __ffs(x) - 1;
+}
+
+// Hands a kernel's results to the host (one thread): the words, then the
+// sequence number it polls for.
+__device__ __forceinline__ void stage_seq(const Stage &st) {
+  __threadfence_system();
+  *(volatile long long *)(st.words + kStageSeq) = st.seq;
+}
+
 // ------------------------------------------------------------ extend
 //
 // Frontiers are column-major (SoA): position c of row r of a frontier with
@@ -377,9 +424,10 @@ __global__ void k_bitmap_emit(const uint32_t *__restrict__ bm, int32_t n_words,
 // (lookback_prefix), so the scan needs no second launch.  lookback:
 // ptiles + kLbExtra zeroed words (tile words, then the ticket, the total,
 // the error word and the count of finished CTAs).  The CTA that finishes
-// last writes woff[R] and, with stage (mapped host memory), stage[0] = the
-// row count, stage[1] = the error words (the producing level's and this
-// scan's, OR-ed), stage[2] = the total and stage[3] = the producing level's
+// last writes woff[R], finishes the level's setup (LevelSetup: a row writes
+// itself into tile_row for every tile that starts among its candidates) and
+// stages [0] = the row count, [1] = the error words (the producing level's
+// and this scan's, OR-ed), [2] = the total and [3] = the producing level's
 // probe bytes.  R_dev: as for launch_pivot_scan.
 constexpr int kPsThreads = 256, kPsIpt = 4;
 constexpr int64_t kPsRows = (int64_t)kPsThreads * kPsIpt;
@@ -387,7 +435,7 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int64_t ld, int64_t R,
     int32_t ptiles, int32_t *__restrict__ pstart, uint8_t *__restrict__ pslot,
     int64_t *__restrict__ woff, const int64_t *R_dev, unsigned long long *lookback,
-    int32_t spin_limit, long long *stage, int32_t stall_tile) {
+    int32_t spin_limit, Stage stage, LevelSetup setup, int32_t stall_tile) {
   __shared__ int64_t s_val[kPsRows];
   __shared__ int64_t s_warp[33];
   __shared__ int32_t s_tile;
@@ -495,24 +543,43 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
 #pragma unroll
     for (int j = 0; j < kPsIpt; ++j) {
       const int64_t r = base + j * kPsThreads + threadIdx.x;
-      if (r < R) woff[r] = s_val[j * kPsThreads + threadIdx.x];
+      if (r >= R) continue;
+      const int64_t s = s_val[j * kPsThreads + threadIdx.x];
+      woff[r] = s;
+      if (best[j] > 0 && s < (int64_t)setup.cap * setup.tile_items) {  // (cap * items < 2^31)
+        const uint32_t items = (uint32_t)setup.tile_items;
+        for (uint32_t t = ((uint32_t)s + items - 1) / items;
+             t < (uint32_t)setup.cap && (int64_t)t * items < s + best[j]; ++t)
+          setup.tile_row[t] = (int32_t)r;
+      }
     }
     __syncthreads();  // s_val and s_tile are reused by the next tile
   }
+  __syncthreads();  // every thread has read s_tile
   if (threadIdx.x == 0) {
     __threadfence();  // this CTA's offsets and look-back words before its count
-    const unsigned long long done = atomicAdd(lookback + ptiles + 3, 1ull);
-    if (done == gridDim.x - 1) {  // every other CTA has finished
-      __threadfence();
-      const long long W = (long long)atomicAdd(lookback + ptiles + 1, 0ull);
-      const long long err = (long long)atomicAdd(lookback + ptiles + 2, 0ull);
-      woff[R] = W;
-      if (stage) {
-        stage[0] = rows_in;
-        stage[1] = lvl_err | err;
-        stage[2] = W;
-        stage[3] = lvl_probes;
-      }
+    s_tile = atomicAdd(lookback + ptiles + 3, 1ull) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_tile) return;  // only the CTA that finishes last goes on
+  const int64_t W = (int64_t)atomicAdd(lookback + ptiles + 1, 0ull);
+  if (setup.cap > 0 && W <= (int64_t)setup.cap * setup.tile_items) {
+    const int64_t tiles = (W + setup.tile_items - 1) / setup.tile_items;
+    const int64_t words =
+        tiles + 2 * kLbExtra + max((int64_t)1, (W + kPsRows - 1) / kPsRows);
+    for (int64_t j = threadIdx.x; j < words; j += kPsThreads) setup.lb[j] = 0;
+    if (threadIdx.x == 0) setup.tile_row[tiles] = (int32_t)(R - 1);
+  }
+  if (threadIdx.x == 0) {
+    const long long err = (long long)atomicAdd(lookback + ptiles + 2, 0ull);
+    woff[R] = W;
+    if (stage.words) {
+      stage.words[0] = rows_in;
+      stage.words[1] = lvl_err | err;
+      stage.words[2] = W;
+      stage.words[3] = lvl_probes;
+      stage_seq(stage);
     }
   }
 }
@@ -731,7 +798,7 @@ __global__ void __launch_bounds__(kMaxThreads,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
     int32_t W, int32_t tiles, unsigned long long *__restrict__ lookback, RowSink sink,
-    bool stage_out, int32_t spin_limit, int32_t stall_tile) {
+    bool stage_out, int32_t spin_limit, int32_t stall_tile, Stage stage) {
   static_assert(kItemsPerThread == 4, "four candidates per thread");
   constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ int32_t smem[];
@@ -849,6 +916,17 @@ __global__ void __launch_bounds__(kMaxThreads,
     buf ^= 1;
   }
   if (pend >= 0) finish(pend, pend_T, pend_buf);
+  if (!stage.words) return;
+  __syncthreads();  // the CTA's rows are written
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(lookback + tiles + 4, 1ull) == gridDim.x - 1) {
+      __threadfence();
+      for (int w = 0; w < 3; ++w)
+        stage.words[w] = (long long)atomicAdd(lookback + tiles + 1 + w, 0ull);
+      stage_seq(stage);
+    }
+  }
 }
 
 __global__ void k_split_points(const int64_t *__restrict__ woff, int64_t R, int64_t step,
@@ -1086,12 +1164,14 @@ void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits,
                                                                                       lab_bits);
 }
 
+bool filter_stages(const GraphDev &g) { return g.thr && g.n > 0; }
+
 void launch_filter(const GraphDev &g, const FilterDesc &d, uint32_t *bitmaps,
-                   unsigned long long *sizes, cudaStream_t s) {
+                   unsigned long long *sizes, cudaStream_t s, Stage stage) {
   const int threads = 256;
   if (g.thr && d.n_words > 0) {
-    k_filter_bits<<<dim3((d.n_words + threads - 1) / threads, d.k), threads, 0, s>>>(g, d, bitmaps,
-                                                                                     sizes);
+    k_filter_bits<<<dim3((d.n_words + threads - 1) / threads, d.k), threads, 0, s>>>(
+        g, d, bitmaps, sizes, stage);
     return;
   }
   int64_t warps_needed = d.n_words;
@@ -1143,19 +1223,28 @@ void launch_bitmap_to_list(const uint32_t *bitmap, int32_t n_words, int32_t *cnt
   k_bitmap_emit<<<grid_for(n_words, 256), 256, 0, s>>>(bitmap, n_words, off, out);
 }
 
+void launch_list_direct(const uint32_t *bitmap, int32_t w0, int32_t w1, int32_t *out,
+                        cudaStream_t s) {
+  if (w1 > w0) k_list_direct<<<(w1 - w0 + 1023) / 1024, 256, 0, s>>>(bitmap, w0, w1, out);
+}
+
 int64_t pivot_scan_words(int64_t R) {
   return std::max<int64_t>(1, (R + kPsRows - 1) / kPsRows) + kLbExtra;
 }
 
+int64_t level_setup_words(int32_t cap, int32_t tile_items) {
+  return (int64_t)cap + kLbExtra + pivot_scan_words((int64_t)cap * tile_items);
+}
+
 void launch_pivot_scan(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                        int64_t R, int32_t *pstart, uint8_t *pslot, int64_t *woff,
-                       unsigned long long *lookback, int32_t spin_limit, void *stage,
-                       int32_t stall_tile, cudaStream_t s, const int64_t *R_dev) {
+                       unsigned long long *lookback, int32_t spin_limit, Stage stage,
+                       const LevelSetup &setup, int32_t stall_tile, cudaStream_t s,
+                       const int64_t *R_dev) {
   const int64_t ptiles = pivot_scan_words(R) - kLbExtra;
   const int grid = (int)std::min<int64_t>(ptiles, 152 * 4);  // the CTAs resident at once
   k_pivot_scan<<<grid, kPsThreads, 0, s>>>(g, d, F, ld, R, (int32_t)ptiles, pstart, pslot, woff,
-                                           R_dev, lookback, spin_limit, (long long *)stage,
-                                           stall_tile);
+                                           R_dev, lookback, spin_limit, stage, setup, stall_tile);
 }
 
 int64_t extend_tiles(int64_t wa, int64_t wb, int32_t block) {
@@ -1265,7 +1354,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
                        const int32_t *tile_row, int64_t wa, int32_t W, int32_t tiles,
                        int32_t block, size_t smem, unsigned long long *lookback,
                        const RowSink &sink, bool stage, int32_t spin_limit, int32_t stall_tile,
-                       cudaStream_t s) {
+                       Stage back, cudaStream_t s) {
   static std::atomic<unsigned long long> attr_set{0};  // bit per device
   // occupancy of the last (block, smem) this host thread launched with
   static thread_local int per_sm_cache[64][2] = {};
@@ -1294,7 +1383,7 @@ void launch_fused_mode(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)std::max(per_sm, 1) * sms);
   k_extend_fused<kMode, kMaxThreads, kProbes, kCheck><<<(unsigned)grid, block, smem, s>>>(
       g, d, F, (int32_t)ld, pstart, pslot, woff, tile_row, wa, W, tiles, lookback, sink, stage,
-      spin_limit, stall_tile);
+      spin_limit, stall_tile, back);
 }
 }  // namespace
 
@@ -1302,7 +1391,7 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
                          int64_t rows, unsigned long long *lookback, const RowSink &sink,
-                         int32_t spin_limit, int32_t stall_tile, cudaStream_t s) {
+                         int32_t spin_limit, int32_t stall_tile, Stage back, cudaStream_t s) {
   const int64_t tiles = extend_tiles(wa, wb, block);
   if (tiles <= 0) return;
   const int32_t W = (int32_t)(wb - wa), T = (int32_t)tiles;
@@ -1323,15 +1412,15 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
     if (sink.mode == kSinkRows)
       launch_fused_mode<kSinkRows, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
                                                  W, T, block, smem, lookback, sink, stage,
-                                                 spin_limit, stall_tile, s);
+                                                 spin_limit, stall_tile, back, s);
     else if (sink.mode == kSinkKeys)
       launch_fused_mode<kSinkKeys, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row, wa,
                                                  W, T, block, smem, lookback, sink, false,
-                                                 spin_limit, stall_tile, s);
+                                                 spin_limit, stall_tile, back, s);
     else
       launch_fused_mode<kSinkColumns, kMax, kP, kC>(g, d, F, ld, pstart, pslot, woff, tile_row,
                                                     wa, W, T, block, smem, lookback, sink, false,
-                                                    spin_limit, stall_tile, s);
+                                                    spin_limit, stall_tile, back, s);
   };
   // the probe-byte accounting is a separate instance, so the default one
   // carries no trace of it

@@ -156,9 +156,21 @@ void launch_label_counts(const GraphDev &g, uint8_t *nlc, int32_t stride, cudaSt
 constexpr int32_t kThrLevels = 4;
 void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits, cudaStream_t s);
 
-// Writes k bitmaps of n_words words and adds |C(u)| into sizes[u].
+// A read-back that a kernel makes by itself: its last CTA writes its results
+// into mapped host memory, then seq into word kStageSeq, which the host polls
+// (a separate copy kernel and a stream synchronisation cost about 10 us).
+constexpr int kStageSeq = 31;
+struct Stage {
+  long long *words = nullptr;  // device view; null: no read-back
+  long long seq = 0;
+};
+
+// Writes k bitmaps of n_words words and adds |C(u)| into sizes[u].  With
+// stage.words (filter_stages(g)): the k sizes go there; sizes[kMaxK], zeroed,
+// counts the CTAs that have finished.
+bool filter_stages(const GraphDev &g);
 void launch_filter(const GraphDev &g, const FilterDesc &d, uint32_t *bitmaps,
-                   unsigned long long *sizes, cudaStream_t s);
+                   unsigned long long *sizes, cudaStream_t s, Stage stage = Stage());
 
 // One refinement round (Sec. 3.2 repeated pruning): v stays in C(u) iff it
 // was there and, for every label group of u's query neighbours, v has at least
@@ -183,6 +195,12 @@ int scan_kernels(int64_t n);
 void launch_scan_i32(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t s);
 void launch_scan_i64(const int64_t *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t s);
 
+// Bitmap words [w0, w1) -> ascending vertex list, for at most kListDirectWords
+// words: one launch, every CTA adds up the words before its own.
+constexpr int32_t kListDirectWords = 32768;
+void launch_list_direct(const uint32_t *bitmap, int32_t w0, int32_t w1, int32_t *out,
+                        cudaStream_t s);
+
 // Bitmap -> ascending vertex list.  cnt: int32[n_words], off: int64[n_words+1]
 // (scratch), tmp: scan_tmp_elems(n_words).
 void launch_bitmap_to_list(const uint32_t *bitmap, int32_t n_words, int32_t *cnt, int64_t *off,
@@ -197,22 +215,38 @@ void launch_bitmap_to_list(const uint32_t *bitmap, int32_t n_words, int32_t *cnt
 // lengths, woff[R] = the level's candidate total.  One launch: the scan uses
 // a decoupled look-back over tiles of rows.  F has leading dimension ld >= R.
 // lookback: pivot_scan_words(R) words, zeroed before the launch (a memset,
-// or launch_tile_rows' extra words); a look-back wait longer than spin_limit
-// polls sets the error word.  stage (optional, device view of mapped host
-// memory, 4 words) receives, once the kernel is done: [0] the row count,
-// [1] non-zero if a wait ran out (this scan's or, with R_dev, the producing
-// level's), [2] woff[R], [3] R_dev[2] (0 without R_dev).  stall_tile (-1 =
-// none) is fault injection for tests: that tile never publishes its
-// look-back word, so the waits of the tiles after it run out.
+// launch_tile_rows' extra words, or the setup of the level before); a
+// look-back wait longer than spin_limit polls sets the error word.  stage
+// (4 words) receives, once the kernel is done: [0] the row count, [1] non-zero
+// if a wait ran out (this scan's or, with R_dev, the producing level's),
+// [2] woff[R], [3] R_dev[2] (0 without R_dev).  setup (cap = 0: none): see
+// LevelSetup.  stall_tile (-1 = none) is fault injection for tests: that tile
+// never publishes its look-back word, so the waits of the tiles after it run
+// out.
 // With R_dev the row count is read on the device (R_dev[0]; R is its upper
 // bound), R_dev[1] is the error word of the level that wrote F (when it is
 // set, some rows were never written and no row is read) and R_dev[2] its
 // probe bytes: the words a single-pass level leaves after its total.
 int64_t pivot_scan_words(int64_t R);
+
+// What a level launched in one piece needs besides its offsets, prepared by
+// its pivot scan when its tiles number at most cap: tile_row (cap + 1
+// entries, as launch_tile_rows writes them) and, zeroed at lb, its look-back
+// words (tiles + kLbExtra) followed by those of the next level's pivot scan
+// (pivot_scan_words(W)).  A larger level, whose time such a launch does not
+// matter to, takes launch_tile_rows.
+struct LevelSetup {
+  int32_t *tile_row = nullptr;
+  unsigned long long *lb = nullptr;
+  int32_t cap = 0;
+  int32_t tile_items = 0;
+};
+int64_t level_setup_words(int32_t cap, int32_t tile_items);  // of lb
 void launch_pivot_scan(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                        int64_t R, int32_t *pstart, uint8_t *pslot, int64_t *woff,
-                       unsigned long long *lookback, int32_t spin_limit, void *stage,
-                       int32_t stall_tile, cudaStream_t s, const int64_t *R_dev = nullptr);
+                       unsigned long long *lookback, int32_t spin_limit, Stage stage,
+                       const LevelSetup &setup, int32_t stall_tile, cudaStream_t s,
+                       const int64_t *R_dev = nullptr);
 
 // Number of extend tiles for candidates [wa, wb).
 int64_t extend_tiles(int64_t wa, int64_t wb, int32_t block);
@@ -325,11 +359,12 @@ void launch_extend_write(const GraphDev &g, const LevelDesc &d, const int32_t *F
 // does it); afterwards word tiles + 1 holds the survivor count, word
 // tiles + 2 is non-zero if a tile gave up waiting for its predecessors (after
 // spin_limit polls) and word tiles + 3 holds the probe bytes (count_probes).
+// These three go to stage, if any, when the last CTA is done.
 // The sink needs room for wb - wa rows.  The grid is persistent (at most the
 // CTAs that fit on the device at once).  stall_tile (-1 = none) is fault
 // injection for tests: that tile never publishes its look-back word, so later
 // tiles' waits run out.
-constexpr int kLbExtra = 4;
+constexpr int kLbExtra = 5;
 constexpr unsigned long long kLbAggregate = 1ull << 62, kLbInclusive = 2ull << 62;
 constexpr unsigned long long kLbValue = (1ull << 62) - 1;
 constexpr int32_t kLbSpinLimit = 1 << 20;  // default bound of a look-back wait (polls)
@@ -337,7 +372,7 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
                          const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
                          int64_t rows, unsigned long long *lookback, const RowSink &sink,
-                         int32_t spin_limit, int32_t stall_tile, cudaStream_t s);
+                         int32_t spin_limit, int32_t stall_tile, Stage stage, cudaStream_t s);
 
 // Row boundaries for work-bounded sub-chunks: bounds[j] = the row r with
 // woff[r] <= j*step < woff[r+1] (clamped to [0, R]); bounds[J] = R.
@@ -377,7 +412,8 @@ void launch_sort_small(const SmallSortItem *items, int32_t nitems, int32_t max_k
 // the remaining columns, which the stable passes keep.  Keys of one or two
 // words (N < 2^30) take single-sweep passes (one histogram launch, then one
 // launch per digit whose tiles find their offsets by a decoupled look-back);
-// wider keys take per-tile histograms and a scan per digit.  scratch:
+// wider keys take per-tile histograms and a scan per digit; at most
+// kSmallSortRows rows take one launch of one CTA.  scratch:
 // sort_scratch_bytes(N, k, bits, sort_cols) bytes of device memory, 256-byte
 // aligned, contents not kept.  err: null, or two words: a look-back wait
 // longer than spin_limit polls (<= 0: the library default) sets err[0] to 1

@@ -453,6 +453,56 @@ __global__ void __launch_bounds__(sweep_threads<NW>(), NW == 1 ? 2 : 3) k_oneswe
   }
 }
 
+// At most kSmallSortRows keys of up to kMaxKeyWords words: one CTA sorts their
+// indexes in shared memory (bitonic, by the whole key: rows are distinct, so
+// the order is total, and a group or prefix rank above the k columns agrees
+// with it) and unpacks the rows.  Bound by the 55 barriers of 1,024 keys, a
+// few us; the digit passes it replaces are one launch each, 7 or more.
+__global__ void __launch_bounds__(512) k_sort_few_keys(const uint64_t *__restrict__ keys,
+                                                       int64_t ld, int32_t N, int32_t nw,
+                                                       int32_t k, int32_t b,
+                                                       int32_t *__restrict__ out) {
+  extern __shared__ __align__(16) uint64_t s_keys[];  // word w of key i at w*N + i
+  __shared__ int16_t s_idx[kSmallSortRows];
+  int32_t P = 1;
+  while (P < N) P <<= 1;
+  for (int32_t e = threadIdx.x; e < N * nw; e += blockDim.x)
+    s_keys[e] = keys[(int64_t)(e / N) * ld + e % N];
+  for (int32_t e = threadIdx.x; e < P; e += blockDim.x) s_idx[e] = (int16_t)(e < N ? e : -1);
+  __syncthreads();
+  auto less = [&](int32_t x, int32_t y) {
+    if (x < 0) return false;  // padding sorts last
+    if (y < 0) return true;
+    for (int32_t w = nw - 1; w >= 0; --w) {
+      const uint64_t a = s_keys[w * N + x], c = s_keys[w * N + y];
+      if (a != c) return a < c;
+    }
+    return false;
+  };
+  for (int32_t size = 2; size <= P; size <<= 1) {
+    for (int32_t stride = size >> 1; stride > 0; stride >>= 1) {
+      for (int32_t t = threadIdx.x; t < (P >> 1); t += blockDim.x) {
+        const int32_t i = 2 * t - (t & (stride - 1));  // lower element of the pair
+        const int32_t j = i + stride;
+        const int32_t x = s_idx[i], y = s_idx[j];
+        if (less(y, x) == ((i & size) == 0)) {
+          s_idx[i] = (int16_t)y;
+          s_idx[j] = (int16_t)x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  const uint64_t mask = (1ull << b) - 1ull;
+  for (int32_t e = threadIdx.x; e < N * k; e += blockDim.x) {
+    const int32_t q = e / k, bp = (k - 1 - (e - q * k)) * b, w = bp >> 6, sh = bp & 63;
+    const int32_t x = s_idx[q];
+    uint64_t v = s_keys[w * N + x] >> sh;
+    if (sh + b > 64) v |= s_keys[(w + 1) * N + x] << (64 - sh);
+    out[e] = (int32_t)(v & mask);
+  }
+}
+
 // flags[i] = 1 where key i's prefix (the key bits selected by m0 in word 0
 // and m1 in word 1) differs from key i-1's; flags[0] = 0.
 template <int NW>
@@ -765,6 +815,19 @@ int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k,
     k_pack_keys<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(a, lda, 1, N, k, bits, nw, keys_a,
                                                             ld);
     ++launches;
+  }
+  if (N <= kSmallSortRows) {
+    constexpr int kMost = (int)(sizeof(uint64_t) * kMaxKeyWords * kSmallSortRows);
+    static std::atomic<unsigned long long> attr_set{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (!((attr_set.load() >> (dev & 63)) & 1ull)) {
+      cudaFuncSetAttribute(k_sort_few_keys, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+      attr_set.fetch_or(1ull << (dev & 63));
+    }
+    k_sort_few_keys<<<1, 512, sizeof(uint64_t) * (size_t)nw * N, s>>>(keys_a, ld, (int32_t)N, nw,
+                                                                       k, bits, out);
+    return launches + 1;
   }
   char *sc = (char *)scratch;
   if (L.rank_bits && !L.ranked) {
