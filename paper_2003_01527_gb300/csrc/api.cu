@@ -1753,49 +1753,38 @@ gsm_status guarded(gsm_ctx *ctx, F &&f) {
 constexpr int32_t kHubMinDegree = 32;
 constexpr int64_t kHubBytesDefault = int64_t(512) << 20;
 
-void build_hubs(gsm_ctx *ctx, const std::vector<int32_t> &h_rp) {
+// high: the vertices of degree >= kHubMinDegree, highest degree first, d_high
+// the same on the device.
+void build_hubs(gsm_ctx *ctx, const std::vector<int32_t> &h_rp, const std::vector<int32_t> &high,
+                const int32_t *d_high) {
   const int32_t n = ctx->n;
   const int64_t budget =
       ctx->opt.hub_bitmap_bytes == 0 ? kHubBytesDefault : ctx->opt.hub_bitmap_bytes;
   const int32_t words = (n + 31) / 32;
   if (budget <= 0 || n == 0) return;
-  const int64_t cap = budget / ((int64_t)words * 4);
-  std::vector<int32_t> hubs;
-  for (int32_t v = 0; v < n; ++v)
-    if (h_rp[v + 1] - h_rp[v] >= kHubMinDegree) hubs.push_back(v);
-  std::sort(hubs.begin(), hubs.end(), [&](int32_t a, int32_t b) {
-    const int32_t da = h_rp[a + 1] - h_rp[a], db = h_rp[b + 1] - h_rp[b];
-    return da != db ? da > db : a < b;
-  });
-  if ((int64_t)hubs.size() > cap) hubs.resize((size_t)cap);
-  if (hubs.empty()) return;
-  const int32_t H = (int32_t)hubs.size();
+  const int32_t H = (int32_t)std::min<int64_t>((int64_t)high.size(), budget / ((int64_t)words * 4));
+  if (H == 0) return;
   std::vector<int32_t> idx(n, -1);
-  for (int32_t h = 0; h < H; ++h) idx[hubs[h]] = h;
+  for (int32_t h = 0; h < H; ++h) idx[high[h]] = h;
   ctx->d_hub = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * n);
   ctx->hub_bits_bytes = (size_t)H * words * sizeof(uint32_t);
   ctx->d_hub_bits = (uint32_t *)dev_alloc(ctx, ctx->hub_bits_bytes);
-  int32_t *d_list = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * H);
   CU(cudaMemcpyAsync(ctx->d_hub, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice,
                      ctx->stream));
-  CU(cudaMemcpyAsync(d_list, hubs.data(), sizeof(int32_t) * H, cudaMemcpyHostToDevice,
-                     ctx->stream));
   GraphDev g = graph_dev(ctx);
-  launch_hub_bitmaps(g, d_list, H, words, ctx->d_hub_bits, ctx->stream);
+  launch_hub_bitmaps(g, d_high, H, words, ctx->d_hub_bits, ctx->stream);
   CU(cudaGetLastError());
   // label segment table of the hubs (labelled graphs, up to 4,096 labels)
   const int64_t L = (int64_t)ctx->label_values.size();
   if (L > 1 && L <= 4096) {
     ctx->hub_seg_bytes = sizeof(int32_t) * (size_t)H * (size_t)(L + 1);
     ctx->d_hub_seg = (int32_t *)dev_alloc(ctx, ctx->hub_seg_bytes);
-    g.num_labels = (int32_t)L;
-    launch_hub_segments(g, d_list, H, ctx->d_hub_seg, ctx->stream);
+    launch_hub_segments(g, d_high, H, ctx->d_hub_seg, ctx->stream);
     CU(cudaGetLastError());
   }
-  CU(cudaStreamSynchronize(ctx->stream));
-  dev_free(ctx, d_list, sizeof(int32_t) * H);
+  CU(cudaStreamSynchronize(ctx->stream));  // idx is copied
   ctx->hub_count = H;
-  ctx->hub_min_deg = h_rp[hubs.back() + 1] - h_rp[hubs.back()];
+  ctx->hub_min_deg = h_rp[high[H - 1] + 1] - h_rp[high[H - 1]];
 }
 
 void clear_all_graphs(gsm_ctx *ctx);
@@ -1819,7 +1808,8 @@ void free_graph(gsm_ctx *ctx) {
   if (ctx->d_rp) dev_free(ctx, ctx->d_rp, sizeof(int32_t) * (ctx->n + 1));
   if (ctx->d_col) dev_free(ctx, ctx->d_col, sizeof(int32_t) * std::max<int64_t>(ctx->nnz, 1));
   if (ctx->d_lab) dev_free(ctx, ctx->d_lab, sizeof(int32_t) * std::max<int32_t>(ctx->n, 1));
-  if (ctx->d_lcol) dev_free(ctx, ctx->d_lcol, sizeof(int32_t) * std::max<int64_t>(ctx->nnz, 1));
+  if (ctx->d_lcol && ctx->d_lcol != ctx->d_col)
+    dev_free(ctx, ctx->d_lcol, sizeof(int32_t) * std::max<int64_t>(ctx->nnz, 1));
   if (ctx->d_llab) dev_free(ctx, ctx->d_llab, sizeof(int32_t) * std::max<int64_t>(ctx->nnz, 1));
   if (ctx->d_hub) dev_free(ctx, ctx->d_hub, sizeof(int32_t) * std::max<int32_t>(ctx->n, 1));
   if (ctx->d_hub_bits) dev_free(ctx, ctx->d_hub_bits, ctx->hub_bits_bytes);
@@ -3013,7 +3003,9 @@ gsm_status gsm_load_graph(gsm_ctx *ctx, int32_t n, int64_t nnz, const int32_t *r
     }
     ctx->max_deg = md;
     // degrees of every label in ascending order: a counting sort by degree,
-    // then a stable split by label
+    // then a stable split by label; and the vertices of degree >=
+    // kHubMinDegree, highest degree first (then lowest id)
+    std::vector<int32_t> high;
     ctx->deg_by_label.assign(vals.size(), {});
     if (n && rp_ok) {
       std::vector<int32_t> start((size_t)md + 2, 0), by_deg(n);
@@ -3024,6 +3016,8 @@ gsm_status gsm_load_graph(gsm_ctx *ctx, int32_t n, int64_t nnz, const int32_t *r
       for (int32_t v = 0; v < n; ++v) per_label[dense[v]]++;
       for (size_t l = 0; l < vals.size(); ++l) ctx->deg_by_label[l].reserve(per_label[l]);
       for (int32_t v : by_deg) ctx->deg_by_label[dense[v]].push_back(h_rp[v + 1] - h_rp[v]);
+      for (int32_t d = md; d >= kHubMinDegree; --d)  // (start[d] is now degree d's end)
+        high.insert(high.end(), by_deg.begin() + start[d - 1], by_deg.begin() + start[d]);
     }
     CU(cudaStreamSynchronize(ctx->stream));
     if (flags & GSM_VALIDATE) {
@@ -3051,42 +3045,66 @@ gsm_status gsm_load_graph(gsm_ctx *ctx, int32_t n, int64_t nnz, const int32_t *r
       free_graph(ctx);
       FAIL(GSM_ERR_INVALID_GRAPH, "row_ptr is not a valid CSR offset array");
     }
-    // label-segmented copy of the rows (ordered by (neighbour label, id))
-    ctx->d_lcol = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * std::max<int64_t>(nnz, 1));
-    ctx->d_llab = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * std::max<int64_t>(nnz, 1));
-    if (nnz > 0) {
-      if (ctx->label_values.size() <= 1) {
-        CU(cudaMemcpyAsync(ctx->d_lcol, ctx->d_col, sizeof(int32_t) * nnz,
-                           cudaMemcpyDeviceToDevice, ctx->stream));
-        CU(cudaMemsetAsync(ctx->d_llab, 0, sizeof(int32_t) * nnz, ctx->stream));
-      } else {
-        const int32_t bits = label_segment_bits(n, (int32_t)ctx->label_values.size());
+    // the vertices of high degree on the device, for the kernels that take a
+    // CTA per long row
+    struct Temp {
+      gsm_ctx *ctx;
+      void *p = nullptr;
+      size_t bytes = 0;
+      ~Temp() {
+        try {
+          dev_free(ctx, p, bytes);
+        } catch (...) {
+        }
+      }
+    } d_high{ctx};
+    if (!high.empty()) {
+      d_high.bytes = sizeof(int32_t) * high.size();
+      d_high.p = dev_alloc(ctx, d_high.bytes);
+      CU(cudaMemcpyAsync(d_high.p, high.data(), d_high.bytes, cudaMemcpyHostToDevice,
+                         ctx->stream));
+    }
+    // label-segmented copy of the rows (ordered by (neighbour label, id)); with
+    // one label it is the rows themselves.  With few labels a partition of
+    // each row, which also counts neighbours per label for the filter.
+    const int32_t L = (int32_t)ctx->label_values.size();
+    if (L <= 1) {
+      ctx->d_lcol = ctx->d_col;
+    } else {
+      ctx->d_lcol = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * std::max<int64_t>(nnz, 1));
+      ctx->d_llab = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * std::max<int64_t>(nnz, 1));
+      if (L <= kNlcMaxLabels) {
+        if ((size_t)n * L <= (size_t(1) << 30)) {
+          ctx->nlc_stride = L;
+          ctx->d_nlc = (uint8_t *)dev_alloc(ctx, std::max<size_t>((size_t)n * L, 1));
+        }
+        int32_t nlong = 0;
+        while (nlong < (int32_t)high.size() &&
+               h_rp[high[nlong] + 1] - h_rp[high[nlong]] > kLongRowDegree)
+          ++nlong;
+        launch_row_segments(graph_dev(ctx), L, (const int32_t *)d_high.p, nlong, ctx->d_lcol,
+                            ctx->d_llab, ctx->d_nlc, ctx->stream);
+        CU(cudaGetLastError());
+      } else if (nnz > 0) {
+        const int32_t bits = label_segment_bits(n, L);
         const int32_t nw = packed_words(3, bits);
         Carve cv;
         const size_t o_cols = cv.add<int32_t>(3 * nnz), o_rows = cv.add<int32_t>(3 * nnz),
                      o_keys = cv.add<uint64_t>(2 * nnz * nw),
                      o_s = cv.add<char>((int64_t)sort_scratch_bytes(nnz, 3, bits, 2));
-        char *tmpbuf = (char *)dev_alloc(ctx, cv.off);
-        GraphDev g = graph_dev(ctx);
-        launch_label_segments(g, (int32_t)ctx->label_values.size(), (int32_t *)(tmpbuf + o_cols),
+        Temp tmp{ctx};
+        tmp.p = dev_alloc(ctx, cv.off);
+        tmp.bytes = cv.off;
+        char *tmpbuf = (char *)tmp.p;
+        launch_label_segments(graph_dev(ctx), L, (int32_t *)(tmpbuf + o_cols),
                               (uint64_t *)(tmpbuf + o_keys), (int32_t *)(tmpbuf + o_rows),
                               tmpbuf + o_s, ctx->d_flags, ctx->d_lcol, ctx->d_llab, ctx->stream);
         CU(cudaGetLastError());
         CU(cudaStreamSynchronize(ctx->stream));
-        dev_free(ctx, tmpbuf, cv.off);
         check_sort_flag(ctx);
       }
-      CU(cudaStreamSynchronize(ctx->stream));
     }
-    build_hubs(ctx, h_rp);
-    // neighbour label counts for the filter (labelled graphs with few labels)
-    const int32_t L = (int32_t)ctx->label_values.size();
-    if (L > 1 && L <= kNlcMaxLabels && (size_t)n * L <= (size_t(1) << 30)) {
-      ctx->nlc_stride = L;
-      ctx->d_nlc = (uint8_t *)dev_alloc(ctx, std::max<size_t>((size_t)n * L, 1));
-      launch_label_counts(graph_dev(ctx), ctx->d_nlc, L, ctx->stream);
-      CU(cudaGetLastError());
-    }
+    build_hubs(ctx, h_rp, high, (const int32_t *)d_high.p);
     if (n > 0 && (L == 1 || ctx->d_nlc)) {
       // (kThrLevels + 1) bitmaps per label, less than the count table's bytes
       const size_t words = (size_t)(n + 31) / 32;

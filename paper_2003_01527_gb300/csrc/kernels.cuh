@@ -136,6 +136,16 @@ int launch_label_segments(const GraphDev &g, int32_t num_labels, int32_t *edge_c
                           int32_t *out_col, int32_t *out_lab, cudaStream_t s);
 int32_t label_segment_bits(int32_t n, int32_t num_labels);
 
+// The same for graphs of at most kNlcMaxLabels labels, row by row without a
+// sort: out_col/out_lab, and nlc (null: not wanted), the neighbour label count
+// table, n * num_labels bytes.  long_rows: the nlong vertices of degree above
+// kLongRowDegree (device).
+constexpr int32_t kNlcMaxLabels = 64;
+constexpr int32_t kLongRowDegree = 1024;
+void launch_row_segments(const GraphDev &g, int32_t num_labels, const int32_t *long_rows,
+                         int32_t nlong, int32_t *out_col, int32_t *out_lab, uint8_t *nlc,
+                         cudaStream_t s);
+
 // Adjacency bitmaps of the H hubs (vertex ids hubs[0..H)): bitmap h (words
 // bits[h * words ..], zeroed here) gets bit w for every neighbour w.
 void launch_hub_bitmaps(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t words,
@@ -144,11 +154,6 @@ void launch_hub_bitmaps(const GraphDev &g, const int32_t *hubs, int32_t H, int32
 // (label, id)-ordered row of hub hubs[h] (l = num_labels: the row's end).
 void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t *seg,
                          cudaStream_t s);
-
-// The neighbour label count table of every vertex (labels < g.num_labels <=
-// stride), from the label-segmented rows.
-constexpr int32_t kNlcMaxLabels = 64;
-void launch_label_counts(const GraphDev &g, uint8_t *nlc, int32_t stride, cudaStream_t s);
 
 // The threshold and label bitmaps of GraphDev (thr: num_labels * kThrLevels,
 // lab_bits: num_labels bitmaps of hub_words words), from the neighbour label

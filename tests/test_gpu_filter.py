@@ -39,3 +39,29 @@ def test_candidates_of_stars(gsm_lib, cuda, n, labels):
             # no bit past the last vertex
             assert int(np.unpackbits(bm.view(np.uint8)).sum()) == int(got.sum())
     m.close()
+
+
+@pytest.mark.parametrize("labels", [2, 64, 65])  # 65: sorted, not partitioned row by row
+def test_label_segments_of_rows(gsm_lib, cuda, labels):
+    """Rows of every length around a warp, the longest row a warp takes (1,024)
+    and beyond, some with one label only: the edges between two labels, listed
+    through the segments, are numpy's."""
+    degrees = [0, 1, 31, 32, 33, 63, 257, 1023, 1024, 1025, 1056, 3001]
+    n = len(degrees) + max(degrees)
+    rng = np.random.default_rng(labels)
+    edges = []
+    for h, d in enumerate(degrees):
+        ends = len(degrees) + rng.permutation(max(degrees))[:d]
+        edges += [(h, int(v)) for v in ends]
+    lab = rng.integers(0, labels, n).astype(np.int32)
+    lab[len(degrees):len(degrees) + 1200] = 1
+    g = I.graph_from_edges(n, edges, lab)
+    m = gsm_lib.Matcher(device=0)
+    m.load_graph(g.row_ptr, g.col, g.labels, validate=True)
+    src = np.repeat(np.arange(n), np.diff(g.row_ptr))
+    for a, b in [(0, 1), (1, 0), (1, 1), (int(lab[0]), int(lab[11])), (labels - 1, 1)]:
+        keep = (g.labels[src] == a) & (g.labels[g.col] == b)
+        want = np.stack([src[keep], g.col[keep]], axis=1)
+        rows, count = m.enumerate(m.query(2, [(0, 1)], [a, b]))
+        assert count == len(want) and np.array_equal(rows, want), (a, b)
+    m.close()
