@@ -3075,15 +3075,16 @@ gsm_status gsm_load_graph(gsm_ctx *ctx, int32_t n, int64_t nnz, const int32_t *r
       ctx->d_llab = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * std::max<int64_t>(nnz, 1));
       if (L <= kNlcMaxLabels) {
         if ((size_t)n * L <= (size_t(1) << 30)) {
-          ctx->nlc_stride = L;
-          ctx->d_nlc = (uint8_t *)dev_alloc(ctx, std::max<size_t>((size_t)n * L, 1));
+          ctx->nlc_stride = (L + 7) & ~7;
+          ctx->d_nlc =
+              (uint8_t *)dev_alloc(ctx, std::max<size_t>((size_t)n * ctx->nlc_stride, 1));
         }
         int32_t nlong = 0;
         while (nlong < (int32_t)high.size() &&
                h_rp[high[nlong] + 1] - h_rp[high[nlong]] > kLongRowDegree)
           ++nlong;
         launch_row_segments(graph_dev(ctx), L, (const int32_t *)d_high.p, nlong, ctx->d_lcol,
-                            ctx->d_llab, ctx->d_nlc, ctx->stream);
+                            ctx->d_llab, ctx->d_nlc, ctx->nlc_stride, ctx->stream);
         CU(cudaGetLastError());
       } else if (nnz > 0) {
         const int32_t bits = label_segment_bits(n, L);

@@ -452,8 +452,14 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
   }
   const int32_t ntiles = (int32_t)((R + kPsRows - 1) / kPsRows);  // <= ptiles
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = (int32_t)atomicAdd(lookback + ptiles, 1ull);
+  // one tile (or none) is CTA 0's, without ticket, look-back or count of
+  // finished CTAs: small levels are a chain of latencies (600 rows: 16.6 -> 11.0
+  // us under ncu, half of it from counted_segment)
+  const bool single = ntiles <= 1;
+  if (single && blockIdx.x > 0) return;
+  int64_t W = 0;
+  for (int32_t turn = 0;; ++turn) {
+    if (threadIdx.x == 0) s_tile = single ? turn : (int32_t)atomicAdd(lookback + ptiles, 1ull);
     __syncthreads();
     const int32_t tile = s_tile;
     if (tile >= ntiles) break;  // uniform across the block
@@ -520,7 +526,10 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
     }
     int64_t total;
     const int64_t ex = block_excl_scan(sum, s_warp, &total);
-    if (warp == 0) {
+    if (single) {
+      W = total;
+      if (threadIdx.x == 0) s_prefix = 0;
+    } else if (warp == 0) {
       // stall_tile (fault injection) adds its work to the total but never
       // publishes its tile word, so the waits of the tiles after it run out
       if (lane == 0) {
@@ -555,15 +564,19 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
     }
     __syncthreads();  // s_val and s_tile are reused by the next tile
   }
-  __syncthreads();  // every thread has read s_tile
-  if (threadIdx.x == 0) {
-    __threadfence();  // this CTA's offsets and look-back words before its count
-    s_tile = atomicAdd(lookback + ptiles + 3, 1ull) == gridDim.x - 1;
-    __threadfence();
+  long long err = 0;
+  if (!single) {
+    __syncthreads();  // every thread has read s_tile
+    if (threadIdx.x == 0) {
+      __threadfence();  // this CTA's offsets and look-back words before its count
+      s_tile = atomicAdd(lookback + ptiles + 3, 1ull) == gridDim.x - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!s_tile) return;  // only the CTA that finishes last goes on
+    W = (int64_t)atomicAdd(lookback + ptiles + 1, 0ull);
+    err = (long long)atomicAdd(lookback + ptiles + 2, 0ull);
   }
-  __syncthreads();
-  if (!s_tile) return;  // only the CTA that finishes last goes on
-  const int64_t W = (int64_t)atomicAdd(lookback + ptiles + 1, 0ull);
   if (setup.cap > 0 && W <= (int64_t)setup.cap * setup.tile_items) {
     const int64_t tiles = (W + setup.tile_items - 1) / setup.tile_items;
     const int64_t words =
@@ -572,7 +585,6 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
     if (threadIdx.x == 0) setup.tile_row[tiles] = (int32_t)(R - 1);
   }
   if (threadIdx.x == 0) {
-    const long long err = (long long)atomicAdd(lookback + ptiles + 2, 0ull);
     woff[R] = W;
     if (stage.words) {
       stage.words[0] = rows_in;
@@ -816,6 +828,8 @@ __global__ void __launch_bounds__(kMaxThreads,
   int32_t pend = -1, pend_T = 0, pend_buf = 0, buf = 0;
 
   // lookback + write of a verified tile whose survivors are in buffer pb
+  // a level of one tile: no ticket, no look-back
+  const bool single = tiles == 1;
   auto finish = [&](int32_t tile, int32_t T, int32_t pb) {
     if (warp == 0) {
       const unsigned long long prefix =
@@ -866,8 +880,8 @@ __global__ void __launch_bounds__(kMaxThreads,
     }
   };
 
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = (int32_t)atomicAdd(lookback + tiles, 1ull);
+  for (int32_t turn = 0;; ++turn) {
+    if (threadIdx.x == 0) s_tile = single ? turn : (int32_t)atomicAdd(lookback + tiles, 1ull);
     __syncthreads();
     const int32_t tile = s_tile;
     if (tile >= tiles) break;  // uniform across the block
@@ -920,7 +934,7 @@ __global__ void __launch_bounds__(kMaxThreads,
   __syncthreads();  // the CTA's rows are written
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(lookback + tiles + 4, 1ull) == gridDim.x - 1) {
+    if (single || atomicAdd(lookback + tiles + 4, 1ull) == gridDim.x - 1) {
       __threadfence();
       for (int w = 0; w < 3; ++w)
         stage.words[w] = (long long)atomicAdd(lookback + tiles + 1 + w, 0ull);
@@ -1017,7 +1031,8 @@ __global__ void __launch_bounds__(128) k_hub_bits(GraphDev g, const int32_t *__r
 template <int kWarps>
 __global__ void __launch_bounds__(kWarps == 1 ? 256 : 1024) k_row_segments(
     GraphDev g, int32_t L, const int32_t *__restrict__ rows, int32_t nrows,
-    int32_t *__restrict__ out_col, int32_t *__restrict__ out_lab, uint8_t *__restrict__ nlc) {
+    int32_t *__restrict__ out_col, int32_t *__restrict__ out_lab, uint8_t *__restrict__ nlc,
+    int32_t nlc_stride) {
   constexpr int kGroups = kWarps == 1 ? 8 : 1;  // rows a CTA works on at once
   __shared__ int32_t s_cnt[kGroups][kWarps][kNlcMaxLabels];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1051,7 +1066,8 @@ __global__ void __launch_bounds__(kWarps == 1 ? 256 : 1024) k_row_segments(
         for (int j = 0; j < 2; ++j) tot[j] += s_cnt[grp][w][2 * lane + j];
       if (nlc)
         for (int j = 0; j < 2; ++j)
-          if (2 * lane + j < L) nlc[(int64_t)v * L + 2 * lane + j] = (uint8_t)min(tot[j], 255);
+          if (2 * lane + j < nlc_stride)  // (labels past L have none)
+            nlc[(int64_t)v * nlc_stride + 2 * lane + j] = (uint8_t)min(tot[j], 255);
       int32_t incl = tot[0] + tot[1];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -1209,13 +1225,13 @@ int launch_prefix_ranks(const int32_t *F, int64_t ld, int64_t rows, int32_t p, P
 
 void launch_row_segments(const GraphDev &g, int32_t num_labels, const int32_t *long_rows,
                          int32_t nlong, int32_t *out_col, int32_t *out_lab, uint8_t *nlc,
-                         cudaStream_t s) {
+                         int32_t nlc_stride, cudaStream_t s) {
   if (g.n <= 0) return;
   k_row_segments<1><<<grid_for((int64_t)g.n * 32, 256, 152 * 64), 256, 0, s>>>(
-      g, num_labels, nullptr, g.n, out_col, out_lab, nlc);
+      g, num_labels, nullptr, g.n, out_col, out_lab, nlc, nlc_stride);
   if (nlong > 0)
     k_row_segments<32><<<(unsigned)nlong, 1024, 0, s>>>(g, num_labels, long_rows, nlong, out_col,
-                                                        out_lab, nlc);
+                                                        out_lab, nlc, nlc_stride);
 }
 
 void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t *seg,

@@ -86,7 +86,8 @@ struct GraphDev {
   const int32_t *hub_seg;
   // neighbour label counts (null: none): nlc[v * nlc_stride + l] = the number
   // of neighbours of v with label l, saturated at 255 (a query needs at most
-  // 15, so the saturated count decides every requirement exactly)
+  // 15, so the saturated count decides every requirement exactly); nlc_stride
+  // is a multiple of 8
   const uint8_t *nlc;
   int32_t nlc_stride;
   // the same as bitmaps over the vertices (null: none): bit v of
@@ -138,13 +139,13 @@ int32_t label_segment_bits(int32_t n, int32_t num_labels);
 
 // The same for graphs of at most kNlcMaxLabels labels, row by row without a
 // sort: out_col/out_lab, and nlc (null: not wanted), the neighbour label count
-// table, n * num_labels bytes.  long_rows: the nlong vertices of degree above
+// table, n * nlc_stride bytes.  long_rows: the nlong vertices of degree above
 // kLongRowDegree (device).
 constexpr int32_t kNlcMaxLabels = 64;
 constexpr int32_t kLongRowDegree = 1024;
 void launch_row_segments(const GraphDev &g, int32_t num_labels, const int32_t *long_rows,
                          int32_t nlong, int32_t *out_col, int32_t *out_lab, uint8_t *nlc,
-                         cudaStream_t s);
+                         int32_t nlc_stride, cudaStream_t s);
 
 // Adjacency bitmaps of the H hubs (vertex ids hubs[0..H)): bitmap h (words
 // bits[h * words ..], zeroed here) gets bit w for every neighbour w.

@@ -7,8 +7,34 @@
 
 namespace gsm {
 
+// The segment of label l in a row [b, e) of at most 254 entries, from the
+// neighbour label counts (none of them saturated): its start is the sum of the
+// counts of the labels before l.  The counts of a vertex are whole 8-byte
+// words (nlc_stride), loaded together, so the lookup is one load deep; two
+// binary searches of the labels are 2 log2(e - b).
+__device__ __forceinline__ int2 counted_segment(const GraphDev &g, int32_t x, int32_t l,
+                                                int32_t b) {
+  const uint2 *row = reinterpret_cast<const uint2 *>(g.nlc + (int64_t)x * g.nlc_stride);
+  uint32_t before = 0, own = 0;
+  for (int32_t w = 0; w <= l >> 3; ++w) {
+    uint2 c = __ldg(row + w);
+    if (w == l >> 3) {  // keep the bytes before l's
+      const uint32_t byte = l & 7;
+      own = ((byte < 4 ? c.x : c.y) >> (8 * (byte & 3))) & 0xffu;
+      c.x = byte >= 4 ? c.x : c.x & ((1u << (8 * byte)) - 1u);
+      c.y = byte >= 4 ? c.y & ((1u << (8 * (byte - 4))) - 1u) : 0u;
+    }
+    before = __dp4a(c.x, 0x01010101u, before);
+    before = __dp4a(c.y, 0x01010101u, before);
+  }
+  return make_int2(b + (int32_t)before, b + (int32_t)(before + own));
+}
+constexpr int32_t kCountedRow = 254;
+
 // [first, second) = the neighbours of x with label l (rows of lcol are
-// ordered by (label, id), so they are one contiguous, id-sorted segment).
+// ordered by (label, id), so they are one contiguous, id-sorted segment): from
+// a hub's segment table, the neighbour label counts of a short row, or two
+// binary searches.
 __device__ __forceinline__ int2 label_segment(const GraphDev &g, int32_t x, int32_t l) {
   if (g.num_labels > 1 && g.hub_seg) {  // a hub: its segment table
     const int32_t h = __ldg(g.hub + x);
@@ -19,6 +45,7 @@ __device__ __forceinline__ int2 label_segment(const GraphDev &g, int32_t x, int3
   }
   const int32_t b = __ldg(g.rp + x), e = __ldg(g.rp + x + 1);
   if (g.num_labels == 1) return make_int2(b, e);
+  if (g.nlc && e - b <= kCountedRow) return counted_segment(g, x, l, b);
   int32_t lo = b, len = e - b;  // first entry with label >= l
   while (len > 0) {
     const int32_t half = len >> 1;
