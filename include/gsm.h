@@ -142,7 +142,11 @@ typedef struct gsm_options {
    * degree >= 32, highest degree first, ceil(n/32) x 4 bytes each), used to
    * check non-tree edges against a hub with one bit probe instead of a binary
    * search of its row.  0 = 512 MiB; negative = no bitmaps.  Built by
-   * gsm_load_graph, outside the memory budget; results do not depend on it. */
+   * gsm_load_graph, outside the memory budget; results do not depend on it.
+   * (The first clique count on a one-label graph with many 2-edge paths also
+   * builds a copy of the rows renumbered by degree, 4 bytes an entry and 12 a
+   * vertex, with up to 128 MiB of bitmaps out of the same allowance; about 25
+   * bytes an entry of scratch are used and given back meanwhile.) */
   int64_t hub_bitmap_bytes;
   /* Host threads gsm_enumerate_many lists its queries with (0 = 6, at most
    * 16): each thread has a worker context of its own (stream, workspace with

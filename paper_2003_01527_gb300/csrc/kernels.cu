@@ -1008,13 +1008,57 @@ __global__ void k_prefix_reset(PrefixState *st) {
 
 // One CTA per hub: every neighbour's bit of the hub's bitmap.
 __global__ void __launch_bounds__(128) k_hub_bits(GraphDev g, const int32_t *__restrict__ hubs,
-                                                  int32_t words, uint32_t *__restrict__ bits) {
-  const int32_t v = hubs[blockIdx.x];
+                                                  int32_t words, uint32_t *__restrict__ bits,
+                                                  int32_t lo) {
+  const int32_t v = hubs ? hubs[blockIdx.x] : lo + (int32_t)blockIdx.x;
   uint32_t *b = bits + (size_t)blockIdx.x * words;
   for (int32_t e = g.rp[v] + threadIdx.x; e < g.rp[v + 1]; e += blockDim.x) {
-    const int32_t w = g.col[e];
-    atomicOr(b + (w >> 5), 1u << (w & 31));
+    const int32_t w = g.col[e] - lo;
+    if (w >= 0) atomicOr(b + (w >> 5), 1u << (w & 31));
   }
+}
+
+// ---- renumbering: rank[order[i]] = i and the degrees in the new order
+__global__ void k_rank_ids(const int32_t *__restrict__ order, const int32_t *__restrict__ rp,
+                           int32_t n, int32_t *__restrict__ rank, int32_t *__restrict__ deg) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const int32_t v = order[i];
+    rank[v] = (int32_t)i;
+    deg[i] = rp[v + 1] - rp[v];
+  }
+}
+
+// One key per edge, new row i after new row i: (new id of the other end, i).  A
+// stable sort on the other end alone leaves every row ascending (the graph is
+// symmetric), which takes half the digits of a sort on both ends.  A warp per
+// row, or with kCta a CTA per row for the `rows` last, long ones.
+template <bool kCta>
+__global__ void __launch_bounds__(256) k_rank_keys(GraphDev g, const int32_t *__restrict__ order,
+                                                   const int32_t *__restrict__ rank,
+                                                   const int64_t *__restrict__ offs, int32_t first,
+                                                   int32_t rows, int32_t bits,
+                                                   uint64_t *__restrict__ keys) {
+  const int t = kCta ? threadIdx.x : threadIdx.x & 31, nt = kCta ? 256 : 32;
+  const int64_t groups = kCta ? gridDim.x : (int64_t)gridDim.x * 8;
+  for (int64_t r = kCta ? blockIdx.x : ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5; r < rows;
+       r += groups) {
+    const int32_t i = first + (int32_t)r, v = order[i];
+    const int32_t b = g.rp[v], d = g.rp[v + 1] - b;
+    const int64_t to = offs[i];
+#pragma unroll 4
+    for (int32_t x = t; x < d; x += nt)
+      keys[to + x] = ((uint64_t)(uint32_t)rank[g.col[b + x]] << bits) | (uint32_t)i;
+  }
+}
+
+__global__ void k_rank_rows(const int64_t *__restrict__ offs, int32_t n,
+                            const int2 *__restrict__ pairs, int64_t nnz,
+                            int32_t *__restrict__ rp2, int32_t *__restrict__ col2) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t i = t; i <= n; i += stride) rp2[i] = (int32_t)offs[i];
+  for (int64_t e = t; e < nnz; e += stride) col2[e] = pairs[e].y;
 }
 
 // Label-segmented rows by a stable partition of every row: a group of kWarps
@@ -1201,10 +1245,29 @@ void launch_validate_rows(const GraphDev &g, int32_t *err, cudaStream_t s) {
 }
 
 void launch_hub_bitmaps(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t words,
-                        uint32_t *bits, cudaStream_t s) {
+                        uint32_t *bits, cudaStream_t s, int32_t lo) {
   if (H <= 0) return;
   cudaMemsetAsync(bits, 0, sizeof(uint32_t) * (size_t)H * words, s);
-  k_hub_bits<<<(unsigned)H, 128, 0, s>>>(g, hubs, words, bits);
+  k_hub_bits<<<(unsigned)H, 128, 0, s>>>(g, hubs, words, bits, lo);
+}
+
+void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int32_t *rank,
+                     int32_t *deg, int64_t *offs, int64_t *tmp, uint64_t *keys, int32_t *pairs,
+                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2,
+                     cudaStream_t s) {
+  const int32_t bits = label_segment_bits(g.n, 1), nshort = g.n - nlong;
+  k_rank_ids<<<grid_for(g.n, 256), 256, 0, s>>>(order, g.rp, g.n, rank, deg);
+  launch_scan_i32(deg, offs, g.n, tmp, s);
+  if (nshort > 0)
+    k_rank_keys<false><<<grid_for((int64_t)nshort * 32, 256, 152 * 64), 256, 0, s>>>(
+        g, order, rank, offs, 0, nshort, bits, keys);
+  if (nlong > 0)
+    k_rank_keys<true><<<grid_for((int64_t)nlong * 256, 256, 152 * 64), 256, 0, s>>>(
+        g, order, rank, offs, nshort, nlong, bits, keys);
+  launch_sort_rows_packed(nullptr, 0, g.nnz, 2, bits, 1, keys, keys + g.nnz, g.nnz, pairs,
+                          sort_scratch, 0, err, -1, s);
+  k_rank_rows<<<grid_for(std::max<int64_t>(g.nnz, g.n + 1), 256), 256, 0, s>>>(
+      offs, g.n, (const int2 *)pairs, g.nnz, rp2, col2);
 }
 
 void launch_prefix_state_reset(PrefixState *st, cudaStream_t s) {

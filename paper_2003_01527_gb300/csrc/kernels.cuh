@@ -80,7 +80,7 @@ struct GraphDev {
   // neighbour of v.  hub = null: no bitmaps, every test searches the row.
   const int32_t *hub;
   const uint32_t *hub_bits;
-  int32_t hub_words;  // ceil(n/32), also without hubs
+  int32_t hub_words;  // words of a hub's bitmap: ceil(n/32) (also without hubs), but see hub_lo
   // label segments of the hubs' rows (null: none): the neighbours of hub h
   // with label l are lcol[hub_seg[h * (num_labels + 1) + l] .. the next entry)
   const int32_t *hub_seg;
@@ -95,6 +95,11 @@ struct GraphDev {
   // neighbours with label l, bit v of lab_bits[l * hub_words ..] iff v's label
   // is l.  One label: its neighbours are all, so thr holds degrees.
   const uint32_t *thr, *lab_bits;
+  // > 0: the graph with its vertices renumbered by degree (RankGraph): the hubs
+  // are the vertices from hub_lo on, and their bitmaps cover those only
+  // (hub_bits points hub_lo / 32 words before the first), so a hub is asked
+  // about vertices >= hub_lo alone
+  int32_t hub_lo;
   // GSM_DEBUG builds: the mapped word a failed bounds check writes its site
   // to (null: not reported)
   uint32_t *dbg;
@@ -149,12 +154,26 @@ void launch_row_segments(const GraphDev &g, int32_t num_labels, const int32_t *l
 
 // Adjacency bitmaps of the H hubs (vertex ids hubs[0..H)): bitmap h (words
 // bits[h * words ..], zeroed here) gets bit w for every neighbour w.
+// lo > 0: the bitmaps cover vertices lo, lo + 1, ... only (bit w - lo), and
+// hubs may be null: hub h is vertex lo + h.
 void launch_hub_bitmaps(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t words,
-                        uint32_t *bits, cudaStream_t s);
+                        uint32_t *bits, cudaStream_t s, int32_t lo = 0);
 // seg[h * (g.num_labels + 1) + l] = start of label l's segment in the
 // (label, id)-ordered row of hub hubs[h] (l = num_labels: the row's end).
 void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int32_t *seg,
                          cudaStream_t s);
+
+// The rows of g renumbered (one-label graphs): new vertex i is order[i].
+// Writes rp2 (n + 1) and col2 (nnz), rows ascending.  order: device; nlong: how
+// many vertices, the last ones of order, have degrees above kLongRowDegree.
+// rank and deg: n ints, offs: n + 1 and tmp: scan_tmp_elems(n) int64, keys: 2 *
+// nnz uint64, pairs: 2 * nnz ints, sort_scratch: sort_scratch_bytes(nnz, 2,
+// bits, 1), all scratch; bits = label_segment_bits(n, 1); err as for
+// launch_sort_rows_packed.
+void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int32_t *rank,
+                     int32_t *deg, int64_t *offs, int64_t *tmp, uint64_t *keys, int32_t *pairs,
+                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2,
+                     cudaStream_t s);
 
 // The threshold and label bitmaps of GraphDev (thr: num_labels * kThrLevels,
 // lab_bits: num_labels bitmaps of hub_words words), from the neighbour label

@@ -163,7 +163,7 @@ __device__ __forceinline__ bool row_contains_l(const GraphDev &g, int32_t x, int
     if (h >= 0) return hub_bit(g, h, w);
   }
   const int32_t b = __ldg(g.rp + x), e = __ldg(g.rp + x + 1);
-  return few ? row_contains_few(g, x, b, e, l, w) : row_search(g, b, e, l, w);
+  return few && !g.hub_lo ? row_contains_few(g, x, b, e, l, w) : row_search(g, b, e, l, w);
 }
 
 }  // namespace gsm

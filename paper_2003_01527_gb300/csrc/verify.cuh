@@ -404,6 +404,7 @@ __device__ __forceinline__ uint32_t check_group(
     sj[j] = slot;
     at[j] = pst + (x - rs);
   }
+  if (g.hub_lo) few = 0;  // bitmaps that do not cover the mapped neighbours
 #pragma unroll
   for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
   if constexpr (kCheck == kCheckAny) {

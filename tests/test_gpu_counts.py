@@ -107,3 +107,31 @@ def test_counts_past_64_bits(gsm_lib, cuda):
         m.count(star(6))
     assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
     m.close()
+
+
+@pytest.mark.parametrize("hub_bytes", [0, -1, 1 << 16])
+def test_cliques_on_the_renumbered_graph(gsm_lib, cuda, hub_bytes):
+    """Unrestricted cliques on a one-label graph with enough 2-edge paths are
+    counted with its vertices renumbered by degree; a partition into root
+    ranges (never renumbered) adds up to the same, and the first one loaded
+    afterwards does not see the old numbering."""
+    m = gsm_lib.Matcher(device=0, hub_bitmap_bytes=hub_bytes)
+    for scale, ef, drop in ((15, 16, 77), (14, 40, 3)):
+        n, rp, col = I.rmat(scale, ef, *I.RMAT_ABC, seed=91)
+        src = np.repeat(np.arange(n), np.diff(rp))
+        keep = (src < n - drop) & (col < n - drop)  # vertices that fill no bitmap word
+        n -= drop
+        rp, col = I.csr_from_pairs(n, src[keep], col[keep])
+        d = np.diff(rp).astype(float)
+        assert (d * d).sum() > 2 ** 28
+        m.load_graph(rp, col, validate=True)
+        for k in (3, 4, 5):
+            edges = [(i, j) for i in range(k) for j in range(i + 1, k)]
+            if k == 5 and scale == 14:
+                continue  # the partition takes long
+            parts = [m.count(m.query(k, edges).restrict(0, *r))
+                     for r in ((0, n // 3), (n // 3, n - 1), (n - 1, n))]
+            assert m.count(m.query(k, edges)) == sum(parts), (scale, k)
+            assert m.count_distinct(m.query(k, edges)) == \
+                (sum(parts) // math.factorial(k), math.factorial(k))
+    m.close()
