@@ -335,10 +335,68 @@ __global__ void __launch_bounds__(256) k_b_pivot_scan(
   zero_words(lb_level, level_tiles + kLbExtra);
 }
 
+// check_candidate of a thread's four candidates (w[j] of row r[j], a row of
+// query q[j], pivot slot s[j]; `alive`: which of them there are), their loads
+// issued together, stage by stage, as in the single-query path's grouped form:
+// a batch's levels are short, and a check is a chain of dependent loads.
+__device__ __forceinline__ uint32_t b_check_group(
+    const GraphDev &g, const BatchQuery *__restrict__ qs, int32_t i,
+    const int32_t *__restrict__ F, int32_t ld, const int32_t (&r)[kItemsPerThread],
+    const int32_t (&q)[kItemsPerThread], const int32_t (&s)[kItemsPerThread],
+    const int32_t (&w)[kItemsPerThread], uint32_t alive, uint32_t few) {
+  constexpr int kN = kItemsPerThread;
+  int32_t lab[kN];
+  int nb = 0, ninj = 0;
+  {
+    const uint32_t *bm[kN];
+    uint32_t word[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const BatchLevel &L = qs[q[j]].lv[i];
+      const bool on = (alive >> j) & 1u;
+      bm[j] = on ? L.bitmap : nullptr;
+      lab[j] = L.lab;
+      nb = max(nb, on ? (int)L.nb : 0);
+      ninj = max(ninj, on ? (int)L.ninj : 0);
+    }
+#pragma unroll
+    for (int j = 0; j < kN; ++j) word[j] = bm[j] ? __ldg(bm[j] + (w[j] >> 5)) : ~0u;
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (!((word[j] >> (w[j] & 31)) & 1u)) alive &= ~(1u << j);
+  }
+  for (int t = 0; t < ninj; ++t) {
+    int32_t y[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const BatchLevel &L = qs[q[j]].lv[i];
+      y[j] = (alive >> j) & 1u && t < L.ninj ? F[L.inj[t] * ld + r[j]] : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (y[j] == w[j]) alive &= ~(1u << j);
+  }
+  for (int o = 0; o + 1 < nb && alive; ++o) {  // neighbours besides the pivot
+    int32_t x[kN];
+    uint32_t now = 0;  // candidates with this many neighbours
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const BatchLevel &L = qs[q[j]].lv[i];
+      x[j] = 0;
+      if ((alive >> j) & 1u && o + 1 < L.nb) {
+        x[j] = F[L.bpos[o + (o >= s[j])] * ld + r[j]];
+        now |= 1u << j;
+      }
+    }
+    alive &= ~now | group_contains(g, x, w, [&](int j) { return lab[j]; }, now, few);
+  }
+  return alive;
+}
+
 // Verification and write pass of one step, in one launch: tiles by ticket; a
 // tile's survivors are ranked, kept in one of two shared buffers and written
 // after the CTA has verified its next tile, when the look-back has its prefix
-// (the single-query path's k_extend_fused, with its check, check_candidate).
+// (the single-query path's k_extend_fused).
 // Survivors of a query at its last level are counted (times their leaf
 // numbers), and for a query that lists its rows written to the result arena;
 // the others become rows of the next level.  Both ranks travel in one
@@ -420,8 +478,9 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
     const int32_t x0 = tile * tile_items, x1 = min(x0 + tile_items, W);
     const TileRows t = stage_rows(woff, tile_row, 0, tile_items, s_woff, tile);
     const int32_t xb = x0 + warp * 128 + lane * kItemsPerThread;
+    constexpr int kN = kItemsPerThread;
     uint32_t bits = 0, fbits = 0;
-    int32_t rj[kItemsPerThread], wj[kItemsPerThread];
+    int32_t rj[kN], wj[kN];
     BatchSum sum;
     if (xb < x1) {
       int32_t rs;
@@ -429,33 +488,44 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
       int32_t rr = r - t.r0;
       int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
       int32_t q = rseg[r], pst = pstart[r], slot = pslot[r];
+      int32_t qj[kN], sj[kN], at[kN];
+      uint32_t alive = 0, few = 0;
 #pragma unroll
-      for (int j = 0; j < kItemsPerThread; ++j) {
-        rj[j] = r;
-        wj[j] = 0;
+      for (int j = 0; j < kN; ++j) {
         const int32_t x = xb + j;
-        if (x >= x1) continue;
-        while (x >= re) {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
-          q = rseg[r];
-          pst = pstart[r];
-          slot = pslot[r];
-        }
-        const BatchQuery &bq = qs[q];
-        const int32_t w = __ldg(g.lcol + pst + (x - rs));
-        rj[j] = r;
-        wj[j] = w;
-        const ColumnRow row{F, ld, r};
-        if (check_candidate(g, bq.lv[i], row, w, slot, re - rs <= kFewCandidates)) {
-          if (i != bq.kc - 1) {
-            bits |= 1u << j;
-          } else {
-            sum.add(q, core_number(g, bq, ExtendedRow<ColumnRow>{row, i, w}, &over), counts);
-            if (bq.enumerate) fbits |= 1u << j;
+        if (x < x1) {
+          if (x >= re) {
+            do {  // next row (rows without work are skipped)
+              ++rr;
+              ++r;
+              rs = re;
+              re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
+            } while (x >= re);
+            q = rseg[r];
+            pst = pstart[r];
+            slot = pslot[r];
           }
+          alive |= 1u << j;
+          if (re - rs <= kFewCandidates) few |= 1u << j;
+        }
+        rj[j] = r;
+        qj[j] = q;
+        sj[j] = slot;
+        at[j] = pst + (x - rs);
+      }
+#pragma unroll
+      for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
+      alive = b_check_group(g, qs, i, F, ld, rj, qj, sj, wj, alive, few);
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        if (!((alive >> j) & 1u)) continue;
+        const BatchQuery &bq = qs[qj[j]];
+        if (i != bq.kc - 1) {
+          bits |= 1u << j;
+        } else {
+          const ColumnRow row{F, ld, rj[j]};
+          sum.add(qj[j], core_number(g, bq, ExtendedRow<ColumnRow>{row, i, wj[j]}, &over), counts);
+          if (bq.enumerate) fbits |= 1u << j;
         }
       }
     }

@@ -333,6 +333,100 @@ struct RowCheck {
 constexpr int kCheckAny = 0, kCheckRow = 0, kCheckGroup = 3;
 constexpr int kMaxRowCheck = 3;
 
+// Which of the `alive` pairs are edges: w[j] (label lab_of(j)) in the row of
+// x[j].  row_contains_l of four pairs, their loads issued together; few (bit
+// j): see row_contains_few.
+template <typename Lab>
+__device__ __forceinline__ uint32_t group_contains(const GraphDev &g,
+                                                   const int32_t (&x)[kItemsPerThread],
+                                                   const int32_t (&w)[kItemsPerThread],
+                                                   const Lab &lab_of, uint32_t alive,
+                                                   uint32_t few) {
+  constexpr int kN = kItemsPerThread;
+  uint32_t open = alive;  // pairs no bitmap has decided
+  if (g.hub) {
+    int32_t h[kN];
+    uint32_t word[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) h[j] = (alive >> j) & 1u ? __ldg(g.hub + x[j]) : -1;
+    uint32_t rev = 0;  // taken from the candidate's bitmap
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (h[j] < 0 && (alive & few) >> j & 1u) {
+        h[j] = __ldg(g.hub + w[j]);
+        rev |= 1u << j;
+      }
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const int32_t v = (rev >> j) & 1u ? x[j] : w[j];
+      word[j] = h[j] >= 0 ? __ldg(g.hub_bits + (size_t)h[j] * g.hub_words + (v >> 5)) >> (v & 31)
+                          : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      if (h[j] >= 0) {
+        open &= ~(1u << j);
+        if (!(word[j] & 1u)) alive &= ~(1u << j);
+      }
+  }
+  if (!open) return alive;
+  // binary searches, step by step together
+  int32_t lo[kN], len[kN], end[kN], key[kN], lab[kN];
+#pragma unroll
+  for (int j = 0; j < kN; ++j) {
+    const bool on = (open >> j) & 1u;
+    lo[j] = on ? __ldg(g.rp + x[j]) : 0;
+    end[j] = on ? __ldg(g.rp + x[j] + 1) : 0;
+    key[j] = w[j];
+    lab[j] = lab_of(j);
+  }
+#pragma unroll
+  for (int j = 0; j < kN; ++j) {
+    if ((few & open) >> j & 1u && end[j] - lo[j] > kLongRow) {
+      const int32_t wb = __ldg(g.rp + w[j]), we = __ldg(g.rp + w[j] + 1);
+      if (we - wb < end[j] - lo[j]) {  // the candidate's row is shorter: x in it
+        lo[j] = wb;
+        end[j] = we;
+        key[j] = x[j];
+        lab[j] = __ldg(g.lab + x[j]);
+      }
+    }
+    len[j] = end[j] - lo[j];
+  }
+  const bool one = g.num_labels == 1;
+  bool more = true;
+  while (more) {
+    more = false;
+    int32_t v[kN], m[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const int32_t mid = lo[j] + (len[j] >> 1);
+      v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
+      m[j] = len[j] > 0 && !one ? __ldg(g.llab + mid) : lab[j];
+    }
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      if (len[j] <= 0) continue;
+      const int32_t half = len[j] >> 1;
+      if (m[j] < lab[j] || (m[j] == lab[j] && v[j] < key[j])) {
+        lo[j] += half + 1;
+        len[j] -= half + 1;
+      } else {
+        len[j] = half;
+      }
+      more = more || len[j] > 0;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kN; ++j) {
+    if (!((open >> j) & 1u)) continue;
+    const bool in = lo[j] < end[j] && __ldg(g.lcol + lo[j]) == key[j] &&
+                    (one || __ldg(g.llab + lo[j]) == lab[j]);
+    if (!in) alive &= ~(1u << j);
+  }
+  return alive;
+}
+
 // The candidates x = xb .. xb + 3 of one thread, below x1: returns a bit for
 // each that passes the level's checks; rj, wj: their rows and vertices.
 // kProbes (kCheckAny only): adds the checks' probe bytes to *probe_bytes.
@@ -441,8 +535,7 @@ __device__ __forceinline__ uint32_t check_group(
   }
 #pragma unroll
   for (int o = 0; o + 1 < kNb; ++o) {  // neighbours besides the pivot
-    int32_t x[kN], h[kN];
-    uint32_t word[kN];
+    int32_t x[kN];
 #pragma unroll
     for (int j = 0; j < kN; ++j) {
       x[j] = (alive >> j) & 1u ? F[d.bpos[o + (o >= sj[j])] * ld + rj[j]] : 0;
@@ -451,85 +544,7 @@ __device__ __forceinline__ uint32_t check_group(
         x[j] = 0;
       }
     }
-    uint32_t open = alive;  // candidates no bitmap has decided
-    if (g.hub) {
-#pragma unroll
-      for (int j = 0; j < kN; ++j) h[j] = (alive >> j) & 1u ? __ldg(g.hub + x[j]) : -1;
-      uint32_t rev = 0;  // taken from the candidate's bitmap
-#pragma unroll
-      for (int j = 0; j < kN; ++j)
-        if (h[j] < 0 && (alive & few) >> j & 1u) {
-          h[j] = __ldg(g.hub + wj[j]);
-          rev |= 1u << j;
-        }
-#pragma unroll
-      for (int j = 0; j < kN; ++j) {
-        const int32_t v = (rev >> j) & 1u ? x[j] : wj[j];
-        word[j] = h[j] >= 0 ? __ldg(g.hub_bits + (size_t)h[j] * g.hub_words + (v >> 5)) >> (v & 31)
-                            : 0u;
-      }
-#pragma unroll
-      for (int j = 0; j < kN; ++j)
-        if (h[j] >= 0) {
-          open &= ~(1u << j);
-          if (!(word[j] & 1u)) alive &= ~(1u << j);
-        }
-    }
-    if (open) {  // binary searches, step by step together
-      int32_t lo[kN], len[kN], end[kN], key[kN], lab[kN];
-#pragma unroll
-      for (int j = 0; j < kN; ++j) {
-        const bool on = (open >> j) & 1u;
-        lo[j] = on ? __ldg(g.rp + x[j]) : 0;
-        end[j] = on ? __ldg(g.rp + x[j] + 1) : 0;
-        key[j] = wj[j];
-        lab[j] = d.lab;
-      }
-#pragma unroll
-      for (int j = 0; j < kN; ++j) {
-        if ((few & open) >> j & 1u && end[j] - lo[j] > kLongRow) {
-          const int32_t wb = __ldg(g.rp + wj[j]), we = __ldg(g.rp + wj[j] + 1);
-          if (we - wb < end[j] - lo[j]) {  // the candidate's row is shorter: x in it
-            lo[j] = wb;
-            end[j] = we;
-            key[j] = x[j];
-            lab[j] = __ldg(g.lab + x[j]);
-          }
-        }
-        len[j] = end[j] - lo[j];
-      }
-      const bool one = g.num_labels == 1;
-      bool more = true;
-      while (more) {
-        more = false;
-        int32_t v[kN], m[kN];
-#pragma unroll
-        for (int j = 0; j < kN; ++j) {
-          const int32_t mid = lo[j] + (len[j] >> 1);
-          v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
-          m[j] = len[j] > 0 && !one ? __ldg(g.llab + mid) : lab[j];
-        }
-#pragma unroll
-        for (int j = 0; j < kN; ++j) {
-          if (len[j] <= 0) continue;
-          const int32_t half = len[j] >> 1;
-          if (m[j] < lab[j] || (m[j] == lab[j] && v[j] < key[j])) {
-            lo[j] += half + 1;
-            len[j] -= half + 1;
-          } else {
-            len[j] = half;
-          }
-          more = more || len[j] > 0;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kN; ++j) {
-        if (!((open >> j) & 1u)) continue;
-        const bool in = lo[j] < end[j] && __ldg(g.lcol + lo[j]) == key[j] &&
-                        (one || __ldg(g.llab + lo[j]) == lab[j]);
-        if (!in) alive &= ~(1u << j);
-      }
-    }
+    alive = group_contains(g, x, wj, [&](int) { return d.lab; }, alive, few);
   }
   return alive;
 }
