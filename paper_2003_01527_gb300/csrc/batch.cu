@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(256) k_b_filter(GraphDev g, const FilterDesc *
 }
 
 // The same from the graph's bitmaps (a thread per word, a CTA row per query).
+template <int kV>
 __global__ void __launch_bounds__(256) k_b_filter_bits(GraphDev g,
                                                        const FilterDesc *__restrict__ fds,
                                                        uint32_t *const *__restrict__ bm_out,
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(256) k_b_filter_bits(GraphDev g,
   for (int j = threadIdx.x; j < (int)(sizeof(FilterDesc) / 4); j += blockDim.x)
     reinterpret_cast<int32_t *>(&s_d)[j] = reinterpret_cast<const int32_t *>(fds + q)[j];
   __syncthreads();
-  filter_words(g, s_d, bm_out[q], sizes ? sizes + (int64_t)q * kMaxK : nullptr, 0, 1);
+  filter_words<kV>(g, s_d, bm_out[q], sizes ? sizes + (int64_t)q * kMaxK : nullptr, 0, 1);
 }
 
 // ---- counts, and what the last CTA of a kernel does
@@ -581,7 +582,11 @@ void launch_filter_many(const GraphDev &g, const FilterDesc *fds, uint32_t *cons
   if (nq <= 0) return;
   if (sizes) cudaMemsetAsync(sizes, 0, sizeof(unsigned long long) * nq * kMaxK, s);
   if (g.thr && n_words > 0) {
-    k_b_filter_bits<<<dim3((n_words + 255) / 256, nq), 256, 0, s>>>(g, fds, bm_out, sizes);
+    const dim3 grid(filter_grid(n_words), nq);
+    if (n_words % 4 == 0)
+      k_b_filter_bits<4><<<grid, 256, 0, s>>>(g, fds, bm_out, sizes);
+    else
+      k_b_filter_bits<1><<<grid, 256, 0, s>>>(g, fds, bm_out, sizes);
     return;
   }
   const int gx = (int)std::min<int64_t>((n_words + 7) / 8, 128);

@@ -27,31 +27,59 @@ __device__ __forceinline__ uint32_t nlc_pass(const Desc &d, uint32_t vneed,
   return pass;
 }
 
-// Word w of C(u) from the graph's threshold and label bitmaps: the filter's
-// tests for 32 vertices are ands of words.  A requirement above kThrLevels
-// neighbours takes the top bitmap and then looks the counts of the vertices
-// left up one by one.  (Enough neighbours of every label are enough
+// Words of a bitmap that one thread of the filter handles together: four (one
+// 16-byte load or store) when the bitmaps' words are a multiple of four, so
+// that every bitmap starts on a 16-byte boundary, else one.
+template <int kV>
+struct FilterWords {
+  uint32_t w[kV];
+  __device__ __forceinline__ void load(const uint32_t *p) {
+    if constexpr (kV == 4) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+      w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+    } else {
+      w[0] = __ldg(p);
+    }
+  }
+  __device__ __forceinline__ void store(uint32_t *p) const {
+    if constexpr (kV == 4)
+      *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+    else
+      *p = w[0];
+  }
+};
+
+// Words at .. at + kV - 1 of C(u) from the graph's threshold and label bitmaps:
+// the filter's tests for 32 vertices are ands of words.  A requirement above
+// kThrLevels neighbours takes the top bitmap and then looks the counts of the
+// vertices left up one by one.  (Enough neighbours of every label are enough
 // neighbours, so the degree needs no test of its own beside them; with one
 // label the bitmaps hold degrees.)
-template <typename Desc>
-__device__ __forceinline__ uint32_t filter_word(const GraphDev &g, const Desc &d, int u,
-                                                int32_t w) {
-  uint32_t word = __ldg(g.lab_bits + (int64_t)d.qlab[u] * d.n_words + w);
-  const int32_t v0 = w * 32;
-  const int32_t lo = d.lo[u] - v0, hi = d.hi[u] - v0;  // the restriction inside the word
-  if (lo > 0) word &= lo < 32 ? ~0u << lo : 0u;
-  if (hi < 32) word &= hi > 0 ? ~0u >> (32 - hi) : 0u;
+template <int kV, typename Desc>
+__device__ __forceinline__ FilterWords<kV> filter_word(const GraphDev &g, const Desc &d, int u,
+                                                       int32_t at) {
+  FilterWords<kV> word;
+  word.load(g.lab_bits + (int64_t)d.qlab[u] * d.n_words + at);
   const bool one = g.num_labels == 1;
   const int nr = one ? (d.qdeg[u] > 0 ? 1 : 0) : d.nreq[u];
   uint32_t deep = 0;  // requirements above the bitmaps' levels
   for (int r = 0; r < nr; ++r) {
     const int32_t l = one ? 0 : d.slot_label[d.req_slot[u][r]];
     const int32_t c = one ? d.qdeg[u] : d.req_cnt[u][r];
-    word &= __ldg(g.thr + ((int64_t)l * kThrLevels + min(c, kThrLevels) - 1) * d.n_words + w);
+    FilterWords<kV> t;
+    t.load(g.thr + ((int64_t)l * kThrLevels + min(c, kThrLevels) - 1) * d.n_words + at);
+#pragma unroll
+    for (int j = 0; j < kV; ++j) word.w[j] &= t.w[j];
     if (c > kThrLevels) deep |= 1u << r;
   }
-  if (deep && word) {
-    for (uint32_t m = word; m; m &= m - 1) {
+#pragma unroll
+  for (int j = 0; j < kV; ++j) {
+    const int32_t v0 = (at + j) * 32;
+    const int32_t lo = d.lo[u] - v0, hi = d.hi[u] - v0;  // the restriction inside the word
+    if (lo > 0) word.w[j] &= lo < 32 ? ~0u << lo : 0u;
+    if (hi < 32) word.w[j] &= hi > 0 ? ~0u >> (32 - hi) : 0u;
+    if (!deep || !word.w[j]) continue;
+    for (uint32_t m = word.w[j]; m; m &= m - 1) {
       const int bit = __ffs(m) - 1;
       const int64_t v = v0 + bit;
       bool ok = true;
@@ -63,35 +91,42 @@ __device__ __forceinline__ uint32_t filter_word(const GraphDev &g, const Desc &d
           ok = (int32_t)__ldg(g.nlc + v * g.nlc_stride + d.slot_label[d.req_slot[u][r]]) >=
                d.req_cnt[u][r];
       }
-      if (!ok) word &= ~(1u << bit);
+      if (!ok) word.w[j] &= ~(1u << bit);
     }
   }
   return word;
 }
 
 // Words of C(u) for u = u0, u0 + du, ... of one query: thread t of the grid's
-// x dimension takes word t (the caller launches a thread per word), so a
-// warp's loads and stores cover 128 consecutive bytes.  sizes (may be null)
-// gains |C(u)|.  Bound by L2 and the bitmaps written: 256 queries on R-MAT 18
-// (13.6 M words) cost a batch about 20 us, where a test per vertex, query and
-// query vertex took 1,435 us (the counted batch: 2,659 -> 1,247 us).
-template <typename Desc>
+// x dimension takes kV words (filter_grid), so a warp's loads and stores are
+// contiguous.  sizes (may be null) gains |C(u)|.  Bound by L2 and the bitmaps
+// written: 256 queries on R-MAT 18 (13.6 M words) take 37 us with four
+// words a thread, 71 with one, where a test per vertex, query and query vertex
+// took 1,435 us (under ncu).
+template <int kV, typename Desc>
 __device__ __forceinline__ void filter_words(const GraphDev &g, const Desc &d,
                                              uint32_t *__restrict__ bitmaps,
                                              unsigned long long *__restrict__ sizes, int u0,
                                              int du) {
-  const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+  const int32_t at = (blockIdx.x * blockDim.x + threadIdx.x) * kV;
   for (int u = u0; u < d.k; u += du) {
-    uint32_t word = 0;
-    if (w < d.n_words) {
-      word = filter_word(g, d, u, w);
-      bitmaps[(int64_t)u * d.n_words + w] = word;
+    int32_t c = 0;
+    if (at < d.n_words) {
+      const FilterWords<kV> word = filter_word<kV>(g, d, u, at);
+      word.store(bitmaps + (int64_t)u * d.n_words + at);
+#pragma unroll
+      for (int j = 0; j < kV; ++j) c += __popc(word.w[j]);
     }
     if (sizes) {
-      const int32_t c = __reduce_add_sync(0xffffffffu, __popc(word));
+      c = __reduce_add_sync(0xffffffffu, c);
       if ((threadIdx.x & 31) == 0 && c) atomicAdd(sizes + u, (unsigned long long)c);
     }
   }
+}
+// CTAs of 256 threads in x for bitmaps of n_words words.
+inline unsigned filter_grid(int32_t n_words) {
+  const int32_t per = n_words % 4 ? 256 : 1024;
+  return (unsigned)((n_words + per - 1) / per);
 }
 
 // One warp handles 32 consecutive data vertices per iteration (warps

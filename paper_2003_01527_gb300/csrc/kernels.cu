@@ -108,11 +108,12 @@ __global__ void __launch_bounds__(256) k_filter(GraphDev g, FilterDesc d,
 
 // The same from the graph's bitmaps: a thread per word, a CTA row per query
 // vertex.
+template <int kV>
 __global__ void __launch_bounds__(256) k_filter_bits(GraphDev g,
                                                      const __grid_constant__ FilterDesc d,
                                                      uint32_t *__restrict__ bitmaps,
                                                      unsigned long long *sizes, Stage stage) {
-  filter_words(g, d, bitmaps, sizes, blockIdx.y, gridDim.y);
+  filter_words<kV>(g, d, bitmaps, sizes, blockIdx.y, gridDim.y);
   if (!stage.words) return;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1315,8 +1316,11 @@ void launch_filter(const GraphDev &g, const FilterDesc &d, uint32_t *bitmaps,
                    unsigned long long *sizes, cudaStream_t s, Stage stage) {
   const int threads = 256;
   if (g.thr && d.n_words > 0) {
-    k_filter_bits<<<dim3((d.n_words + threads - 1) / threads, d.k), threads, 0, s>>>(
-        g, d, bitmaps, sizes, stage);
+    const dim3 grid(filter_grid(d.n_words), d.k);
+    if (d.n_words % 4 == 0)
+      k_filter_bits<4><<<grid, threads, 0, s>>>(g, d, bitmaps, sizes, stage);
+    else
+      k_filter_bits<1><<<grid, threads, 0, s>>>(g, d, bitmaps, sizes, stage);
     return;
   }
   int64_t warps_needed = d.n_words;
