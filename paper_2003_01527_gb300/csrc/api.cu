@@ -764,6 +764,8 @@ struct Run {
   // 0..rank_p-1, placed first in that order) when rank_p > 0: ranks of the
   // rows of the last level's input piece in `rank`, running state in prefix
   int32_t rank_p = 0, rank_pos = 0;
+  // leaf levels: the left-out entries of the rows of the level being processed
+  const int2 *excl[kMaxK] = {};
   PrefixState *prefix = nullptr;
   const int32_t *rank = nullptr;
 };
@@ -820,6 +822,81 @@ void ensure_acc(Run &R, uint64_t rows) {
   R.acc_ld = ld;
 }
 
+// Room for a leaf level's left-out entries, `rows` of them at most (null if the
+// level is not a leaf's, or its rows have none).
+int2 *push_excl(Run &R, int32_t i, int64_t rows) {
+  if (!R.lv[i].leaf || R.lv[i].ninj == 0) return nullptr;
+  return (int2 *)stack_push(R.ctx, sizeof(int2) * rows);
+}
+size_t excl_bytes(const Run &R, int32_t i, int64_t rows) {
+  return R.lv[i].leaf && R.lv[i].ninj > 0 ? align_up(sizeof(int2) * (size_t)rows) : 0;
+}
+
+// A leaf level: its W output rows are known, none is checked.  Rows are split
+// in halves until their output fits.
+void process_leaf(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t *pstart,
+                  const int64_t *woff, int64_t ra, int64_t rb, int64_t wa, int64_t wb,
+                  const LevelSetup &setup) {
+  gsm_ctx *ctx = R.ctx;
+  const Range range(level_range(i));
+  const LevelDesc &d = R.lv[i];
+  const bool last = i == R.k - 1;
+  const int64_t W = wb - wa, nrows = rb - ra;
+  if (W <= 0) return;
+  const int32_t w_out = i + 1;
+  const size_t bytes = (size_t)W * w_out * sizeof(int32_t);
+  if (!last) {
+    // the frontier and the next level's per-row arrays
+    const size_t need = align_up(bytes) + align_up(4 * (size_t)W) + align_up((size_t)W) +
+                        align_up(8 * ((size_t)W + 1)) + excl_bytes(R, i + 1, W);
+    if (W * w_out >= (int64_t(1) << 31) - 1 || !stack_fits(ctx, need)) {
+      if (nrows <= 1)
+        FAIL(GSM_ERR_BUDGET, "the %lld partial results of one row need %zu bytes, over the budget",
+             (long long)W, bytes);
+      const int64_t mid = ra + nrows / 2;
+      const int64_t wmid = read_i64(ctx, woff + mid);
+      process_leaf(R, i, F, ld, pstart, woff, ra, mid, wa, wmid, LevelSetup());
+      process_leaf(R, i, F, ld, pstart, woff, mid, rb, wmid, wb, LevelSetup());
+      return;
+    }
+  }
+  ctx->run.chunks += 1;
+  const int64_t tiles = extend_tiles(wa, wb, R.block);
+  const int32_t *tile_row = setup.tile_row;
+  if (tiles > setup.cap) {
+    int32_t *rows = (int32_t *)scratch_get(ctx, sizeof(int32_t) * (tiles + 1));
+    timed(ctx, K_PIVOT, 8.0 * (nrows + tiles), (uint64_t)tiles, 1, [&] {
+      launch_tile_rows(woff, ra, rb, wa, wb, R.block, rows, nullptr, ctx->stream);
+    });
+    tile_row = rows;
+  }
+  const Mark mk = stack_mark(ctx);
+  RowSink sink;
+  int32_t *Fn = nullptr;
+  if (last) {
+    ensure_acc(R, R.acc_rows + (uint64_t)W);
+    sink = RowSink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
+                   ctx->acc[0]};
+    sink.rank = R.rank;
+    sink.rank_pos = R.rank_pos;
+  } else {
+    Fn = (int32_t *)stack_push(ctx, bytes);
+    sink = RowSink{kSinkColumns, w_out, 0, 0, W, 0, Fn};
+  }
+  const double out_bytes = last ? (double)W * (double)R.acc_row_bytes() : 4.0 * (double)W * w_out;
+  timed(ctx, K_FUSED, (double)nrows * (4.0 * i + 12.0) + 4.0 * (double)W + out_bytes, (uint64_t)W,
+        1, [&] {
+    launch_leaf_expand(R.g, d, F, ld, pstart, R.excl[i], woff, tile_row, wa, wb, R.block, sink,
+                       ctx->stream);
+  });
+  if (last) {
+    R.acc_rows += (uint64_t)W;
+    return;
+  }
+  recurse(R, i + 1, Fn, W, W);
+  stack_release(ctx, mk);
+}
+
 void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t *pstart,
                  const uint8_t *pslot, const int64_t *woff, int64_t ra, int64_t rb, int64_t wa,
                  int64_t wb, const LevelSetup &setup = LevelSetup()) {
@@ -829,6 +906,10 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   const bool last = i == R.k - 1;
   const int64_t W = wb - wa, nrows = rb - ra;
   if (W <= 0) return;
+  if (d.leaf) {
+    process_leaf(R, i, F, ld, pstart, woff, ra, rb, wa, wb, setup);
+    return;
+  }
   const int64_t tile_items = (int64_t)R.block * kItemsPerThread;
   const int64_t tiles = extend_tiles(wa, wb, R.block);
   const double read_bytes = (double)nrows * (4.0 * i + 13.0) + 4.0 * (double)W;
@@ -845,7 +926,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
     } else {
       const size_t need = align_up((size_t)W * w_out * sizeof(int32_t)) +
                           align_up(4 * (size_t)W) + align_up((size_t)W) +
-                          align_up(8 * ((size_t)W + 1));
+                          align_up(8 * ((size_t)W + 1)) + excl_bytes(R, i + 1, W);
       fits = (int64_t)W * w_out < (int64_t(1) << 31) - 1 && stack_fits(ctx, need);
     }
     if (fits) {
@@ -901,7 +982,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   const size_t bytes = (size_t)S * w_out * sizeof(int32_t);
   // the next level also pushes pivot start, pivot slot and work offsets
   const size_t need = align_up(bytes) + align_up(4 * (size_t)S) + align_up((size_t)S) +
-                      align_up(8 * ((size_t)S + 1));
+                      align_up(8 * ((size_t)S + 1)) + excl_bytes(R, i + 1, S);
   // elements of a frontier are indexed with 32 bits inside the kernels
   const bool too_many = (int64_t)S * w_out >= (int64_t(1) << 31) - 1;
   if (too_many || !stack_fits(ctx, need)) {
@@ -993,11 +1074,14 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   int32_t *pstart2 = (int32_t *)stack_push(ctx, sizeof(int32_t) * W);
   uint8_t *pslot2 = (uint8_t *)stack_push(ctx, W);
   int64_t *woff2 = (int64_t *)stack_push(ctx, sizeof(int64_t) * (W + 1));
+  int2 *excl = push_excl(R, i + 1, W);
   const LevelSetup next = push_setup(R, W);
   timed(ctx, K_PIVOT, 0.0, 0, 1, [&] {
     launch_pivot_scan(R.g, dn, Fn, W, W, pstart2, pslot2, woff2, lb + tiles + kLbExtra,
-                      R.spin_limit, next_stage(ctx), next, R.scan_stall_tile, ctx->stream, S_dev);
+                      R.spin_limit, next_stage(ctx), next, R.scan_stall_tile, ctx->stream, S_dev,
+                      excl);
   });
+  R.excl[i + 1] = excl;
   wait_stage(ctx);
   const int64_t S = ((volatile int64_t *)ctx->h_stage)[0];
   if (((volatile int64_t *)ctx->h_stage)[1])
@@ -1073,12 +1157,14 @@ void recurse(Run &R, int32_t i, const int32_t *F, int64_t ld, int64_t rows) {
   const int64_t pwords = pivot_scan_words(rows);
   auto *plb = (unsigned long long *)scratch_get(ctx, sizeof(unsigned long long) * pwords);
   CU(cudaMemsetAsync(plb, 0, sizeof(unsigned long long) * pwords, ctx->stream));
+  int2 *excl = push_excl(R, i, rows);
   const LevelSetup setup = push_setup(R, rows);
   timed(ctx, K_PIVOT, (double)rows * (4.0 * d.nb + 8.0 * d.nb + 13.0), (uint64_t)rows, 1,
         [&] {
     launch_pivot_scan(R.g, d, F, ld, rows, pstart, pslot, woff, plb, R.spin_limit,
-                      next_stage(ctx), setup, R.scan_stall_tile, ctx->stream);
+                      next_stage(ctx), setup, R.scan_stall_tile, ctx->stream, nullptr, excl);
   });
+  R.excl[i] = excl;
   wait_stage(ctx);
   if (((volatile int64_t *)ctx->h_stage)[1])
     FAIL(GSM_ERR_TIMEOUT, "a work-scan tile waited too long for its predecessors");
@@ -1610,6 +1696,12 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     for (int32_t j = 0; j <= i; ++j) d.out_col[j] = (i == q->k - 1) ? R.order[j] : j;
     // a leaf's candidates are all entries of its parent's cut label segment
     d.bitmap = popc(q->adj[u]) == 1 ? nullptr : bm + (size_t)u * nw;
+    // ... and its level needs no checks (listings; fault injection, the probe
+    // accounting and the two-pass form keep their levels)
+    d.leaf = enumerate && d.bitmap == nullptr && d.ninj <= kLeafExcl && !ctx->opt.lookahead &&
+             R.block <= 256 &&
+             !(ctx->opt.flags & (GSM_OPT_COMPRESSED_FRONTIERS | GSM_OPT_TWO_PASS |
+                                 GSM_OPT_COUNT_PROBES | GSM_OPT_INJECT_LOOKBACK_STALL));
     d.lab = dense[u];
     d.rlo = std::max<int32_t>(0, q->lo[u]);
     d.rhi = std::min<int32_t>(ctx->n, q->hi[u]);

@@ -436,7 +436,8 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int64_t ld, int64_t R,
     int32_t ptiles, int32_t *__restrict__ pstart, uint8_t *__restrict__ pslot,
     int64_t *__restrict__ woff, const int64_t *R_dev, unsigned long long *lookback,
-    int32_t spin_limit, Stage stage, LevelSetup setup, int32_t stall_tile) {
+    int32_t spin_limit, Stage stage, LevelSetup setup, int32_t stall_tile,
+    int2 *__restrict__ excl) {
   __shared__ int64_t s_val[kPsRows];
   __shared__ int64_t s_warp[33];
   __shared__ int32_t s_tile;
@@ -505,6 +506,35 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
           bstart[j] = seg.x;
           bslot[j] = b;
         }
+      }
+    }
+    if (d.leaf) {  // leave out the images the segment holds
+#pragma unroll
+      for (int j = 0; j < kPsIpt; ++j) {
+        const int64_t r = base + j * kPsThreads + threadIdx.x;
+        if (r >= R) continue;
+        int2 out = make_int2(INT_MAX, INT_MAX);
+        int32_t left = best[j];
+        for (int t = 0; t < d.ninj; ++t) {
+          const int32_t y = F[(int64_t)d.inj[t] * ld + r];
+          int32_t at = bstart[j], len = best[j];
+          while (len > 0) {
+            const int32_t half = len >> 1;
+            if (__ldg(g.lcol + at + half) < y) {
+              at += half + 1;
+              len -= half + 1;
+            } else {
+              len = half;
+            }
+          }
+          if (at < bstart[j] + best[j] && __ldg(g.lcol + at) == y) {
+            const int32_t off = at - bstart[j];
+            out = off < out.x ? make_int2(off, out.x) : make_int2(out.x, off);
+            --left;
+          }
+        }
+        if (d.ninj > 0) excl[r] = out;
+        best[j] = left;
       }
     }
 #pragma unroll
@@ -940,6 +970,73 @@ __global__ void __launch_bounds__(kMaxThreads,
       for (int w = 0; w < 3; ++w)
         stage.words[w] = (long long)atomicAdd(lookback + tiles + 1 + w, 0ull);
       stage_seq(stage);
+    }
+  }
+}
+
+// The level of a leaf: output row x of the tile is its row's (x - offset)-th
+// segment entry that is not left out.  Nothing is checked, ranked or waited
+// for.  A thread first finds the rows of four consecutive outputs (one search)
+// and leaves them in shared memory; then thread t writes outputs t, t + B, ...,
+// so that a warp's stores cover 32 consecutive rows.  Bound by the output's
+// write and the parent row's gathers (L1): 16.7 M rows of four (268 MB) take 89 us,
+// where the checking level took 135.
+template <int kMode>
+__global__ void __launch_bounds__(256, 8) k_leaf_expand(
+    GraphDev g, const __grid_constant__ LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
+    const int32_t *__restrict__ pstart, const int2 *__restrict__ excl,
+    const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
+    int32_t W, RowSink sink) {
+  extern __shared__ int32_t smem[];
+  const int32_t B = blockDim.x;
+  const int32_t tile_items = B * kItemsPerThread;
+  int32_t *s_woff = smem;                  // tile_items + 4
+  int32_t *s_row = s_woff + tile_items + 4;  // row - r0 of every output of the tile
+  const int32_t tile = blockIdx.x;
+  const int32_t x0 = tile * tile_items, n = min(tile_items, W - x0);
+  const TileRows t = stage_rows(woff, tile_row, wa, tile_items, s_woff, tile);
+  const int32_t first = threadIdx.x * kItemsPerThread;
+  if (first < n) {
+    int32_t rs;
+    int32_t rr = item_row(t, s_woff, woff, wa, x0 + first, &rs) - t.r0;
+#pragma unroll
+    for (int j = 0; j < kItemsPerThread; ++j) {
+      if (first + j >= n) break;
+      while (x0 + first + j >=
+             (t.staged ? s_woff[rr + 1] : (int32_t)(woff[t.r0 + rr + 1] - wa)))
+        ++rr;
+      s_row[first + j] = rr;
+    }
+  }
+  __syncthreads();
+  const int32_t i = d.i, k = sink.k;
+  for (int32_t x = threadIdx.x; x < n; x += B) {
+    const int32_t rr = s_row[x], r = t.r0 + rr;
+    int32_t at = x0 + x - (t.staged ? s_woff[rr] : (int32_t)(woff[r] - wa));
+    if (d.ninj > 0) {
+      const int2 out = excl[r];
+      at += at >= out.x;
+      at += at >= out.y;
+    }
+    if (!GSM_IN_BOUNDS(g.dbg, pstart[r] + at >= 0 && pstart[r] + at < g.nnz, kDbgCandidate) ||
+        !GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
+      continue;
+    const int32_t w = __ldg(g.lcol + pstart[r] + at);
+    const int64_t to = sink.row0 + x0 + x;
+    if (kMode == kSinkRows && (k & 1) == 0) {
+      // (rows are only written directly in the matching order)
+      int32_t *dst = (int32_t *)sink.out + to * k;
+      auto col = [&](int c) { return c < i ? F[c * ld + r] : w; };
+      if ((k & 3) == 0) {
+        for (int c = 0; c < k; c += 4)
+          *reinterpret_cast<int4 *>(dst + c) = make_int4(col(c), col(c + 1), col(c + 2),
+                                                         col(c + 3));
+      } else {
+        for (int c = 0; c < k; c += 2)
+          *reinterpret_cast<int2 *>(dst + c) = make_int2(col(c), col(c + 1));
+      }
+    } else {
+      put_row<kMode>(sink, d, ColumnRow{F, ld, r}, w, to);
     }
   }
 }
@@ -1389,11 +1486,11 @@ void launch_pivot_scan(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
                        int64_t R, int32_t *pstart, uint8_t *pslot, int64_t *woff,
                        unsigned long long *lookback, int32_t spin_limit, Stage stage,
                        const LevelSetup &setup, int32_t stall_tile, cudaStream_t s,
-                       const int64_t *R_dev) {
+                       const int64_t *R_dev, int2 *excl) {
   const int64_t ptiles = pivot_scan_words(R) - kLbExtra;
   const int grid = (int)std::min<int64_t>(ptiles, 152 * 4);  // the CTAs resident at once
   k_pivot_scan<<<grid, kPsThreads, 0, s>>>(g, d, F, ld, R, (int32_t)ptiles, pstart, pslot, woff,
-                                           R_dev, lookback, spin_limit, stage, setup, stall_tile);
+                                           R_dev, lookback, spin_limit, stage, setup, stall_tile, excl);
 }
 
 int64_t extend_tiles(int64_t wa, int64_t wb, int32_t block) {
@@ -1595,6 +1692,25 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
     go(false_type{}, false_type{}, any);
   else
     go(false_type{}, true_type{}, any);
+}
+
+void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
+                        const int32_t *pstart, const int2 *excl, const int64_t *woff,
+                        const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
+                        const RowSink &sink, cudaStream_t s) {
+  const int64_t tiles = extend_tiles(wa, wb, block);
+  if (tiles <= 0) return;
+  const size_t smem = sizeof(int32_t) * (2 * (size_t)block * kItemsPerThread + 4);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)tiles, block, smem, s>>>(g, d, F, (int32_t)ld, pstart, excl, woff, tile_row,
+                                                wa, (int32_t)(wb - wa), sink);
+  };
+  if (sink.mode == kSinkRows)
+    go(k_leaf_expand<kSinkRows>);
+  else if (sink.mode == kSinkKeys)
+    go(k_leaf_expand<kSinkKeys>);
+  else
+    go(k_leaf_expand<kSinkColumns>);
 }
 
 void launch_split_points(const int64_t *woff, int64_t R, int64_t step, int64_t J,

@@ -60,6 +60,13 @@ struct LevelDesc {
   uint32_t la_pos[kMaxK], la_uq[kMaxK];
   const uint32_t *cand;
   int32_t n_words;
+  // 1: pi_i is a query leaf with at most kLeafExcl same-label, non-adjacent
+  // positions, so that all entries of its parent's cut label segment extend
+  // the row but those that are images of such positions.  The pivot scan then
+  // counts exactly (work = entries left) and notes where in the segment the
+  // left-out entries stand; the level itself (launch_leaf_expand) checks
+  // nothing and needs no compaction.
+  int32_t leaf;
   // 1 (GSM_OPT_COUNT_PROBES): the single-pass level adds the algorithmic
   // bytes of its non-tree edge checks, 4 * ceil(log2 deg) per check made
   // (the binary-search probes of the byte model), to lookback word tiles + 3
@@ -254,6 +261,10 @@ void launch_bitmap_to_list(const uint32_t *bitmap, int32_t n_words, int32_t *cnt
 // probe bytes: the words a single-pass level leaves after its total.
 int64_t pivot_scan_words(int64_t R);
 
+// Leaf levels (LevelDesc::leaf): excl[r] = the offsets in row r's segment of
+// the entries left out, ascending (INT32_MAX: none), for rows [0, R).
+constexpr int32_t kLeafExcl = 2;
+
 // What a level launched in one piece needs besides its offsets, prepared by
 // its pivot scan when its tiles number at most cap: tile_row (cap + 1
 // entries, as launch_tile_rows writes them) and, zeroed at lb, its look-back
@@ -271,7 +282,7 @@ void launch_pivot_scan(const GraphDev &g, const LevelDesc &d, const int32_t *F, 
                        int64_t R, int32_t *pstart, uint8_t *pslot, int64_t *woff,
                        unsigned long long *lookback, int32_t spin_limit, Stage stage,
                        const LevelSetup &setup, int32_t stall_tile, cudaStream_t s,
-                       const int64_t *R_dev = nullptr);
+                       const int64_t *R_dev = nullptr, int2 *excl = nullptr);
 
 // Number of extend tiles for candidates [wa, wb).
 int64_t extend_tiles(int64_t wa, int64_t wb, int32_t block);
@@ -398,6 +409,14 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
                          const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
                          int64_t rows, unsigned long long *lookback, const RowSink &sink,
                          int32_t spin_limit, int32_t stall_tile, Stage stage, cudaStream_t s);
+
+// A leaf level (LevelDesc::leaf) over output rows [wa, wb): output row x comes
+// from the row whose work offsets hold it and goes to sink row sink.row0 + x -
+// wa.  tile_row: as for the other levels.
+void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
+                        const int32_t *pstart, const int2 *excl, const int64_t *woff,
+                        const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
+                        const RowSink &sink, cudaStream_t s);
 
 // Row boundaries for work-bounded sub-chunks: bounds[j] = the row r with
 // woff[r] <= j*step < woff[r+1] (clamped to [0, R]); bounds[J] = R.
