@@ -764,6 +764,13 @@ struct Run {
   // 0..rank_p-1, placed first in that order) when rank_p > 0: ranks of the
   // rows of the last level's input piece in `rank`, running state in prefix
   int32_t rank_p = 0, rank_pos = 0;
+  // direct: the final rows so far stand in `out`, the caller's device buffer of
+  // out_cap rows (listings whose rows nothing reads from library buffers
+  // afterwards): the last level or the sort's last pass writes there, with no
+  // copy of the result
+  bool direct = false;
+  int32_t *out = nullptr;
+  uint64_t out_cap = 0;
   // leaf levels: the left-out entries of the rows of the level being processed
   const int2 *excl[kMaxK] = {};
   PrefixState *prefix = nullptr;
@@ -822,6 +829,21 @@ void ensure_acc(Run &R, uint64_t rows) {
   R.acc_ld = ld;
 }
 
+// The result does not go straight to the caller's buffer after all: brings the
+// rows written there so far into the accumulator.
+void rows_to_acc(Run &R) {
+  if (!R.direct) return;
+  gsm_ctx *ctx = R.ctx;
+  R.direct = false;
+  const uint64_t done = R.acc_rows;
+  R.acc_rows = 0;
+  ensure_acc(R, done);
+  R.acc_rows = done;
+  if (done)
+    CU(cudaMemcpyAsync(ctx->acc[0], R.out, done * R.acc_row_bytes(), cudaMemcpyDeviceToDevice,
+                       ctx->stream));
+}
+
 // Room for a leaf level's left-out entries, `rows` of them at most (null if the
 // level is not a leaf's, or its rows have none).
 int2 *push_excl(Run &R, int32_t i, int64_t rows) {
@@ -874,9 +896,10 @@ void process_leaf(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t
   RowSink sink;
   int32_t *Fn = nullptr;
   if (last) {
-    ensure_acc(R, R.acc_rows + (uint64_t)W);
+    if (R.direct && R.acc_rows + (uint64_t)W > R.out_cap) rows_to_acc(R);
+    if (!R.direct) ensure_acc(R, R.acc_rows + (uint64_t)W);
     sink = RowSink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
-                   ctx->acc[0]};
+                   R.direct ? R.out : ctx->acc[0]};
     sink.rank = R.rank;
     sink.rank_pos = R.rank_pos;
   } else {
@@ -967,6 +990,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   const int64_t S = read_i64(ctx, tile_off + tiles);
   if (S == 0) return;
   if (last) {
+    rows_to_acc(R);
     ensure_acc(R, R.acc_rows + (uint64_t)S);
     RowSink sink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
                  ctx->acc[0]};
@@ -1040,6 +1064,7 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   RowSink sink;
   int32_t *Fn = nullptr;
   if (last) {
+    rows_to_acc(R);
     ensure_acc(R, R.acc_rows + (uint64_t)W);
     sink = RowSink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
                    ctx->acc[0]};
@@ -1569,7 +1594,8 @@ bool counts_by_rank(const gsm_ctx *ctx, const gsm_query *q) {
 }
 
 // The whole matcher for one query.  out == nullptr and !enumerate: count only;
-// distinct_of = |Aut(Q)| divides the count (distinct subgraphs).
+// distinct_of = |Aut(Q)| divides the count (distinct subgraphs).  keep_rows =
+// false: gsm_last_rows will not be asked for these rows.
 // pre (optional): the query's candidate bitmaps and sizes, already computed
 // by a batched filter launch (gsm_enumerate_many).
 struct Prefiltered {
@@ -1580,7 +1606,7 @@ struct Prefiltered {
 void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, uint64_t cap_rows,
                int32_t flags, uint64_t *count_out, bool *truncated,
                bool copy_async = false, const Prefiltered *pre = nullptr,
-               uint64_t distinct_of = 1) {
+               uint64_t distinct_of = 1, bool keep_rows = true) {
   if (!ctx->has_graph) FAIL(GSM_ERR_NO_GRAPH, "no data graph loaded");
   const Range range(enumerate ? "gsm query (list)" : "gsm query (count)");
   std::memset(&ctx->run, 0, sizeof(ctx->run));
@@ -1661,6 +1687,13 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   R.acc_mode = sort_cols == 0 ? kSinkRows : kSinkKeys;
   R.key_bits = key_bits;
   R.key_nw = packed_words(q->k, key_bits);
+  // straight into the caller's buffer, if it takes the kernels' widest store
+  const bool to_out = enumerate && !keep_rows && (flags & GSM_OUT_DEVICE) && q->k > 1 &&
+                      ((uintptr_t)out & 15) == 0 &&
+                      !(ctx->opt.flags & GSM_OPT_COMPRESSED_FRONTIERS);
+  R.out = out;
+  R.out_cap = cap_rows;
+  R.direct = to_out && R.acc_mode == kSinkRows;
   // rows leave the levels sorted by the columns of query vertices 0..p-1 when
   // the matching order starts with them; the last level then writes their
   // dense rank into the keys' spare bits (any int32 fits), so that the sort
@@ -1804,12 +1837,15 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   // order), or their packed keys are sorted on columns 0 .. sort_cols-1 and
   // unpacked row-major into acc[1]
   int32_t *rows = (int32_t *)ctx->acc[0];
+  bool placed = R.direct;  // the rows are in `out`
   if (R.acc_mode == kSinkKeys && total > 0) {
     const int32_t nw = R.key_nw;
     const size_t bytes = (size_t)total * q->k * sizeof(int32_t);
     const size_t key_bytes = (size_t)R.acc_ld * nw * sizeof(uint64_t);
     ensure_buf(ctx, &ctx->sort_keys, &ctx->sort_keys_cap, key_bytes, false, 0);
-    ensure_buf(ctx, &ctx->acc[1], &ctx->acc_cap[1], bytes, false, 0);
+    placed = to_out && total <= cap_rows;
+    if (!placed) ensure_buf(ctx, &ctx->acc[1], &ctx->acc_cap[1], bytes, false, 0);
+    rows = placed ? out : (int32_t *)ctx->acc[1];
     // the rows leave the levels sorted by the columns the matching order
     // places first in id order (0, 1, ..., p-1), with at most |F_p|
     // distinct prefixes
@@ -1833,16 +1869,16 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     timed(ctx, K_SORT, moved + (double)bytes, total, 0, [&] {
       launches = launch_sort_rows_packed(nullptr, 0, (int64_t)total, q->k, R.key_bits, sort_cols,
                                          (uint64_t *)ctx->acc[0], (uint64_t *)ctx->sort_keys,
-                                         R.acc_ld, (int32_t *)ctx->acc[1], ctx->sort_tmp,
-                                         R.spin_limit, ctx->d_flags, sort_stall_tile(ctx),
-                                         ctx->stream, pre);
+                                         R.acc_ld, rows, ctx->sort_tmp, R.spin_limit,
+                                         ctx->d_flags, sort_stall_tile(ctx), ctx->stream, pre);
     });
     ctx->run.kernel_launches += launches;
-    rows = (int32_t *)ctx->acc[1];
   }
-  ctx->last_rows = rows;
-  ctx->last_count = total;
-  const uint64_t ncopy = std::min<uint64_t>(total, cap_rows);
+  if (keep_rows) {
+    ctx->last_rows = rows;
+    ctx->last_count = total;
+  }
+  const uint64_t ncopy = placed ? 0 : std::min<uint64_t>(total, cap_rows);
   const cudaMemcpyKind kind =
       (flags & GSM_OUT_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   if (copy_async) {
@@ -3573,8 +3609,9 @@ void list_many(gsm_ctx *ctx, ManyState &M, uint64_t *launches, uint64_t *peak, b
     next_result_slot(c, slots);
     bool trunc = false;
     const Prefiltered *p = (M.pre && (*M.pre)[j].bitmaps) ? &(*M.pre)[j] : nullptr;
+    // (only the call's last result is kept for gsm_last_rows)
     run_query(c, M.queries[j], true, M.outs[j], M.cap_rows[j], M.flags, &M.counts[j], &trunc,
-              true, p);
+              true, p, 1, j == M.nq - 1);
     *launches += c->run.kernel_launches;
     *peak = std::max<uint64_t>(*peak, c->peak_bytes);
     if (trunc) {
