@@ -418,15 +418,22 @@ void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F,
                         const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
                         const RowSink &sink, cudaStream_t s);
 
+// The last level of a clique counted on the renumbered graph (d.nb = 2 or 3
+// mapped neighbours, all other vertices of the row): adds the number of
+// candidates of rows [ra, rb) that are neighbours of all of them into *total.
+void launch_clique_count(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
+                         const int32_t *pstart, const uint8_t *pslot, const int64_t *woff,
+                         int64_t ra, int64_t rb, unsigned long long *total, cudaStream_t s);
+
 // Row boundaries for work-bounded sub-chunks: bounds[j] = the row r with
 // woff[r] <= j*step < woff[r+1] (clamped to [0, R]); bounds[J] = R.
 void launch_split_points(const int64_t *woff, int64_t R, int64_t step, int64_t J,
                          int64_t *bounds, int64_t *bound_w, cudaStream_t s);
 
-// Copies `bytes` (a multiple of 4, at most 4096) from src to dst with one
-// small kernel; dst is typically the device view of mapped pinned host memory,
-// so small reads back to the host do not queue behind copy-engine transfers.
-void launch_fetch(const void *src, void *dst, size_t bytes, cudaStream_t s);
+// Copies `bytes` (a multiple of 4, at most 8 * kStageSeq) from src to the stage
+// with one small kernel, so that small reads back to the host do not queue
+// behind copy-engine transfers.
+void launch_fetch(const void *src, size_t bytes, Stage stage, cudaStream_t s);
 
 // Sorting many small results at once (one CTA each): rows src (count x k,
 // row-major) into canonical lexicographic order at dst (count x k); sort = 0
