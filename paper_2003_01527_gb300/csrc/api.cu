@@ -769,6 +769,10 @@ struct Run {
   // afterwards): the last level or the sort's last pass writes there, with no
   // copy of the result
   bool direct = false;
+  // twin: the final rows so far stand in the accumulator and in `out` (the
+  // rows of gsm_enumerate, which gsm_last_rows may be asked for): written
+  // twice by the kernel that makes them instead of copied
+  bool twin = false;
   int32_t *out = nullptr;
   uint64_t out_cap = 0;
   // leaf levels: the left-out entries of the rows of the level being processed
@@ -902,6 +906,7 @@ void process_leaf(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t
   int32_t *Fn = nullptr;
   if (last) {
     if (R.direct && R.acc_rows + (uint64_t)W > R.out_cap) rows_to_acc(R);
+    if (R.acc_rows + (uint64_t)W > R.out_cap) R.twin = false;
     if (!R.direct) ensure_acc(R, R.acc_rows + (uint64_t)W);
     sink = RowSink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
                    R.direct ? R.out : ctx->acc[0]};
@@ -915,7 +920,7 @@ void process_leaf(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t
   timed(ctx, K_FUSED, (double)nrows * (4.0 * i + 12.0) + 4.0 * (double)W + out_bytes, (uint64_t)W,
         1, [&] {
     launch_leaf_expand(R.g, d, F, ld, pstart, R.excl[i], woff, tile_row, wa, wb, R.block, sink,
-                       ctx->stream);
+                       last && R.twin ? R.out : nullptr, ctx->stream);
   });
   if (last) {
     R.acc_rows += (uint64_t)W;
@@ -1004,6 +1009,7 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   if (S == 0) return;
   if (last) {
     rows_to_acc(R);
+    R.twin = false;
     ensure_acc(R, R.acc_rows + (uint64_t)S);
     RowSink sink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
                  ctx->acc[0]};
@@ -1078,6 +1084,7 @@ void process_fused(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_
   int32_t *Fn = nullptr;
   if (last) {
     rows_to_acc(R);
+    R.twin = false;  // (a level that waits may fail: nothing reaches the caller before)
     ensure_acc(R, R.acc_rows + (uint64_t)W);
     sink = RowSink{R.acc_mode, R.k, R.key_bits, R.key_nw, R.acc_ld, (int64_t)R.acc_rows,
                    ctx->acc[0]};
@@ -1702,12 +1709,14 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   R.key_bits = key_bits;
   R.key_nw = packed_words(q->k, key_bits);
   // straight into the caller's buffer, if it takes the kernels' widest store
-  const bool to_out = enumerate && !keep_rows && (flags & GSM_OUT_DEVICE) && q->k > 1 &&
-                      ((uintptr_t)out & 15) == 0 &&
-                      !(ctx->opt.flags & GSM_OPT_COMPRESSED_FRONTIERS);
+  const bool wide = enumerate && (flags & GSM_OUT_DEVICE) && q->k > 1 && cap_rows > 0 &&
+                    ((uintptr_t)out & 15) == 0 &&
+                    !(ctx->opt.flags & GSM_OPT_COMPRESSED_FRONTIERS);
+  const bool to_out = wide && !keep_rows;
   R.out = out;
   R.out_cap = cap_rows;
   R.direct = to_out && R.acc_mode == kSinkRows;
+  R.twin = wide && keep_rows && R.acc_mode == kSinkRows;
   // rows leave the levels sorted by the columns of query vertices 0..p-1 when
   // the matching order starts with them; the last level then writes their
   // dense rank into the keys' spare bits (any int32 fits), so that the sort
@@ -1851,15 +1860,16 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   // order), or their packed keys are sorted on columns 0 .. sort_cols-1 and
   // unpacked row-major into acc[1]
   int32_t *rows = (int32_t *)ctx->acc[0];
-  bool placed = R.direct;  // the rows are in `out`
+  bool placed = R.direct || R.twin;  // the rows are in `out`
   if (R.acc_mode == kSinkKeys && total > 0) {
     const int32_t nw = R.key_nw;
     const size_t bytes = (size_t)total * q->k * sizeof(int32_t);
     const size_t key_bytes = (size_t)R.acc_ld * nw * sizeof(uint64_t);
     ensure_buf(ctx, &ctx->sort_keys, &ctx->sort_keys_cap, key_bytes, false, 0);
-    placed = to_out && total <= cap_rows;
-    if (!placed) ensure_buf(ctx, &ctx->acc[1], &ctx->acc_cap[1], bytes, false, 0);
-    rows = placed ? out : (int32_t *)ctx->acc[1];
+    placed = wide && total <= cap_rows;
+    const bool only_out = placed && !keep_rows;
+    if (!only_out) ensure_buf(ctx, &ctx->acc[1], &ctx->acc_cap[1], bytes, false, 0);
+    rows = only_out ? out : (int32_t *)ctx->acc[1];
     // the rows leave the levels sorted by the columns the matching order
     // places first in id order (0, 1, ..., p-1), with at most |F_p|
     // distinct prefixes
@@ -1884,7 +1894,8 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
       launches = launch_sort_rows_packed(nullptr, 0, (int64_t)total, q->k, R.key_bits, sort_cols,
                                          (uint64_t *)ctx->acc[0], (uint64_t *)ctx->sort_keys,
                                          R.acc_ld, rows, ctx->sort_tmp, R.spin_limit,
-                                         ctx->d_flags, sort_stall_tile(ctx), ctx->stream, pre);
+                                         ctx->d_flags, sort_stall_tile(ctx), ctx->stream, pre,
+                                         placed && !only_out ? out : nullptr);
     });
     ctx->run.kernel_launches += launches;
   }

@@ -986,7 +986,7 @@ __global__ void __launch_bounds__(256, 8) k_leaf_expand(
     GraphDev g, const __grid_constant__ LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const int2 *__restrict__ excl,
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t wa,
-    int32_t W, RowSink sink) {
+    int32_t W, RowSink sink, int32_t *__restrict__ copy) {
   extern __shared__ int32_t smem[];
   const int32_t B = blockDim.x;
   const int32_t tile_items = B * kItemsPerThread;
@@ -1025,18 +1025,28 @@ __global__ void __launch_bounds__(256, 8) k_leaf_expand(
     const int64_t to = sink.row0 + x0 + x;
     if (kMode == kSinkRows && (k & 1) == 0) {
       // (rows are only written directly in the matching order)
-      int32_t *dst = (int32_t *)sink.out + to * k;
+      int32_t *dst = (int32_t *)sink.out + to * k, *dst2 = copy + to * k;
       auto col = [&](int c) { return c < i ? F[c * ld + r] : w; };
       if ((k & 3) == 0) {
-        for (int c = 0; c < k; c += 4)
-          *reinterpret_cast<int4 *>(dst + c) = make_int4(col(c), col(c + 1), col(c + 2),
-                                                         col(c + 3));
+        for (int c = 0; c < k; c += 4) {
+          const int4 v = make_int4(col(c), col(c + 1), col(c + 2), col(c + 3));
+          *reinterpret_cast<int4 *>(dst + c) = v;
+          if (copy) *reinterpret_cast<int4 *>(dst2 + c) = v;
+        }
       } else {
-        for (int c = 0; c < k; c += 2)
-          *reinterpret_cast<int2 *>(dst + c) = make_int2(col(c), col(c + 1));
+        for (int c = 0; c < k; c += 2) {
+          const int2 v = make_int2(col(c), col(c + 1));
+          *reinterpret_cast<int2 *>(dst + c) = v;
+          if (copy) *reinterpret_cast<int2 *>(dst2 + c) = v;
+        }
       }
     } else {
       put_row<kMode>(sink, d, ColumnRow{F, ld, r}, w, to);
+      if (kMode == kSinkRows && copy) {
+        RowSink second = sink;
+        second.out = copy;
+        put_row<kMode>(second, d, ColumnRow{F, ld, r}, w, to);
+      }
     }
   }
 }
@@ -1790,13 +1800,13 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
 void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                         const int32_t *pstart, const int2 *excl, const int64_t *woff,
                         const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                        const RowSink &sink, cudaStream_t s) {
+                        const RowSink &sink, int32_t *copy, cudaStream_t s) {
   const int64_t tiles = extend_tiles(wa, wb, block);
   if (tiles <= 0) return;
   const size_t smem = sizeof(int32_t) * (2 * (size_t)block * kItemsPerThread + 4);
   auto go = [&](auto kernel) {
     kernel<<<(unsigned)tiles, block, smem, s>>>(g, d, F, (int32_t)ld, pstart, excl, woff, tile_row,
-                                                wa, (int32_t)(wb - wa), sink);
+                                                wa, (int32_t)(wb - wa), sink, copy);
   };
   if (sink.mode == kSinkRows)
     go(k_leaf_expand<kSinkRows>);

@@ -412,11 +412,12 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
 
 // A leaf level (LevelDesc::leaf) over output rows [wa, wb): output row x comes
 // from the row whose work offsets hold it and goes to sink row sink.row0 + x -
-// wa.  tile_row: as for the other levels.
+// wa.  tile_row: as for the other levels.  copy (kSinkRows only, may be null):
+// a second buffer that takes the same rows.
 void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
                         const int32_t *pstart, const int2 *excl, const int64_t *woff,
                         const int32_t *tile_row, int64_t wa, int64_t wb, int32_t block,
-                        const RowSink &sink, cudaStream_t s);
+                        const RowSink &sink, int32_t *copy, cudaStream_t s);
 
 // The last level of a clique counted on the renumbered graph (d.nb = 2 or 3
 // mapped neighbours, all other vertices of the row): adds the number of
@@ -471,8 +472,9 @@ void launch_sort_small(const SmallSortItem *items, int32_t nitems, int32_t max_k
 // and leaves the rows out of order, every write still inside `out`; a failed
 // bounds check of the GSM_DEBUG build writes its site to err[1].
 // stall_tile >= 0 (fault injection for tests): that tile of every
-// single-sweep pass never publishes its counts.  Returns the number of
-// kernels launched.
+// single-sweep pass never publishes its counts.  copy (may be null): a second
+// buffer that takes the same rows as `out`.  Returns the number of kernels
+// launched.
 // Optional knowledge of the input order: the rows already stand sorted by
 // their first `cols` columns (1 <= cols < sort_cols), with at most `groups`
 // distinct prefixes.  The sort then orders those columns by the prefix's
@@ -520,6 +522,7 @@ int32_t sort_digit_passes(int64_t N, int32_t k, int32_t bits, int32_t sort_cols,
 int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k, int32_t bits,
                             int32_t sort_cols, uint64_t *keys_a, uint64_t *keys_b, int64_t ld,
                             int32_t *out, void *scratch, int32_t spin_limit, uint32_t *err,
-                            int32_t stall_tile, cudaStream_t s, SortPrefix pre = SortPrefix());
+                            int32_t stall_tile, cudaStream_t s, SortPrefix pre = SortPrefix(),
+                            int32_t *copy = nullptr);
 
 }  // namespace gsm

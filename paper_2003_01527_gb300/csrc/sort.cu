@@ -97,8 +97,8 @@ __global__ void __launch_bounds__(kSortThreads) k_hist_keys(const uint64_t *__re
 template <bool kUnpack>
 __global__ void __launch_bounds__(kSortThreads) k_scatter_keys(
     const uint64_t *__restrict__ in, uint64_t *__restrict__ out_keys,
-    int32_t *__restrict__ out_rows, int64_t ld, int64_t N, int32_t nw, int32_t k, int32_t b,
-    int32_t p, const int64_t *__restrict__ hist_off, int64_t nblocks) {
+    int32_t *__restrict__ out_rows, int32_t *__restrict__ copy, int64_t ld, int64_t N, int32_t nw,
+    int32_t k, int32_t b, int32_t p, const int64_t *__restrict__ hist_off, int64_t nblocks) {
   __shared__ int64_t s_base[kBins];
   __shared__ int32_t s_wcnt[kSortThreads / 32][kBins + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(kSortThreads) k_scatter_keys(
             if (i == wi + 1 && sh + b > 64) v |= wv[i] << (64 - sh);
           }
           dst[j] = (int32_t)(v & mask_b);
+          if (copy) copy[pos * k + j] = (int32_t)(v & mask_b);
         }
       } else {
         for (int32_t i = 0; i < nw; ++i) out_keys[(int64_t)i * ld + pos] = in[(int64_t)i * ld + idx];
@@ -316,8 +317,8 @@ __host__ __device__ constexpr int sweep_threads() {
 template <int NW, bool kUnpack>
 __global__ void __launch_bounds__(sweep_threads<NW>(), NW == 1 ? 2 : 3) k_onesweep(
     const uint64_t *__restrict__ in, uint64_t *__restrict__ out_keys,
-    int32_t *__restrict__ out_rows, int64_t ld, int64_t N, int32_t k, int32_t b, int32_t p,
-    const uint32_t *__restrict__ gexcl, uint32_t *status, uint32_t *ticket, int32_t spin_limit,
+    int32_t *__restrict__ out_rows, int32_t *__restrict__ copy, int64_t ld, int64_t N, int32_t k,
+    int32_t b, int32_t p, const uint32_t *__restrict__ gexcl, uint32_t *status, uint32_t *ticket, int32_t spin_limit,
     uint32_t *err, int64_t stall_tile) {
   constexpr int kT = sweep_threads<NW>();
   constexpr int kTile = kT * kSortChunks;
@@ -440,11 +441,16 @@ __global__ void __launch_bounds__(sweep_threads<NW>(), NW == 1 ? 2 : 3) k_oneswe
     if (kUnpack) {
       int32_t *dst = out_rows + pos * k;
       if ((k & 1) == 0) {
-        for (int32_t j = 0; j < k; j += 2)
-          *reinterpret_cast<int2 *>(dst + j) =
-              make_int2(key_column<NW>(kk, k, b, j), key_column<NW>(kk, k, b, j + 1));
+        for (int32_t j = 0; j < k; j += 2) {
+          const int2 v = make_int2(key_column<NW>(kk, k, b, j), key_column<NW>(kk, k, b, j + 1));
+          *reinterpret_cast<int2 *>(dst + j) = v;
+          if (copy) *reinterpret_cast<int2 *>(copy + pos * k + j) = v;
+        }
       } else {
-        for (int32_t j = 0; j < k; ++j) dst[j] = key_column<NW>(kk, k, b, j);
+        for (int32_t j = 0; j < k; ++j) {
+          dst[j] = key_column<NW>(kk, k, b, j);
+          if (copy) copy[pos * k + j] = dst[j];
+        }
       }
     } else {
 #pragma unroll
@@ -461,7 +467,8 @@ __global__ void __launch_bounds__(sweep_threads<NW>(), NW == 1 ? 2 : 3) k_oneswe
 __global__ void __launch_bounds__(512) k_sort_few_keys(const uint64_t *__restrict__ keys,
                                                        int64_t ld, int32_t N, int32_t nw,
                                                        int32_t k, int32_t b,
-                                                       int32_t *__restrict__ out) {
+                                                       int32_t *__restrict__ out,
+                                                       int32_t *__restrict__ copy) {
   extern __shared__ __align__(16) uint64_t s_keys[];  // word w of key i at w*N + i
   __shared__ int16_t s_idx[kSmallSortRows];
   int32_t P = 1;
@@ -500,6 +507,7 @@ __global__ void __launch_bounds__(512) k_sort_few_keys(const uint64_t *__restric
     uint64_t v = s_keys[w * N + x] >> sh;
     if (sh + b > 64) v |= s_keys[(w + 1) * N + x] << (64 - sh);
     out[e] = (int32_t)(v & mask);
+    if (copy) copy[e] = (int32_t)(v & mask);
   }
 }
 
@@ -763,7 +771,7 @@ int sm_count() {
 }
 
 template <int NW>
-void sweep_pass(bool last, const uint64_t *src, uint64_t *dst, int32_t *out, int64_t ld,
+void sweep_pass(bool last, const uint64_t *src, uint64_t *dst, int32_t *out, int32_t *copy, int64_t ld,
                 int64_t N, int32_t k, int32_t bits, int32_t p, const uint32_t *gexcl,
                 uint32_t *status, uint32_t *ticket, int32_t spin_limit, uint32_t *err,
                 int64_t stall_tile, int64_t tiles, cudaStream_t s) {
@@ -783,10 +791,10 @@ void sweep_pass(bool last, const uint64_t *src, uint64_t *dst, int32_t *out, int
   }
   if (last)
     k_onesweep<NW, true><<<(unsigned)tiles, kT, kDyn, s>>>(
-        src, dst, out, ld, N, k, bits, p, gexcl, status, ticket, spin_limit, err, stall_tile);
+        src, dst, out, copy, ld, N, k, bits, p, gexcl, status, ticket, spin_limit, err, stall_tile);
   else
     k_onesweep<NW, false><<<(unsigned)tiles, kT, kDyn, s>>>(
-        src, dst, out, ld, N, k, bits, p, gexcl, status, ticket, spin_limit, err, stall_tile);
+        src, dst, out, copy, ld, N, k, bits, p, gexcl, status, ticket, spin_limit, err, stall_tile);
 }
 
 }  // namespace
@@ -806,7 +814,7 @@ int32_t sort_digit_passes(int64_t N, int32_t k, int32_t bits, int32_t sort_cols,
 int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k, int32_t bits,
                             int32_t sort_cols, uint64_t *keys_a, uint64_t *keys_b, int64_t ld,
                             int32_t *out, void *scratch, int32_t spin_limit, uint32_t *err,
-                            int32_t stall_tile, cudaStream_t s, SortPrefix pre) {
+                            int32_t stall_tile, cudaStream_t s, SortPrefix pre, int32_t *copy) {
   if (N <= 0) return 0;
   int launches = 0;
   const SortLayout L = sort_layout(N, k, bits, sort_cols, pre);
@@ -826,7 +834,7 @@ int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k,
       attr_set.fetch_or(1ull << (dev & 63));
     }
     k_sort_few_keys<<<1, 512, sizeof(uint64_t) * (size_t)nw * N, s>>>(keys_a, ld, (int32_t)N, nw,
-                                                                       k, bits, out);
+                                                                       k, bits, out, copy);
     return launches + 1;
   }
   char *sc = (char *)scratch;
@@ -876,10 +884,10 @@ int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k,
       const bool last = dg == L.digits - 1;
       uint32_t *st = status + (size_t)dg * (size_t)L.tiles * kBins;
       if (nw == 1)
-        sweep_pass<1>(last, src, dst, out, ld, N, k, bits, p, gexcl + dg * kBins, st, ticket + dg,
+        sweep_pass<1>(last, src, dst, out, copy, ld, N, k, bits, p, gexcl + dg * kBins, st, ticket + dg,
                       spin_limit, err, stall_tile, L.tiles, s);
       else
-        sweep_pass<2>(last, src, dst, out, ld, N, k, bits, p, gexcl + dg * kBins, st, ticket + dg,
+        sweep_pass<2>(last, src, dst, out, copy, ld, N, k, bits, p, gexcl + dg * kBins, st, ticket + dg,
                       spin_limit, err, stall_tile, L.tiles, s);
       ++launches;
       std::swap(src, dst);
@@ -897,11 +905,11 @@ int launch_sort_rows_packed(const int32_t *a, int64_t lda, int64_t N, int32_t k,
     launch_scan_i32(hist, hist_off, nb * kBins, tmp, s);
     const bool last = dg == L.digits - 1;
     if (last)
-      k_scatter_keys<true><<<(unsigned)nb, kSortThreads, 0, s>>>(src, dst, out, ld, N, nw, k,
-                                                                 bits, p, hist_off, nb);
+      k_scatter_keys<true><<<(unsigned)nb, kSortThreads, 0, s>>>(src, dst, out, copy, ld, N, nw,
+                                                                 k, bits, p, hist_off, nb);
     else
-      k_scatter_keys<false><<<(unsigned)nb, kSortThreads, 0, s>>>(src, dst, out, ld, N, nw, k,
-                                                                  bits, p, hist_off, nb);
+      k_scatter_keys<false><<<(unsigned)nb, kSortThreads, 0, s>>>(src, dst, out, copy, ld, N, nw,
+                                                                  k, bits, p, hist_off, nb);
     launches += 5;
     std::swap(src, dst);
   }
