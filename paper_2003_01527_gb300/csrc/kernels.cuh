@@ -107,6 +107,7 @@ struct GraphDev {
   // (hub_bits points hub_lo / 32 words before the first), so a hub is asked
   // about vertices >= hub_lo alone
   int32_t hub_lo;
+  const int32_t *up;  // ... and up[v] = where the neighbours above v start in v's row (else null)
   // GSM_DEBUG builds: the mapped word a failed bounds check writes its site
   // to (null: not reported)
   uint32_t *dbg;
@@ -171,7 +172,7 @@ void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int3
                          cudaStream_t s);
 
 // The rows of g renumbered (one-label graphs): new vertex i is order[i].
-// Writes rp2 (n + 1) and col2 (nnz), rows ascending.  order: device; nlong: how
+// Writes rp2 (n + 1), col2 (nnz), rows ascending, and up (n, GraphDev).  order: device; nlong: how
 // many vertices, the last ones of order, have degrees above kLongRowDegree.
 // rank and deg: n ints, offs: n + 1 and tmp: scan_tmp_elems(n) int64, keys: 2 *
 // nnz uint64, pairs: 2 * nnz ints, sort_scratch: sort_scratch_bytes(nnz, 2,
@@ -179,7 +180,7 @@ void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int3
 // launch_sort_rows_packed.
 void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int32_t *rank,
                      int32_t *deg, int64_t *offs, int64_t *tmp, uint64_t *keys, int32_t *pairs,
-                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2,
+                     void *sort_scratch, uint32_t *err, int32_t *rp2, int32_t *col2, int32_t *up,
                      cudaStream_t s);
 
 // The threshold and label bitmaps of GraphDev (thr: num_labels * kThrLevels,
