@@ -915,11 +915,17 @@ __global__ void __launch_bounds__(kMaxThreads,
     }
   };
 
+  // (thread 0) the ticket after the current tile's, taken while that one is
+  // verified.  Tiles are only waited for by later ones, and a CTA's waits are
+  // for tiles before the one it holds, so a held ticket cannot close a circle.
+  int32_t ahead = -1;
   for (int32_t turn = 0;; ++turn) {
-    if (threadIdx.x == 0) s_tile = single ? turn : (int32_t)atomicAdd(lookback + tiles, 1ull);
+    if (threadIdx.x == 0)
+      s_tile = single ? turn : ahead >= 0 ? ahead : (int32_t)atomicAdd(lookback + tiles, 1ull);
     __syncthreads();
     const int32_t tile = s_tile;
     if (tile >= tiles) break;  // uniform across the block
+    if (threadIdx.x == 0 && !single) ahead = (int32_t)atomicAdd(lookback + tiles, 1ull);
     const int32_t x0 = tile * tile_items;
     const int32_t x1 = min(x0 + tile_items, W);
     const TileRows t = stage_rows(woff, tile_row, wa, tile_items, s_woff, tile);

@@ -499,9 +499,9 @@ __device__ __forceinline__ uint32_t check_group(
     at[j] = pst + (x - rs);
   }
   if (g.hub_lo) few = 0;  // bitmaps that do not cover the mapped neighbours
-#pragma unroll
-  for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
   if constexpr (kCheck == kCheckAny) {
+#pragma unroll
+    for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
 #pragma unroll
     for (int j = 0; j < kN; ++j) {
       if (!((alive >> j) & 1u)) continue;
@@ -515,6 +515,25 @@ __device__ __forceinline__ uint32_t check_group(
     }
     return alive;
   }
+  // what depends on the row alone is loaded beside the candidates
+  int32_t x[kNb > 1 ? kNb - 1 : 1][kN], y[2][kN];
+#pragma unroll
+  for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
+#pragma unroll
+  for (int o = 0; o + 1 < kNb; ++o)
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      x[o][j] = (alive >> j) & 1u ? F[d.bpos[o + (o >= sj[j])] * ld + rj[j]] : 0;
+      if (!GSM_IN_BOUNDS(g.dbg, x[o][j] >= 0 && x[o][j] < g.n, kDbgNeighbour)) {
+        alive &= ~(1u << j);
+        x[o][j] = 0;
+      }
+    }
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int j = 0; j < kN; ++j)
+      y[t][j] = t < d.ninj && (alive >> j) & 1u ? F[d.inj[t] * ld + rj[j]] : -1;
   if (d.bitmap) {
     uint32_t word[kN];
 #pragma unroll
@@ -524,28 +543,12 @@ __device__ __forceinline__ uint32_t check_group(
     for (int j = 0; j < kN; ++j)
       if (!((word[j] >> (wj[j] & 31)) & 1u)) alive &= ~(1u << j);
   }
-  for (int i = 0; i < d.ninj; ++i) {
-    const int32_t *col = F + d.inj[i] * ld;
-    int32_t y[kN];
 #pragma unroll
-    for (int j = 0; j < kN; ++j) y[j] = (alive >> j) & 1u ? col[rj[j]] : -1;
+  for (int j = 0; j < kN; ++j)
+    if (y[0][j] == wj[j] || y[1][j] == wj[j]) alive &= ~(1u << j);
 #pragma unroll
-    for (int j = 0; j < kN; ++j)
-      if (y[j] == wj[j]) alive &= ~(1u << j);
-  }
-#pragma unroll
-  for (int o = 0; o + 1 < kNb; ++o) {  // neighbours besides the pivot
-    int32_t x[kN];
-#pragma unroll
-    for (int j = 0; j < kN; ++j) {
-      x[j] = (alive >> j) & 1u ? F[d.bpos[o + (o >= sj[j])] * ld + rj[j]] : 0;
-      if (!GSM_IN_BOUNDS(g.dbg, x[j] >= 0 && x[j] < g.n, kDbgNeighbour)) {
-        alive &= ~(1u << j);
-        x[j] = 0;
-      }
-    }
-    alive = group_contains(g, x, wj, [&](int) { return d.lab; }, alive, few);
-  }
+  for (int o = 0; o + 1 < kNb; ++o)  // neighbours besides the pivot
+    alive = group_contains(g, x[o], wj, [&](int) { return d.lab; }, alive, few);
   return alive;
 }
 
