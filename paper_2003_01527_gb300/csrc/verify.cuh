@@ -2,6 +2,8 @@
 // pass): tile row staging, the candidate check and the row writer.
 #pragma once
 
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "segments.cuh"
 
@@ -394,29 +396,38 @@ __device__ __forceinline__ uint32_t group_contains(const GraphDev &g,
     len[j] = end[j] - lo[j];
   }
   const bool one = g.num_labels == 1;
-  bool more = true;
-  while (more) {
-    more = false;
-    int32_t v[kN], m[kN];
+  auto search = [&](auto plain) {  // plain: one label, ids alone order a row
+    bool more = true;
+    while (more) {
+      more = false;
+      int32_t v[kN], m[kN];
 #pragma unroll
-    for (int j = 0; j < kN; ++j) {
-      const int32_t mid = lo[j] + (len[j] >> 1);
-      v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
-      m[j] = len[j] > 0 && !one ? __ldg(g.llab + mid) : lab[j];
-    }
-#pragma unroll
-    for (int j = 0; j < kN; ++j) {
-      if (len[j] <= 0) continue;
-      const int32_t half = len[j] >> 1;
-      if (m[j] < lab[j] || (m[j] == lab[j] && v[j] < key[j])) {
-        lo[j] += half + 1;
-        len[j] -= half + 1;
-      } else {
-        len[j] = half;
+      for (int j = 0; j < kN; ++j) {
+        const int32_t mid = lo[j] + (len[j] >> 1);
+        v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
+        if constexpr (!decltype(plain)::value) m[j] = len[j] > 0 ? __ldg(g.llab + mid) : lab[j];
       }
-      more = more || len[j] > 0;
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        if (len[j] <= 0) continue;
+        const int32_t half = len[j] >> 1;
+        bool below = v[j] < key[j];
+        if constexpr (!decltype(plain)::value)
+          below = m[j] < lab[j] || (m[j] == lab[j] && below);
+        if (below) {
+          lo[j] += half + 1;
+          len[j] -= half + 1;
+        } else {
+          len[j] = half;
+        }
+        more = more || len[j] > 0;
+      }
     }
-  }
+  };
+  if (one)
+    search(std::true_type{});
+  else
+    search(std::false_type{});
 #pragma unroll
   for (int j = 0; j < kN; ++j) {
     if (!((open >> j) & 1u)) continue;
