@@ -1599,10 +1599,11 @@ GraphDev rank_dev(const gsm_ctx *ctx);
 void make_rank_graph(gsm_ctx *ctx);
 
 // Is q counted on the renumbered graph?  Cliques of at least three vertices,
-// unrestricted, on a one-label graph with enough 2-edge paths.  Their symmetry constraints put every vertex of the clique
-// above the ones before it, so a hub's bitmap is only asked about higher
-// vertices, which it covers; ids do not matter to a count.  Candidate sets
-// refined or looked ahead at read other bitmaps and stay on the plain graph.
+// unrestricted, on a one-label graph with enough 2-edge paths.  Their symmetry
+// constraints put every vertex of the clique above the ones before it, so a
+// hub's bitmap is only asked about higher vertices, which it covers; ids do not
+// matter to a count.  Candidate sets refined or looked ahead at read other
+// bitmaps and stay on the plain graph.
 bool counts_by_rank(const gsm_ctx *ctx, const gsm_query *q) {
   if (ctx->label_values.size() > 1 || ctx->by_degree.empty() ||
       ctx->degree_squares < kRankSquares || ctx->opt.lookahead > 0 ||
@@ -1663,9 +1664,14 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   uint64_t sizes[kMaxK] = {};
   if (!dense_labels(ctx, q, dense)) return;  // a query label absent from G: no embedding
   if (!enumerate && counts_by_rank(ctx, q)) {
-    if (!ctx->rankg.ready) make_rank_graph(ctx);
-    R.g = rank_dev(ctx);
-    R.ranked = true;
+    try {
+      if (!ctx->rankg.ready) make_rank_graph(ctx);
+      R.g = rank_dev(ctx);
+      R.ranked = true;
+    } catch (const Fail &e) {
+      if (e.code != GSM_ERR_OOM) throw;
+      ctx->err.clear();  // no room for it: the plain graph counts too
+    }
   }
   if (pre)
     std::memcpy(sizes, pre->sizes, sizeof(uint64_t) * q->k);
@@ -2071,14 +2077,15 @@ void make_rank_graph(gsm_ctx *ctx) {
     GraphDev g = rank_dev(ctx);
     g.hub_words = words;
     launch_threshold_bits(g, r.thr, r.thr + (size_t)words * kThrLevels, ctx->stream);
-    // hubs: the highest vertices, from a multiple of 32 on
+    // hubs: the highest vertices, from a multiple of 32 on (not from 0, which
+    // stands for a graph in its own numbering)
     const int64_t budget =
         ctx->opt.hub_bitmap_bytes == 0 ? kHubBytesDefault : ctx->opt.hub_bitmap_bytes;
     int32_t H = std::min(n, kRankHubs);
     while (H > 0 && (int64_t)H * ((H + 63) / 32) * 4 > budget) H /= 2;
     if (H > 0) {
-      r.hub_lo = (n - H) / 32 * 32;
-      if (r.hub_lo > 0) {
+      r.hub_lo = std::max(32, (n - H) / 32 * 32);
+      if (r.hub_lo < n) {
         H = n - r.hub_lo;
         r.hub_words = (H + 31) / 32;
         r.bits_bytes = sizeof(uint32_t) * (size_t)H * r.hub_words;
