@@ -327,8 +327,9 @@ struct RowCheck {
 //                  the steps of the binary searches
 // A check is a chain of dependent loads.  With few candidates a row they miss
 // L1 and the chains' latency bounds the level: grouped, the last level of a
-// 5-cycle listing on R-MAT 20 (four candidates a row) takes 1.46 instead of
-// 1.67 ms.  With many, the row's adjacency stays in L1 and the grouped form's
+// 5-cycle listing on R-MAT 20 (four candidates a row) took 1.46 instead of
+// 1.67 ms; about 1.15 with searches that compare ids alone and halve by length
+// (the listing 1,981 -> 1,834 -> 1,721 us).  With many, the row's adjacency stays in L1 and the grouped form's
 // registers cost more warps than it gains: ordered triangles of R-MAT 20 (146
 // a row) 24.1 against 19.9 ms, 4-cliques of R-MAT 16 12.5 against 9.8 ms.
 // Hence grouped up to kFewCandidates candidates a row on average.
@@ -394,47 +395,58 @@ __device__ __forceinline__ uint32_t group_contains(const GraphDev &g,
       }
     }
     len[j] = end[j] - lo[j];
+    if (len[j] <= 0) {  // an empty row, or none to search
+      if ((open >> j) & 1u) alive &= ~(1u << j);
+      open &= ~(1u << j);
+      len[j] = 0;
+    }
   }
+  // The part [lo, lo + len) that can hold the key is halved with its longer
+  // side kept, so that its length does not depend on what was read: a step is a
+  // load, a compare and an add, and the longest of the four rows counts the
+  // steps for all.
   const bool one = g.num_labels == 1;
+  int32_t longest = len[0];
+#pragma unroll
+  for (int j = 1; j < kN; ++j) longest = max(longest, len[j]);
   auto search = [&](auto plain) {  // plain: one label, ids alone order a row
-    bool more = true;
-    while (more) {
-      more = false;
+    for (; longest > 1; longest -= longest >> 1) {
       int32_t v[kN], m[kN];
 #pragma unroll
       for (int j = 0; j < kN; ++j) {
-        const int32_t mid = lo[j] + (len[j] >> 1);
-        v[j] = len[j] > 0 ? __ldg(g.lcol + mid) : 0;
-        if constexpr (!decltype(plain)::value) m[j] = len[j] > 0 ? __ldg(g.llab + mid) : lab[j];
+        const int32_t half = len[j] >> 1;
+        v[j] = half > 0 ? __ldg(g.lcol + lo[j] + half - 1) : key[j];
+        if constexpr (!decltype(plain)::value)
+          m[j] = half > 0 ? __ldg(g.llab + lo[j] + half - 1) : lab[j];
       }
 #pragma unroll
       for (int j = 0; j < kN; ++j) {
-        if (len[j] <= 0) continue;
         const int32_t half = len[j] >> 1;
         bool below = v[j] < key[j];
         if constexpr (!decltype(plain)::value)
           below = m[j] < lab[j] || (m[j] == lab[j] && below);
-        if (below) {
-          lo[j] += half + 1;
-          len[j] -= half + 1;
-        } else {
-          len[j] = half;
-        }
-        more = more || len[j] > 0;
+        if (below) lo[j] += half;
+        len[j] -= half;
       }
+    }
+    int32_t v[kN], m[kN];
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      v[j] = (open >> j) & 1u ? __ldg(g.lcol + lo[j]) : key[j];
+      if constexpr (!decltype(plain)::value)
+        m[j] = (open >> j) & 1u ? __ldg(g.llab + lo[j]) : lab[j];
+    }
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      bool in = v[j] == key[j];
+      if constexpr (!decltype(plain)::value) in = in && m[j] == lab[j];
+      if (!in) alive &= ~(1u << j);
     }
   };
   if (one)
     search(std::true_type{});
   else
     search(std::false_type{});
-#pragma unroll
-  for (int j = 0; j < kN; ++j) {
-    if (!((open >> j) & 1u)) continue;
-    const bool in = lo[j] < end[j] && __ldg(g.lcol + lo[j]) == key[j] &&
-                    (one || __ldg(g.llab + lo[j]) == lab[j]);
-    if (!in) alive &= ~(1u << j);
-  }
   return alive;
 }
 
