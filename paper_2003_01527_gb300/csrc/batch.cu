@@ -496,12 +496,8 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
         const int32_t x = xb + j;
         if (x < x1) {
           if (x >= re) {
-            do {  // next row (rows without work are skipped)
-              ++rr;
-              ++r;
-              rs = re;
-              re = t.staged ? s_woff[rr + 1] : (int32_t)woff[r + 1];
-            } while (x >= re);
+            next_row(t, s_woff, woff, 0, x, &rr, &rs, &re);
+            r = t.r0 + rr;
             q = rseg[r];
             pst = pstart[r];
             slot = pslot[r];

@@ -91,12 +91,8 @@ __global__ void __launch_bounds__(1024) k_cextend(
       const int32_t x = xb + j;
       if (x >= x1) continue;
       if (x >= re) {
-        while (x >= re) {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-        }
+        next_row(t, s_woff, woff, wa, x, &rr, &rs, &re);
+        r = t.r0 + rr;
         pst = pstart[r];
         slot = pslot[r];
         decode_row(f, i, r, vals);

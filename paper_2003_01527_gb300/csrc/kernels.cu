@@ -1009,12 +1009,11 @@ __global__ void __launch_bounds__(256, 8) k_leaf_expand(
   if (first < n) {
     int32_t rs;
     int32_t rr = item_row(t, s_woff, woff, wa, x0 + first, &rs) - t.r0;
+    int32_t re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[t.r0 + rr + 1] - wa);
 #pragma unroll
     for (int j = 0; j < kItemsPerThread; ++j) {
       if (first + j >= n) break;
-      while (x0 + first + j >=
-             (t.staged ? s_woff[rr + 1] : (int32_t)(woff[t.r0 + rr + 1] - wa)))
-        ++rr;
+      if (x0 + first + j >= re) next_row(t, s_woff, woff, wa, x0 + first + j, &rr, &rs, &re);
       s_row[first + j] = rr;
     }
   }

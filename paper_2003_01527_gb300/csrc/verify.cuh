@@ -64,6 +64,32 @@ __device__ __forceinline__ int32_t item_row(const TileRows &t, const int32_t *s_
   return t.r0 + lo;
 }
 
+// From row r0 + rr, whose candidates end at re <= x, to the row of item x, and
+// where its candidates start and end.  Mostly the next; rows without work are
+// stepped over four at a time, longer runs by a search: bounds cut off a row's
+// segment leave runs of millions (counting the 5-cycles of two low roots of
+// R-MAT 20, whose symmetry orders two vertices, one thread stepped through
+// most of 6.5 M rows: 237 ms, 0.56 with the search).
+__device__ __forceinline__ void next_row(const TileRows &t, const int32_t *s_woff,
+                                         const int64_t *__restrict__ woff, int64_t wa, int32_t x,
+                                         int32_t *rr, int32_t *rs, int32_t *re) {
+  auto offset = [&](int32_t j) { return t.staged ? s_woff[j] : (int32_t)(woff[t.r0 + j] - wa); };
+  for (int32_t step = 0; step < 4; ++step) {
+    ++*rr;
+    *rs = *re;
+    *re = offset(*rr + 1);
+    if (x < *re) return;
+  }
+  int32_t lo = *rr + 1, hi = t.span;  // (the tile's last item lies before offset(span))
+  while (hi - lo > 1) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (offset(mid) <= x) lo = mid; else hi = mid;
+  }
+  *rr = lo;
+  *rs = offset(lo);
+  *re = offset(lo + 1);
+}
+
 // A row extended by one vertex at position i.
 template <typename Row>
 struct ExtendedRow {
@@ -328,7 +354,7 @@ struct RowCheck {
 // A check is a chain of dependent loads.  With few candidates a row they miss
 // L1 and the chains' latency bounds the level: grouped, the last level of a
 // 5-cycle listing on R-MAT 20 (four candidates a row) took 1.46 instead of
-// 1.67 ms; about 1.15 with searches that compare ids alone and halve by length
+// 1.67 ms; 1.17 with searches that compare ids alone and halve by length
 // (the listing 1,981 -> 1,834 -> 1,721 us).  With many, the row's adjacency stays in L1 and the grouped form's
 // registers cost more warps than it gains: ordered triangles of R-MAT 20 (146
 // a row) 24.1 against 19.9 ms, 4-cliques of R-MAT 16 12.5 against 9.8 ms.
@@ -476,12 +502,8 @@ __device__ __forceinline__ uint32_t check_group(
       const int32_t x = xb + j;
       if (x >= x1) break;
       if (x >= re) {
-        do {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-        } while (x >= re);
+        next_row(t, s_woff, woff, wa, x, &rr, &rs, &re);
+        r = t.r0 + rr;
         pst = pstart[r];
         slot = pslot[r];
         check.load(g, d, ColumnRow{F, ld, r}, slot);
@@ -503,12 +525,8 @@ __device__ __forceinline__ uint32_t check_group(
     const int32_t x = xb + j;
     if (x < x1) {
       if (x >= re) {
-        do {  // next row (rows without work are skipped)
-          ++rr;
-          ++r;
-          rs = re;
-          re = t.staged ? s_woff[rr + 1] : (int32_t)(woff[r + 1] - wa);
-        } while (x >= re);
+        next_row(t, s_woff, woff, wa, x, &rr, &rs, &re);
+        r = t.r0 + rr;
         pst = pstart[r];
         slot = pslot[r];
       }

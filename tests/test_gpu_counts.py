@@ -135,3 +135,38 @@ def test_cliques_on_the_renumbered_graph(gsm_lib, cuda, hub_bytes):
             assert m.count_distinct(m.query(k, edges)) == \
                 (sum(parts) // math.factorial(k), math.factorial(k))
     m.close()
+
+
+@pytest.mark.parametrize("opts", [{}, {"two_pass": True}, {"compressed": True},
+                                  {"block_size": 1024}, {"lookahead": 1}])
+def test_long_runs_of_rows_without_candidates(gsm_lib, cuda, opts):
+    """A range on the last vertex leaves most rows of a level without
+    candidates, in runs longer than a tile's rows, with single rows and short
+    gaps between them."""
+    n, spokes = 6010, 6000
+    pairs = [(0, a) for a in range(1, spokes + 1)]
+    for z, at in ((6001, [1, 2, 4, 9, 15, 2500]), (6002, [3, 2501, 2507, 6000]), (6003, [5999]),
+                  (6004, [1, 6000])):
+        pairs += [(z, a) for a in at] + [(0, z)]
+    g = I.graph_from_edges(n, pairs)
+    m = gsm_lib.Matcher(device=0, **opts)
+    m.load_graph(g.row_ptr, g.col, g.labels)
+    windows = [(1, (6001, 6005)), (2, (6001, 6005)), (2, (6003, 6010))]
+    for shape in ("path3", "triangle", "cycle4", "diamond"):
+        k, edges = SHAPES[shape]
+        q = I.query_from_edges(k, edges)
+        for u, (lo, hi) in windows:
+            ranges = {v: (0, 1) for v in [0] if shape != "diamond"}
+            ranges[u] = (lo, hi)
+            want, rows, rc = oracle.match(g, q, root_range=ranges.get(0, (0, n)),
+                                          ranges={u: (lo, hi)})
+            assert rc == oracle.OK
+            Q = m.query(k, edges)
+            for v, r in ranges.items():
+                Q.restrict(v, *r)
+            assert m.count(Q) == want, (shape, u)
+            got, count = m.enumerate(Q)
+            assert count == want and np.array_equal(got, rows), (shape, u)
+            if not opts:
+                assert m.run_batch([Q, Q]) == [want, want]
+    m.close()
