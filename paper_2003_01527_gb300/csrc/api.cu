@@ -849,10 +849,11 @@ void rows_to_acc(Run &R) {
                        ctx->stream));
 }
 
-// Candidates a row on average from which k_clique_count beats the general
-// count kernel: triangles of R-MAT 20 (78 a row) 3.0 against 5.1 ms, 4-cliques
-// of R-MAT 16 (28 a row, less than a warp's lanes) 3.1 against 2.3.
-constexpr int64_t kCliqueRow = 48;
+// Candidates a row on average from which k_clique_count beats the general count
+// kernel: triangles of R-MAT 20 (78 a row) 3.0 against 5.1 ms without the common
+// words of bitmaps and 2.4 with them, 4-cliques of R-MAT 16 (28 a row) 3.36 ->
+// 2.48 ms altogether; below half a warp's lanes they would idle.
+constexpr int64_t kCliqueRow = 16;
 
 // Room for a leaf level's left-out entries, `rows` of them at most (null if the
 // level is not a leaf's, or its rows have none).
@@ -1997,8 +1998,8 @@ void clear_all_graphs(gsm_ctx *ctx);
 // hubs: their bitmaps need to cover the kRankHubs highest vertices only, 4 KB
 // each, which stay in L1 and L2.  Triangles of R-MAT 20: 1.2e9 checks instead
 // of 2.3e9, 6.2 instead of 17.5 ms (the first count also renumbers: + 2 ms),
-// and 3.7 with k_clique_count and GraphDev::up; distinct 4-cliques of R-MAT 16
-// 3.6 instead of 9.4 ms, and 3.4 with up.
+// and 3.05 with k_clique_count and GraphDev::up; distinct 4-cliques of R-MAT 16
+// 3.6 instead of 9.4 ms, and 2.5 with both.
 constexpr int32_t kRankHubs = 32768;
 
 void free_rank_graph(gsm_ctx *ctx) {
@@ -2077,17 +2078,18 @@ void make_rank_graph(gsm_ctx *ctx) {
     GraphDev g = rank_dev(ctx);
     g.hub_words = words;
     launch_threshold_bits(g, r.thr, r.thr + (size_t)words * kThrLevels, ctx->stream);
-    // hubs: the highest vertices, from a multiple of 32 on (not from 0, which
-    // stands for a graph in its own numbering)
+    // hubs: the highest vertices, from a multiple of 128 on (not from 0, which
+    // stands for a graph in its own numbering); their bitmaps' lengths are
+    // multiples of four words too, so that any part starts on 16 bytes
     const int64_t budget =
         ctx->opt.hub_bitmap_bytes == 0 ? kHubBytesDefault : ctx->opt.hub_bitmap_bytes;
     int32_t H = std::min(n, kRankHubs);
-    while (H > 0 && (int64_t)H * ((H + 63) / 32) * 4 > budget) H /= 2;
+    while (H > 0 && (int64_t)(H + 127) * ((H + 255) / 32) * 4 > budget) H /= 2;
     if (H > 0) {
-      r.hub_lo = std::max(32, (n - H) / 32 * 32);
+      r.hub_lo = std::max(128, (n - H) / 128 * 128);
       if (r.hub_lo < n) {
         H = n - r.hub_lo;
-        r.hub_words = (H + 31) / 32;
+        r.hub_words = (H + 127) / 128 * 4;
         r.bits_bytes = sizeof(uint32_t) * (size_t)H * r.hub_words;
         r.bits = (uint32_t *)dev_alloc(ctx, r.bits_bytes);
         std::vector<int32_t> idx(n, -1);
