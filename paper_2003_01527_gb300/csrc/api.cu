@@ -850,9 +850,10 @@ void rows_to_acc(Run &R) {
 }
 
 // Candidates a row on average from which k_clique_count beats the general count
-// kernel: triangles of R-MAT 20 (78 a row) 3.0 against 5.1 ms without the common
-// words of bitmaps and 2.4 with them, 4-cliques of R-MAT 16 (28 a row) 3.36 ->
-// 2.48 ms altogether; below half a warp's lanes they would idle.
+// kernel: the kernel alone 3.0 against 5.1 ms for triangles of R-MAT 20 (78 a
+// row) before it took common words of bitmaps; with those the count of distinct
+// 4-cliques of R-MAT 16 (28 a row) went from 3.36 to 2.48 ms.  Below half a
+// warp's lanes a row the lanes would idle.
 constexpr int64_t kCliqueRow = 16;
 
 // Room for a leaf level's left-out entries, `rows` of them at most (null if the
