@@ -239,8 +239,9 @@ gsm_status gsm_count_distinct(gsm_ctx *ctx, const gsm_query *q, uint64_t *count,
  * per row and about 1.5 bytes per row of histograms.  A single-pass last
  * level reserves room for one row per candidate it checks (at most 4 GiB;
  * beyond that it takes two passes), so the staging can exceed the count.
- * A device `out` on a 16-byte boundary may be written by the kernels that
- * produce the rows; on an error other than GSM_ERR_TRUNCATED its contents are
+ * A device `out` on a 16-byte boundary in the context's device memory may be
+ * written by the kernels that produce the rows (any other gets them by a copy);
+ * on an error other than GSM_ERR_TRUNCATED its contents are
  * unspecified.  Errors: as gsm_count, plus GSM_ERR_TRUNCATED. */
 gsm_status gsm_enumerate(gsm_ctx *ctx, const gsm_query *q, int32_t *out, uint64_t cap_rows,
                          uint64_t *count, int32_t flags);

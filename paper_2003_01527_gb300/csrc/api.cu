@@ -30,6 +30,7 @@
 #include "gsm.h"
 #include "compressed.cuh"
 #include "kernels.cuh"
+#include "out_access.h"
 #include "query_access.h"
 
 using namespace gsm;
@@ -1617,6 +1618,17 @@ bool counts_by_rank(const gsm_ctx *ctx, const gsm_query *q) {
   return true;
 }
 
+// kernels_may_store of a caller's buffer; memory CUDA does not know (an error
+// here) is left to the copy.
+bool stores_reach(const gsm_ctx *ctx, const void *out) {
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, out) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return kernels_may_store(attr, out, ctx->device);
+}
+
 // The whole matcher for one query.  out == nullptr and !enumerate: count only;
 // distinct_of = |Aut(Q)| divides the count (distinct subgraphs).  keep_rows =
 // false: gsm_last_rows will not be asked for these rows.
@@ -1717,10 +1729,10 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   R.acc_mode = sort_cols == 0 ? kSinkRows : kSinkKeys;
   R.key_bits = key_bits;
   R.key_nw = packed_words(q->k, key_bits);
-  // straight into the caller's buffer, if it takes the kernels' widest store
+  // straight into the caller's buffer, if kernels may store there
   const bool wide = enumerate && (flags & GSM_OUT_DEVICE) && q->k > 1 && cap_rows > 0 &&
-                    ((uintptr_t)out & 15) == 0 &&
-                    !(ctx->opt.flags & GSM_OPT_COMPRESSED_FRONTIERS);
+                    !(ctx->opt.flags & GSM_OPT_COMPRESSED_FRONTIERS) &&
+                    stores_reach(ctx, out);
   const bool to_out = wide && !keep_rows;
   R.out = out;
   R.out_cap = cap_rows;
