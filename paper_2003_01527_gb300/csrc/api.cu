@@ -1947,17 +1947,23 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   *truncated = total > cap_rows;
 }
 
+// Runs the body of an entry point (or of a listing worker).  After a failure
+// the context's stream is waited for: kernels launched before it may still be
+// storing rows into the caller's buffers, which are the caller's again on
+// return, and into blocks that the allocator may hand to another stream.
 template <typename F>
 gsm_status guarded(gsm_ctx *ctx, F &&f) {
+  gsm_status st = GSM_OK;
   try {
     f();
-    return GSM_OK;
   } catch (const Fail &e) {
-    return e.code;
+    st = e.code;
   } catch (const std::exception &e) {
     set_err(ctx, "internal error: %s", e.what());
-    return GSM_ERR_OOM;
+    st = GSM_ERR_OOM;
   }
+  if (st != GSM_OK && ctx->stream) cudaStreamSynchronize(ctx->stream);
+  return st;
 }
 
 // Adjacency bitmaps of the hubs: vertices of degree >= kHubMinDegree, the
@@ -3778,7 +3784,8 @@ gsm_status gsm_enumerate_many(gsm_ctx *ctx, int32_t nq, const gsm_query *const *
     ctx->run.kernel_launches = launches;
     ctx->run.peak_bytes = peak;
   });
-  // no copy into the caller's buffers outlives the call, whatever happened
+  // no copy into the caller's buffers outlives the call, whatever happened (and
+  // no kernel: guarded)
   if (ctx->copy_stream) cudaStreamSynchronize(ctx->copy_stream);
   ctx->active_pending = false;
   for (auto &p : ctx->parked) p.pending = false;
