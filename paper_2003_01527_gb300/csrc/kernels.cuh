@@ -322,8 +322,9 @@ struct LeafDesc {
   LeafGroup grp[kMaxK];
 };
 // Where a count goes: words [0] += the low and [1] += the high 32 bits of each
-// embedding's number (sums of fewer than 2^32 values stay exact), [2] != 0 if
-// one embedding's number exceeds 64 bits, [3 + l] += the number of partial
+// embedding's number, [2] != 0 if one embedding's number exceeds 64 bits or one
+// of the two sums wrapped (it can with more than 2^32 embeddings, and the count
+// is then past 64 bits), [3 + l] += the number of partial
 // embeddings with the core and l leaves placed (l < nleaves, modulo 2^64).
 constexpr int32_t kCountWords = 3 + kMaxK;
 

@@ -109,6 +109,30 @@ def test_counts_past_64_bits(gsm_lib, cuda):
     m.close()
 
 
+def test_sums_of_halves_past_64_bits(gsm_lib, cuda):
+    """In K_n, a vertex with three leaves and a tail of two has n (n-1) (n-2)
+    core embeddings, each with (n-3) (n-4) (n-5) images of the leaves.  At n =
+    1,629 that is more than 2^32 embeddings of just under 2^32 each: their
+    numbers' low halves add up past 64 bits, the high ones to nothing."""
+    edges = [(0, 1), (0, 2), (0, 3), (0, 4), (4, 5)]
+    m = gsm_lib.Matcher(device=0)
+    for n in (1626, 1629):
+        ids = np.arange(n * n, dtype=np.int64)
+        src, dst = ids // n, ids % n
+        rp, col = I.csr_from_pairs(n, src[src != dst], dst[src != dst])
+        m.load_graph(rp, col)
+        assert n * (n - 1) * (n - 2) > 2 ** 32 - 2 ** 28
+        assert (n - 3) * (n - 4) * (n - 5) < 2 ** 32
+        want = math.perm(n, 6)
+        if want < 2 ** 64:
+            assert m.count(m.query(6, edges)) == want
+            continue
+        with pytest.raises(gsm_lib.GsmError) as e:
+            m.count(m.query(6, edges))
+        assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+    m.close()
+
+
 @pytest.mark.parametrize("hub_bytes", [0, -1, 1 << 16])
 def test_cliques_on_the_renumbered_graph(gsm_lib, cuda, hub_bytes):
     """Unrestricted cliques on a one-label graph with enough 2-edge paths are
