@@ -352,7 +352,8 @@ void gsm_result_free(gsm_ctx *ctx, gsm_result *r);
  * for that shape.  nq <= 65535.
  * Errors: GSM_ERR_INVALID_ARG, GSM_ERR_NO_GRAPH, GSM_ERR_OOM, GSM_ERR_CUDA, and
  * the errors of gsm_count / gsm_enumerate on the fallback path (on an error
- * no rows are left allocated). */
+ * no rows are left allocated).  After GSM_ERR_OVERFLOW every count is set
+ * nevertheless; those that exceed 2^64 - 1 read 2^64 - 1. */
 gsm_status gsm_run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *counts,
                          gsm_result *results, int32_t flags);
 
@@ -378,7 +379,8 @@ gsm_status gsm_batch_configure(gsm_ctx *ctx, uint64_t cap_rows, uint64_t cap_ele
  * frontier capacity -- at least one query per batch, at most max_batch.
  * Queries that arrive while batches run are admitted as soon as a lane frees,
  * so their work overlaps the running batches on the device.  A batch that
- * overflows its workspace is rerun query by query.  Every result equals
+ * overflows its workspace is rerun query by query, and a query that fails
+ * there fails alone (gsm_result.status).  Every result equals
  * gsm_count's (gsm_enumerate's rows) for that query.
  */
 

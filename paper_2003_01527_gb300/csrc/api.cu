@@ -2892,9 +2892,11 @@ void run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *c
   ctx->bstats.tuned = tuned ? 1 : 0;
   ctx->bstats.block_size = cfg.first;
   ctx->bstats.grid = cfg.second;
+  bool past = false;  // a count past 64 bits
   try {
     if (overflow) {
-      // the workspace was too small for this batch: run it query by query
+      // the workspace was too small for this batch (or a count exceeds 64
+      // bits): run it query by query
       ctx->bstats.overflowed = 1;
       ctx->bstats.fallbacks += 1;
       for (int32_t t = 0; t < L.m; ++t) {
@@ -2905,7 +2907,13 @@ void run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *c
         } else {
           uint64_t c = 0;
           bool trunc = false;
-          run_query(ctx, qs[j], false, nullptr, 0, 0, &c, &trunc);
+          try {
+            run_query(ctx, qs[j], false, nullptr, 0, 0, &c, &trunc);
+          } catch (const Fail &e) {  // past 64 bits: the others' counts stay good
+            if (e.code != GSM_ERR_OVERFLOW) throw;
+            c = UINT64_MAX;
+            past = true;
+          }
           counts[j] = c;
         }
       }
@@ -2932,6 +2940,7 @@ void run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *c
     for (int32_t j = 0; j < nq; ++j) results[j].count = counts[j];
   ctx->bstats.last_ms =
       std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+  if (past) FAIL(GSM_ERR_OVERFLOW, "a count of the batch exceeds 2^64 - 1");
 }
 
 }  // namespace
@@ -2993,19 +3002,28 @@ void server_complete(gsm_ctx *ctx, gsm_ctx::Server &S, Lane &L) {
   }
   const size_t nr = L.tickets.size();
   std::vector<uint64_t> counts(nr, 0);
+  std::vector<gsm_status> status(nr, GSM_OK);
   std::vector<gsm_result> res(nr);
   for (auto &r : res) std::memset(&r, 0, sizeof(r));
   gsm_status st = guarded(ctx, [&] {
     try {
       if (lane_counts(ctx, L)) {
         ctx->bstats.fallbacks += 1;
+        // one request's failure (a count past 64 bits, rows over the memory) is
+        // its own: the others of the lane have other submitters
         for (size_t t = 0; t < nr; ++t) {
-          if (modes[t] == GSM_MODE_ENUMERATE) {
-            single_query_rows(ctx, qs[t], false, &res[t]);
-            counts[t] = res[t].count;
-          } else {
-            bool trunc = false;
-            run_query(ctx, qs[t], false, nullptr, 0, 0, &counts[t], &trunc);
+          status[t] = guarded(ctx, [&] {
+            if (modes[t] == GSM_MODE_ENUMERATE) {
+              single_query_rows(ctx, qs[t], false, &res[t]);
+              counts[t] = res[t].count;
+            } else {
+              bool trunc = false;
+              run_query(ctx, qs[t], false, nullptr, 0, 0, &counts[t], &trunc);
+            }
+          });
+          if (status[t] != GSM_OK) {
+            release_rows(ctx, &res[t]);
+            counts[t] = 0;
           }
         }
       } else {
@@ -3039,7 +3057,7 @@ void server_complete(gsm_ctx *ctx, gsm_ctx::Server &S, Lane &L) {
     auto node = S.inflight.extract(L.tickets[t]);
     node.mapped().count = counts[t];
     node.mapped().rows = res[t].rows;
-    node.mapped().status = st;
+    node.mapped().status = st != GSM_OK ? st : status[t];
     node.mapped().t_done = t_done;
     S.finished.insert(std::move(node));
   }

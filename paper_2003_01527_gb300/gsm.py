@@ -358,12 +358,19 @@ class _DevicePtr:
 def gsm_run_batch(ctx: int, queries, flags: int = 0, enumerate: bool = False):
     """queries: sequence of gsm_query handles.  Returns uint64 counts, or with
     enumerate=True (counts, rows): rows[j] = the sorted rows of query j, a
-    numpy array (host) or, with flags & GSM_OUT_DEVICE, a CUDA tensor."""
+    numpy array (host) or, with flags & GSM_OUT_DEVICE, a CUDA tensor.  The
+    GsmError of a batch with counts past 64 bits (GSM_ERR_OVERFLOW) carries all
+    counts as `counts`; those read 2^64 - 1."""
     nq = len(queries)
     arr = (ctypes.c_void_p * max(nq, 1))(*queries)
     counts = np.zeros(max(nq, 1), dtype=np.uint64)
     res = (gsm_result * max(nq, 1))() if enumerate else None
-    _check(ctx, _lib.gsm_run_batch(ctx, arr, nq, _ptr(counts), res, flags))
+    try:
+        _check(ctx, _lib.gsm_run_batch(ctx, arr, nq, _ptr(counts), res, flags))
+    except GsmError as e:
+        if e.status == GSM_ERR_OVERFLOW:
+            e.counts = counts[:nq]
+        raise
     if not enumerate:
         return counts[:nq]
     rows = _take_all(ctx, [res[j] for j in range(nq)])

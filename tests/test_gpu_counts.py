@@ -4,6 +4,7 @@ different labels, restricted leaves), queries with symmetries (one of every
 set of symmetric embeddings is counted; candidates outside the ordering
 constraints are never generated), and counts past 64 bits."""
 import math
+import time
 
 import numpy as np
 import pytest
@@ -106,6 +107,46 @@ def test_counts_past_64_bits(gsm_lib, cuda):
     with pytest.raises(gsm_lib.GsmError) as e:
         m.count(star(6))
     assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+    m.close()
+
+
+def test_one_count_past_64_bits_is_not_the_others(gsm_lib, cuda):
+    """A batch with a count past 64 bits reports it, with every other count;
+    in the served form only that request fails, listings beside it too."""
+    d = 2000
+    g = I.graph_from_edges(d + 4, [(0, v) for v in range(1, d + 1)] +
+                           [(d + 1, d + 2), (d + 2, d + 3), (d + 1, d + 3)])
+    m = gsm_lib.Matcher(device=0)
+    m.load_graph(g.row_ptr, g.col, g.labels)
+    star = [m.query(x + 1, [(0, j + 1) for j in range(x)]) for x in range(1, 9)]
+    triangle = m.query(3, [(0, 1), (1, 2), (0, 2)])
+    want = [math.perm(d, x) + (6 if x < 3 else 0) for x in range(1, 9)] + [6]
+    want[0] = 2 * (d + 3)
+    capped = [min(c, 2 ** 64 - 1) for c in want]
+    assert capped.count(2 ** 64 - 1) == 3
+    for _ in range(2):
+        with pytest.raises(gsm_lib.GsmError) as e:
+            m.run_batch(star + [triangle])
+        assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+        assert [int(c) for c in e.value.counts] == capped
+    assert m.run_batch(star[:5] + [triangle]) == want[:5] + [6]
+    tri = [[d + 1 + a, d + 1 + b, d + 1 + c] for a, b, c in
+           [(0, 1, 2), (0, 2, 1), (1, 0, 2), (1, 2, 0), (2, 0, 1), (2, 1, 0)]]
+    gsm_lib.gsm_server_start(m.ctx, 2, 16)
+    tickets = [gsm_lib.gsm_submit(m.ctx, q.handle) for q in star]
+    tickets.append(gsm_lib.gsm_submit(m.ctx, triangle.handle, gsm_lib.GSM_MODE_ENUMERATE))
+    done = [None] * len(tickets)
+    deadline = time.time() + 60
+    while None in done and time.time() < deadline:
+        done = [r or gsm_lib.gsm_poll(m.ctx, t) for r, t in zip(done, tickets)]
+    gsm_lib.gsm_server_stop(m.ctx)
+    assert None not in done
+    for r, c in zip(done, want):
+        if c < 2 ** 64:
+            assert (r["status"], r["count"]) == (gsm_lib.GSM_OK, c)
+        else:
+            assert r["status"] == gsm_lib.GSM_ERR_OVERFLOW
+    assert done[-1]["rows"].tolist() == tri
     m.close()
 
 
