@@ -734,6 +734,13 @@ uint64_t symmetry_constraints(int32_t k, const uint32_t *adj, const int32_t *lab
 
 // ------------------------------------------------------------------ driver
 
+// How a run uses the budgeted stack (run_query tries them in turn).
+enum class Thrift {
+  kNone,     // with level setups and leaf levels
+  kLean,     // frontiers and their rows' arrays only
+  kCareful,  // ... in pieces that leave every later level room for one row's output
+};
+
 struct Run {
   gsm_ctx *ctx;
   const gsm_query *q;
@@ -743,6 +750,8 @@ struct Run {
   LevelDesc lv[kMaxK];
   GraphDev g;
   bool ranked = false;  // g is the graph renumbered by degree
+  Thrift thrift = Thrift::kNone;
+  bool spared = false;  // a level setup or a leaf's left-out entries were pushed
   int32_t block;
   int32_t spin_limit;  // polls a look-back wait may take
   int32_t stall_tile;  // GSM_OPT_INJECT_LOOKBACK_STALL: the tile that withholds its count
@@ -802,7 +811,8 @@ LevelSetup push_setup(Run &R, int64_t rows) {
   st.cap = (int32_t)std::min<int64_t>(8192, 64 + rows / 8);
   const size_t words = sizeof(unsigned long long) * level_setup_words(st.cap, st.tile_items);
   const size_t bytes = align_up(words) + align_up(sizeof(int32_t) * (size_t)(st.cap + 1));
-  if (!stack_fits(ctx, bytes)) return LevelSetup();
+  if (R.thrift != Thrift::kNone || !stack_fits(ctx, bytes)) return LevelSetup();
+  R.spared = true;
   char *p = (char *)stack_push(ctx, bytes);
   st.lb = (unsigned long long *)p;
   st.tile_row = (int32_t *)(p + align_up(words));
@@ -861,10 +871,38 @@ constexpr int64_t kCliqueRow = 16;
 // level is not a leaf's, or its rows have none).
 int2 *push_excl(Run &R, int32_t i, int64_t rows) {
   if (!R.lv[i].leaf || R.lv[i].ninj == 0) return nullptr;
+  R.spared = true;
   return (int2 *)stack_push(R.ctx, sizeof(int2) * rows);
 }
 size_t excl_bytes(const Run &R, int32_t i, int64_t rows) {
   return R.lv[i].leaf && R.lv[i].ninj > 0 ? align_up(sizeof(int2) * (size_t)rows) : 0;
+}
+
+// The stack bytes of a frontier of `rows` rows of width w, with the next
+// level's per-row arrays.
+size_t frontier_bytes(int64_t rows, int32_t w) {
+  return align_up((size_t)rows * w * sizeof(int32_t)) + align_up(4 * (size_t)rows) +
+         align_up((size_t)rows) + align_up(8 * ((size_t)rows + 1));
+}
+// ... of the prefix ranks of the last level's input of `rows` rows.
+size_t rank_bytes(const Run &R, int64_t rows) {
+  if (R.rank_p == 0) return 0;
+  return 2 * align_up(4 * (size_t)rows) + align_up(8 * ((size_t)rows + 1)) +
+         align_up(8 * (size_t)scan_tmp_elems(rows));
+}
+// What the levels after level i need for the output of one row each, at most
+// (a row has at most max_deg candidates).
+size_t later_bytes(const Run &R, int32_t i) {
+  size_t b = 0;
+  for (int32_t j = i + 1; j < R.k - 1; ++j)
+    b += frontier_bytes(R.ctx->max_deg, j + 1) + (j == R.k - 2 ? rank_bytes(R, R.ctx->max_deg) : 0);
+  return b;
+}
+// ... and what a piece of several rows of level i with `rows` output rows leaves
+// free for them in a careful run.
+size_t room_bytes(const Run &R, int32_t i, int64_t nrows, int64_t rows) {
+  if (R.thrift != Thrift::kCareful || nrows <= 1) return 0;
+  return later_bytes(R, i) + (i == R.k - 2 ? rank_bytes(R, rows) : 0);
 }
 
 // A leaf level: its W output rows are known, none is checked.  Rows are split
@@ -882,8 +920,7 @@ void process_leaf(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t
   const size_t bytes = (size_t)W * w_out * sizeof(int32_t);
   if (!last) {
     // the frontier and the next level's per-row arrays
-    const size_t need = align_up(bytes) + align_up(4 * (size_t)W) + align_up((size_t)W) +
-                        align_up(8 * ((size_t)W + 1)) + excl_bytes(R, i + 1, W);
+    const size_t need = frontier_bytes(W, w_out) + excl_bytes(R, i + 1, W);
     if (W * w_out >= (int64_t(1) << 31) - 1 || !stack_fits(ctx, need)) {
       if (nrows <= 1)
         FAIL(GSM_ERR_BUDGET, "the %lld partial results of one row need %zu bytes, over the budget",
@@ -961,9 +998,8 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
     if (last) {
       fits = (double)W * (double)R.acc_row_bytes() <= kFusedResultBytes;
     } else {
-      const size_t need = align_up((size_t)W * w_out * sizeof(int32_t)) +
-                          align_up(4 * (size_t)W) + align_up((size_t)W) +
-                          align_up(8 * ((size_t)W + 1)) + excl_bytes(R, i + 1, W);
+      const size_t need = frontier_bytes(W, w_out) + excl_bytes(R, i + 1, W) +
+                          room_bytes(R, i, nrows, W);
       fits = (int64_t)W * w_out < (int64_t(1) << 31) - 1 && stack_fits(ctx, need);
     }
     if (fits) {
@@ -1028,8 +1064,8 @@ void process_sub(Run &R, int32_t i, const int32_t *F, int64_t ld, const int32_t 
   }
   const size_t bytes = (size_t)S * w_out * sizeof(int32_t);
   // the next level also pushes pivot start, pivot slot and work offsets
-  const size_t need = align_up(bytes) + align_up(4 * (size_t)S) + align_up((size_t)S) +
-                      align_up(8 * ((size_t)S + 1)) + excl_bytes(R, i + 1, S);
+  const size_t need = frontier_bytes(S, w_out) + excl_bytes(R, i + 1, S) +
+                      room_bytes(R, i, nrows, S);
   // elements of a frontier are indexed with 32 bits inside the kernels
   const bool too_many = (int64_t)S * w_out >= (int64_t(1) << 31) - 1;
   if (too_many || !stack_fits(ctx, need)) {
@@ -1271,7 +1307,8 @@ void process_c(Run &R, int32_t i, const CFrontier &f, const int32_t *pstart, con
       fits = (double)W * (double)R.acc_row_bytes() <= kFusedResultBytes;
     } else {
       const size_t need = 2 * align_up(4 * (size_t)W) + align_up(4 * (size_t)W) +
-                          align_up((size_t)W) + align_up(8 * ((size_t)W + 1));
+                          align_up((size_t)W) + align_up(8 * ((size_t)W + 1)) +
+                          room_bytes(R, i, nrows, W);
       fits = stack_fits(ctx, need);
     }
     if (!fits) {
@@ -1639,10 +1676,17 @@ struct Prefiltered {
   const uint64_t *sizes;
 };
 
-void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, uint64_t cap_rows,
-               int32_t flags, uint64_t *count_out, bool *truncated,
-               bool copy_async = false, const Prefiltered *pre = nullptr,
-               uint64_t distinct_of = 1, bool keep_rows = true) {
+//
+// One attempt at it.  What a next one could do: spared = this one pushed what a
+// lean run does without; careful = a careful run is sure to fit the stack.
+struct Attempt {
+  Thrift thrift = Thrift::kNone;
+  bool spared = false, careful = false;
+};
+void run_query_once(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out,
+                    uint64_t cap_rows, int32_t flags, uint64_t *count_out, bool *truncated,
+                    bool copy_async, const Prefiltered *pre, uint64_t distinct_of, bool keep_rows,
+                    Attempt *attempt) {
   if (!ctx->has_graph) FAIL(GSM_ERR_NO_GRAPH, "no data graph loaded");
   const Range range(enumerate ? "gsm query (list)" : "gsm query (count)");
   std::memset(&ctx->run, 0, sizeof(ctx->run));
@@ -1670,6 +1714,12 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
                              std::min<int64_t>((int64_t(1) << 30) - 4096,
                                                (int64_t)(ctx->scratch_limit / 2) * 7));
   R.d_total = ctx->d_small + kSmallCount;
+  R.thrift = attempt->thrift;
+  struct Note {  // (also when an exception ends the attempt)
+    const Run &run;
+    Attempt *to;
+    ~Note() { to->spared = run.spared; }
+  } note{R, attempt};
   ctx->run.k = q->k;
   *truncated = false;
   *count_out = 0;
@@ -1775,8 +1825,8 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     d.bitmap = popc(q->adj[u]) == 1 ? nullptr : bm + (size_t)u * nw;
     // ... and its level needs no checks (listings; fault injection, the probe
     // accounting and the two-pass form keep their levels)
-    d.leaf = enumerate && d.bitmap == nullptr && d.ninj <= kLeafExcl && !ctx->opt.lookahead &&
-             R.block <= 256 &&
+    d.leaf = enumerate && R.thrift == Thrift::kNone && d.bitmap == nullptr && d.ninj <= kLeafExcl &&
+             !ctx->opt.lookahead && R.block <= 256 &&
              !(ctx->opt.flags & (GSM_OPT_COMPRESSED_FRONTIERS | GSM_OPT_TWO_PASS |
                                  GSM_OPT_COUNT_PROBES | GSM_OPT_INJECT_LOOKBACK_STALL));
     d.lab = dense[u];
@@ -1819,6 +1869,8 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
   // (run_filter has zeroed the count's words; a listing adds up none)
   const Mark mk = stack_mark(ctx);
   const int64_t R1 = (int64_t)sizes[R.order[0]];
+  attempt->careful = frontier_bytes(R1, 1) + (R.k == 2 ? rank_bytes(R, R1) : 0) +
+                         later_bytes(R, 0) <= ctx->stack_limit;
   int32_t *F1 = (int32_t *)stack_push(ctx, sizeof(int32_t) * R1);
   // only words that the root's restriction reaches can be non-zero
   const int32_t w0 = std::min(std::max(0, q->lo[R.order[0]]), ctx->n) / 32,
@@ -1945,6 +1997,37 @@ void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, u
     check_sort_flag(ctx);
   }
   *truncated = total > cap_rows;
+}
+
+// What speeds a level up (LevelSetup, a leaf level's left-out entries) takes
+// room on the stack that later levels may need: with it the listing of the
+// tailed triangles of 2,000 vertices of degree 16 needed 586 KB of budget
+// instead of 84 KB.  So a run that does not fit the budget with it is made again
+// without.  Even then a piece may fill the stack so far that a later level's
+// smallest piece does not fit, for one budget and not for a smaller one, and
+// counts have other pieces since they break symmetries; hence the careful run,
+// wherever it is sure to end well.
+void run_query(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *out, uint64_t cap_rows,
+               int32_t flags, uint64_t *count_out, bool *truncated,
+               bool copy_async = false, const Prefiltered *pre = nullptr,
+               uint64_t distinct_of = 1, bool keep_rows = true) {
+  Attempt a;
+  for (;;) {
+    try {
+      run_query_once(ctx, q, enumerate, out, cap_rows, flags, count_out, truncated, copy_async,
+                     pre, distinct_of, keep_rows, &a);
+      return;
+    } catch (const Fail &e) {
+      if (e.code != GSM_ERR_BUDGET) throw;
+      if (a.thrift == Thrift::kNone && a.spared)
+        a.thrift = Thrift::kLean;
+      else if (a.thrift != Thrift::kCareful && a.careful)
+        a.thrift = Thrift::kCareful;
+      else
+        throw;
+    }
+    ctx->err.clear();
+  }
 }
 
 // Runs the body of an entry point (or of a listing worker).  After a failure
