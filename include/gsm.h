@@ -76,9 +76,9 @@ typedef void (*gsm_free_fn)(void *alloc_ctx, void *ptr, size_t bytes, void *stre
  * (rows are split until one row per candidate fits). */
 #define GSM_OPT_COMPRESSED_FRONTIERS 4
 /* Fault injection for tests of the bounded waits: in every single-pass level
- * of the default frontier layout, the second tile never publishes its
- * survivor count, so the waits of the tiles after it run out
- * (lookback_spin_limit) and the call returns GSM_ERR_TIMEOUT.  Nothing hangs
+ * of the default frontier layout, and of the batched form, the second tile
+ * never publishes its survivor count, so the waits of the tiles after it run
+ * out (lookback_spin_limit) and the call returns GSM_ERR_TIMEOUT.  Nothing hangs
  * and every row stays inside its buffer; the context stays usable. */
 #define GSM_OPT_INJECT_LOOKBACK_STALL 8
 /* The same for the final sort of listing calls: in every single-sweep pass
@@ -95,7 +95,8 @@ typedef void (*gsm_free_fn)(void *alloc_ctx, void *ptr, size_t bytes, void *stre
  * tile never publishes its work total, so the waits of the tiles after it
  * run out; the call returns GSM_ERR_TIMEOUT, no offset is used, and the
  * context stays usable.  Only levels of more than 1,024 rows have a second
- * tile. */
+ * tile (of the batched form: of more than 256 rows, and its list of level 1
+ * with more than 1,024 bitmap words). */
 #define GSM_OPT_INJECT_SCAN_STALL 64
 
 typedef struct gsm_options {
@@ -125,9 +126,12 @@ typedef struct gsm_options {
    * buffers of one query's rows until they are copied out, so up to this
    * many of a worker's queries can be ahead of its copies. */
   int32_t copy_slots;
-  /* Bound of every wait of a single-pass level on the counts of earlier
-   * tiles (polls of about 32 ns; 0 = 2^20).  A wait that runs out ends the
-   * call with GSM_ERR_TIMEOUT; the rows written stay inside the buffers. */
+  /* Bound of every wait of a kernel's tile on the counts of earlier tiles
+   * (polls of about 32 ns; 0 = 2^20): single-pass levels, the work scans
+   * between levels, the final sort, and the list, work scans and levels of the
+   * batched and served forms.  A wait that runs out ends the call (of the
+   * served form: the requests of that batch) with GSM_ERR_TIMEOUT; the rows
+   * written stay inside the buffers. */
   int32_t lookback_spin_limit;
   /* k-look-ahead of the verification levels (Sec. 3.2, "1- and 2-look-ahead";
    * 0 = off, 1, 2): a candidate w for pi_i is dropped when the query
@@ -350,10 +354,11 @@ void gsm_result_free(gsm_ctx *ctx, gsm_result *r);
  * GSM_BATCH_AUTOTUNE, the first batch of a shape is run once per candidate
  * configuration (every run gives the same results) and the fastest is kept
  * for that shape.  nq <= 65535.
- * Errors: GSM_ERR_INVALID_ARG, GSM_ERR_NO_GRAPH, GSM_ERR_OOM, GSM_ERR_CUDA, and
- * the errors of gsm_count / gsm_enumerate on the fallback path (on an error
- * no rows are left allocated).  After GSM_ERR_OVERFLOW every count is set
- * nevertheless; those that exceed 2^64 - 1 read 2^64 - 1. */
+ * Errors: GSM_ERR_INVALID_ARG, GSM_ERR_NO_GRAPH, GSM_ERR_OOM, GSM_ERR_CUDA,
+ * GSM_ERR_TIMEOUT (lookback_spin_limit), and the errors of gsm_count /
+ * gsm_enumerate on the fallback path (on an error no rows are left allocated).
+ * After GSM_ERR_OVERFLOW every count is set nevertheless; those that exceed
+ * 2^64 - 1 read 2^64 - 1. */
 gsm_status gsm_run_batch(gsm_ctx *ctx, const gsm_query *const *qs, int32_t nq, uint64_t *counts,
                          gsm_result *results, int32_t flags);
 

@@ -2493,6 +2493,8 @@ cudaGraphExec_t lane_graph(gsm_ctx *ctx, Lane &L, int32_t m, int32_t kmax, int32
   BatchArgs a = L.a;
   if (!L.enumerate) a.final_rows = nullptr;
   a.spin_limit = ctx->opt.lookback_spin_limit > 0 ? ctx->opt.lookback_spin_limit : kLbSpinLimit;
+  a.stall_tile = (ctx->opt.flags & GSM_OPT_INJECT_LOOKBACK_STALL) ? 1 : -1;
+  a.scan_stall_tile = (ctx->opt.flags & GSM_OPT_INJECT_SCAN_STALL) ? 1 : -1;
   a.nq = m;
   a.kmax = kmax;
   a.n_words = n_words;

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) k_b_list(GraphDev g, const BatchQuery *__
                                                 unsigned long long *counts,
                                                 unsigned long long *lb,
                                                 unsigned long long *lb_pivot, int32_t spin_limit,
-                                                int32_t *overflow) {
+                                                int32_t stall_tile, int32_t *overflow) {
   constexpr int kWords = kBatchListTile / 256;  // of a thread, consecutive
   __shared__ int32_t s_warp[33];
   __shared__ int32_t s_tile, s_q;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_b_list(GraphDev g, const BatchQuery *__
     const int32_t rank = block_rank(c, s_warp, &T);
     if (warp == 0) {
       const unsigned long long p = lookback_prefix(lb, tile, tiles, (unsigned long long)T, lane,
-                                                   spin_limit);
+                                                   spin_limit, tile != stall_tile);
       if (lane == 0) s_prefix = p;
     }
     __syncthreads();
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(256) k_b_pivot_scan(
     int32_t *__restrict__ pstart, uint8_t *__restrict__ pslot, int64_t *__restrict__ woff,
     int32_t *__restrict__ tile_row, int32_t tile_items, int64_t cap_rows, int64_t cap_elems,
     int64_t cap_items, unsigned long long *lb, unsigned long long *lb_level, int32_t spin_limit,
-    int32_t *overflow) {
+    int32_t stall_tile, int32_t *overflow) {
   __shared__ int64_t s_warp[33];
   __shared__ int32_t s_tile;
   __shared__ unsigned long long s_prefix;
@@ -305,7 +305,8 @@ __global__ void __launch_bounds__(256) k_b_pivot_scan(
       }
       if (lane < 8) s_warp[lane] = vi - v;
       const unsigned long long T = (unsigned long long)__shfl_sync(kFull, vi, 7);
-      const unsigned long long p = lookback_prefix(lb, tile, tiles, T, lane, spin_limit);
+      const unsigned long long p =
+          lookback_prefix(lb, tile, tiles, T, lane, spin_limit, tile != stall_tile);
       if (lane == 0) s_prefix = p;
     }
     __syncthreads();
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
     const int64_t *__restrict__ woff, const int32_t *__restrict__ tile_row, int64_t cap_rows,
     int64_t cap_elems, int64_t cap_final, unsigned long long *counts, int32_t *__restrict__ Fn,
     int32_t *__restrict__ rseg_n, int32_t *__restrict__ final_rows, unsigned long long *lb,
-    unsigned long long *lb_pivot, int32_t spin_limit, int32_t *overflow) {
+    unsigned long long *lb_pivot, int32_t spin_limit, int32_t stall_tile, int32_t *overflow) {
   static_assert(kItemsPerThread == 4, "four candidates per thread");
   extern __shared__ int32_t smem[];
   __shared__ int32_t s_tile;
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
     if (warp == 0) {
       const unsigned long long p = lookback_resolve(
           lb, tile, tiles, ((unsigned long long)tf << kPackBits) | (unsigned long long)tn, lane,
-          spin_limit);
+          spin_limit, tile != stall_tile);
       if (lane == 0) s_prefix = p;
     }
     __syncthreads();
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 4 : 1) k_b_l
         s_pair[2 * at + 1] = wj[j];
       }
     }
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0 && tile != stall_tile)
       lookback_publish(lb, tile, tiles,
                        ((unsigned long long)((uint32_t)T >> 16) << kPackBits) |
                            (unsigned long long)(T & 0xffff));
@@ -611,20 +612,20 @@ int batch_enqueue(const GraphDev &g, const BatchArgs &a, cudaStream_t s) {
   // level 1: every query's candidate list for its first matched vertex
   k_b_list<<<(unsigned)std::max<int64_t>(std::min<int64_t>(list_tiles, G), 1), 256, 0, s>>>(
       g, a.qs, a.nq, a.list_off, a.state, std::min(a.cap_rows, a.cap_elems), a.F[0], a.rseg[0],
-      a.counts, a.lb_list, a.lb_pivot, a.spin_limit, a.overflow);
+      a.counts, a.lb_list, a.lb_pivot, a.spin_limit, a.scan_stall_tile, a.overflow);
   int launches = 3;
   for (int32_t i = 1; i < a.kmax; ++i) {
     const int cur = (i - 1) & 1, nxt = i & 1;
     k_b_pivot_scan<<<G, 256, 0, s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart,
                                      a.pslot, a.woff, a.tile_row, tile_items, a.cap_rows,
                                      a.cap_elems, a.cap_items, a.lb_pivot, a.lb_level,
-                                     a.spin_limit, a.overflow);
+                                     a.spin_limit, a.scan_stall_tile, a.overflow);
     auto level = [&](auto kernel) {
       kernel<<<G, B, level_smem(B), s>>>(g, a.qs, i, a.state, a.F[cur], a.rseg[cur], a.pstart,
                                          a.pslot, a.woff, a.tile_row, a.cap_rows, a.cap_elems,
                                          a.cap_final, a.counts, a.F[nxt], a.rseg[nxt],
                                          a.final_rows, a.lb_level, a.lb_pivot, a.spin_limit,
-                                         a.overflow);
+                                         a.stall_tile, a.overflow);
     };
     B <= 256 ? level(k_b_level<256>) : level(k_b_level<1024>);
     launches += 2;

@@ -69,6 +69,9 @@ struct BatchArgs {
   unsigned long long *lb_pivot;   // [cap_rows / kBatchPivotTile + 1 + kLbExtra]
   unsigned long long *lb_level;   // [cap_items / kBatchMinTile + 1 + kLbExtra]
   int32_t spin_limit;
+  // fault injection (-1: none): tiles that never publish their look-back words,
+  // of the levels, and of the list and the pivot scans
+  int32_t stall_tile, scan_stall_tile;
   // enumerate batches: result rows of the queries that list them (null: a
   // counting batch).  The rows of step i (queries with k = i + 1) are
   // row-major, k ints each, in query-id column order, from element

@@ -759,14 +759,21 @@ __device__ __forceinline__ unsigned long long lookback_resolve(unsigned long lon
   return prefix;
 }
 
-// Both halves at once (the tile waits for its prefix right after counting).
+// Both halves at once (the tile waits for its prefix right after counting);
+// publish = false: as above, and the total gains T all the same.
 __device__ __forceinline__ unsigned long long lookback_prefix(unsigned long long *lookback,
                                                               int32_t tile, int32_t tiles,
                                                               unsigned long long T, int lane,
-                                                              int32_t spin_limit) {
-  if (lane == 0) lookback_publish(lookback, tile, tiles, T);
+                                                              int32_t spin_limit,
+                                                              bool publish = true) {
+  if (lane == 0) {
+    if (publish)
+      lookback_publish(lookback, tile, tiles, T);
+    else if (T)
+      atomicAdd(lookback + tiles + 1, T);
+  }
   __syncwarp();
-  return lookback_resolve(lookback, tile, tiles, T, lane, spin_limit);
+  return lookback_resolve(lookback, tile, tiles, T, lane, spin_limit, publish);
 }
 
 }  // namespace gsm

@@ -18,6 +18,7 @@ waits -- no GPU fault and no hang:
   counts exactly.
 """
 import hashlib
+import time
 
 import numpy as np
 import pytest
@@ -170,6 +171,49 @@ def test_work_scan_wait_runs_out(gsm_lib, cuda):
     # query has no level and so no work scan
     assert m.count(m.query(1, [], [0])) == int((g.labels == 0).sum())
     m.close()
+
+
+@pytest.mark.parametrize("where", ["level", "work_scan", "list"])
+def test_batched_wait_runs_out(gsm_lib, cuda, where):
+    """The look-backs of the batched form: its levels, the pivot scans between
+    them, and the list of level 1.  The batch ends in GSM_ERR_TIMEOUT, served
+    requests with that status each, and the context still counts exactly."""
+    import bench
+    g, queries = bench.load_workload()
+    sl = queries[0]
+    ones = int((g.labels == 0).sum())
+    stall = "inject_lookback_stall" if where == "level" else "inject_scan_stall"
+    for opts in ({}, {stall: True}):
+        m = gsm_lib.Matcher(device=0, lookback_spin_limit=4096, **opts)
+        m.load_graph(g.row_ptr, g.col, g.labels)
+        one = m.query(1, [], [0])
+        if where == "list":  # 6 tiles of 1,024 words
+            Qs, want = [one] * 3, [ones] * 3
+        else:
+            Q = m.query(sl["k"], sl["edges"], sl["labels"]).restrict(0, 0, sl["root_hi"])
+            Qs, want = [Q], [sl["count"]]
+        if not opts:  # the same batch without the injection, under the same bound
+            assert m.run_batch(Qs) == want
+            assert m.run_batch(Qs, enumerate=True, device=True)[0] == want
+            m.close()
+            continue
+        for listing in (True, False) if where == "list" else (True,):
+            with pytest.raises(gsm_lib.GsmError) as e:
+                m.run_batch(Qs, enumerate=listing)
+            assert e.value.status == gsm_lib.GSM_ERR_TIMEOUT
+            assert "batch" in str(e.value)
+        assert m.run_batch([one]) == [ones]
+        gsm_lib.gsm_server_start(m.ctx, 1, 4)
+        tickets = [gsm_lib.gsm_submit(m.ctx, q.handle, gsm_lib.GSM_MODE_ENUMERATE) for q in Qs]
+        done, deadline = [None] * len(Qs), time.time() + 60
+        while None in done and time.time() < deadline:
+            done = [r or gsm_lib.gsm_poll(m.ctx, t) for r, t in zip(done, tickets)]
+        gsm_lib.gsm_server_stop(m.ctx)
+        status = {r["status"] for r in done}
+        # (requests admitted one by one need no third tile)
+        assert status <= ({gsm_lib.GSM_ERR_TIMEOUT} if where != "list"
+                          else {gsm_lib.GSM_ERR_TIMEOUT, gsm_lib.GSM_OK})
+        m.close()
 
 
 def test_invalid_spin_limit(gsm_lib, cuda):
