@@ -1,6 +1,8 @@
 """The batched form (gsm_run_batch): every count equals the single-query
 path's and the oracle's, whatever the batch mix, launch configuration or
 workspace size."""
+import math
+
 import numpy as np
 import pytest
 
@@ -193,4 +195,55 @@ def test_batched_workload_full_size(gsm_lib, cuda):
     for q, r in zip(gold["queries"], rows):
         got = np.ascontiguousarray(r.cpu().numpy(), dtype="<i4").reshape(-1)
         assert hashlib.sha256(got.tobytes()).hexdigest() == q["rows_sha256"]
+    m.close()
+
+
+def test_batched_counts_multiply_leaves_out(gsm_lib, cuda):
+    """Leaves, alike and different, restricted and not, of one and several
+    parents, counted in one batch; and sums near 64 bits."""
+    shapes = {
+        "edge": (2, [(0, 1)]),
+        "path3": (3, [(0, 1), (1, 2)]),
+        "path5": (5, [(0, 1), (1, 2), (2, 3), (3, 4)]),
+        "star5": (6, [(0, 1), (0, 2), (0, 3), (0, 4), (0, 5)]),
+        "bull": (5, [(0, 1), (1, 2), (0, 2), (0, 3), (1, 4)]),
+        "triangle_two_tails": (5, [(0, 1), (1, 2), (0, 2), (2, 3), (2, 4)]),
+        "caterpillar": (7, [(0, 1), (1, 2), (0, 3), (1, 4), (1, 5), (2, 6)]),
+    }
+    n, rp, col = I.erdos_renyi(90, 500, seed=58)
+    m = gsm_lib.Matcher(device=0)
+    for labels in (1, 2, 3):
+        lab = np.arange(n, dtype=np.int32) % labels
+        g = I.make_graph(n, rp, col, lab)
+        m.load_graph(g.row_ptr, g.col, g.labels)
+        Qs, want = [], []
+        for k, edges in shapes.values():
+            q = I.query_from_edges(k, edges, np.arange(k) % labels)
+            for ranges in [{}] + [{u: (11, 64)} for u in range(k)] + \
+                    [{u: (5, 60 + 3 * u) for u in range(k)}]:
+                c = oracle.match(g, q, enumerate=False, root_range=ranges.get(0, (0, n)),
+                                 ranges={u: r for u, r in ranges.items() if u})[0]
+                Q = m.query(q.k, q.edges, q.labels)
+                for u, r in ranges.items():
+                    Q.restrict(u, *r)
+                Qs.append(Q)
+                want.append(c)
+        assert m.run_batch(Qs) == want
+        assert [m.count(Q) for Q in Qs] == want
+    # hubs of 4,000 leaves: each hub's number fits in 64 bits, and their sum
+    d, hubs = 4000, 40
+    g = I.graph_from_edges(hubs * (d + 1), [((d + 1) * h, (d + 1) * h + v) for h in range(hubs)
+                                            for v in range(1, d + 1)])
+    m.load_graph(g.row_ptr, g.col, g.labels)
+
+    def star(x):
+        return m.query(x + 1, [(0, j + 1) for j in range(x)])
+
+    assert m.run_batch([star(4), star(2)]) == [hubs * math.perm(d, 4), hubs * math.perm(d, 2)]
+    assert m.batch_stats()["overflowed"] == 0
+    assert math.perm(d, 5) < 2 ** 64 < hubs * math.perm(d, 5)
+    with pytest.raises(gsm_lib.GsmError) as e:
+        m.run_batch([star(5), star(4)])
+    assert e.value.status == gsm_lib.GSM_ERR_OVERFLOW
+    assert int(e.value.counts[1]) == hubs * math.perm(d, 4)
     m.close()
