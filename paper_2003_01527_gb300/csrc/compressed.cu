@@ -53,8 +53,8 @@ __global__ void k_cpivot(GraphDev g, LevelDesc d, CFrontier f, int32_t i, int64_
 
 // Tiles, candidate order and survivor order as k_extend_fused; the row of a
 // candidate is decoded once per thread and row change.
-template <int kMode>
-__global__ void __launch_bounds__(1024) k_cextend(
+template <int kMode, int kMaxThreads>
+__global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_cextend(
     GraphDev g, LevelDesc d, CFrontier f, int32_t i, const int32_t *__restrict__ pstart,
     const uint8_t *__restrict__ pslot, const int64_t *__restrict__ woff,
     const int32_t *__restrict__ tile_row, int64_t wa, int32_t W, int32_t tiles,
@@ -167,24 +167,21 @@ void launch_cextend(const GraphDev &g, const LevelDesc &d, const CFrontier &f, i
   // the staged work offsets, later the survivor pairs (2 ints per item)
   const size_t smem = (size_t)((int64_t)block * kItemsPerThread * 2 + 1) * sizeof(int32_t);
   const int32_t W = (int32_t)(wb - wa), T = (int32_t)tiles;
-  switch (sink.mode) {
-    case kCSinkPairs:
-      k_cextend<kCSinkPairs><<<(unsigned)tiles, block, smem, s>>>(
-          g, d, f, i, pstart, pslot, woff, tile_row, wa, W, T, lookback, sink, spin_limit);
-      break;
-    case kCSinkRows:
-      k_cextend<kCSinkRows><<<(unsigned)tiles, block, smem, s>>>(
-          g, d, f, i, pstart, pslot, woff, tile_row, wa, W, T, lookback, sink, spin_limit);
-      break;
-    case kCSinkKeys:
-      k_cextend<kCSinkKeys><<<(unsigned)tiles, block, smem, s>>>(
-          g, d, f, i, pstart, pslot, woff, tile_row, wa, W, T, lookback, sink, spin_limit);
-      break;
-    default:
-      k_cextend<kCSinkCount><<<(unsigned)tiles, block, smem, s>>>(
-          g, d, f, i, pstart, pslot, woff, tile_row, wa, W, T, lookback, sink, spin_limit);
-      break;
-  }
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)tiles, block, smem, s>>>(g, d, f, i, pstart, pslot, woff, tile_row, wa, W,
+                                                T, lookback, sink, spin_limit);
+  };
+  auto by_mode = [&](auto threads) {
+    constexpr int kMax = decltype(threads)::value;
+    switch (sink.mode) {
+      case kCSinkPairs: return go(k_cextend<kCSinkPairs, kMax>);
+      case kCSinkRows: return go(k_cextend<kCSinkRows, kMax>);
+      case kCSinkKeys: return go(k_cextend<kCSinkKeys, kMax>);
+      default: return go(k_cextend<kCSinkCount, kMax>);
+    }
+  };
+  block <= 256 ? by_mode(std::integral_constant<int, 256>{})
+               : by_mode(std::integral_constant<int, 1024>{});
 }
 
 }  // namespace gsm
