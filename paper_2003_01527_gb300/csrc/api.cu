@@ -1919,7 +1919,10 @@ void run_query_once(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *o
     std::memcpy(w, ctx->h_stage, sizeof(w));
     // (without leaves word 0 is the sum itself)
     unsigned __int128 sum = (unsigned __int128)w[0] + ((unsigned __int128)w[1] << 32);
-    const bool big = w[2] || sum > ~(unsigned __int128)0 / core_aut;
+    double approx;
+    std::memcpy(&approx, &w[kCountApprox], sizeof(approx));
+    const bool big = w[2] || sum > ~(unsigned __int128)0 / core_aut ||
+                     approx - (double)(uint64_t)sum >= 9223372036854775808.0;
     sum = sum * core_aut / distinct_of;
     if (big || sum >> 64) FAIL(GSM_ERR_OVERFLOW, "the count exceeds 2^64 - 1");
     total = (uint64_t)sum;

@@ -322,11 +322,18 @@ struct LeafDesc {
   LeafGroup grp[kMaxK];
 };
 // Where a count goes: words [0] += the low and [1] += the high 32 bits of each
-// embedding's number, [2] != 0 if one embedding's number exceeds 64 bits or one
-// of the two sums wrapped (it can with more than 2^32 embeddings, and the count
-// is then past 64 bits), [3 + l] += the number of partial
-// embeddings with the core and l leaves placed (l < nleaves, modulo 2^64).
-constexpr int32_t kCountWords = 3 + kMaxK;
+// embedding's number, [2] != 0 if one embedding's number exceeds 64 bits,
+// [3 + l] += the number of partial embeddings with the core and l leaves placed
+// (l < nleaves), all modulo 2^64.  The sums wrap with more than 2^32 embeddings
+// of large numbers, so [kCountApprox] += the numbers as doubles: the count is
+// past 64 bits when that is half of 2^64 or more above what words 0 and 1 say.
+// Warps whose numbers add up to less than kCountSmall leave it alone (2^43 of
+// them would be needed to matter), which spares counts of few leaf images an
+// atomic; adds that return the old word, to see it wrap, cost a count of
+// 5-cliques with a tail 14 % (2.57 -> 2.93 ms).
+constexpr int32_t kCountApprox = 3 + kMaxK;
+constexpr double kCountSmall = 1048576.0;
+constexpr int32_t kCountWords = 4 + kMaxK;
 
 // Adds up the leaf numbers of rows [0, rows) of F (core rows of width w).
 void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,

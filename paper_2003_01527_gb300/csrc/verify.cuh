@@ -222,15 +222,16 @@ struct LeafSums {
   __device__ __forceinline__ void flush(const LeafDesc &leaf, unsigned long long *total) {
     constexpr unsigned kAll = 0xffffffffu;
     const bool first = (threadIdx.x & 31) == 0;
-    // (true: the word wrapped; a warp's own sums of fewer than 2^31 halves of
-    // 32 bits do not)
     auto sum = [&](unsigned long long v, unsigned long long *to) {
 #pragma unroll
       for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kAll, v, o);
-      return first && v && atomicAdd(to, v) + v < v;
+      if (first && v) atomicAdd(to, v);
+      return v;
     };
-    const bool wrapped = sum(lo, total) | sum(hi, total + 1);
-    if (__any_sync(kAll, over || wrapped) && first) atomicOr(total + 2, 1ull);
+    // (a warp's own sums of fewer than 2^31 halves of 32 bits do not wrap)
+    const double v = (double)sum(lo, total) + 4294967296.0 * (double)sum(hi, total + 1);
+    if (first && v >= kCountSmall) atomicAdd((double *)(total + kCountApprox), v);
+    if (__any_sync(kAll, over) && first) atomicOr(total + 2, 1ull);
 #pragma unroll
     for (int l = 0; l < kLeaves; ++l)
       if (l < leaf.nleaves) sum(part[l], total + 3 + l);
