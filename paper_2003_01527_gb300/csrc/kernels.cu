@@ -660,9 +660,16 @@ __global__ void k_tile_rows(const int64_t *__restrict__ woff, int64_t ra, int64_
 // latency with warps: eight CTAs of 256 threads an SM (32 registers).  At 34
 // registers, six CTAs, the distinct 4-cliques of R-MAT 16 took 11.8 instead
 // of 9.8 ms.
+// The forms for every shape likewise, although they spill at eight: 5-cliques of
+// R-MAT 15 with three labels 7.64 ms with eight, 8.4 with six, 9.5 with five; a
+// 5-clique with a tail, counted by its leaf, 2.30 with six, 2.49 with five.
+constexpr int count_ctas(int leaves, int check) {  // at least so many an SM
+  if (check <= kCheckWide) return leaves ? 1 : 2;
+  if (check == kCheckAnyFew) return leaves ? 5 : 6;
+  return check > kCheckGroup ? 4 : leaves ? 6 : 8;
+}
 template <bool kMasks, int kLeaves, int kCheck>
-__global__ void __launch_bounds__(kCheck ? 256 : 1024,
-                                  kCheck > kCheckGroup ? 4 : !kCheck ? 1 : kLeaves ? 6 : 8)
+__global__ void __launch_bounds__(kCheck <= kCheckWide ? 1024 : 256, count_ctas(kLeaves, kCheck))
     k_extend_count(
     GraphDev g, LevelDesc d, const int32_t *__restrict__ F, int32_t ld,
     const int32_t *__restrict__ pstart, const uint8_t *__restrict__ pslot,
@@ -684,7 +691,8 @@ __global__ void __launch_bounds__(kCheck ? 256 : 1024,
   uint32_t bits = 0;
   if (xb < x1) {
     int32_t rj[kItemsPerThread], wj[kItemsPerThread];
-    bits = check_group<kCheck>(g, d, F, ld, t, s_woff, woff, wa, pstart, pslot, xb, x1, rj, wj);
+    bits = check_group<kCheck, false, 1>(g, d, F, ld, t, s_woff, woff, wa, pstart, pslot, xb, x1,
+                                         rj, wj);
     if constexpr (kLeaves > 0) {
 #pragma unroll
       for (int j = 0; j < kItemsPerThread; ++j)
@@ -1686,8 +1694,11 @@ void launch_tile_rows(const int64_t *woff, int64_t ra, int64_t rb, int64_t wa, i
 // rows, for CTAs of up to 256 threads (the default; the other instances are
 // bounded to it).
 static int check_form(const LevelDesc &d, int32_t block, int64_t W, int64_t rows) {
-  if (block > 256 || d.nb > kMaxRowCheck || d.ninj > 2 || d.la || d.count_probes) return kCheckAny;
-  return d.nb >= 2 && W <= kFewCandidates * rows ? kCheckGroup + d.nb : kCheckRow + d.nb;
+  const bool few = d.nb >= 2 && W <= kFewCandidates * rows;
+  if (block > 256) return few ? kCheckWideFew : kCheckWide;
+  if (d.nb > kMaxRowCheck || d.ninj > 2 || d.la || d.count_probes)
+    return few ? kCheckAnyFew : kCheckAny;
+  return few ? kCheckGroup + d.nb : kCheckRow + d.nb;
 }
 
 void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,
@@ -1707,12 +1718,20 @@ void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F
   auto by_form = [&](auto masked, auto leaves) {
     constexpr bool kM = decltype(masked)::value;
     constexpr int kL = decltype(leaves)::value;
+    if constexpr (kL <= 1) {  // (more leaves: any shape's form)
+      switch (form) {
+        case kCheckRow + 1: return go(k_extend_count<kM, kL, kCheckRow + 1>);
+        case kCheckRow + 2: return go(k_extend_count<kM, kL, kCheckRow + 2>);
+        case kCheckRow + 3: return go(k_extend_count<kM, kL, kCheckRow + 3>);
+        case kCheckGroup + 2: return go(k_extend_count<kM, kL, kCheckGroup + 2>);
+        case kCheckGroup + 3: return go(k_extend_count<kM, kL, kCheckGroup + 3>);
+        default: break;
+      }
+    }
     switch (form) {
-      case kCheckRow + 1: return go(k_extend_count<kM, kL, kCheckRow + 1>);
-      case kCheckRow + 2: return go(k_extend_count<kM, kL, kCheckRow + 2>);
-      case kCheckRow + 3: return go(k_extend_count<kM, kL, kCheckRow + 3>);
-      case kCheckGroup + 2: return go(k_extend_count<kM, kL, kCheckGroup + 2>);
-      case kCheckGroup + 3: return go(k_extend_count<kM, kL, kCheckGroup + 3>);
+      case kCheckWide: return go(k_extend_count<kM, kL, kCheckWide>);
+      case kCheckWideFew: return go(k_extend_count<kM, kL, kCheckWideFew>);
+      case kCheckAnyFew: return go(k_extend_count<kM, kL, kCheckAnyFew>);
       default: return go(k_extend_count<kM, kL, kCheckAny>);
     }
   };
@@ -1724,9 +1743,9 @@ void launch_extend_count(const GraphDev &g, const LevelDesc &d, const int32_t *F
   else if (leaf->nleaves == 1)
     by_form(std::false_type{}, integral_constant<int, 1>{});
   else if (leaf->nleaves <= 3)
-    go(k_extend_count<false, 3, kCheckAny>);
+    by_form(std::false_type{}, integral_constant<int, 3>{});
   else
-    go(k_extend_count<false, kMaxK, kCheckAny>);
+    by_form(std::false_type{}, integral_constant<int, kMaxK>{});
 }
 
 void launch_leaf_rows(const GraphDev &g, const LeafDesc &leaf, const int32_t *F, int64_t ld,
@@ -1846,7 +1865,8 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
   using std::false_type;
   using std::integral_constant;
   using std::true_type;
-  switch (check_form(d, block, W, rows)) {
+  const int form = check_form(d, block, W, rows);
+  switch (form) {
     case kCheckRow + 1: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 1>{});
     case kCheckRow + 2: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 2>{});
     case kCheckRow + 3: return go(true_type{}, false_type{}, integral_constant<int, kCheckRow + 3>{});
@@ -1856,15 +1876,18 @@ void launch_extend_fused(const GraphDev &g, const LevelDesc &d, const int32_t *F
       return go(true_type{}, false_type{}, integral_constant<int, kCheckGroup + 3>{});
     default: break;
   }
-  const integral_constant<int, kCheckAny> any;
-  if (block <= 256 && !d.count_probes)
-    go(true_type{}, false_type{}, any);
-  else if (block <= 256)
-    go(true_type{}, true_type{}, any);
-  else if (!d.count_probes)
-    go(false_type{}, false_type{}, any);
-  else
-    go(false_type{}, true_type{}, any);
+  auto by_block = [&](auto check) {  // (the wide forms differ in the count kernel only)
+    if (block <= 256 && !d.count_probes)
+      go(true_type{}, false_type{}, check);
+    else if (block <= 256)
+      go(true_type{}, true_type{}, check);
+    else if (!d.count_probes)
+      go(false_type{}, false_type{}, check);
+    else
+      go(false_type{}, true_type{}, check);
+  };
+  form == kCheckAny || form == kCheckWide ? by_block(integral_constant<int, kCheckAny>{})
+                                          : by_block(integral_constant<int, kCheckAnyFew>{});
 }
 
 void launch_leaf_expand(const GraphDev &g, const LevelDesc &d, const int32_t *F, int64_t ld,

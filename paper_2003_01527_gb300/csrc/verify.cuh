@@ -66,15 +66,16 @@ __device__ __forceinline__ int32_t item_row(const TileRows &t, const int32_t *s_
 
 // From row r0 + rr, whose candidates end at re <= x, to the row of item x, and
 // where its candidates start and end.  Mostly the next; rows without work are
-// stepped over four at a time, longer runs by a search: bounds cut off a row's
+// stepped over (kSteps rows), longer runs by a search: bounds cut off a row's
 // segment leave runs of millions (counting the 5-cycles of two low roots of
 // R-MAT 20, whose symmetry orders two vertices, one thread stepped through
 // most of 6.5 M rows: 237 ms, 0.56 with the search).
+template <int kSteps = 4>
 __device__ __forceinline__ void next_row(const TileRows &t, const int32_t *s_woff,
                                          const int64_t *__restrict__ woff, int64_t wa, int32_t x,
                                          int32_t *rr, int32_t *rs, int32_t *re) {
   auto offset = [&](int32_t j) { return t.staged ? s_woff[j] : (int32_t)(woff[t.r0 + j] - wa); };
-  for (int32_t step = 0; step < 4; ++step) {
+  for (int32_t step = 0; step < kSteps; ++step) {
     ++*rr;
     *rs = *re;
     *re = offset(*rr + 1);
@@ -346,7 +347,10 @@ struct RowCheck {
 
 // How a level's launch checks its candidates.
 //   kCheckAny      every shape: check_candidate and the look-ahead, one
-//                  candidate after the other, the row read again for each
+//                  candidate after the other, the row read again for each;
+//                  kCheckAnyFew: also from the candidate's side
+//                  (row_contains_few), with the candidates loaded together
+//   kCheckWide, kCheckWideFew: the same two in CTAs of more than 256 threads
 //   kCheckRow + n  n = 1..3 mapped neighbours, at most two injectivity tests,
 //                  no look-ahead: RowCheck
 //   kCheckGroup+n  the same shapes, n = 2, 3: the loads of a thread's four
@@ -360,8 +364,12 @@ struct RowCheck {
 // (the listing 1,981 -> 1,834 -> 1,721 us).  With many, the row's adjacency stays in L1 and the grouped form's
 // registers cost more warps than it gains: ordered triangles of R-MAT 20 (146
 // a row) 24.1 against 19.9 ms, 4-cliques of R-MAT 16 12.5 against 9.8 ms.
-// Hence grouped up to kFewCandidates candidates a row on average.
-constexpr int kCheckAny = 0, kCheckRow = 0, kCheckGroup = 3;
+// Hence grouped up to kFewCandidates candidates a row on average.  The forms for
+// every shape go by the same line: one candidate after the other with eight CTAs
+// an SM counts the 6-cliques of R-MAT 15 with three labels in 44.3 ms, four
+// loaded together and looked at from both sides, at four CTAs, in 57.4.
+constexpr int kCheckWideFew = -3, kCheckWide = -2, kCheckAnyFew = -1, kCheckAny = 0, kCheckRow = 0,
+              kCheckGroup = 3;
 constexpr int kMaxRowCheck = 3;
 
 // Which of the `alive` pairs are edges: w[j] (label lab_of(j)) in the row of
@@ -481,7 +489,8 @@ __device__ __forceinline__ uint32_t group_contains(const GraphDev &g,
 // The candidates x = xb .. xb + 3 of one thread, below x1: returns a bit for
 // each that passes the level's checks; rj, wj: their rows and vertices.
 // kProbes (kCheckAny only): adds the checks' probe bytes to *probe_bytes.
-template <int kCheck, bool kProbes = false>
+// kSteps (kCheckAny, kCheckWide): next_row's.
+template <int kCheck, bool kProbes = false, int kSteps = 4>
 __device__ __forceinline__ uint32_t check_group(
     const GraphDev &g, const LevelDesc &d, const int32_t *__restrict__ F, int32_t ld,
     const TileRows &t, const int32_t *s_woff, const int64_t *__restrict__ woff, int64_t wa,
@@ -520,6 +529,34 @@ __device__ __forceinline__ uint32_t check_group(
     }
     return bits;
   }
+  if constexpr (kCheck == kCheckAny || kCheck == kCheckWide) {  // (rj, wj: as above)
+    uint32_t bits = 0;
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const int32_t x = xb + j;
+      if (x >= x1) break;
+      if (x >= re) {
+        next_row<kSteps>(t, s_woff, woff, wa, x, &rr, &rs, &re);
+        r = t.r0 + rr;
+        pst = pstart[r];
+        slot = pslot[r];
+      }
+      if (!GSM_IN_BOUNDS(g.dbg, pst + (x - rs) >= 0 && pst + (x - rs) < g.nnz, kDbgCandidate) ||
+          !GSM_IN_BOUNDS(g.dbg, r >= 0 && r < ld, kDbgRow))
+        continue;
+      const int32_t w = __ldg(g.lcol + pst + (x - rs));
+      rj[j] = r;
+      wj[j] = w;
+      const ColumnRow row{F, ld, r};
+      bool ok;
+      if constexpr (kProbes)
+        ok = check_candidate_probes(g, d, row, w, slot, false, probe_bytes);
+      else
+        ok = check_candidate(g, d, row, w, slot, false);
+      if (ok && (!d.la || lookahead_ok(g, d, row, w))) bits |= 1u << j;
+    }
+    return bits;
+  }
   int32_t at[kN], sj[kN];
   uint32_t alive = 0, few = 0;
 #pragma unroll
@@ -542,7 +579,7 @@ __device__ __forceinline__ uint32_t check_group(
     at[j] = pst + (x - rs);
   }
   if (g.hub_lo) few = 0;  // bitmaps that do not cover the mapped neighbours
-  if constexpr (kCheck == kCheckAny) {
+  if constexpr (kCheck < kCheckAny) {
 #pragma unroll
     for (int j = 0; j < kN; ++j) wj[j] = (alive >> j) & 1u ? __ldg(g.lcol + at[j]) : 0;
 #pragma unroll
