@@ -53,8 +53,14 @@ __global__ void k_cpivot(GraphDev g, LevelDesc d, CFrontier f, int32_t i, int64_
 
 // Tiles, candidate order and survivor order as k_extend_fused; the row of a
 // candidate is decoded once per thread and row change.
+// Latency-bound.  CTAs an SM: six write rows without spilling (40 registers; the
+// 20 slices of R-MAT 16 5.78 ms, with five 6.05, with four 6.52); counts take
+// eight although they spill (6-cliques of R-MAT 15 with three labels 49.4 ms,
+// with six 55.2; cliques of five with a tail 63.7 and 73.4).
 template <int kMode, int kMaxThreads>
-__global__ void __launch_bounds__(kMaxThreads, kMaxThreads == 256 ? 6 : 1) k_cextend(
+__global__ void __launch_bounds__(kMaxThreads, kMaxThreads != 256        ? 1
+                                               : kMode == kCSinkCount ? 8
+                                                                      : 6) k_cextend(
     GraphDev g, LevelDesc d, CFrontier f, int32_t i, const int32_t *__restrict__ pstart,
     const uint8_t *__restrict__ pslot, const int64_t *__restrict__ woff,
     const int32_t *__restrict__ tile_row, int64_t wa, int32_t W, int32_t tiles,
