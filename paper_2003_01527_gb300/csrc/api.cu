@@ -1948,7 +1948,8 @@ void run_query_once(gsm_ctx *ctx, const gsm_query *q, bool enumerate, int32_t *o
     ensure_buf(ctx, &ctx->sort_keys, &ctx->sort_keys_cap, key_bytes, false, 0);
     // rows of an odd width leave the sort in 4-byte stores, and a second buffer
     // of them takes longer than a copy when it is large (7 columns, 543 MB: 565
-    // against 170 us; 3 columns, 43 MB: 11 against 26)
+    // against 170 us; 5 columns, 329 MB: 160 against 108); a small copy is a
+    // launch and little else
     const bool twice = q->k % 2 == 0 || bytes <= kTwiceBytes;
     placed = wide && total <= cap_rows && (!keep_rows || twice);
     const bool only_out = placed && !keep_rows;
@@ -2188,8 +2189,7 @@ void make_rank_graph(gsm_ctx *ctx) {
                     (uint64_t *)(b + o_keys), (int32_t *)(b + o_pairs), b + o_s, ctx->d_flags,
                     r.rp, r.col, r.up, ctx->stream);
     CU(cudaGetLastError());
-    GraphDev g = rank_dev(ctx);
-    g.hub_words = words;
+    const GraphDev g = rank_dev(ctx);
     launch_threshold_bits(g, r.thr, r.thr + (size_t)words * kThrLevels, ctx->stream);
     // hubs: the highest vertices, from a multiple of 128 on (not from 0, which
     // stands for a graph in its own numbering); their bitmaps' lengths are

@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(256) k_threshold_bits(GraphDev g, uint32_t *__
                                                         uint32_t *__restrict__ lab_bits) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < g.hub_words;
-       w += warps) {
+  const int64_t words = ((int64_t)g.n + 31) / 32;
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < words; w += warps) {
     const int64_t v = w * 32 + lane;
     const bool valid = v < g.n;
     const int32_t lv = valid ? g.lab[v] : -1;
@@ -143,10 +143,10 @@ __global__ void __launch_bounds__(256) k_threshold_bits(GraphDev g, uint32_t *__
 #pragma unroll
       for (int t = 0; t < kThrLevels; ++t) {
         const uint32_t word = __ballot_sync(kFull, c > t);
-        if (lane == t) thr[((int64_t)l * kThrLevels + t) * g.hub_words + w] = word;
+        if (lane == t) thr[((int64_t)l * kThrLevels + t) * words + w] = word;
       }
       const uint32_t word = __ballot_sync(kFull, lv == l);
-      if (lane == 0) lab_bits[(int64_t)l * g.hub_words + w] = word;
+      if (lane == 0) lab_bits[(int64_t)l * words + w] = word;
     }
   }
 }
@@ -1584,8 +1584,7 @@ void launch_hub_segments(const GraphDev &g, const int32_t *hubs, int32_t H, int3
 
 void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits, cudaStream_t s) {
   if (g.n <= 0) return;
-  k_threshold_bits<<<grid_for((int64_t)g.hub_words * 32, 256, 152 * 16), 256, 0, s>>>(g, thr,
-                                                                                      lab_bits);
+  k_threshold_bits<<<grid_for(g.n, 256, 152 * 16), 256, 0, s>>>(g, thr, lab_bits);
 }
 
 bool filter_stages(const GraphDev &g) { return g.thr && g.n > 0; }

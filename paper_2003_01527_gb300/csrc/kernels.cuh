@@ -98,8 +98,8 @@ struct GraphDev {
   const uint8_t *nlc;
   int32_t nlc_stride;
   // the same as bitmaps over the vertices (null: none): bit v of
-  // thr[(l * kThrLevels + c - 1) * hub_words ..] is set iff v has at least c
-  // neighbours with label l, bit v of lab_bits[l * hub_words ..] iff v's label
+  // thr[(l * kThrLevels + c - 1) * ceil(n/32) ..] is set iff v has at least c
+  // neighbours with label l, bit v of lab_bits[l * ceil(n/32) ..] iff v's label
   // is l.  One label: its neighbours are all, so thr holds degrees.
   const uint32_t *thr, *lab_bits;
   // > 0: the graph with its vertices renumbered by degree (RankGraph): the hubs
@@ -184,7 +184,7 @@ void launch_renumber(const GraphDev &g, const int32_t *order, int32_t nlong, int
                      cudaStream_t s);
 
 // The threshold and label bitmaps of GraphDev (thr: num_labels * kThrLevels,
-// lab_bits: num_labels bitmaps of hub_words words), from the neighbour label
+// lab_bits: num_labels bitmaps of ceil(n/32) words), from the neighbour label
 // counts, or with one label from the degrees.
 constexpr int32_t kThrLevels = 4;
 void launch_threshold_bits(const GraphDev &g, uint32_t *thr, uint32_t *lab_bits, cudaStream_t s);
