@@ -215,7 +215,12 @@ void gsm_query_destroy(gsm_query *q);
  * Errors: GSM_ERR_INVALID_ARG (u out of range, lo > hi, negative bound). */
 gsm_status gsm_query_restrict(gsm_query *q, int32_t u, int32_t lo, int32_t hi);
 
-/* Counts the embeddings of q in the loaded graph.  Query vertices of degree 1
+/* (gsm_count, gsm_enumerate and the other synchronous calls poll mapped memory
+ * for their kernels' small results, for up to about a millisecond each before
+ * they block on the stream: the calling thread, and every listing worker, is
+ * busy while its call runs.)
+ *
+ * Counts the embeddings of q in the loaded graph.  Query vertices of degree 1
  * are counted in closed form where that is possible, so a count may exceed
  * 64 bits (GSM_ERR_OVERFLOW).
  * Errors: GSM_ERR_NO_GRAPH, GSM_ERR_BUDGET, GSM_ERR_OOM, GSM_ERR_OVERFLOW,
@@ -500,7 +505,9 @@ typedef struct gsm_run_stats {
   int32_t k;
   int32_t order[16];
   uint64_t cand_size[16];    /* |C(u)| per query vertex id */
-  uint64_t frontier[16];     /* partial embeddings of i vertices (i = 1..k; [0] unused) */
+  uint64_t frontier[16];     /* partial embeddings of i vertices (i = 1..k; [0] unused).  Counts
+                                keep one of each set that a symmetry of the query maps to one
+                                another: those kept, for i < k */
   uint64_t candidates[16];   /* candidates checked while extending level i -> i+1 (0 for
                                 levels counted in closed form) */
   uint64_t chunks;           /* extend sub-chunks launched */

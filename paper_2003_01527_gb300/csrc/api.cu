@@ -1636,7 +1636,12 @@ void run_filter(gsm_ctx *ctx, const gsm_query *q, const int32_t *dense, uint64_t
 constexpr size_t kTwiceBytes = size_t(32) << 20;
 
 // Graphs below this sum of squared degrees (the 2-edge paths, what a clique
-// count starts from) count in about the time that renumbering takes.
+// count starts from) are not renumbered.  The line is a compromise between a
+// first count, which renumbers (0.3 ms for R-MAT 15), and the next ones: R-MAT 15
+// (1.65 times the line) counts triangles in 490 us first and 149 then, plain in
+// 227 and 204; 4-cliques in 1.55 and 1.12 ms, plain in 3.14 and 2.99.  R-MAT 14
+// (0.58 times) 321 and 119 against 156 and 145; 0.79 and 0.53 against 1.26 and
+// 1.08.  R-MAT 18 (35 times) triangles 1.33 and 0.66 ms against 2.24 and 2.16.
 constexpr double kRankSquares = 1 << 28;
 
 GraphDev rank_dev(const gsm_ctx *ctx);
