@@ -844,7 +844,8 @@ constexpr size_t kFusedStageMax = 96 * 1024;   // ... with the tile's result row
 
 // kMaxThreads = 256: up to 256 threads per CTA, registers capped so that six
 // CTAs fit on an SM; 1024: any block size.
-// kCheck: the form of check_group (kCheckAny with kProbes).
+// kCheck: the form of check_group (kCheckAny or kCheckAnyFew with kProbes and in
+// CTAs of more than 256 threads).
 template <int kMode, int kMaxThreads, bool kProbes, int kCheck>
 __global__ void __launch_bounds__(kMaxThreads,
                                   kMaxThreads == 256 ? (kCheck > kCheckGroup ? 4 : 6) : 1)
@@ -1690,8 +1691,8 @@ void launch_tile_rows(const int64_t *woff, int64_t ra, int64_t rb, int64_t wa, i
 }
 
 // The form of check_group for a level's launch over W candidates of `rows`
-// rows, for CTAs of up to 256 threads (the default; the other instances are
-// bounded to it).
+// rows (all but the wide ones are bounded to CTAs of up to 256 threads, the
+// default).
 static int check_form(const LevelDesc &d, int32_t block, int64_t W, int64_t rows) {
   const bool few = d.nb >= 2 && W <= kFewCandidates * rows;
   if (block > 256) return few ? kCheckWideFew : kCheckWide;

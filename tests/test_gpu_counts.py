@@ -235,3 +235,37 @@ def test_long_runs_of_rows_without_candidates(gsm_lib, cuda, opts):
             if not opts:
                 assert m.run_batch([Q, Q]) == [want, want]
     m.close()
+
+
+@pytest.mark.parametrize("opts", [{}, {"lookahead": 1}, {"block_size": 128}, {"block_size": 512},
+                                  {"block_size": 1024, "lookahead": 2}, {"two_pass": True},
+                                  {"compressed": True}, {"count_probes": True},
+                                  {"hub_bitmap_bytes": -1}])
+def test_checks_of_many_neighbours(gsm_lib, cuda, opts):
+    """More than three mapped neighbours, with many candidates a row (a dense
+    graph) and few (a sparse one with cliques in it), counted and listed, with
+    and without a leaf."""
+    rng = np.random.default_rng(23)
+    cliques = [(int(a), int(b)) for _ in range(30)
+               for c in [np.sort(rng.choice(600, 7, replace=False))]
+               for i, a in enumerate(c) for b in c[i + 1:]]
+    sparse = sorted(set(cliques + [(u, u + 1) for u in range(599)]))
+    n, rp, col = I.erdos_renyi(70, 1500, seed=29)
+    k5 = [(a, b) for a in range(5) for b in range(a + 1, 5)]
+    wheel = [(0, i) for i in range(1, 6)] + [(1, 2), (2, 3), (3, 4), (4, 5), (1, 5)]
+    shapes = [(5, k5), (6, wheel), (6, k5 + [(4, 5)]),
+              (6, [(a, b) for a in range(6) for b in range(a + 1, 6)])]
+    m = gsm_lib.Matcher(device=0, **opts)
+    for g in (I.make_graph(n, rp, col, np.arange(n, dtype=np.int32) % 3),
+              I.graph_from_edges(600, sparse, np.arange(600, dtype=np.int32) % 2)):
+        m.load_graph(g.row_ptr, g.col, g.labels)
+        for k, edges in shapes:
+            q = I.query_from_edges(k, edges, np.arange(k) % (int(g.labels.max()) + 1))
+            hi = 24 if g.n == n else g.n
+            want, rows, rc = oracle.match(g, q, root_range=(0, hi))
+            assert rc == oracle.OK and want > 0
+            Q = m.query(q.k, q.edges, q.labels).restrict(0, 0, hi)
+            assert m.count(Q) == want, (k, len(edges))
+            got, count = m.enumerate(Q)
+            assert count == want and np.array_equal(got, rows), (k, len(edges))
+    m.close()
